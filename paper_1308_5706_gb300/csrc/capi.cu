@@ -117,6 +117,7 @@ void kernels_prepare(bool fp64, bool pair) {
   }
   if (pair && !(done_pair & bit)) {
     ck(pair_prepare());
+    ck(contract_direct_prepare());
     done_pair |= bit;
   }
 }
@@ -262,6 +263,16 @@ struct Lists {
   std::vector<std::pair<int, std::pair<void*, int>>> tiles_w;
   void* tiles_phi = nullptr;
   int ntiles_phi = 0;
+  // direct FP32 contraction: per N the analysis and synthesis tasks of the
+  // wavelet scales; dir_phi (N = 1): those of the scaling parts, launched with
+  // the first group
+  struct DirGroup {
+    int N = 1, rt = 4;
+    void* task[2] = {nullptr, nullptr};  // analysis, synthesis
+    int n[2] = {0, 0};
+  };
+  std::vector<DirGroup> dir_w;
+  DirGroup dir_phi;
   static constexpr int NK = 16;  // chirp-z 0..3, direct alpha 4..5, single-FFT beta 6..7, segmented alpha 8..9,
                                  // MW-grid synthesis beta 10..12, half-length beta 13..15
   void* segs[NK] = {};
@@ -361,6 +372,7 @@ struct s2dw_plan_s {
   std::vector<unsigned char> desc_w_host, desc_phi_host;
   std::vector<TileTask> tiles_w_host, tiles_phi_host;  // FP64 plans
   std::vector<PairTask> ptasks_w_host, ptasks_phi_host;  // FP32 plans
+  bool direct_w = false, direct_phi = false;  // FP32: those tasks run the direct contraction (one tile each)
   int pair_shape = kPairShapePair;  // FP32: the contraction's CTA shape (a launch method; N > 5: one tile)
   Lists own;
   // stage timing (s2dw_profile): one set of events per call, up to kProfCalls
@@ -438,6 +450,23 @@ void evict_batches() {  // g_batch_mu held; called before an insertion
   }
 }
 
+// Gamma factors [k N + g], n_k = -(N-1) + 2k, gamma_g = pi g / N, eta = 1 (N
+// odd) or i: analysis conj(eta) i^{n_k} e^{i n_k gamma_g} (Eq. (28)), synthesis
+// eta (2 pi/N) i^{-n_k} e^{-i n_k gamma_g} (Eq. (39)).
+template <typename T>
+void gamma_factors(int N, cx<T>* ana, cx<T>* syn) {
+  const double pi = 3.14159265358979323846;
+  for (int k = 0; k < N; ++k)
+    for (int g = 0; g < N; ++g) {
+      const int n = -(N - 1) + 2 * k;
+      // n g pi / N + n pi/2 - (N even) pi/2 in units of pi/(2N), reduced exactly
+      const int u = (((2 * n * g + n * N - (N % 2 == 0 ? N : 0)) % (4 * N)) + 4 * N) % (4 * N);
+      const double c = std::cos(pi * u / (2 * N)), s = std::sin(pi * u / (2 * N)), sc = 2.0 * pi / N;
+      ana[k * N + g] = mkc<T>((T)c, (T)s);
+      syn[k * N + g] = mkc<T>((T)(c * sc), (T)(-s * sc));
+    }
+}
+
 template <typename T>
 void fill_desc(s2dw_plan_s* p, ContractDesc<T>& dw, ContractDesc<T>& dp, const T* delta) {
   std::memset(&dw, 0, sizeof(dw));
@@ -457,6 +486,8 @@ void fill_desc(s2dw_plan_s* p, ContractDesc<T>& dw, ContractDesc<T>& dp, const T
   dw.N = p->N;
   dw.nslot = 2;
   dw.eta_odd = (p->N % 2 == 0) ? 1 : 0;
+  gamma_factors<T>(p->N, dw.cga, dw.cgs);
+  gamma_factors<T>(1, dp.cga, dp.cgs);
   for (int j = 0; j < p->nscale; ++j) {
     dw.Lj[j] = p->Lj[j];
     dw.Y[j] = reinterpret_cast<cx<T>*>(p->Y[j]);
@@ -543,6 +574,75 @@ void build_pair_tasks(int Lband, int lend, bool two, int table_Lmax, std::vector
     }
   auto work = [two](const PairTask& t) { return (long long)(t.lend - t.lstart + 1) * (two && t.p != t.q ? 2 : 1); };
   std::stable_sort(out.begin(), out.end(), [&](const PairTask& a, const PairTask& b) { return work(a) > work(b); });
+}
+
+// Direct contraction tasks of one plan's wavelet scales or scaling part (d:
+// its descriptor, band Lband, last l lend): every tile, for the analysis once
+// per scale over the scale's l (its [lo, hi] from the l-segments), for the
+// synthesis once per l-segment.
+void build_direct_tasks(const ContractDesc<float>& d, int prob, int Lband, int lend, int table_Lmax,
+                        std::vector<DirTask>& ana, std::vector<DirTask>& syn) {
+  if (Lband <= 0 || lend < 0) return;
+  int lo[MAXS], hi[MAXS], nj = 0;
+  for (int j = 0; j < MAXS; ++j) lo[j] = hi[j] = -1;
+  for (int i = 0; i < d.nseg; ++i)
+    for (int s = 0; s < d.nslot; ++s) {
+      const int j = d.seg[i].j[s];
+      if (j < 0) continue;
+      if (lo[j] < 0) lo[j] = d.seg[i].lo;
+      hi[j] = d.seg[i].hi;
+      nj = std::max(nj, j + 1);
+    }
+  const int nb = (Lband + 31) / 32;
+  for (int q = 0; q < nb; ++q)
+    for (int p = 0; p <= q; ++p) {
+      const long long base = pair_run_base(p, q, table_Lmax);  // l = 32 q
+      for (int half = 0; half <= (p == q ? 0 : 1); ++half) {
+        auto add = [&](std::vector<DirTask>& v, int a, int b, int j, int j2, int slot) {
+          a = std::max(a, 32 * q);
+          b = std::min(b, lend);
+          if (a <= b) v.push_back(DirTask{prob, p, q, half, a, b, j, j2, slot, 0, base + 1024LL * (a - 32 * q)});
+        };
+        for (int j = 0; j < nj; ++j)
+          if (hi[j] >= 0) add(ana, lo[j], hi[j], j, -1, j % 2);
+        for (int i = 0; i < d.nseg; ++i) add(syn, d.seg[i].lo, d.seg[i].hi, d.seg[i].j[0], d.seg[i].j[1], 0);
+      }
+    }
+}
+
+// Analysis rows per thread and synthesis l ranges of a direct launch, from the
+// number of tasks over all its plans (neither enters the arithmetic).
+// Analysis: rt rows per thread, so 32 / (8 rt) CTAs of 8 warps per task (8 CTAs
+// of 4 warps at rt = 1): fewer rows per thread while the tasks alone would
+// leave SMs idle (a thread's R loads serve its rt rows).  Synthesis: pieces of
+// a multiple of 16 l, about four CTAs per SM over the launch.
+int direct_split(std::vector<DirTask>& ana, std::vector<DirTask>& syn, int sms) {
+  const long long n = (long long)ana.size();
+  long long total = 0;
+  for (const DirTask& t : syn) total += t.lend - t.lstart + 1;
+  const int ls = round_up((int)std::min<long long>(std::max<long long>((total + 4LL * sms - 1) / (4LL * sms), 1), 4096), 16);
+  std::vector<DirTask> cut;
+  for (const DirTask& t : syn)
+    for (int l = t.lstart; l <= t.lend; l += ls) {
+      DirTask u = t;
+      u.lstart = l;
+      u.lend = std::min(t.lend, l + ls - 1);
+      u.dbase = t.dbase + 1024LL * (l - t.lstart);
+      cut.push_back(u);
+    }
+  syn.swap(cut);
+  // longest first (a counting sort on the length)
+  for (std::vector<DirTask>* v : {&ana, &syn}) {
+    int maxlen = 0;
+    for (const DirTask& t : *v) maxlen = std::max(maxlen, t.lend - t.lstart);
+    std::vector<size_t> at(maxlen + 2, 0);
+    for (const DirTask& t : *v) ++at[maxlen - (t.lend - t.lstart) + 1];
+    for (int i = 0; i <= maxlen; ++i) at[i + 1] += at[i];
+    std::vector<DirTask> sorted(v->size());
+    for (const DirTask& t : *v) sorted[at[maxlen - (t.lend - t.lstart)]++] = t;
+    v->swap(sorted);
+  }
+  return n >= 2 * sms ? 4 : (n >= sms / 2 ? 2 : 1);
 }
 
 void sort_tiles(std::vector<TileTask>& t) {
@@ -714,6 +814,13 @@ Lists* build_lists(const std::vector<s2dw_plan_t>& plans) {
   std::vector<ContractDesc<T>> dw(nj), dp(nj);
   std::map<int, std::vector<Task>> tw_byN;
   std::vector<Task> tphi;
+  struct DirBuild {  // direct FP32 contraction: analysis and synthesis tasks
+    std::vector<DirTask> task[2];
+    int rt = 4;
+    size_t off[2] = {0, 0};
+  };
+  std::map<int, DirBuild> dir_byN;
+  DirBuild dir_phi;
   std::vector<CztSeg<T>> segs[Lists::NK];
   int start[Lists::NK] = {};
   Lists* ls = new Lists();
@@ -732,7 +839,13 @@ Lists* build_lists(const std::vector<s2dw_plan_t>& plans) {
       tps = &p->tiles_phi_host;
     }
     const int key = p->N | ((sizeof(T) == sizeof(float)) ? (p->pair_shape << kShapeShift) : 0);
-    for (Task t : *tws) {
+    if constexpr (sizeof(T) == sizeof(float)) {
+      if (p->direct_w)
+        build_direct_tasks(dw[i], i, p->L0, p->lend_w, p->tab->Lmax, dir_byN[p->N].task[0], dir_byN[p->N].task[1]);
+      if (p->direct_phi)
+        build_direct_tasks(dp[i], i, p->Lphi, p->lphi, p->tab->Lmax, dir_phi.task[0], dir_phi.task[1]);
+    }
+    for (Task t : *tws) {  // (empty where the direct contraction runs)
       t.prob = i;
       tw_byN[key].push_back(t);
     }
@@ -743,8 +856,10 @@ Lists* build_lists(const std::vector<s2dw_plan_t>& plans) {
     for (int k = 0; k < Lists::NK; ++k) build_segs<T>(p, i, k, segs[k], start[k]);
     ls->maxlogM = std::max(ls->maxlogM, p->logM);
     ls->Lmax = std::max(ls->Lmax, p->L);
-    ls->nbmax = std::max(ls->nbmax, (p->L + 31) / 32);
-    ls->Lrmax = std::max(ls->Lrmax, p->Lrf);
+    if (p->fP) {  // packed f: plans with a tile-pair contraction
+      ls->nbmax = std::max(ls->nbmax, (p->L + 31) / 32);
+      ls->Lrmax = std::max(ls->Lrmax, p->Lrf);
+    }
     if (p->mw) ls->odd = CZT_ODD_ROWS;
   }
   for (int k = CZT_BETA_ANA_DCT; k <= CZT_BETA_RS_DCT; ++k) {
@@ -784,6 +899,15 @@ Lists* build_lists(const std::vector<s2dw_plan_t>& plans) {
   };
   for (auto& kv : tw_byN) by_work(kv.second, kv.first);
   by_work(tphi, 1);
+  int sms = 152;
+  {
+    int dev = 0;
+    if (cudaGetDevice(&dev) == cudaSuccess) cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+  }
+  std::vector<DirBuild*> dirs;
+  for (auto& kv : dir_byN) dirs.push_back(&kv.second);
+  dirs.push_back(&dir_phi);  // always the last
+  for (DirBuild* b : dirs) b->rt = direct_split(b->task[0], b->task[1], sms);
   // one allocation for everything
   size_t off = 0;
   const size_t o_dw = off;
@@ -797,6 +921,11 @@ Lists* build_lists(const std::vector<s2dw_plan_t>& plans) {
   }
   const size_t o_tp = off;
   off = align256(off + tphi.size() * sizeof(Task));
+  for (DirBuild* b : dirs)
+    for (int d = 0; d < 2; ++d) {
+      b->off[d] = off;
+      off = align256(off + b->task[d].size() * sizeof(DirTask));
+    }
   size_t o_sg[Lists::NK];
   for (int k = 0; k < Lists::NK; ++k) {
     o_sg[k] = off;
@@ -811,6 +940,9 @@ Lists* build_lists(const std::vector<s2dw_plan_t>& plans) {
     ++q;
   }
   if (!tphi.empty()) std::memcpy(host.data() + o_tp, tphi.data(), tphi.size() * sizeof(Task));
+  for (DirBuild* b : dirs)
+    for (int d = 0; d < 2; ++d)
+      if (!b->task[d].empty()) std::memcpy(host.data() + b->off[d], b->task[d].data(), b->task[d].size() * sizeof(DirTask));
   for (int k = 0; k < Lists::NK; ++k)
     if (!segs[k].empty()) std::memcpy(host.data() + o_sg[k], segs[k].data(), segs[k].size() * sizeof(CztSeg<T>));
   try {
@@ -832,6 +964,18 @@ Lists* build_lists(const std::vector<s2dw_plan_t>& plans) {
   }
   ls->tiles_phi = base + o_tp;
   ls->ntiles_phi = (int)tphi.size();
+  auto dir_group = [&](int N, const DirBuild& b) {
+    Lists::DirGroup g;
+    g.N = N;
+    g.rt = b.rt;
+    for (int d = 0; d < 2; ++d) {
+      g.task[d] = base + b.off[d];
+      g.n[d] = (int)b.task[d].size();
+    }
+    return g;
+  };
+  for (auto& kv : dir_byN) ls->dir_w.push_back(dir_group(kv.first, kv.second));
+  ls->dir_phi = dir_group(1, dir_phi);
   for (int k = 0; k < Lists::NK; ++k) {
     ls->segs[k] = base + o_sg[k];
     ls->nseg[k] = (int)segs[k].size();
@@ -857,6 +1001,24 @@ inline void mark_use(s2dw_plan_t p, cudaStream_t st) {
   if (!capturing(st)) cudaEventRecord(p->last_use, st);
 }
 
+// Direct FP32 contraction launches of one direction (the scaling parts ride
+// with the first group); the number of launches.
+int direct_groups(const Lists& ls) { return (int)ls.dir_w.size() + (ls.dir_w.empty() && ls.dir_phi.n[0] > 0 ? 1 : 0); }
+void run_direct(const Lists& ls, bool syn, const ContractDesc<float>* dw, const ContractDesc<float>* dp,
+                const CallPtrs& ptrs, cudaStream_t st) {
+  const int d = syn ? 1 : 0;
+  const DirTasks phi{dp, reinterpret_cast<const DirTask*>(ls.dir_phi.task[d]), ls.dir_phi.n[d]};
+  DirTasks none = phi;
+  none.n = 0;
+  bool first = true;
+  for (const auto& g : ls.dir_w) {
+    launch_contract_direct(g.N, syn, g.rt, DirTasks{dw, reinterpret_cast<const DirTask*>(g.task[d]), g.n[d]},
+                           first ? phi : none, ptrs, st);
+    first = false;
+  }
+  if (first) launch_contract_direct(1, syn, ls.dir_phi.rt, DirTasks{dw, nullptr, 0}, phi, ptrs, st);
+}
+
 // Analysis stages: [contraction + gamma | scaling contraction | beta | alpha chirp-z full-band | segmented
 // | alpha direct].
 // the half-length beta launches of a kind, one per transform length
@@ -874,6 +1036,7 @@ void run_analysis(const Lists& ls, const CallPtrs& ptrs, cudaStream_t st, cudaEv
   rec(ev, 0, st);
   if constexpr (sizeof(T) == sizeof(float)) {
     launch_fpack(dw, ls.njobs, ls.nbmax, ls.Lrmax, ptrs, st);
+    run_direct(ls, false, dw, dp, ptrs, st);
     for (auto& t : ls.tiles_w)
       launch_contract_pair(t.first & 0xff, 2, false, t.first >> kShapeShift, dw,
                            reinterpret_cast<const PairTask*>(t.second.first), t.second.second, ptrs, st);
@@ -937,6 +1100,7 @@ void run_synthesis(const Lists& ls, const CallPtrs& ptrs, const ReduceJobs& rj, 
   launch_dct_parts<T>(ls, CZT_BETA_SYN_DCT, ptrs, st);
   rec(ev, 4, st);
   if constexpr (sizeof(T) == sizeof(float)) {
+    run_direct(ls, true, dw, dp, ptrs, st);
     for (auto& t : ls.tiles_w)
       launch_contract_pair(t.first & 0xff, 2, true, t.first >> kShapeShift, dw,
                            reinterpret_cast<const PairTask*>(t.second.first), t.second.second, ptrs, st);
@@ -970,6 +1134,8 @@ void own_lists_build(s2dw_plan_s* p) {
   p->own.tiles_w = ls->tiles_w;
   p->own.tiles_phi = ls->tiles_phi;
   p->own.ntiles_phi = ls->ntiles_phi;
+  p->own.dir_w = ls->dir_w;
+  p->own.dir_phi = ls->dir_phi;
   for (int k = 0; k < Lists::NK; ++k) {
     p->own.segs[k] = ls->segs[k];
     p->own.nseg[k] = ls->nseg[k];
@@ -1007,7 +1173,10 @@ void plan_build_typed(s2dw_plan_s* p, const double* kap_d, const double* phi_d, 
   const size_t o_RSphi = pairc ? take(0) : take((size_t)p->Lphi * p->Lphip * sizeof(T));
   const size_t o_RSp = pairc ? take((size_t)nbw * p->Lr * 2 * NH * 32 * sizeof(float)) : take(0);
   const size_t o_RSphi_p = pairc ? take((size_t)nbp * p->Lrphi * 32 * sizeof(float)) : take(0);
-  const size_t o_fP = pairc ? take((size_t)nbw * p->Lrf * 32 * sizeof(cx<T>)) : take(0);
+  p->direct_w = pairc && p->L0 <= kContractDirectMaxL;
+  p->direct_phi = pairc && p->Lphi <= kContractDirectMaxL;
+  const bool packf = pairc && !(p->direct_w && p->direct_phi);  // the direct contraction reads f itself
+  const size_t o_fP = packf ? take((size_t)nbw * p->Lrf * 32 * sizeof(cx<T>)) : take(0);
   std::vector<size_t> o_Y(p->nscale + 1), o_X(p->nscale + 1);
   for (int j = 0; j <= p->nscale; ++j) {
     const int Nj = (j == p->nscale) ? 1 : N;
@@ -1077,7 +1246,7 @@ void plan_build_typed(s2dw_plan_s* p, const double* kap_d, const double* phi_d, 
   p->RSphi = pairc ? nullptr : b + o_RSphi;
   p->RSp = pairc ? b + o_RSp : nullptr;
   p->RSphi_p = pairc ? b + o_RSphi_p : nullptr;
-  p->fP = pairc ? b + o_fP : nullptr;
+  p->fP = packf ? b + o_fP : nullptr;
   p->Y.resize(p->nscale + 1);
   p->X.resize(p->nscale + 1);
   for (int j = 0; j <= p->nscale; ++j) {
@@ -1248,8 +1417,9 @@ void plan_build_typed(s2dw_plan_s* p, const double* kap_d, const double* phi_d, 
       if (!pair_two_tiles(N) || npairs < 3LL * sms) p->pair_shape = kPairShapeTile;
       else p->pair_shape = N >= 4 ? kPairShapePair : kPairShapeTile2;
     }
-    build_pair_tasks(p->L0, p->lend_w, p->pair_shape == kPairShapePair, p->tab->Lmax, p->ptasks_w_host);
-    build_pair_tasks(p->Lphi, p->lphi, true, p->tab->Lmax, p->ptasks_phi_host);
+    if (!p->direct_w)
+      build_pair_tasks(p->L0, p->lend_w, p->pair_shape == kPairShapePair, p->tab->Lmax, p->ptasks_w_host);
+    if (!p->direct_phi) build_pair_tasks(p->Lphi, p->lphi, true, p->tab->Lmax, p->ptasks_phi_host);
   } else {
     build_tiles(p->L0, p->lend_w, p->TMP, 0, p->tiles_w_host);
     build_tiles(p->Lphi, p->lphi, p->TMP, 0, p->tiles_phi_host);
@@ -1648,7 +1818,8 @@ static void choices_put(s2dw_plan_t p, const int* c) {
     const int shape = c[choices_count(p) - 1];
     if (shape != p->pair_shape) {
       p->pair_shape = shape;
-      build_pair_tasks(p->L0, p->lend_w, shape == kPairShapePair, p->tab->Lmax, p->ptasks_w_host);
+      if (!p->direct_w)
+        build_pair_tasks(p->L0, p->lend_w, shape == kPairShapePair, p->tab->Lmax, p->ptasks_w_host);
     }
   }
   drop_batches_with(p);
@@ -1877,7 +2048,7 @@ int s2dw_wait_probe(long long limit_cycles, void* stream) {
 int s2dw_launch_counts(s2dw_plan_t p, int* analysis, int* synthesis) {
   if (!p) return S2DW_EINVAL;
   const Lists& ls = p->own;
-  int contract = ls.ntiles_phi > 0 ? 1 : 0;
+  int contract = (ls.ntiles_phi > 0 ? 1 : 0) + direct_groups(ls);
   for (auto& t : ls.tiles_w) contract += t.second.second > 0 ? 1 : 0;
   auto has = [&](int k) {
     if (k >= CZT_BETA_ANA_DCT && k <= CZT_BETA_RS_DCT) return (int)ls.dct_parts[k - CZT_BETA_ANA_DCT].size();

@@ -1,0 +1,451 @@
+// FP32 l-contraction for small and middle band-limits (Sec. 3.2 Eq. (27);
+// Sec. 3.3 Eqs. (34), (32)): the sums of contract_pair.cuh, organised for
+// latency instead of for one long stream per CTA.
+//
+// What bounds it.  At L <= kContractDirectMaxL a whole contraction is a few
+// microseconds of FP32 work; the tile-pair ring kernel has one CTA per 32 x 32
+// tile (pair) and walks its l one stage after the other, so at L = 128 it kept
+// 16 of 152 SMs busy for 128 dependent steps.  Here
+//   analysis: a task is one scale of one tile over that scale's own l range, so
+//     the scales run side by side and the gamma step runs once, at the end; a
+//     thread owns RT rows x 1 column and keeps its accumulators; a task is cut
+//     into 32 / (RT warps) CTAs, RT chosen so that the launch fills the SMs
+//     (RT does not enter the arithmetic);
+//   synthesis: a tile's l range is cut at the changes of scale and further (the
+//     sums over m' of different l are independent), each CTA loading the H
+//     values of its own range once.
+// Delta goes from the pair table straight to registers, the next l group in
+// flight while the current one is summed; the R rows and f values of 16 l are
+// staged in shared memory by cp.async, double-buffered, one barrier per 16 l.
+// Lanes run along the second index of the stored block D_l[r][c] =
+// Delta^l_{32p+r, 32q+c} in both tiles of a pair, so every Delta load is one
+// 128-byte line: tile A (m' in p, m in q) has lanes along m, tile B
+// (m' in q, m in p; Delta_{m'm} = (-1)^{m'-m} Delta_{mm'}) lanes along m'.
+// The scaling part's tiles (N = 1, one slot) ride in the same launch.
+#include "contract.cuh"
+
+namespace s2dw {
+
+namespace {
+
+constexpr int kDirLC = 16;  // l per shared-memory stage
+
+// f(integral_constant<0>) .. f(integral_constant<K - 1>), unrolled
+template <int K, typename F>
+__device__ __forceinline__ void dir_unroll(F&& f) {
+  if constexpr (K > 0) {
+    dir_unroll<K - 1>(f);
+    f(std::integral_constant<int, K - 1>());
+  }
+}
+
+__device__ __forceinline__ void cp_async8_zf(void* smem, const void* gmem, int src_bytes) {
+  const unsigned s = static_cast<unsigned>(__cvta_generic_to_shared(smem));
+  asm volatile("cp.async.ca.shared.global [%0], [%1], 8, %2;\n" ::"r"(s), "l"(gmem), "r"(src_bytes) : "memory");
+}
+
+// c + a b, complex, with the fused order fixed (so that every instantiation
+// rounds alike: a batched call equals the single one bit for bit)
+__device__ __forceinline__ float2 cfma_rn(float2 a, float2 b, float2 c) {
+  c.x = __fmaf_rn(a.x, b.x, c.x);
+  c.y = __fmaf_rn(a.x, b.y, c.y);
+  c.x = __fmaf_rn(-a.y, b.y, c.x);
+  c.y = __fmaf_rn(a.y, b.x, c.y);
+  return c;
+}
+
+template <int RT>
+__device__ __forceinline__ void lds_rows(const float* p, float (&r)[RT]) {
+  if constexpr (RT == 4) {
+    const float4 v = *reinterpret_cast<const float4*>(p);
+    r[0] = v.x, r[1] = v.y, r[2] = v.z, r[3] = v.w;
+  } else if constexpr (RT == 2) {
+    const float2 v = *reinterpret_cast<const float2*>(p);
+    r[0] = v.x, r[1] = v.y;
+  } else {
+    r[0] = *p;
+  }
+}
+
+// One scale of one tile: G^j over l in [lstart, lend], then the gamma step.
+// nslot: slots of the R rows (the scale's values sit in slot tk.slot).
+template <int N, int RT, int NW, bool ISB>
+__device__ __forceinline__ void dir_ana_tile(const ContractDesc<float>* __restrict__ D, int nslot, const DirTask& tk, int sub,
+                                             const float2* __restrict__ f, float2* cg, float* Rs0, float2* fs0) {
+  constexpr int NH = (N + 1) / 2, ZH = N & 1, NP = N / 2, RW = NH * 32, LC = kDirLC;
+  constexpr int NTH = 32 * NW, U = RT == 4 ? 4 : 8;
+  static_assert(LC % U == 0 && U % 2 == 0, "the parity of a position is its l's relative to lstart");
+  const int t = threadIdx.x, w = t >> 5, lane = t & 31;
+  const int rw = (sub * NW + w) * RT;  // first row of the stored block
+  const int l_start = tk.lstart, l_end = tk.lend, rrow = nslot * RW;
+  const float* __restrict__ dp = D->dpair + tk.dbase + rw * 32 + lane;
+  const float* __restrict__ Rg = D->RSp + ((size_t)(ISB ? tk.q : tk.p) * D->Lr + l_start) * rrow + tk.slot * RW;
+  const int mb = 32 * (ISB ? tk.p : tk.q);  // m block of f
+  const int Lj = D->Lj[tk.j];
+  float2* __restrict__ Y = D->Y[tk.j];
+  for (int i = t; i < N * N; i += NTH) cg[i] = D->cga[i];
+
+  auto stage = [&](int ch) {  // R rows and f of l_start + 16 ch .., zero past l_end
+    float* Rs = Rs0 + (ch & 1) * LC * RW;
+    float2* fs = fs0 + (ch & 1) * LC * 32;
+    const int l0 = l_start + ch * LC;
+    const float* src = Rg + (size_t)ch * LC * rrow;
+    for (int i = t; i < LC * (RW / 4); i += NTH) {
+      const int r = i / (RW / 4), c = 4 * (i % (RW / 4));
+      const bool ok = l0 + r <= l_end;
+      cp_async16(Rs + r * RW + c, src + (ok ? (size_t)r * rrow + c : 0), ok ? 16 : 0);
+    }
+    for (int i = t; i < LC * 32; i += NTH) {
+      const int l = l0 + (i >> 5), m = mb + (i & 31);
+      const bool ok = m <= l && l <= l_end;
+      cp_async8_zf(fs + i, f + (ok ? (size_t)l * l + l + m : 0), ok ? 8 : 0);
+    }
+    cp_async_commit();
+  };
+
+  float ax[RT][N], ay[RT][N];
+#pragma unroll
+  for (int e = 0; e < RT; ++e)
+#pragma unroll
+    for (int k = 0; k < N; ++k) ax[e][k] = ay[e][k] = 0.f;
+
+  float dn[U][RT], dc[U][RT] = {};  // Delta of the next and the current group
+  auto fetch = [&](int l) {
+#pragma unroll
+    for (int u = 0; u < U; ++u)
+#pragma unroll
+      for (int e = 0; e < RT; ++e) dn[u][e] = l + u <= l_end ? __ldg(dp + (size_t)(l - l_start + u) * 1024 + e * 32) : 0.f;
+  };
+  auto compute = [&](const float* Rl, const float2* fl, auto uu) {
+    constexpr int u = decltype(uu)::value, BQ = (u & 1) * NP;
+    float tx[RT], ty[RT];
+    if constexpr (!ISB) {
+      const float2 fv = fl[lane];
+#pragma unroll
+      for (int e = 0; e < RT; ++e) tx[e] = __fmul_rn(dc[u][e], fv.x), ty[e] = __fmul_rn(dc[u][e], fv.y);
+    } else {
+#pragma unroll
+      for (int e = 0; e < RT; ++e) {
+        const float2 fv = fl[rw + e];
+        tx[e] = __fmul_rn(dc[u][e], fv.x), ty[e] = __fmul_rn(dc[u][e], fv.y);
+      }
+    }
+#pragma unroll
+    for (int h = 0; h < NH; ++h) {
+      const int q = (ZH && h == 0) ? 2 * NP : BQ + h - ZH;
+      float r[RT];
+      if constexpr (!ISB) {
+        lds_rows<RT>(Rl + h * 32 + rw, r);
+      } else {
+        const float r0 = Rl[h * 32 + lane];
+#pragma unroll
+        for (int e = 0; e < RT; ++e) r[e] = r0;
+      }
+#pragma unroll
+      for (int e = 0; e < RT; ++e) {
+        ax[e][q] = __fmaf_rn(tx[e], r[e], ax[e][q]);
+        ay[e][q] = __fmaf_rn(ty[e], r[e], ay[e][q]);
+      }
+    }
+  };
+
+  stage(0);
+  fetch(l_start);
+  const int nch = (l_end - l_start) / LC + 1;
+  for (int ch = 0; ch < nch; ++ch) {
+    cp_async_wait<0>();
+    __syncthreads();  // this chunk's rows visible, the previous buffer free
+    if (ch + 1 < nch) stage(ch + 1);
+    const float* Rs = Rs0 + (ch & 1) * LC * RW;
+    const float2* fs = fs0 + (ch & 1) * LC * 32;
+#pragma unroll 1
+    for (int gi = 0; gi < LC; gi += U) {
+      const int l0 = l_start + ch * LC + gi;
+      if (l0 > l_end) break;
+#pragma unroll
+      for (int u = 0; u < U; ++u)
+#pragma unroll
+        for (int e = 0; e < RT; ++e) dc[u][e] = dn[u][e];
+      fetch(l0 + U);
+      dir_unroll<U>([&](auto uu) { compute(Rs + (gi + decltype(uu)::value) * RW, fs + (gi + decltype(uu)::value) * 32, uu); });
+    }
+  }
+
+  // gamma step (Eq. (28)): G_{+n} = B0 + B1, G_{-n} = (-1)^{m' + lstart} (B0 - B1)
+  // from the sums over the l of lstart's parity (B0) and of the other (B1)
+#pragma unroll
+  for (int e = 0; e < RT; ++e) {
+    const int mp = ISB ? 32 * tk.q + lane : 32 * tk.p + rw + e;
+    const int m = ISB ? 32 * tk.p + rw + e : 32 * tk.q + lane;
+    if (mp >= Lj || m >= Lj) continue;
+    float2 gk[N];
+    if (ZH) gk[N / 2] = make_float2(ax[e][2 * NP], ay[e][2 * NP]);
+    const float sgn = ((mp + l_start) & 1) ? -1.f : 1.f;
+#pragma unroll
+    for (int p = 0; p < NP; ++p) {
+      gk[(N + 1) / 2 + p] = make_float2(ax[e][p] + ax[e][NP + p], ay[e][p] + ay[e][NP + p]);
+      gk[N / 2 - 1 - p] = make_float2(sgn * (ax[e][p] - ax[e][NP + p]), sgn * (ay[e][p] - ay[e][NP + p]));
+    }
+    const float fs = (ISB && ((mp + m) & 1)) ? -1.f : 1.f;
+#pragma unroll
+    for (int g = 0; g < N; ++g) {
+      float2 v = make_float2(0.f, 0.f);
+#pragma unroll
+      for (int k = 0; k < N; ++k) v = cfma_rn(gk[k], cg[k * N + g], v);
+      Y[((size_t)g * Lj + m) * Lj + mp] = cscale<float>(cmul_ipow<float>(v, (-m) & 3), fs);
+    }
+  }
+}
+
+template <int N, int RT, int NW>
+__global__ void __launch_bounds__(32 * NW)
+k_contract_dir_ana(const ContractDesc<float>* __restrict__ dw, const DirTask* __restrict__ tw, int nw,
+                   const ContractDesc<float>* __restrict__ dphi, const DirTask* __restrict__ tp, CallPtrs ptrs) {
+  constexpr int SUB = 32 / (RT * NW), RW = ((N + 1) / 2) * 32;
+  __shared__ float2 cg[64];
+  __shared__ __align__(16) float Rs[2 * kDirLC * RW];
+  __shared__ __align__(16) float2 fs[2 * kDirLC * 32];
+  const int i = blockIdx.x / SUB, sub = blockIdx.x % SUB;
+  if (i < nw) {
+    const DirTask tk = tw[i];
+    const float2* f = reinterpret_cast<const float2*>(ptrs.f[tk.prob]);
+    if (tk.half == 0) dir_ana_tile<N, RT, NW, false>(dw + tk.prob, 2, tk, sub, f, cg, Rs, fs);
+    else dir_ana_tile<N, RT, NW, true>(dw + tk.prob, 2, tk, sub, f, cg, Rs, fs);
+  } else {
+    const DirTask tk = tp[i - nw];
+    const float2* f = reinterpret_cast<const float2*>(ptrs.f[tk.prob]);
+    if (tk.half == 0) dir_ana_tile<1, RT, NW, false>(dphi + tk.prob, 1, tk, sub, f, cg, Rs, fs);
+    else dir_ana_tile<1, RT, NW, true>(dphi + tk.prob, 1, tk, sub, f, cg, Rs, fs);
+  }
+}
+
+// Synthesis of one tile over l in [lstart, lend], a range on which the two
+// slots hold constant scales (tk.j, tk.j2; -1: empty).  8 warps x 4 rows of the
+// stored block.  Tile A sums its rows m' in the thread, then over the warps in
+// shared memory; tile B's rows m' are the lanes: a butterfly that halves the
+// values with the lanes leaves one column part per four lanes.
+template <int N, int NSLOT, bool ISB>
+__device__ __forceinline__ void dir_syn_tile(const ContractDesc<float>* __restrict__ D, const DirTask& tk, float2* cg,
+                                             float* Rs0, float2* red) {
+  constexpr int NH = (N + 1) / 2, ZH = N & 1, NP = N / 2, RROW = NSLOT * NH * 32, LC = kDirLC;
+  constexpr int NTH = 256, RT = 4, U = 4;
+  const int t = threadIdx.x, w = t >> 5, lane = t & 31, rw = 4 * w;
+  const int l_start = tk.lstart, l_end = tk.lend;
+  const int rb = ISB ? tk.q : tk.p, cb = ISB ? tk.p : tk.q, L = D->L, Lp32 = D->Lp32;
+  const float* __restrict__ dp = D->dpair + tk.dbase + rw * 32 + lane;
+  const float* __restrict__ Rg = D->RSp + ((size_t)rb * D->Lr + l_start) * RROW;
+  float2* __restrict__ P = D->P + ((size_t)rb * L + l_start) * Lp32 + 32 * cb;
+
+  auto stage = [&](int ch) {
+    float* Rs = Rs0 + (ch & 1) * LC * RROW;
+    const int nl = l_end - l_start - ch * LC + 1;
+    const float* src = Rg + (size_t)ch * LC * RROW;
+    for (int i = t; i < LC * (RROW / 4); i += NTH) {
+      const bool ok = i / (RROW / 4) < nl;
+      cp_async16(Rs + 4 * i, src + (ok ? 4 * i : 0), ok ? 16 : 0);
+    }
+    cp_async_commit();
+  };
+  float dn[U][RT], dc[U][RT] = {};
+  auto fetch = [&](int l) {
+#pragma unroll
+    for (int u = 0; u < U; ++u)
+#pragma unroll
+      for (int e = 0; e < RT; ++e) dn[u][e] = l + u <= l_end ? __ldg(dp + (size_t)(l - l_start + u) * 1024 + e * 32) : 0.f;
+  };
+  stage(0);
+  fetch(l_start);
+  for (int i = t; i < N * N; i += NTH) cg[i] = D->cgs[i];
+  __syncthreads();
+
+  // gamma adjoint (Eq. (39)) of both slots, folded into the parity banks
+  float hx[RT][NSLOT][N], hy[RT][NSLOT][N];
+#pragma unroll
+  for (int s = 0; s < NSLOT; ++s) {
+    const int j = s == 0 ? tk.j : tk.j2;
+    const int Lj = j >= 0 ? D->Lj[j] : 0;
+    const float2* __restrict__ V = j >= 0 ? D->Y[j] : nullptr;
+#pragma unroll
+    for (int e = 0; e < RT; ++e) {
+      const int mp = ISB ? 32 * tk.q + lane : 32 * tk.p + rw + e;
+      const int m = ISB ? 32 * tk.p + rw + e : 32 * tk.q + lane;
+      float2 h[N];
+#pragma unroll
+      for (int k = 0; k < N; ++k) h[k] = make_float2(0.f, 0.f);
+      if (mp < Lj && m < Lj) {
+        float2 vg[N];
+#pragma unroll
+        for (int g = 0; g < N; ++g) vg[g] = V[((size_t)g * Lj + mp) * Lj + m];
+#pragma unroll
+        for (int g = 0; g < N; ++g)
+#pragma unroll
+          for (int k = 0; k < N; ++k) h[k] = cfma_rn(vg[g], cg[k * N + g], h[k]);
+        const float fs = (ISB && ((mp + m) & 1)) ? -1.f : 1.f;
+#pragma unroll
+        for (int k = 0; k < N; ++k) h[k] = cscale<float>(cmul_ipow<float>(h[k], m & 3), fs);
+      }
+      const float sgn = ((mp + l_start) & 1) ? -1.f : 1.f;
+#pragma unroll
+      for (int p = 0; p < NP; ++p) {
+        const float2 hp = h[(N + 1) / 2 + p], hm = h[N / 2 - 1 - p];
+        hx[e][s][p] = hp.x + sgn * hm.x;
+        hy[e][s][p] = hp.y + sgn * hm.y;
+        hx[e][s][NP + p] = hp.x - sgn * hm.x;
+        hy[e][s][NP + p] = hp.y - sgn * hm.y;
+      }
+      if (ZH) hx[e][s][2 * NP] = h[N / 2].x, hy[e][s][2 * NP] = h[N / 2].y;
+    }
+  }
+  auto compute = [&](const float* Rl, int li, int l, auto uu) {
+    constexpr int u = decltype(uu)::value, BQ = (u & 1) * NP;
+    float px[RT], py[RT];
+#pragma unroll
+    for (int e = 0; e < RT; ++e) px[e] = py[e] = 0.f;
+#pragma unroll
+    for (int s = 0; s < NSLOT; ++s)
+#pragma unroll
+      for (int h = 0; h < NH; ++h) {
+        const int q = (ZH && h == 0) ? 2 * NP : BQ + h - ZH;
+        float r[RT];
+        if constexpr (!ISB) {
+          lds_rows<RT>(Rl + (s * NH + h) * 32 + rw, r);
+        } else {
+          const float r0 = Rl[(s * NH + h) * 32 + lane];
+#pragma unroll
+          for (int e = 0; e < RT; ++e) r[e] = r0;
+        }
+#pragma unroll
+        for (int e = 0; e < RT; ++e) {
+          px[e] = __fmaf_rn(hx[e][s][q], r[e], px[e]);
+          py[e] = __fmaf_rn(hy[e][s][q], r[e], py[e]);
+        }
+      }
+    if constexpr (!ISB) {
+      float2 v = make_float2(__fmul_rn(dc[u][0], px[0]), __fmul_rn(dc[u][0], py[0]));
+#pragma unroll
+      for (int e = 1; e < RT; ++e) v.x = __fmaf_rn(dc[u][e], px[e], v.x), v.y = __fmaf_rn(dc[u][e], py[e], v.y);
+      red[(li * 8 + w) * 32 + lane] = v;
+    } else {
+      float v[8];
+#pragma unroll
+      for (int e = 0; e < RT; ++e) v[2 * e] = __fmul_rn(dc[u][e], px[e]), v[2 * e + 1] = __fmul_rn(dc[u][e], py[e]);
+      const bool h16 = lane & 16, h8 = lane & 8, h4 = lane & 4;
+      float a[4], b[2], c;
+#pragma unroll
+      for (int i = 0; i < 4; ++i) a[i] = (h16 ? v[i + 4] : v[i]) + __shfl_xor_sync(0xffffffffu, h16 ? v[i] : v[i + 4], 16);
+#pragma unroll
+      for (int i = 0; i < 2; ++i) b[i] = (h8 ? a[i + 2] : a[i]) + __shfl_xor_sync(0xffffffffu, h8 ? a[i] : a[i + 2], 8);
+      c = (h4 ? b[1] : b[0]) + __shfl_xor_sync(0xffffffffu, h4 ? b[0] : b[1], 4);
+      c += __shfl_xor_sync(0xffffffffu, c, 2);
+      c += __shfl_xor_sync(0xffffffffu, c, 1);
+      if ((lane & 3) == 0 && l <= l_end) reinterpret_cast<float*>(P + (size_t)(l - l_start) * Lp32 + rw)[lane >> 2] = c;
+    }
+  };
+
+  const int nch = (l_end - l_start) / LC + 1;
+  for (int ch = 0; ch < nch; ++ch) {
+    cp_async_wait<0>();
+    __syncthreads();
+    if (ch + 1 < nch) stage(ch + 1);
+    const float* Rs = Rs0 + (ch & 1) * LC * RROW;
+    const int lc0 = l_start + ch * LC;
+#pragma unroll 1
+    for (int gi = 0; gi < LC; gi += U) {
+      const int l0 = lc0 + gi;
+      if (l0 > l_end) break;
+#pragma unroll
+      for (int u = 0; u < U; ++u)
+#pragma unroll
+        for (int e = 0; e < RT; ++e) dc[u][e] = dn[u][e];
+      fetch(l0 + U);
+      dir_unroll<U>([&](auto uu) {
+        constexpr int u = decltype(uu)::value;
+        compute(Rs + (gi + u) * RROW, gi + u, l0 + u, uu);
+      });
+    }
+    if constexpr (!ISB) {
+      __syncthreads();
+      const int nl = min(LC, l_end - lc0 + 1);
+      for (int i = w; i < nl; i += 8) {
+        float2 sum = red[i * 256 + lane];
+#pragma unroll
+        for (int r2 = 1; r2 < 8; ++r2) {
+          const float2 v = red[i * 256 + r2 * 32 + lane];
+          sum.x += v.x;
+          sum.y += v.y;
+        }
+        P[(size_t)(lc0 - l_start + i) * Lp32 + lane] = sum;
+      }
+    }
+  }
+}
+
+template <int N>
+constexpr size_t dir_syn_smem() {
+  return (size_t)2 * kDirLC * 2 * ((N + 1) / 2) * 32 * sizeof(float) + (size_t)kDirLC * 8 * 32 * sizeof(float2);
+}
+
+template <int N>
+__global__ void __launch_bounds__(256)
+k_contract_dir_syn(const ContractDesc<float>* __restrict__ dw, const DirTask* __restrict__ tw, int nw,
+                   const ContractDesc<float>* __restrict__ dphi, const DirTask* __restrict__ tp) {
+  extern __shared__ __align__(16) unsigned char dir_smem[];
+  __shared__ float2 cg[64];
+  float2* red = reinterpret_cast<float2*>(dir_smem);
+  float* Rs = reinterpret_cast<float*>(dir_smem + (size_t)kDirLC * 8 * 32 * sizeof(float2));
+  const int i = blockIdx.x;
+  if (i < nw) {
+    const DirTask tk = tw[i];
+    if (tk.half == 0) dir_syn_tile<N, 2, false>(dw + tk.prob, tk, cg, Rs, red);
+    else dir_syn_tile<N, 2, true>(dw + tk.prob, tk, cg, Rs, red);
+  } else {
+    const DirTask tk = tp[i - nw];
+    if (tk.half == 0) dir_syn_tile<1, 1, false>(dphi + tk.prob, tk, cg, Rs, red);
+    else dir_syn_tile<1, 1, true>(dphi + tk.prob, tk, cg, Rs, red);
+  }
+}
+
+template <int N>
+void dir_launch(bool syn, int rt, const DirTasks& w, const DirTasks& p, const CallPtrs& ptrs, cudaStream_t st) {
+  const int n = w.n + p.n;
+  const ContractDesc<float>* dw = w.descs;
+  const ContractDesc<float>* dp = p.descs;
+  if (syn) k_contract_dir_syn<N><<<n, 256, dir_syn_smem<N>(), st>>>(dw, w.tasks, w.n, dp, p.tasks);
+  else if (rt == 4) k_contract_dir_ana<N, 4, 8><<<n, 256, 0, st>>>(dw, w.tasks, w.n, dp, p.tasks, ptrs);
+  else if (rt == 2) k_contract_dir_ana<N, 2, 8><<<2 * n, 256, 0, st>>>(dw, w.tasks, w.n, dp, p.tasks, ptrs);
+  else k_contract_dir_ana<N, 1, 4><<<8 * n, 128, 0, st>>>(dw, w.tasks, w.n, dp, p.tasks, ptrs);
+}
+
+template <int N>
+cudaError_t dir_attr() {
+  return cudaFuncSetAttribute(k_contract_dir_syn<N>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)dir_syn_smem<N>());
+}
+
+}  // namespace
+
+// One launch over the tasks of w (N orders, two slots) and p (scaling parts).
+void launch_contract_direct(int N, bool syn, int rt, const DirTasks& w, const DirTasks& p, const CallPtrs& ptrs,
+                            cudaStream_t st) {
+  if (w.n + p.n <= 0) return;
+  switch (N) {
+    case 1: dir_launch<1>(syn, rt, w, p, ptrs, st); break;
+    case 2: dir_launch<2>(syn, rt, w, p, ptrs, st); break;
+    case 3: dir_launch<3>(syn, rt, w, p, ptrs, st); break;
+    case 4: dir_launch<4>(syn, rt, w, p, ptrs, st); break;
+    case 5: dir_launch<5>(syn, rt, w, p, ptrs, st); break;
+    case 6: dir_launch<6>(syn, rt, w, p, ptrs, st); break;
+    case 7: dir_launch<7>(syn, rt, w, p, ptrs, st); break;
+    case 8: dir_launch<8>(syn, rt, w, p, ptrs, st); break;
+    default: break;
+  }
+}
+
+cudaError_t contract_direct_prepare() {
+  cudaError_t (*fns[])() = {dir_attr<1>, dir_attr<2>, dir_attr<3>, dir_attr<4>,
+                            dir_attr<5>, dir_attr<6>, dir_attr<7>, dir_attr<8>};
+  for (auto f : fns)
+    if (cudaError_t e = f(); e != cudaSuccess) return e;
+  return cudaSuccess;
+}
+
+}  // namespace s2dw

@@ -10,7 +10,7 @@ __global__ void __launch_bounds__(256) k_fpack(const ContractDesc<float>* __rest
   const int job = blockIdx.z, b = blockIdx.y;
   const ContractDesc<float>* D = descs + job;
   const int L = D->L, Lrf = D->Lrf;
-  if (32 * b >= L) return;
+  if (!D->fP || 32 * b >= L) return;  // (a plan of the direct contraction reads f itself)
   const int l = blockIdx.x * 8 + (threadIdx.x >> 5), c = threadIdx.x & 31;
   if (l >= Lrf) return;
   const int m = 32 * b + c;

@@ -32,6 +32,9 @@ struct ContractDesc {
   int L, Lp, Lp32, nbr;
   int nseg;
   int N, nslot, eta_odd;   // eta_odd: N even -> eta = i
+  // gamma factors [k N + g]: analysis conj(eta) i^{n_k} e^{i n_k gamma_g},
+  // synthesis eta (2 pi/N) i^{-n_k} e^{-i n_k gamma_g} (direct FP32 contraction)
+  cx<T> cga[64], cgs[64];
   int Lj[MAXS];            // per scale band-limit (support hi + 1)
   cx<T>* Y[MAXS];          // per scale cube [N][Lj][Lj] (analysis out / synthesis in)
   LSeg seg[2 * MAXS + 2];
@@ -188,6 +191,35 @@ void launch_fpack(const ContractDesc<float>* descs, int njobs, int nbmax, int Lr
 cudaError_t launch_pair_table(float* out, const double* d64, int Lmax, cudaStream_t st);
 cudaError_t launch_rtable_pair(float* RSp, const double* d64, const double* kap, const double* sabs,
                                const int* slotj, int L, int Lr, int N, int nslot, int kapL, cudaStream_t st);
+// FP32 contraction of small and middle band-limits (contract_direct.cu): one
+// launch over the tiles of the plans' wavelet scales (N orders) and of their
+// scaling parts.  rt: rows per thread of the analysis (1, 2 or 4).
+// A task is one 32 x 32 tile (half 0: m' in block p, m in q; half 1: the
+// other way round) over l in [lstart, lend]; dbase: pair-table entry of lstart.
+// Analysis: scale j, held in slot `slot` of the R rows.  Synthesis: the two
+// slots hold scales j and j2 (-1: none) over the whole range.
+struct DirTask {
+  int prob, p, q, half;
+  int lstart, lend;
+  int j, j2, slot, pad;
+  long long dbase;
+};
+struct DirTasks {
+  const ContractDesc<float>* descs;
+  const DirTask* tasks;
+  int n;
+};
+// Band-limits up to this run it.  Contraction per call, GB300 (tile-pair ring
+// kernel with its scaling launch -> direct, analysis / synthesis, us): L = 32,
+// N = 3 34 / 38 -> 8 / 13; L = 128, N = 5 62 / 77 -> 15 / 17; L = 256, N = 5
+// 85 / 106 -> 28 / 40; L = 512, N = 5 144 / 170 -> 101 / 139; L = 640, N = 3
+// 149 / 161 -> 137 / 119.  Above, Delta no longer stays in L2 between the two
+// halves and the scales: L = 800, N = 3 246 / 268 against 250 / 205, L = 1024,
+// N = 5 406 / 400 against 648 / 705.
+constexpr int kContractDirectMaxL = 640;
+void launch_contract_direct(int N, bool syn, int rt, const DirTasks& w, const DirTasks& p, const CallPtrs& ptrs,
+                            cudaStream_t st);
+cudaError_t contract_direct_prepare();
 cudaError_t pair_prepare();
 cudaError_t pair_timeouts(int* count);  // reads and resets the device count
 template <typename T>
