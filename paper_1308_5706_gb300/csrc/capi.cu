@@ -116,7 +116,7 @@ void kernels_prepare(bool fp64, bool pair) {
     done_czt[fp64 ? 1 : 0] |= bit;
   }
   if (pair && !(done_pair & bit)) {
-    ck(pair_prepare());
+    ck(contract_tile_prepare());
     ck(contract_direct_prepare());
     done_pair |= bit;
   }
@@ -156,7 +156,7 @@ struct DeltaTab {
   size_t bytes;
   double* raw64 = nullptr;  // the allocations
   float* raw32 = nullptr;
-  float* pair32 = nullptr;  // pair table of the FP32 tile-pair contraction (built for the first FP32 plan)
+  float* pair32 = nullptr;  // pair table of the FP32 contraction (built for the first FP32 plan)
 };
 std::mutex g_mu;
 std::vector<DeltaTab*> g_tabs;
@@ -251,28 +251,25 @@ void delta_release(DeltaTab* t) {
   }
 }
 
-// launch-list keys of the FP32 contraction tasks: N | (CTA shape << 8)
-constexpr int kShapeShift = 8;
-
 // Device-resident launch lists for a set of jobs (one plan = one job).
 struct Lists {
   void* mem = nullptr;
   void* desc_w = nullptr;     // ContractDesc<T>[njobs]
   void* desc_phi = nullptr;   // ContractDesc<T>[njobs]
-  // (N, or N | shape << kShapeShift for the FP32 contraction, (tiles, count))
+  // FP64: (N, (tiles, count))
   std::vector<std::pair<int, std::pair<void*, int>>> tiles_w;
   void* tiles_phi = nullptr;
   int ntiles_phi = 0;
-  // direct FP32 contraction: per N the analysis and synthesis tasks of the
-  // wavelet scales; dir_phi (N = 1): those of the scaling parts, launched with
-  // the first group
-  struct DirGroup {
+  // FP32 contraction, direct and tile kernel: per N the analysis and synthesis
+  // tasks of the wavelet scales; *_phi (N = 1): those of the scaling parts (the
+  // direct ones are launched with the first direct group)
+  struct FpGroup {
     int N = 1, rt = 4;
     void* task[2] = {nullptr, nullptr};  // analysis, synthesis
     int n[2] = {0, 0};
   };
-  std::vector<DirGroup> dir_w;
-  DirGroup dir_phi;
+  std::vector<FpGroup> dir_w, tile_w;
+  FpGroup dir_phi, tile_phi;
   static constexpr int NK = 16;  // chirp-z 0..3, direct alpha 4..5, single-FFT beta 6..7, segmented alpha 8..9,
                                  // MW-grid synthesis beta 10..12, half-length beta 13..15
   void* segs[NK] = {};
@@ -363,7 +360,7 @@ struct s2dw_plan_s {
   std::vector<int> alpha_mode[2];
   // [nscale + 1]: tensor-core basis images of the direct alpha sums (FP32 plans)
   std::vector<void*> tc_ana, tc_syn;
-  // FP32 plans: R rows and packed f of the tile-pair contraction
+  // FP32 plans: R rows and packed f of the FP32 contraction
   void* RSp = nullptr;
   void* RSphi_p = nullptr;
   void* fP = nullptr;
@@ -371,9 +368,8 @@ struct s2dw_plan_s {
   // host copies of the static descriptors (device copies live in `own`)
   std::vector<unsigned char> desc_w_host, desc_phi_host;
   std::vector<TileTask> tiles_w_host, tiles_phi_host;  // FP64 plans
-  std::vector<PairTask> ptasks_w_host, ptasks_phi_host;  // FP32 plans
-  bool direct_w = false, direct_phi = false;  // FP32: those tasks run the direct contraction (one tile each)
-  int pair_shape = kPairShapePair;  // FP32: the contraction's CTA shape (a launch method; N > 5: one tile)
+  bool direct_w = false, direct_phi = false;  // FP32: the direct contraction (else the tile kernel)
+  int pair_shape = kPairShapePair;  // FP32: CTA-shape value of s2dw_plan_choices
   Lists own;
   // stage timing (s2dw_profile): one set of events per call, up to kProfCalls
   static constexpr int kProfCalls = 256;
@@ -488,7 +484,16 @@ void fill_desc(s2dw_plan_s* p, ContractDesc<T>& dw, ContractDesc<T>& dp, const T
   dw.eta_odd = (p->N % 2 == 0) ? 1 : 0;
   gamma_factors<T>(p->N, dw.cga, dw.cgs);
   gamma_factors<T>(1, dp.cga, dp.cgs);
+  for (int j = 0; j < MAXS; ++j) {
+    dw.jlo[j] = dp.jlo[j] = 0;
+    dw.jhi[j] = dp.jhi[j] = -1;
+  }
+  dp.jhi[0] = p->Lphi - 1;
   for (int j = 0; j < p->nscale; ++j) {
+    if (p->hi[j] >= 0) {
+      dw.jlo[j] = p->lo[j];
+      dw.jhi[j] = p->hi[j];
+    }
     dw.Lj[j] = p->Lj[j];
     dw.Y[j] = reinterpret_cast<cx<T>*>(p->Y[j]);
   }
@@ -551,29 +556,67 @@ void build_tiles(int Lband, int lend, int TMP, int prob, std::vector<TileTask>& 
     }
 }
 
-// Tile pairs (p <= q) of a band Lband with l in [32 q, lend]; a pair whose
-// tiles run on separate CTAs (N > 5) becomes two tasks.  Sorted by decreasing
-// work (two tiles count double) so that the long ones start first.
-// two: one task per pair of tiles (both computed by one CTA, N <= 5), else
-// one task per tile
-void build_pair_tasks(int Lband, int lend, bool two, int table_Lmax, std::vector<PairTask>& out) {
-  out.clear();
+CTask make_task(int prob, int p, int q, int half, int lstart, int lend, int j, int j2, int slot, int table_Lmax) {
+  CTask t;
+  std::memset(&t, 0, sizeof(t));
+  t.prob = (uint8_t)prob, t.p = (uint8_t)p, t.q = (uint8_t)q, t.half = (uint8_t)half;
+  t.j = (int8_t)j, t.j2 = (int8_t)j2, t.slot = (int8_t)slot;
+  t.lstart = (int16_t)lstart, t.lend = (int16_t)lend, t.Lmax = (int16_t)table_Lmax;
+  return t;
+}
+
+// Tasks of the contraction of large band-limits (contract_tile.cuh): per block
+// pair (and tile, where a CTA computes one), the analysis by pairs of adjacent
+// scales 2i, 2i + 1 (one per slot) over the union of their l ranges, the
+// synthesis by l ranges on which each slot holds one scale (an l-segment
+// where a slot is empty joins its neighbour).
+void build_tile_tasks(const ContractDesc<float>& d, int prob, int Lband, int lend, int table_Lmax,
+                      std::vector<CTask>& ana, std::vector<CTask>& syn) {
   if (Lband <= 0 || lend < 0) return;
+  struct Range { int lo, hi, j, j2; };
+  std::vector<Range> ra, rs;
+  for (int j = 0; j < MAXS; j += d.nslot) {
+    const int j2 = d.nslot == 2 ? j + 1 : -1;
+    const bool a = d.jhi[j] >= d.jlo[j], b = j2 >= 0 && j2 < MAXS && d.jhi[j2] >= d.jlo[j2];
+    if (!a && !b) continue;
+    ra.push_back({a && b ? std::min(d.jlo[j], d.jlo[j2]) : (a ? d.jlo[j] : d.jlo[j2]),
+                  a && b ? std::max(d.jhi[j], d.jhi[j2]) : (a ? d.jhi[j] : d.jhi[j2]), a ? j : -1, b ? j2 : -1});
+  }
+  for (int i = 0; i < d.nseg; ++i) {
+    const LSeg& g = d.seg[i];
+    const int n2 = d.nslot == 2 ? g.j[1] : -1;
+    auto fits = [](int cur, int next) { return cur == next || cur < 0 || next < 0; };
+    if (!rs.empty() && fits(rs.back().j, g.j[0]) && fits(rs.back().j2, n2)) {
+      rs.back().hi = g.hi;
+      rs.back().j = std::max(rs.back().j, g.j[0]);
+      rs.back().j2 = std::max(rs.back().j2, n2);
+    } else {
+      rs.push_back({g.lo, g.hi, g.j[0], n2});
+    }
+  }
   const int nb = (Lband + 31) / 32;
+  const bool both = tile_both_halves(d.N);
   for (int q = 0; q < nb; ++q)
     for (int p = 0; p <= q; ++p) {
-      const int ls = 32 * q;
-      if (ls > lend) continue;
-      const long long base = pair_run_base(p, q, table_Lmax);
-      if (two || p == q) {
-        out.push_back(PairTask{0, p, q, ls, lend, 0, base});
-      } else {
-        out.push_back(PairTask{0, p, q, ls, lend, 0, base});
-        out.push_back(PairTask{0, p, q, ls, lend, 1, base});
-      }
+      for (int half = 0; half <= (both || p == q ? 0 : 1); ++half)
+        for (int dir = 0; dir < 2; ++dir)
+          for (const Range& r : dir ? rs : ra) {
+            const int a = std::max(r.lo, 32 * q), b = std::min(r.hi, lend);
+            if (a <= b) (dir ? syn : ana).push_back(make_task(prob, p, q, half, a, b, r.j, r.j2, 0, table_Lmax));
+          }
     }
-  auto work = [two](const PairTask& t) { return (long long)(t.lend - t.lstart + 1) * (two && t.p != t.q ? 2 : 1); };
-  std::stable_sort(out.begin(), out.end(), [&](const PairTask& a, const PairTask& b) { return work(a) > work(b); });
+}
+
+// longest first (a counting sort on the length of the l range)
+void sort_tasks(std::vector<CTask>& v) {
+  int maxlen = 0;
+  for (const CTask& t : v) maxlen = std::max(maxlen, t.lend - t.lstart);
+  std::vector<size_t> at(maxlen + 2, 0);
+  for (const CTask& t : v) ++at[maxlen - (t.lend - t.lstart) + 1];
+  for (int i = 0; i <= maxlen; ++i) at[i + 1] += at[i];
+  std::vector<CTask> sorted(v.size());
+  for (const CTask& t : v) sorted[at[maxlen - (t.lend - t.lstart)]++] = t;
+  v.swap(sorted);
 }
 
 // Direct contraction tasks of one plan's wavelet scales or scaling part (d:
@@ -581,30 +624,19 @@ void build_pair_tasks(int Lband, int lend, bool two, int table_Lmax, std::vector
 // per scale over the scale's l (its [lo, hi] from the l-segments), for the
 // synthesis once per l-segment.
 void build_direct_tasks(const ContractDesc<float>& d, int prob, int Lband, int lend, int table_Lmax,
-                        std::vector<DirTask>& ana, std::vector<DirTask>& syn) {
+                        std::vector<CTask>& ana, std::vector<CTask>& syn) {
   if (Lband <= 0 || lend < 0) return;
-  int lo[MAXS], hi[MAXS], nj = 0;
-  for (int j = 0; j < MAXS; ++j) lo[j] = hi[j] = -1;
-  for (int i = 0; i < d.nseg; ++i)
-    for (int s = 0; s < d.nslot; ++s) {
-      const int j = d.seg[i].j[s];
-      if (j < 0) continue;
-      if (lo[j] < 0) lo[j] = d.seg[i].lo;
-      hi[j] = d.seg[i].hi;
-      nj = std::max(nj, j + 1);
-    }
   const int nb = (Lband + 31) / 32;
   for (int q = 0; q < nb; ++q)
     for (int p = 0; p <= q; ++p) {
-      const long long base = pair_run_base(p, q, table_Lmax);  // l = 32 q
       for (int half = 0; half <= (p == q ? 0 : 1); ++half) {
-        auto add = [&](std::vector<DirTask>& v, int a, int b, int j, int j2, int slot) {
+        auto add = [&](std::vector<CTask>& v, int a, int b, int j, int j2, int slot) {
           a = std::max(a, 32 * q);
           b = std::min(b, lend);
-          if (a <= b) v.push_back(DirTask{prob, p, q, half, a, b, j, j2, slot, 0, base + 1024LL * (a - 32 * q)});
+          if (a <= b) v.push_back(make_task(prob, p, q, half, a, b, j, j2, slot, table_Lmax));
         };
-        for (int j = 0; j < nj; ++j)
-          if (hi[j] >= 0) add(ana, lo[j], hi[j], j, -1, j % 2);
+        for (int j = 0; j < MAXS; ++j)
+          if (d.jhi[j] >= d.jlo[j]) add(ana, d.jlo[j], d.jhi[j], j, -1, j % 2);
         for (int i = 0; i < d.nseg; ++i) add(syn, d.seg[i].lo, d.seg[i].hi, d.seg[i].j[0], d.seg[i].j[1], 0);
       }
     }
@@ -616,32 +648,22 @@ void build_direct_tasks(const ContractDesc<float>& d, int prob, int Lband, int l
 // of 4 warps at rt = 1): fewer rows per thread while the tasks alone would
 // leave SMs idle (a thread's R loads serve its rt rows).  Synthesis: pieces of
 // a multiple of 16 l, about four CTAs per SM over the launch.
-int direct_split(std::vector<DirTask>& ana, std::vector<DirTask>& syn, int sms) {
+int direct_split(std::vector<CTask>& ana, std::vector<CTask>& syn, int sms) {
   const long long n = (long long)ana.size();
   long long total = 0;
-  for (const DirTask& t : syn) total += t.lend - t.lstart + 1;
+  for (const CTask& t : syn) total += t.lend - t.lstart + 1;
   const int ls = round_up((int)std::min<long long>(std::max<long long>((total + 4LL * sms - 1) / (4LL * sms), 1), 4096), 16);
-  std::vector<DirTask> cut;
-  for (const DirTask& t : syn)
+  std::vector<CTask> cut;
+  for (const CTask& t : syn)
     for (int l = t.lstart; l <= t.lend; l += ls) {
-      DirTask u = t;
-      u.lstart = l;
-      u.lend = std::min(t.lend, l + ls - 1);
-      u.dbase = t.dbase + 1024LL * (l - t.lstart);
+      CTask u = t;
+      u.lstart = (int16_t)l;
+      u.lend = (int16_t)std::min((int)t.lend, l + ls - 1);
       cut.push_back(u);
     }
   syn.swap(cut);
-  // longest first (a counting sort on the length)
-  for (std::vector<DirTask>* v : {&ana, &syn}) {
-    int maxlen = 0;
-    for (const DirTask& t : *v) maxlen = std::max(maxlen, t.lend - t.lstart);
-    std::vector<size_t> at(maxlen + 2, 0);
-    for (const DirTask& t : *v) ++at[maxlen - (t.lend - t.lstart) + 1];
-    for (int i = 0; i <= maxlen; ++i) at[i + 1] += at[i];
-    std::vector<DirTask> sorted(v->size());
-    for (const DirTask& t : *v) sorted[at[maxlen - (t.lend - t.lstart)]++] = t;
-    v->swap(sorted);
-  }
+  sort_tasks(ana);
+  sort_tasks(syn);
   return n >= 2 * sms ? 4 : (n >= sms / 2 ? 2 : 1);
 }
 
@@ -807,20 +829,20 @@ void build_segs(s2dw_plan_s* p, int job, int kind, std::vector<CztSeg<T>>& out, 
 // Build the device launch lists for a set of plans (same precision).
 template <typename T>
 Lists* build_lists(const std::vector<s2dw_plan_t>& plans) {
-  // FP32 plans run the tile-pair contraction (PairTask), FP64 plans the
-  // eighth-domain one (TileTask)
-  using Task = typename std::conditional<sizeof(T) == sizeof(float), PairTask, TileTask>::type;
+  // FP64 plans: eighth-domain tiles; FP32 plans: the tile kernel or, for small
+  // and middle band-limits, the direct one, each with its own tasks
+  using Task = TileTask;
   const int nj = (int)plans.size();
   std::vector<ContractDesc<T>> dw(nj), dp(nj);
   std::map<int, std::vector<Task>> tw_byN;
   std::vector<Task> tphi;
-  struct DirBuild {  // direct FP32 contraction: analysis and synthesis tasks
-    std::vector<DirTask> task[2];
+  struct FpTasks {  // FP32 contraction: analysis and synthesis tasks
+    std::vector<CTask> task[2];
     int rt = 4;
     size_t off[2] = {0, 0};
   };
-  std::map<int, DirBuild> dir_byN;
-  DirBuild dir_phi;
+  std::map<int, FpTasks> dir_byN, tile_byN;
+  FpTasks dir_phi, tile_phi;
   std::vector<CztSeg<T>> segs[Lists::NK];
   int start[Lists::NK] = {};
   Lists* ls = new Lists();
@@ -829,34 +851,24 @@ Lists* build_lists(const std::vector<s2dw_plan_t>& plans) {
     s2dw_plan_s* p = plans[i];
     std::memcpy(&dw[i], p->desc_w_host.data(), sizeof(ContractDesc<T>));
     std::memcpy(&dp[i], p->desc_phi_host.data(), sizeof(ContractDesc<T>));
-    const std::vector<Task>* tws;
-    const std::vector<Task>* tps;
     if constexpr (sizeof(T) == sizeof(float)) {
-      tws = &p->ptasks_w_host;
-      tps = &p->ptasks_phi_host;
-    } else {
-      tws = &p->tiles_w_host;
-      tps = &p->tiles_phi_host;
+      FpTasks& w = (p->direct_w ? dir_byN : tile_byN)[p->N];
+      (p->direct_w ? build_direct_tasks : build_tile_tasks)(dw[i], i, p->L0, p->lend_w, p->tab->Lmax, w.task[0], w.task[1]);
+      FpTasks& f = p->direct_phi ? dir_phi : tile_phi;
+      (p->direct_phi ? build_direct_tasks : build_tile_tasks)(dp[i], i, p->Lphi, p->lphi, p->tab->Lmax, f.task[0], f.task[1]);
     }
-    const int key = p->N | ((sizeof(T) == sizeof(float)) ? (p->pair_shape << kShapeShift) : 0);
-    if constexpr (sizeof(T) == sizeof(float)) {
-      if (p->direct_w)
-        build_direct_tasks(dw[i], i, p->L0, p->lend_w, p->tab->Lmax, dir_byN[p->N].task[0], dir_byN[p->N].task[1]);
-      if (p->direct_phi)
-        build_direct_tasks(dp[i], i, p->Lphi, p->lphi, p->tab->Lmax, dir_phi.task[0], dir_phi.task[1]);
-    }
-    for (Task t : *tws) {  // (empty where the direct contraction runs)
+    for (Task t : p->tiles_w_host) {  // (FP64 plans)
       t.prob = i;
-      tw_byN[key].push_back(t);
+      tw_byN[p->N].push_back(t);
     }
-    for (Task t : *tps) {
+    for (Task t : p->tiles_phi_host) {
       t.prob = i;
       tphi.push_back(t);
     }
     for (int k = 0; k < Lists::NK; ++k) build_segs<T>(p, i, k, segs[k], start[k]);
     ls->maxlogM = std::max(ls->maxlogM, p->logM);
     ls->Lmax = std::max(ls->Lmax, p->L);
-    if (p->fP) {  // packed f: plans with a tile-pair contraction
+    if (p->fP) {  // packed f: plans that run the tile contraction
       ls->nbmax = std::max(ls->nbmax, (p->L + 31) / 32);
       ls->Lrmax = std::max(ls->Lrmax, p->Lrf);
     }
@@ -884,30 +896,24 @@ Lists* build_lists(const std::vector<s2dw_plan_t>& plans) {
       if (sg.logM != u) u = 0;
     ls->ulogM[k] = u;
   }
-  // longest tasks first (a CTA computing both tiles of a pair counts double)
-  auto by_work = [](std::vector<Task>& v, int key) {
-    if constexpr (sizeof(T) == sizeof(float)) {
-      const bool two = (key >> kShapeShift) == kPairShapePair;
-      auto work = [two](const PairTask& t) {
-        return (long long)(t.lend - t.lstart + 1) * (two && t.p != t.q ? 2 : 1);
-      };
-      std::stable_sort(v.begin(), v.end(), [&](const PairTask& a, const PairTask& b) { return work(a) > work(b); });
-    } else {
-      (void)key;
-      sort_tiles(v);
-    }
-  };
-  for (auto& kv : tw_byN) by_work(kv.second, kv.first);
-  by_work(tphi, 1);
+  for (auto& kv : tw_byN) sort_tiles(kv.second);
+  sort_tiles(tphi);
   int sms = 152;
   {
     int dev = 0;
     if (cudaGetDevice(&dev) == cudaSuccess) cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
   }
-  std::vector<DirBuild*> dirs;
-  for (auto& kv : dir_byN) dirs.push_back(&kv.second);
-  dirs.push_back(&dir_phi);  // always the last
-  for (DirBuild* b : dirs) b->rt = direct_split(b->task[0], b->task[1], sms);
+  std::vector<FpTasks*> fp;
+  for (auto& kv : dir_byN) fp.push_back(&kv.second);
+  fp.push_back(&dir_phi);
+  for (FpTasks* b : fp) b->rt = direct_split(b->task[0], b->task[1], sms);
+  const size_t ndir = fp.size();
+  for (auto& kv : tile_byN) fp.push_back(&kv.second);
+  fp.push_back(&tile_phi);
+  for (size_t i = ndir; i < fp.size(); ++i) {
+    sort_tasks(fp[i]->task[0]);
+    sort_tasks(fp[i]->task[1]);
+  }
   // one allocation for everything
   size_t off = 0;
   const size_t o_dw = off;
@@ -921,10 +927,10 @@ Lists* build_lists(const std::vector<s2dw_plan_t>& plans) {
   }
   const size_t o_tp = off;
   off = align256(off + tphi.size() * sizeof(Task));
-  for (DirBuild* b : dirs)
+  for (FpTasks* b : fp)
     for (int d = 0; d < 2; ++d) {
       b->off[d] = off;
-      off = align256(off + b->task[d].size() * sizeof(DirTask));
+      off = align256(off + b->task[d].size() * sizeof(CTask));
     }
   size_t o_sg[Lists::NK];
   for (int k = 0; k < Lists::NK; ++k) {
@@ -940,9 +946,9 @@ Lists* build_lists(const std::vector<s2dw_plan_t>& plans) {
     ++q;
   }
   if (!tphi.empty()) std::memcpy(host.data() + o_tp, tphi.data(), tphi.size() * sizeof(Task));
-  for (DirBuild* b : dirs)
+  for (FpTasks* b : fp)
     for (int d = 0; d < 2; ++d)
-      if (!b->task[d].empty()) std::memcpy(host.data() + b->off[d], b->task[d].data(), b->task[d].size() * sizeof(DirTask));
+      if (!b->task[d].empty()) std::memcpy(host.data() + b->off[d], b->task[d].data(), b->task[d].size() * sizeof(CTask));
   for (int k = 0; k < Lists::NK; ++k)
     if (!segs[k].empty()) std::memcpy(host.data() + o_sg[k], segs[k].data(), segs[k].size() * sizeof(CztSeg<T>));
   try {
@@ -964,8 +970,8 @@ Lists* build_lists(const std::vector<s2dw_plan_t>& plans) {
   }
   ls->tiles_phi = base + o_tp;
   ls->ntiles_phi = (int)tphi.size();
-  auto dir_group = [&](int N, const DirBuild& b) {
-    Lists::DirGroup g;
+  auto group = [&](int N, const FpTasks& b) {
+    Lists::FpGroup g;
     g.N = N;
     g.rt = b.rt;
     for (int d = 0; d < 2; ++d) {
@@ -974,8 +980,10 @@ Lists* build_lists(const std::vector<s2dw_plan_t>& plans) {
     }
     return g;
   };
-  for (auto& kv : dir_byN) ls->dir_w.push_back(dir_group(kv.first, kv.second));
-  ls->dir_phi = dir_group(1, dir_phi);
+  for (auto& kv : dir_byN) ls->dir_w.push_back(group(kv.first, kv.second));
+  for (auto& kv : tile_byN) ls->tile_w.push_back(group(kv.first, kv.second));
+  ls->dir_phi = group(1, dir_phi);
+  ls->tile_phi = group(1, tile_phi);
   for (int k = 0; k < Lists::NK; ++k) {
     ls->segs[k] = base + o_sg[k];
     ls->nseg[k] = (int)segs[k].size();
@@ -1007,12 +1015,12 @@ int direct_groups(const Lists& ls) { return (int)ls.dir_w.size() + (ls.dir_w.emp
 void run_direct(const Lists& ls, bool syn, const ContractDesc<float>* dw, const ContractDesc<float>* dp,
                 const CallPtrs& ptrs, cudaStream_t st) {
   const int d = syn ? 1 : 0;
-  const DirTasks phi{dp, reinterpret_cast<const DirTask*>(ls.dir_phi.task[d]), ls.dir_phi.n[d]};
+  const DirTasks phi{dp, reinterpret_cast<const CTask*>(ls.dir_phi.task[d]), ls.dir_phi.n[d]};
   DirTasks none = phi;
   none.n = 0;
   bool first = true;
   for (const auto& g : ls.dir_w) {
-    launch_contract_direct(g.N, syn, g.rt, DirTasks{dw, reinterpret_cast<const DirTask*>(g.task[d]), g.n[d]},
+    launch_contract_direct(g.N, syn, g.rt, DirTasks{dw, reinterpret_cast<const CTask*>(g.task[d]), g.n[d]},
                            first ? phi : none, ptrs, st);
     first = false;
   }
@@ -1037,12 +1045,10 @@ void run_analysis(const Lists& ls, const CallPtrs& ptrs, cudaStream_t st, cudaEv
   if constexpr (sizeof(T) == sizeof(float)) {
     launch_fpack(dw, ls.njobs, ls.nbmax, ls.Lrmax, ptrs, st);
     run_direct(ls, false, dw, dp, ptrs, st);
-    for (auto& t : ls.tiles_w)
-      launch_contract_pair(t.first & 0xff, 2, false, t.first >> kShapeShift, dw,
-                           reinterpret_cast<const PairTask*>(t.second.first), t.second.second, ptrs, st);
+    for (auto& g : ls.tile_w)
+      launch_contract_tile(g.N, 2, false, dw, reinterpret_cast<const CTask*>(g.task[0]), g.n[0], st);
     rec(ev, 1, st);
-    launch_contract_pair(1, 1, false, kPairShapePair, dp, reinterpret_cast<const PairTask*>(ls.tiles_phi), ls.ntiles_phi, ptrs,
-                         st);
+    launch_contract_tile(1, 1, false, dp, reinterpret_cast<const CTask*>(ls.tile_phi.task[0]), ls.tile_phi.n[0], st);
   } else {
     for (auto& t : ls.tiles_w)
       launch_contract<T>(t.first, 2, false, dw, reinterpret_cast<const TileTask*>(t.second.first), t.second.second,
@@ -1101,12 +1107,10 @@ void run_synthesis(const Lists& ls, const CallPtrs& ptrs, const ReduceJobs& rj, 
   rec(ev, 4, st);
   if constexpr (sizeof(T) == sizeof(float)) {
     run_direct(ls, true, dw, dp, ptrs, st);
-    for (auto& t : ls.tiles_w)
-      launch_contract_pair(t.first & 0xff, 2, true, t.first >> kShapeShift, dw,
-                           reinterpret_cast<const PairTask*>(t.second.first), t.second.second, ptrs, st);
+    for (auto& g : ls.tile_w)
+      launch_contract_tile(g.N, 2, true, dw, reinterpret_cast<const CTask*>(g.task[1]), g.n[1], st);
     rec(ev, 5, st);
-    launch_contract_pair(1, 1, true, kPairShapePair, dp, reinterpret_cast<const PairTask*>(ls.tiles_phi), ls.ntiles_phi, ptrs,
-                         st);
+    launch_contract_tile(1, 1, true, dp, reinterpret_cast<const CTask*>(ls.tile_phi.task[1]), ls.tile_phi.n[1], st);
   } else {
     for (auto& t : ls.tiles_w)
       launch_contract<T>(t.first, 2, true, dw, reinterpret_cast<const TileTask*>(t.second.first), t.second.second,
@@ -1135,7 +1139,9 @@ void own_lists_build(s2dw_plan_s* p) {
   p->own.tiles_phi = ls->tiles_phi;
   p->own.ntiles_phi = ls->ntiles_phi;
   p->own.dir_w = ls->dir_w;
+  p->own.tile_w = ls->tile_w;
   p->own.dir_phi = ls->dir_phi;
+  p->own.tile_phi = ls->tile_phi;
   for (int k = 0; k < Lists::NK; ++k) {
     p->own.segs[k] = ls->segs[k];
     p->own.nseg[k] = ls->nseg[k];
@@ -1163,9 +1169,9 @@ void plan_build_typed(s2dw_plan_s* p, const double* kap_d, const double* phi_d, 
     off = align256(off + bytes);
     return o;
   };
-  const bool pairc = sizeof(T) == sizeof(float);  // tile-pair contraction (FP32 plans)
+  const bool pairc = sizeof(T) == sizeof(float);  // FP32 contraction (pair table)
   const int NH = (N + 1) / 2;
-  p->Lr = L + kPairPadL;  // read-ahead rows of the tile-pair contraction
+  p->Lr = L + kPairPadL;  // read-ahead rows of the tile contraction
   p->Lrphi = p->Lphi + kPairPadL;
   p->Lrf = L + kPairPadL;
   const int nbw = (L + 31) / 32, nbp = (p->Lphi + 31) / 32;
@@ -1414,12 +1420,9 @@ void plan_build_typed(s2dw_plan_s* p, const double* kap_d, const double* phi_d, 
       ck(cudaGetDevice(&dev));
       ck(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
       const long long nbk = (p->L0 + 31) / 32, npairs = nbk * (nbk + 1) / 2;
-      if (!pair_two_tiles(N) || npairs < 3LL * sms) p->pair_shape = kPairShapeTile;
+      if (!pair_shapes_offered(N) || npairs < 3LL * sms) p->pair_shape = kPairShapeTile;
       else p->pair_shape = N >= 4 ? kPairShapePair : kPairShapeTile2;
     }
-    if (!p->direct_w)
-      build_pair_tasks(p->L0, p->lend_w, p->pair_shape == kPairShapePair, p->tab->Lmax, p->ptasks_w_host);
-    if (!p->direct_phi) build_pair_tasks(p->Lphi, p->lphi, true, p->tab->Lmax, p->ptasks_phi_host);
   } else {
     build_tiles(p->L0, p->lend_w, p->TMP, 0, p->tiles_w_host);
     build_tiles(p->Lphi, p->lphi, p->TMP, 0, p->tiles_phi_host);
@@ -1787,7 +1790,7 @@ static bool choice_valid(s2dw_plan_t p, int idx, int v) {
   if (idx < 2) return v == 0 || v == 1;  // grids without half-length transforms keep the FFT
   if (idx == choices_count(p) - 1) {  // contraction CTA shape (FP32 plans with N <= 5 have three)
     if (p->fp64) return v == 0;
-    return pair_two_tiles(p->N) ? (v >= kPairShapePair && v <= kPairShapeTile2) : v == kPairShapeTile;
+    return pair_shapes_offered(p->N) ? (v >= kPairShapePair && v <= kPairShapeTile2) : v == kPairShapeTile;
   }
   const int j = (idx - 2) / 2, d = (idx - 2) % 2;
   const int Lj = p->Ycols[j];
@@ -1814,14 +1817,7 @@ static void choices_put(s2dw_plan_t p, const int* c) {
     p->alpha_mode[0][j] = c[2 + 2 * j];
     p->alpha_mode[1][j] = c[3 + 2 * j];
   }
-  if (!p->fp64) {
-    const int shape = c[choices_count(p) - 1];
-    if (shape != p->pair_shape) {
-      p->pair_shape = shape;
-      if (!p->direct_w)
-        build_pair_tasks(p->L0, p->lend_w, shape == kPairShapePair, p->tab->Lmax, p->ptasks_w_host);
-    }
-  }
+  if (!p->fp64) p->pair_shape = c[choices_count(p) - 1];
   drop_batches_with(p);
   if (p->fp64) own_lists_build<double>(p);
   else own_lists_build<float>(p);
@@ -1983,21 +1979,6 @@ int s2dw_plan_tune(s2dw_plan_t p, int reps, int* choices, int* n) {
           }
         }
       }
-    // the contraction's CTA shape (both directions)
-    {
-      const int idx = nc - 1;
-      for (int v = 0; v < 3; ++v) {
-        if (v == cur[idx] || !choice_valid(p, idx, v)) continue;
-        std::vector<int> trial(cur);
-        trial[idx] = v;
-        choices_put(p, trial.data());
-        double ms[5];
-        if (better(ms, 4, base)) {
-          cur = trial;
-          base[4] = ms[4];
-        }
-      }
-    }
     choices_put(p, cur.data());
     ck(cudaStreamSynchronize(st));
   } catch (const CudaFail& e) {
@@ -2048,7 +2029,8 @@ int s2dw_wait_probe(long long limit_cycles, void* stream) {
 int s2dw_launch_counts(s2dw_plan_t p, int* analysis, int* synthesis) {
   if (!p) return S2DW_EINVAL;
   const Lists& ls = p->own;
-  int contract = (ls.ntiles_phi > 0 ? 1 : 0) + direct_groups(ls);
+  int contract = (ls.ntiles_phi > 0 ? 1 : 0) + direct_groups(ls) + (ls.tile_phi.n[0] > 0 ? 1 : 0);
+  for (auto& g : ls.tile_w) contract += g.n[0] > 0 ? 1 : 0;
   for (auto& t : ls.tiles_w) contract += t.second.second > 0 ? 1 : 0;
   auto has = [&](int k) {
     if (k >= CZT_BETA_ANA_DCT && k <= CZT_BETA_RS_DCT) return (int)ls.dct_parts[k - CZT_BETA_ANA_DCT].size();

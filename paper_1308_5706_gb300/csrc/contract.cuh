@@ -42,6 +42,63 @@ constexpr int kMaxStages = 8;
 constexpr size_t kCtaSmemBudget = 112 * 1024;  // two CTAs per SM (228 KB, 1 KB reserved each)
 
 
+// Gamma step of one element (Eq. (28)) from its two parity banks: b0 holds the
+// sums over the l of l_start's parity, b1 the others, orders n_k >= 0.  With
+// G_{+n} = b0 + b1, G_{-n} = sgn (b0 - b1), sgn = (-1)^{m' + l_start}, and the
+// factors conj(eta) i^{+-n} e^{+-in gamma} = eps (cos + i sin), tau eps (cos - i
+// sin) (eps = +-1, tau = (-1)^{N-1}), an order pair contributes
+//   2 eps (P cos + i Q sin), (P, Q) = (b0, b1) if tau sgn = 1 else (b1, b0):
+// four multiply-adds per pair and sample.  cg[k N + g]: the factors of n_k.
+// (Fused operations are explicit, so that every instantiation rounds alike: a
+// batched call equals the single one bit for bit.)
+template <int N>
+__device__ __forceinline__ void gamma_ana(const float2 (&b0)[(N + 1) / 2], const float2 (&b1)[(N + 1) / 2], bool plus,
+                                          const float2* cg, float2 (&y)[N]) {
+  constexpr int NH = (N + 1) / 2, ZH = N & 1;
+  float2 P[NH], Q[NH];
+#pragma unroll
+  for (int q = ZH; q < NH; ++q) {
+    const float2 p = plus ? b0[q] : b1[q], r = plus ? b1[q] : b0[q];
+    P[q] = make_float2(2.f * p.x, 2.f * p.y);
+    Q[q] = make_float2(2.f * r.x, 2.f * r.y);
+  }
+#pragma unroll
+  for (int g = 0; g < N; ++g) {
+    float2 z = ZH ? make_float2(b0[0].x + b1[0].x, b0[0].y + b1[0].y) : make_float2(0.f, 0.f);
+#pragma unroll
+    for (int q = ZH; q < NH; ++q) {
+      const float2 c = cg[(N / 2 + q) * N + g];
+      z.x = __fmaf_rn(P[q].x, c.x, z.x);
+      z.x = __fmaf_rn(-Q[q].y, c.y, z.x);
+      z.y = __fmaf_rn(P[q].y, c.x, z.y);
+      z.y = __fmaf_rn(Q[q].x, c.y, z.y);
+    }
+    y[g] = z;
+  }
+}
+
+// Its adjoint (Eq. (39)): one bank's share of sample g, value v (with i^m and
+// the tile's sign applied): 2 Re(factor) v where plus (tau sgn = 1, with
+// l_start's parity or the other one for the other bank), else 2 i Im(factor) v;
+// n = 0: the factor itself.
+template <int N>
+__device__ __forceinline__ void gamma_syn_add(float2 (&h)[(N + 1) / 2], float2 v, bool plus, const float2* cg, int g) {
+  constexpr int NH = (N + 1) / 2, ZH = N & 1;
+  if (ZH) {
+    const float c = cg[(N / 2) * N + g].x;
+    h[0].x = __fmaf_rn(v.x, c, h[0].x);
+    h[0].y = __fmaf_rn(v.y, c, h[0].y);
+  }
+  const float2 u = plus ? make_float2(2.f * v.x, 2.f * v.y) : make_float2(-2.f * v.y, 2.f * v.x);
+#pragma unroll
+  for (int q = ZH; q < NH; ++q) {
+    const float2 f = cg[(N / 2 + q) * N + g];
+    const float c = plus ? f.x : f.y;
+    h[q].x = __fmaf_rn(u.x, c, h[q].x);
+    h[q].y = __fmaf_rn(u.y, c, h[q].y);
+  }
+}
+
 // E consecutive values from 16-byte aligned shared memory.
 template <typename T, int E> struct VecLdS;
 template <> struct VecLdS<float, 4> {

@@ -1,11 +1,11 @@
 // FP32 l-contraction for small and middle band-limits (Sec. 3.2 Eq. (27);
-// Sec. 3.3 Eqs. (34), (32)): the sums of contract_pair.cuh, organised for
+// Sec. 3.3 Eqs. (34), (32)): the sums of contract_tile.cuh, organised for
 // latency instead of for one long stream per CTA.
 //
 // What bounds it.  At L <= kContractDirectMaxL a whole contraction is a few
-// microseconds of FP32 work; the tile-pair ring kernel has one CTA per 32 x 32
-// tile (pair) and walks its l one stage after the other, so at L = 128 it kept
-// 16 of 152 SMs busy for 128 dependent steps.  Here
+// microseconds of FP32 work; a ring kernel with one CTA per 32 x 32 tile (pair)
+// walks its l one stage after the other, at L = 128 on 16 of 152 SMs for 128
+// dependent steps.  Here
 //   analysis: a task is one scale of one tile over that scale's own l range, so
 //     the scales run side by side and the gamma step runs once, at the end; a
 //     thread owns RT rows x 1 column and keeps its accumulators; a task is cut
@@ -44,16 +44,6 @@ __device__ __forceinline__ void cp_async8_zf(void* smem, const void* gmem, int s
   asm volatile("cp.async.ca.shared.global [%0], [%1], 8, %2;\n" ::"r"(s), "l"(gmem), "r"(src_bytes) : "memory");
 }
 
-// c + a b, complex, with the fused order fixed (so that every instantiation
-// rounds alike: a batched call equals the single one bit for bit)
-__device__ __forceinline__ float2 cfma_rn(float2 a, float2 b, float2 c) {
-  c.x = __fmaf_rn(a.x, b.x, c.x);
-  c.y = __fmaf_rn(a.x, b.y, c.y);
-  c.x = __fmaf_rn(-a.y, b.y, c.x);
-  c.y = __fmaf_rn(a.y, b.x, c.y);
-  return c;
-}
-
 template <int RT>
 __device__ __forceinline__ void lds_rows(const float* p, float (&r)[RT]) {
   if constexpr (RT == 4) {
@@ -70,7 +60,7 @@ __device__ __forceinline__ void lds_rows(const float* p, float (&r)[RT]) {
 // One scale of one tile: G^j over l in [lstart, lend], then the gamma step.
 // nslot: slots of the R rows (the scale's values sit in slot tk.slot).
 template <int N, int RT, int NW, bool ISB>
-__device__ __forceinline__ void dir_ana_tile(const ContractDesc<float>* __restrict__ D, int nslot, const DirTask& tk, int sub,
+__device__ __forceinline__ void dir_ana_tile(const ContractDesc<float>* __restrict__ D, int nslot, const CTask& tk, int sub,
                                              const float2* __restrict__ f, float2* cg, float* Rs0, float2* fs0) {
   constexpr int NH = (N + 1) / 2, ZH = N & 1, NP = N / 2, RW = NH * 32, LC = kDirLC;
   constexpr int NTH = 32 * NW, U = RT == 4 ? 4 : 8;
@@ -78,7 +68,7 @@ __device__ __forceinline__ void dir_ana_tile(const ContractDesc<float>* __restri
   const int t = threadIdx.x, w = t >> 5, lane = t & 31;
   const int rw = (sub * NW + w) * RT;  // first row of the stored block
   const int l_start = tk.lstart, l_end = tk.lend, rrow = nslot * RW;
-  const float* __restrict__ dp = D->dpair + tk.dbase + rw * 32 + lane;
+  const float* __restrict__ dp = D->dpair + tk.dbase() + rw * 32 + lane;
   const float* __restrict__ Rg = D->RSp + ((size_t)(ISB ? tk.q : tk.p) * D->Lr + l_start) * rrow + tk.slot * RW;
   const int mb = 32 * (ISB ? tk.p : tk.q);  // m block of f
   const int Lj = D->Lj[tk.j];
@@ -171,48 +161,43 @@ __device__ __forceinline__ void dir_ana_tile(const ContractDesc<float>* __restri
     }
   }
 
-  // gamma step (Eq. (28)): G_{+n} = B0 + B1, G_{-n} = (-1)^{m' + lstart} (B0 - B1)
-  // from the sums over the l of lstart's parity (B0) and of the other (B1)
+  // gamma step (Eq. (28)) from the sums over the l of lstart's parity and of the other
 #pragma unroll
   for (int e = 0; e < RT; ++e) {
     const int mp = ISB ? 32 * tk.q + lane : 32 * tk.p + rw + e;
     const int m = ISB ? 32 * tk.p + rw + e : 32 * tk.q + lane;
     if (mp >= Lj || m >= Lj) continue;
-    float2 gk[N];
-    if (ZH) gk[N / 2] = make_float2(ax[e][2 * NP], ay[e][2 * NP]);
-    const float sgn = ((mp + l_start) & 1) ? -1.f : 1.f;
+    float2 b0[NH], b1[NH], y[N];
 #pragma unroll
-    for (int p = 0; p < NP; ++p) {
-      gk[(N + 1) / 2 + p] = make_float2(ax[e][p] + ax[e][NP + p], ay[e][p] + ay[e][NP + p]);
-      gk[N / 2 - 1 - p] = make_float2(sgn * (ax[e][p] - ax[e][NP + p]), sgn * (ay[e][p] - ay[e][NP + p]));
+    for (int h = 0; h < NH; ++h) {
+      const int q0 = (ZH && h == 0) ? 2 * NP : h - ZH, q1 = (ZH && h == 0) ? -1 : NP + h - ZH;
+      b0[h] = make_float2(ax[e][q0], ay[e][q0]);
+      b1[h] = q1 < 0 ? make_float2(0.f, 0.f) : make_float2(ax[e][q1 < 0 ? 0 : q1], ay[e][q1 < 0 ? 0 : q1]);
     }
+    gamma_ana<N>(b0, b1, ((mp + l_start + N - 1) & 1) == 0, cg, y);
     const float fs = (ISB && ((mp + m) & 1)) ? -1.f : 1.f;
 #pragma unroll
-    for (int g = 0; g < N; ++g) {
-      float2 v = make_float2(0.f, 0.f);
-#pragma unroll
-      for (int k = 0; k < N; ++k) v = cfma_rn(gk[k], cg[k * N + g], v);
-      Y[((size_t)g * Lj + m) * Lj + mp] = cscale<float>(cmul_ipow<float>(v, (-m) & 3), fs);
-    }
+    for (int g = 0; g < N; ++g)
+      Y[((size_t)g * Lj + m) * Lj + mp] = cscale<float>(cmul_ipow<float>(y[g], (-m) & 3), fs);
   }
 }
 
 template <int N, int RT, int NW>
 __global__ void __launch_bounds__(32 * NW)
-k_contract_dir_ana(const ContractDesc<float>* __restrict__ dw, const DirTask* __restrict__ tw, int nw,
-                   const ContractDesc<float>* __restrict__ dphi, const DirTask* __restrict__ tp, CallPtrs ptrs) {
+k_contract_dir_ana(const ContractDesc<float>* __restrict__ dw, const CTask* __restrict__ tw, int nw,
+                   const ContractDesc<float>* __restrict__ dphi, const CTask* __restrict__ tp, CallPtrs ptrs) {
   constexpr int SUB = 32 / (RT * NW), RW = ((N + 1) / 2) * 32;
   __shared__ float2 cg[64];
   __shared__ __align__(16) float Rs[2 * kDirLC * RW];
   __shared__ __align__(16) float2 fs[2 * kDirLC * 32];
   const int i = blockIdx.x / SUB, sub = blockIdx.x % SUB;
   if (i < nw) {
-    const DirTask tk = tw[i];
+    const CTask tk = tw[i];
     const float2* f = reinterpret_cast<const float2*>(ptrs.f[tk.prob]);
     if (tk.half == 0) dir_ana_tile<N, RT, NW, false>(dw + tk.prob, 2, tk, sub, f, cg, Rs, fs);
     else dir_ana_tile<N, RT, NW, true>(dw + tk.prob, 2, tk, sub, f, cg, Rs, fs);
   } else {
-    const DirTask tk = tp[i - nw];
+    const CTask tk = tp[i - nw];
     const float2* f = reinterpret_cast<const float2*>(ptrs.f[tk.prob]);
     if (tk.half == 0) dir_ana_tile<1, RT, NW, false>(dphi + tk.prob, 1, tk, sub, f, cg, Rs, fs);
     else dir_ana_tile<1, RT, NW, true>(dphi + tk.prob, 1, tk, sub, f, cg, Rs, fs);
@@ -225,14 +210,14 @@ k_contract_dir_ana(const ContractDesc<float>* __restrict__ dw, const DirTask* __
 // shared memory; tile B's rows m' are the lanes: a butterfly that halves the
 // values with the lanes leaves one column part per four lanes.
 template <int N, int NSLOT, bool ISB>
-__device__ __forceinline__ void dir_syn_tile(const ContractDesc<float>* __restrict__ D, const DirTask& tk, float2* cg,
+__device__ __forceinline__ void dir_syn_tile(const ContractDesc<float>* __restrict__ D, const CTask& tk, float2* cg,
                                              float* Rs0, float2* red) {
   constexpr int NH = (N + 1) / 2, ZH = N & 1, NP = N / 2, RROW = NSLOT * NH * 32, LC = kDirLC;
   constexpr int NTH = 256, RT = 4, U = 4;
   const int t = threadIdx.x, w = t >> 5, lane = t & 31, rw = 4 * w;
   const int l_start = tk.lstart, l_end = tk.lend;
   const int rb = ISB ? tk.q : tk.p, cb = ISB ? tk.p : tk.q, L = D->L, Lp32 = D->Lp32;
-  const float* __restrict__ dp = D->dpair + tk.dbase + rw * 32 + lane;
+  const float* __restrict__ dp = D->dpair + tk.dbase() + rw * 32 + lane;
   const float* __restrict__ Rg = D->RSp + ((size_t)rb * D->Lr + l_start) * RROW;
   float2* __restrict__ P = D->P + ((size_t)rb * L + l_start) * Lp32 + 32 * cb;
 
@@ -269,31 +254,28 @@ __device__ __forceinline__ void dir_syn_tile(const ContractDesc<float>* __restri
     for (int e = 0; e < RT; ++e) {
       const int mp = ISB ? 32 * tk.q + lane : 32 * tk.p + rw + e;
       const int m = ISB ? 32 * tk.p + rw + e : 32 * tk.q + lane;
-      float2 h[N];
+      float2 h0[NH], h1[NH];  // banks of lstart's parity and of the other
 #pragma unroll
-      for (int k = 0; k < N; ++k) h[k] = make_float2(0.f, 0.f);
+      for (int h = 0; h < NH; ++h) h0[h] = h1[h] = make_float2(0.f, 0.f);
       if (mp < Lj && m < Lj) {
         float2 vg[N];
 #pragma unroll
         for (int g = 0; g < N; ++g) vg[g] = V[((size_t)g * Lj + mp) * Lj + m];
-#pragma unroll
-        for (int g = 0; g < N; ++g)
-#pragma unroll
-          for (int k = 0; k < N; ++k) h[k] = cfma_rn(vg[g], cg[k * N + g], h[k]);
         const float fs = (ISB && ((mp + m) & 1)) ? -1.f : 1.f;
+        const bool plus = ((mp + l_start + N - 1) & 1) == 0;
 #pragma unroll
-        for (int k = 0; k < N; ++k) h[k] = cscale<float>(cmul_ipow<float>(h[k], m & 3), fs);
+        for (int g = 0; g < N; ++g) {
+          const float2 v = cscale<float>(cmul_ipow<float>(vg[g], m & 3), fs);
+          gamma_syn_add<N>(h0, v, plus, cg, g);
+          gamma_syn_add<N>(h1, v, !plus, cg, g);
+        }
       }
-      const float sgn = ((mp + l_start) & 1) ? -1.f : 1.f;
 #pragma unroll
-      for (int p = 0; p < NP; ++p) {
-        const float2 hp = h[(N + 1) / 2 + p], hm = h[N / 2 - 1 - p];
-        hx[e][s][p] = hp.x + sgn * hm.x;
-        hy[e][s][p] = hp.y + sgn * hm.y;
-        hx[e][s][NP + p] = hp.x - sgn * hm.x;
-        hy[e][s][NP + p] = hp.y - sgn * hm.y;
+      for (int h = 0; h < NH; ++h) {
+        const int q0 = (ZH && h == 0) ? 2 * NP : h - ZH;
+        hx[e][s][q0] = h0[h].x, hy[e][s][q0] = h0[h].y;
+        if (!(ZH && h == 0)) hx[e][s][q0 + NP] = h1[h].x, hy[e][s][q0 + NP] = h1[h].y;
       }
-      if (ZH) hx[e][s][2 * NP] = h[N / 2].x, hy[e][s][2 * NP] = h[N / 2].y;
     }
   }
   auto compute = [&](const float* Rl, int li, int l, auto uu) {
@@ -387,19 +369,19 @@ constexpr size_t dir_syn_smem() {
 
 template <int N>
 __global__ void __launch_bounds__(256)
-k_contract_dir_syn(const ContractDesc<float>* __restrict__ dw, const DirTask* __restrict__ tw, int nw,
-                   const ContractDesc<float>* __restrict__ dphi, const DirTask* __restrict__ tp) {
+k_contract_dir_syn(const ContractDesc<float>* __restrict__ dw, const CTask* __restrict__ tw, int nw,
+                   const ContractDesc<float>* __restrict__ dphi, const CTask* __restrict__ tp) {
   extern __shared__ __align__(16) unsigned char dir_smem[];
   __shared__ float2 cg[64];
   float2* red = reinterpret_cast<float2*>(dir_smem);
   float* Rs = reinterpret_cast<float*>(dir_smem + (size_t)kDirLC * 8 * 32 * sizeof(float2));
   const int i = blockIdx.x;
   if (i < nw) {
-    const DirTask tk = tw[i];
+    const CTask tk = tw[i];
     if (tk.half == 0) dir_syn_tile<N, 2, false>(dw + tk.prob, tk, cg, Rs, red);
     else dir_syn_tile<N, 2, true>(dw + tk.prob, tk, cg, Rs, red);
   } else {
-    const DirTask tk = tp[i - nw];
+    const CTask tk = tp[i - nw];
     if (tk.half == 0) dir_syn_tile<1, 1, false>(dphi + tk.prob, tk, cg, Rs, red);
     else dir_syn_tile<1, 1, true>(dphi + tk.prob, tk, cg, Rs, red);
   }

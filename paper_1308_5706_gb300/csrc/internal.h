@@ -1,6 +1,8 @@
 // Internal descriptors shared by the plan, the launchers and the kernels.
 #pragma once
 
+#include <cstdint>
+
 #include "common.cuh"
 
 namespace s2dw {
@@ -22,10 +24,10 @@ struct LSeg {
 template <typename T>
 struct ContractDesc {
   const T* delta;    // Delta table (padded eighth domain), working precision
-  // FP32 plans (tile-pair contraction, contract_pair.cuh):
+  // FP32 plans (contract_tile.cuh, contract_direct.cu):
   const float* dpair;  // Delta pair table of the plan's shared table
   const float* RSp;    // [nb][Lr][nslot][(N+1)/2][32]: R rows per 32-block of m', l outermost
-  const cx<T>* fP;     // [nb][Lrf][32]: f_lm per 32-block of m (zero for m > l), packed per call
+  const cx<T>* fP;     // [nb][Lrf][re, im][32] (as floats): f_lm per 32-block of m (zero for m > l), packed per call
   int Lr, Lrf;         // l rows of RSp and fP (>= L + 7: a stage may read seven l past the last)
   const T* RS;       // [L][nslot][(N+1)/2][Lp]: Delta^l_{m',n_k} kappa^j(l) |s_{l,n_k}|, n_k >= 0
   cx<T>* P;          // synthesis partials [nbr][L][Lp32]
@@ -38,20 +40,10 @@ struct ContractDesc {
   int Lj[MAXS];            // per scale band-limit (support hi + 1)
   cx<T>* Y[MAXS];          // per scale cube [N][Lj][Lj] (analysis out / synthesis in)
   LSeg seg[2 * MAXS + 2];
+  int jlo[MAXS], jhi[MAXS];  // per scale first and last l with a nonzero kernel (empty: jhi < jlo)
 };
 
-// One tile pair of the FP32 contraction: blocks p <= q of 32 rows / columns;
-// tile A = (m' block p, m block q), tile B = (q, p).  dbase: entry of the
-// pair table holding l = lstart = 32 q (1024 entries per l follow).
-struct PairTask {
-  int prob;
-  int p, q;
-  int lstart, lend;
-  int half;  // one-tile launches (N > 5): 0 = tile A, 1 = tile B
-  long long dbase;
-};
-
-// l rows of padding after the tables the tile-pair contraction streams (the
+// l rows of padding after the tables the FP32 contraction streams (the
 // pair table's last run, the R rows and f values of each block): a pipeline
 // stage of up to eight l may read seven l past a tile's last l; the values
 // read there never enter the sums.
@@ -69,6 +61,22 @@ __host__ __device__ __forceinline__ long long pair_run_base(int p, int q, int Lm
 __host__ __device__ __forceinline__ long long pair_table_entries(int Lmax) {
   return pair_run_base(0, Lmax / 32, Lmax) + kPairPadL * 1024;
 }
+
+// One task of the FP32 contractions: a tile of the block pair p <= q (half 0: m'
+// in block p, m in q; half 1: the other way round), or both tiles
+// (tile_both_halves), over l in [lstart, lend].  j, j2: scales of the two slots
+// (-1: none); the direct analysis takes one scale, j, held in R slot `slot`.
+// 16 bytes: a batch of 64 transforms has some 1e5 tasks, built and copied to
+// the device when its plan set is first used.
+struct CTask {
+  uint8_t prob, p, q, half;
+  int8_t j, j2, slot, pad;
+  int16_t lstart, lend, Lmax, pad2;  // Lmax: reach of the pair table
+  __host__ __device__ __forceinline__ long long dbase() const {  // pair-table entry of lstart
+    return pair_run_base(p, q, Lmax) + 1024LL * (lstart - 32 * q);
+  }
+};
+static_assert(sizeof(CTask) == 16 && MAXB <= 256 && MAXS <= 127, "task fields");
 
 struct TileTask {
   int prob;    // index into the descriptor array of the launch
@@ -177,15 +185,13 @@ struct ReduceJobs {
 template <typename T>
 void launch_contract(int N, int nslot, bool syn, const ContractDesc<T>* descs, const TileTask* tiles,
                      int ntiles, const CallPtrs& ptrs, cudaStream_t st);
-// FP32 tile-pair contraction and its tables (contract_pair.cu)
-bool pair_two_tiles(int N);  // a CTA may compute both tiles of a pair (N <= 5)
-// CTA shapes of the FP32 contraction: the tasks name pairs and each CTA
-// computes both tiles (N <= 5 only), or each task names one tile (its half),
-// at one CTA per SM (the only shape for N > 5) or at two (N <= 5, 128
-// registers per thread)
+// FP32 contraction of large band-limits and its tables (contract_tile.cu)
+bool tile_both_halves(int N);  // a CTA computes both tiles of a block pair
+// CTA-shape values of s2dw_plan_choices (FP32 plans), see there
 constexpr int kPairShapePair = 0, kPairShapeTile = 1, kPairShapeTile2 = 2;
-void launch_contract_pair(int N, int nslot, bool syn, int shape, const ContractDesc<float>* descs,
-                          const PairTask* tasks, int ntasks, const CallPtrs& ptrs, cudaStream_t st);
+inline bool pair_shapes_offered(int N) { return N <= 5; }
+void launch_contract_tile(int N, int nslot, bool syn, const ContractDesc<float>* descs, const CTask* tasks, int ntasks,
+                          cudaStream_t st);
 void launch_fpack(const ContractDesc<float>* descs, int njobs, int nbmax, int Lrmax, const CallPtrs& ptrs,
                   cudaStream_t st);
 cudaError_t launch_pair_table(float* out, const double* d64, int Lmax, cudaStream_t st);
@@ -194,19 +200,9 @@ cudaError_t launch_rtable_pair(float* RSp, const double* d64, const double* kap,
 // FP32 contraction of small and middle band-limits (contract_direct.cu): one
 // launch over the tiles of the plans' wavelet scales (N orders) and of their
 // scaling parts.  rt: rows per thread of the analysis (1, 2 or 4).
-// A task is one 32 x 32 tile (half 0: m' in block p, m in q; half 1: the
-// other way round) over l in [lstart, lend]; dbase: pair-table entry of lstart.
-// Analysis: scale j, held in slot `slot` of the R rows.  Synthesis: the two
-// slots hold scales j and j2 (-1: none) over the whole range.
-struct DirTask {
-  int prob, p, q, half;
-  int lstart, lend;
-  int j, j2, slot, pad;
-  long long dbase;
-};
 struct DirTasks {
   const ContractDesc<float>* descs;
-  const DirTask* tasks;
+  const CTask* tasks;
   int n;
 };
 // Band-limits up to this run it.  Contraction per call, GB300 (tile-pair ring
@@ -220,7 +216,7 @@ constexpr int kContractDirectMaxL = 640;
 void launch_contract_direct(int N, bool syn, int rt, const DirTasks& w, const DirTasks& p, const CallPtrs& ptrs,
                             cudaStream_t st);
 cudaError_t contract_direct_prepare();
-cudaError_t pair_prepare();
+cudaError_t contract_tile_prepare();
 cudaError_t pair_timeouts(int* count);  // reads and resets the device count
 template <typename T>
 void launch_czt(int kind, const CztSeg<T>* segs, int nseg, int total_items, int maxlogM,

@@ -246,7 +246,7 @@ __global__ void k_rtable(T* RS, const double* d64, const double* kap, const doub
   RS[idx] = (T)v;
 }
 
-// Pair table (FP32) of the tile-pair contraction from the FP64 table: block
+// Pair table (FP32) of the FP32 contraction from the FP64 table: block
 // (pair (p, q), l) is [r][c] = Delta^l_{32p+r, 32q+c}, zero where an index
 // exceeds l.  Grid (Lmax, number of pairs); CTAs with l < 32 q exit.  Each
 // thread writes 4 consecutive c (one 16-byte store).
@@ -281,7 +281,7 @@ cudaError_t launch_pair_table(float* out, const double* d64, int Lmax, cudaStrea
   return cudaMemsetAsync(out + pair_run_base(0, B, Lmax), 0, (size_t)kPairPadL * 1024 * sizeof(float), st);
 }
 
-// R rows in the layout of the tile-pair contraction:
+// R rows in the layout of the FP32 contraction:
 // RSp[b][l][s][h][c] = R at (l, m' = 32 b + c, slot s, order n_k, k = N/2 + h),
 // as k_rtable (zero for l >= L, m' > l, inactive slots).
 __global__ void k_rtable_pair(float* RSp, const double* d64, const double* kap, const double* sabs, const int* slotj,

@@ -1,4 +1,4 @@
-"""The FP32 contraction of small and middle band-limits: Fourier cube, scaling
+"""The FP32 contractions (L <= 640 and above): Fourier cube, scaling
 part and synthesis against the FP64 plan at the edges of its 32-blocks, of its
 range (L = 640 | 641) and for every N, within the 1e-5 that the mixed path keeps
 (FP32 sums of at most L terms); and independence of how a launch cuts its tasks
@@ -15,7 +15,8 @@ pytestmark = pytest.mark.gpu
 
 @pytest.mark.parametrize("L,N,lam,J0", [(2, 1, 2.0, 0), (9, 8, 2.0, 1), (31, 2, 2.0, 0), (32, 3, 1.5, 0), (33, 4, 2.0, 2),
                                         (63, 7, 3.0, 0), (65, 6, 2.0, 4), (97, 5, 2.0, 0), (193, 1, 2.0, 7),
-                                        (640, 3, 2.0, 1), (641, 2, 2.0, 1)])
+                                        (640, 3, 2.0, 1), (641, 2, 2.0, 1), (655, 7, 2.0, 0), (672, 8, 3.0, 0),
+                                        (705, 6, 1.7, 2), (800, 5, 2.0, 0), (673, 1, 2.0, 0)])
 def test_direct_contraction_vs_fp64(L, N, lam, J0):
     f = flm_gaussian(L, 17, "unit")
     pm, p64 = B.Plan(L, N, lam, J0, "mixed"), B.Plan(L, N, lam, J0, "fp64")
