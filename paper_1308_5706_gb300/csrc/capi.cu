@@ -118,6 +118,7 @@ void kernels_prepare(bool fp64, bool pair) {
   if (pair && !(done_pair & bit)) {
     ck(contract_tile_prepare());
     ck(contract_direct_prepare());
+    ck(split_gemm_prepare());
     done_pair |= bit;
   }
 }
@@ -270,11 +271,12 @@ struct Lists {
   };
   std::vector<FpGroup> dir_w, tile_w;
   FpGroup dir_phi, tile_phi;
-  static constexpr int NK = 16;  // chirp-z 0..3, direct alpha 4..5, single-FFT beta 6..7, segmented alpha 8..9,
-                                 // MW-grid synthesis beta 10..12, half-length beta 13..15
+  static constexpr int NK = 21;  // chirp-z 0..3, direct alpha 4..5, single-FFT beta 6..7, segmented alpha 8..9,
+                                 // MW-grid synthesis beta 10..12, half-length beta 13..15, split products 16..20
   void* segs[NK] = {};
   int nseg[NK] = {};
   int items[NK] = {};
+  int stages[NK] = {};  // data stages of the split products
   int ulogM[NK] = {};  // the segments' common transform length log2 (0: lengths differ)
   // half-length beta kinds (13..15): the segments ordered by transform length,
   // one launch per length {first segment, segments, items, log2 length}, so
@@ -337,6 +339,11 @@ struct s2dw_plan_s {
     void* bfft = nullptr;    // e^{i pi m'/(4Lg)} (|m'| < Lg), then q_b (b < 2Lg): single-FFT beta
     void* tw2 = nullptr;     // FFT twiddles of length 2Lg (half-length beta)
     void* Hs = nullptr;      // 4 x M spectra
+    // FP32 plans: basis tables of the split products (beta analysis, beta
+    // synthesis, alpha analysis, alpha synthesis, MW: beta evaluation on the
+    // DH grid), where some launch uses them
+    void* sg[5] = {};
+    bool sg_beta[2] = {false, false};  // the beta sums of a direction run as products
   };
   bool multires = false;       // every scale on the grid of its own band-limit
   bool mw = false;             // L beta samples per grid (McEwen-Wiaux), not 2L
@@ -357,7 +364,10 @@ struct s2dw_plan_s {
   // alpha_mode[dir][j] 0 = direct sums (L_j <= 32), 1 = chirp-z of the grid's
   // length, 2 = segmented chirp-z (where its tables exist); dir 0 = analysis
   int beta_mode[2] = {1, 1};
-  std::vector<int> alpha_mode[2];
+  std::vector<int> alpha_mode[2], alpha_default[2];
+  // FP32: the alpha sums of scale j run as split products (while its method is the default one)
+  std::vector<char> alpha_sg[2];
+  void* sg_data = nullptr;  // operand images of the product launch under way
   // [nscale + 1]: tensor-core basis images of the direct alpha sums (FP32 plans)
   std::vector<void*> tc_ana, tc_syn;
   // FP32 plans: R rows and packed f of the FP32 contraction
@@ -674,7 +684,7 @@ void sort_tiles(std::vector<TileTask>& t) {
 }
 
 template <typename T>
-void build_segs(s2dw_plan_s* p, int job, int kind, std::vector<CztSeg<T>>& out, int& start) {
+void build_segs(s2dw_plan_s* p, int job, int kind, std::vector<CztSeg<T>>& out, int& start, int& stages) {
   // kinds 4 / 5 collect the alpha segments of scales with Lj <= kDirectMaxLjAna
   // (analysis) or kDirectMaxLj (synthesis),
   // kinds 6 / 7 the beta segments of plans whose FFT length M is 4L
@@ -682,20 +692,29 @@ void build_segs(s2dw_plan_s* p, int job, int kind, std::vector<CztSeg<T>>& out, 
   // kinds 10..12 (MW grid only) the synthesis-side resampling of V from the L
   // MW beta samples to the DH beta grid (torus coefficients, then their
   // evaluation on the DH grid by the analysis beta kernels)
-  if ((kind == CZT_BETA_MW_DFT || kind == CZT_BETA_RS_FFT || kind == CZT_BETA_RS || kind == CZT_BETA_RS_DCT) &&
+  if ((kind == CZT_BETA_MW_DFT || kind == CZT_BETA_RS_FFT || kind == CZT_BETA_RS || kind == CZT_BETA_RS_DCT ||
+       kind == SG_KIND_BETA_RS) &&
       !p->mw)
     return;
-  const int base_kind = (kind == CZT_ALPHA_ANA_DIRECT || kind == CZT_ALPHA_ANA_SEG) ? CZT_ALPHA_ANA
-                        : (kind == CZT_ALPHA_SYN_DIRECT || kind == CZT_ALPHA_SYN_SEG) ? CZT_ALPHA_SYN
+  const int base_kind = (kind == CZT_ALPHA_ANA_DIRECT || kind == CZT_ALPHA_ANA_SEG || kind == SG_KIND_ALPHA_ANA)
+                            ? CZT_ALPHA_ANA
+                        : (kind == CZT_ALPHA_SYN_DIRECT || kind == CZT_ALPHA_SYN_SEG || kind == SG_KIND_ALPHA_SYN)
+                            ? CZT_ALPHA_SYN
+                        : (kind == SG_KIND_BETA_ANA || kind == SG_KIND_BETA_RS) ? CZT_BETA_ANA
+                        : kind == SG_KIND_BETA_SYN                              ? CZT_BETA_SYN
                         : (kind == CZT_BETA_ANA_FFT || kind == CZT_BETA_RS_FFT || kind == CZT_BETA_RS ||
                            kind == CZT_BETA_MW_DFT || kind == CZT_BETA_ANA_DCT || kind == CZT_BETA_RS_DCT)
                             ? CZT_BETA_ANA
                         : (kind == CZT_BETA_SYN_FFT || kind == CZT_BETA_SYN_DCT) ? CZT_BETA_SYN
                                                                                   : kind;
-  const bool rs_list = kind == CZT_BETA_RS_FFT || kind == CZT_BETA_RS || kind == CZT_BETA_RS_DCT;
+  const bool sg_list = kind >= SG_KIND_BETA_ANA && kind <= SG_KIND_BETA_RS;
+  if (sg_list && sizeof(T) != sizeof(float)) return;
+  const bool rs_list =
+      kind == CZT_BETA_RS_FFT || kind == CZT_BETA_RS || kind == CZT_BETA_RS_DCT || kind == SG_KIND_BETA_RS;
   const bool dct_list = kind == CZT_BETA_ANA_DCT || kind == CZT_BETA_SYN_DCT || kind == CZT_BETA_RS_DCT;
   const bool direct_list = kind == CZT_ALPHA_ANA_DIRECT || kind == CZT_ALPHA_SYN_DIRECT;
   const bool seg_list = kind == CZT_ALPHA_ANA_SEG || kind == CZT_ALPHA_SYN_SEG;
+  size_t sg_used = 0;  // data stages of this plan so far
   const bool fft_list = kind == CZT_BETA_ANA_FFT || kind == CZT_BETA_SYN_FFT || kind == CZT_BETA_RS_FFT;
   for (int j = 0; j <= p->nscale; ++j) {
     const bool phi = (j == p->nscale);
@@ -715,9 +734,13 @@ void build_segs(s2dw_plan_s* p, int job, int kind, std::vector<CztSeg<T>>& out, 
     const bool dct_faster = bdir == 0 ? L >= 128 : (L >= 128 && L <= 1024);
     const bool beta_dct = beta_pow2 && L >= 16 && p->beta_mode[bdir] == 1 && dct_faster;
     const bool beta_fft = beta_pow2 && !beta_dct;
-    if ((base_kind == CZT_BETA_ANA || base_kind == CZT_BETA_SYN) && kind != CZT_BETA_MW_DFT &&
-        (beta_fft != fft_list || beta_dct != dct_list))
-      continue;
+    const bool is_beta = base_kind == CZT_BETA_ANA || base_kind == CZT_BETA_SYN;
+    if (is_beta && kind != CZT_BETA_MW_DFT) {
+      // split products on the grids where they are faster, in mode 1 (the default)
+      const bool sg = p->beta_mode[bdir] == 1 && (rs_list ? G.sg[4] != nullptr : G.sg_beta[bdir]);
+      if (sg != sg_list) continue;
+      if (!sg && (beta_fft != fft_list || beta_dct != dct_list)) continue;
+    }
     const cx<T>* Hs = reinterpret_cast<const cx<T>*>(G.Hs);
     CztSeg<T> s;
     std::memset(&s, 0, sizeof(s));
@@ -735,7 +758,12 @@ void build_segs(s2dw_plan_s* p, int job, int kind, std::vector<CztSeg<T>>& out, 
     const int amode = is_alpha ? p->alpha_mode[base_kind == CZT_ALPHA_SYN ? 1 : 0][j] : -1;
     const bool direct = is_alpha && amode == 0;
     if (direct != direct_list) continue;
-    if (is_alpha && !direct && (amode == 2) != seg_list) continue;
+    if (is_alpha && !direct) {
+      const int d = base_kind == CZT_ALPHA_SYN ? 1 : 0;
+      const bool sg = p->alpha_sg[d][j] && amode == p->alpha_default[d][j];
+      if (sg != sg_list) continue;
+      if (!sg && (amode == 2) != seg_list) continue;
+    }
     switch (base_kind) {
       case CZT_BETA_ANA:
         s.P = beta_czt_cols(G.logM, sizeof(T) == 8);  // columns per CTA of the chirp-z beta kernels
@@ -819,6 +847,25 @@ void build_segs(s2dw_plan_s* p, int job, int kind, std::vector<CztSeg<T>>& out, 
       }
       s.pre = reinterpret_cast<const cx<T>*>(G.root_a);
     }
+    if constexpr (sizeof(T) == sizeof(float)) {
+      if (sg_list) {
+        const int k = kind - SG_KIND_BETA_ANA, mode = k == 4 ? 0 : k;
+        const SgDims d = sg_dims(mode, L, Lj, Nj, s.nb);
+        const SgTable t = sg_table(mode, L);
+        s.items = d.data_tiles * d.basis_tiles;
+        s.P = d.basis_tiles;
+        s.nsegs = d.stages;
+        s.tabP = t.tiles;
+        s.tabK = t.stages;
+        s.H = reinterpret_cast<const cx<T>*>(G.sg[k]);
+        s.scale = sg_out_scale(mode, L);
+        s.tabD = stages;
+        // this plan's images of the launch: one buffer, its segments in turn
+        s.pre = reinterpret_cast<const cx<T>*>(reinterpret_cast<const char*>(p->sg_data) + sg_used * kSgDataBytes);
+        stages += d.data_tiles * d.stages;
+        sg_used += (size_t)d.data_tiles * d.stages;
+      }
+    }
     if (s.items <= 0) continue;
     s.start = start;
     start += s.items;
@@ -844,7 +891,7 @@ Lists* build_lists(const std::vector<s2dw_plan_t>& plans) {
   std::map<int, FpTasks> dir_byN, tile_byN;
   FpTasks dir_phi, tile_phi;
   std::vector<CztSeg<T>> segs[Lists::NK];
-  int start[Lists::NK] = {};
+  int start[Lists::NK] = {}, stages[Lists::NK] = {};
   Lists* ls = new Lists();
   ls->njobs = nj;
   for (int i = 0; i < nj; ++i) {
@@ -865,7 +912,7 @@ Lists* build_lists(const std::vector<s2dw_plan_t>& plans) {
       t.prob = i;
       tphi.push_back(t);
     }
-    for (int k = 0; k < Lists::NK; ++k) build_segs<T>(p, i, k, segs[k], start[k]);
+    for (int k = 0; k < Lists::NK; ++k) build_segs<T>(p, i, k, segs[k], start[k], stages[k]);
     ls->maxlogM = std::max(ls->maxlogM, p->logM);
     ls->Lmax = std::max(ls->Lmax, p->L);
     if (p->fP) {  // packed f: plans that run the tile contraction
@@ -988,6 +1035,7 @@ Lists* build_lists(const std::vector<s2dw_plan_t>& plans) {
     ls->segs[k] = base + o_sg[k];
     ls->nseg[k] = (int)segs[k].size();
     ls->items[k] = start[k];
+    ls->stages[k] = stages[k];
   }
   return ls;
 }
@@ -1037,6 +1085,14 @@ void launch_dct_parts(const Lists& ls, int kind, const CallPtrs& ptrs, cudaStrea
     launch_czt<T>(kind, segs + pt[0], pt[1], pt[2], ls.maxlogM, ptrs, st, pt[3]);
 }
 
+// split matrix products of a kind (FP32 plans)
+template <typename T>
+void launch_products(const Lists& ls, int kind, const CallPtrs& ptrs, cudaStream_t st) {
+  if constexpr (sizeof(T) == sizeof(float))
+    launch_split_gemm(kind == SG_KIND_BETA_RS ? 0 : kind - SG_KIND_BETA_ANA, reinterpret_cast<const CztSeg<T>*>(ls.segs[kind]),
+                      ls.nseg[kind], ls.items[kind], ls.stages[kind], ptrs, st);
+}
+
 template <typename T>
 void run_analysis(const Lists& ls, const CallPtrs& ptrs, cudaStream_t st, cudaEvent_t* ev = nullptr) {
   const ContractDesc<T>* dw = reinterpret_cast<const ContractDesc<T>*>(ls.desc_w);
@@ -1062,7 +1118,9 @@ void run_analysis(const Lists& ls, const CallPtrs& ptrs, cudaStream_t st, cudaEv
   launch_czt<T>(CZT_BETA_ANA_FFT, reinterpret_cast<const CztSeg<T>*>(ls.segs[6]), ls.nseg[6], ls.items[6],
                 ls.maxlogM, ptrs, st, ls.ulogM[6]);
   launch_dct_parts<T>(ls, CZT_BETA_ANA_DCT, ptrs, st);
+  launch_products<T>(ls, SG_KIND_BETA_ANA, ptrs, st);
   rec(ev, 3, st);
+  launch_products<T>(ls, SG_KIND_ALPHA_ANA, ptrs, st);
   launch_czt<T>(CZT_ALPHA_ANA | ls.odd, reinterpret_cast<const CztSeg<T>*>(ls.segs[1]), ls.nseg[1], ls.items[1],
                 ls.maxlogM, ptrs, st, ls.ulogM[1]);
   rec(ev, 4, st);
@@ -1085,6 +1143,7 @@ void run_synthesis(const Lists& ls, const CallPtrs& ptrs, const ReduceJobs& rj, 
   launch_czt<T>(CZT_ALPHA_SYN_DIRECT, reinterpret_cast<const CztSeg<T>*>(ls.segs[5]), ls.nseg[5], ls.items[5],
                 ls.maxlogM, ptrs, st, ls.ulogM[5]);
   rec(ev, 1, st);
+  launch_products<T>(ls, SG_KIND_ALPHA_SYN, ptrs, st);
   launch_czt<T>(CZT_ALPHA_SYN, reinterpret_cast<const CztSeg<T>*>(ls.segs[2]), ls.nseg[2], ls.items[2], ls.maxlogM,
                 ptrs, st, ls.ulogM[2]);
   rec(ev, 2, st);
@@ -1097,6 +1156,7 @@ void run_synthesis(const Lists& ls, const CallPtrs& ptrs, const ReduceJobs& rj, 
   launch_czt<T>(CZT_BETA_RS_FFT, reinterpret_cast<const CztSeg<T>*>(ls.segs[11]), ls.nseg[11], ls.items[11],
                 ls.maxlogM, ptrs, st, ls.ulogM[11]);
   launch_dct_parts<T>(ls, CZT_BETA_RS_DCT, ptrs, st);
+  launch_products<T>(ls, SG_KIND_BETA_RS, ptrs, st);
   launch_czt<T>(CZT_BETA_RS, reinterpret_cast<const CztSeg<T>*>(ls.segs[12]), ls.nseg[12], ls.items[12],
                 ls.maxlogM, ptrs, st, ls.ulogM[12]);
   launch_czt<T>(CZT_BETA_SYN, reinterpret_cast<const CztSeg<T>*>(ls.segs[3]), ls.nseg[3], ls.items[3], ls.maxlogM,
@@ -1104,6 +1164,7 @@ void run_synthesis(const Lists& ls, const CallPtrs& ptrs, const ReduceJobs& rj, 
   launch_czt<T>(CZT_BETA_SYN_FFT, reinterpret_cast<const CztSeg<T>*>(ls.segs[7]), ls.nseg[7], ls.items[7],
                 ls.maxlogM, ptrs, st, ls.ulogM[7]);
   launch_dct_parts<T>(ls, CZT_BETA_SYN_DCT, ptrs, st);
+  launch_products<T>(ls, SG_KIND_BETA_SYN, ptrs, st);
   rec(ev, 4, st);
   if constexpr (sizeof(T) == sizeof(float)) {
     run_direct(ls, true, dw, dp, ptrs, st);
@@ -1146,6 +1207,7 @@ void own_lists_build(s2dw_plan_s* p) {
     p->own.segs[k] = ls->segs[k];
     p->own.nseg[k] = ls->nseg[k];
     p->own.items[k] = ls->items[k];
+    p->own.stages[k] = ls->stages[k];
     p->own.ulogM[k] = ls->ulogM[k];
   }
   for (int k = 0; k < 3; ++k) p->own.dct_parts[k] = ls->dct_parts[k];
@@ -1190,7 +1252,6 @@ void plan_build_typed(s2dw_plan_s* p, const double* kap_d, const double* phi_d, 
     o_Y[j] = take((size_t)Nj * Lj * Lj * sizeof(cx<T>));
     o_X[j] = take((size_t)Nj * 2 * p->gt[p->grid_of[j]].L * Lj * sizeof(cx<T>));
   }
-  const size_t o_P = take((size_t)p->nbr * L * p->Lp32 * sizeof(cx<T>));
   const size_t o_Pphi = take((size_t)p->nbr_phi * p->Lphi * p->Lphip32 * sizeof(cx<T>));
   // per grid: twiddles, chirps, roots, beta phases and weights, spectra
   struct GridOff { size_t tw, ca, pb, qb, pS, qS, root, bf, H, pm, tw2; };
@@ -1229,12 +1290,55 @@ void plan_build_typed(s2dw_plan_s* p, const double* kap_d, const double* phi_d, 
   // was chosen above, else the grid's chirp-z
   for (int d = 0; d < 2; ++d) {
     p->alpha_mode[d].assign(p->nscale + 1, 1);
+    p->alpha_sg[d].assign(p->nscale + 1, 0);
     for (int j = 0; j <= p->nscale; ++j) {
       const int Lj = p->Ycols[j];
       if (Lj <= (d == 0 ? kDirectMaxLjAna : kDirectMaxLj)) p->alpha_mode[d][j] = 0;
       else if (p->seg[j].S > 0) p->alpha_mode[d][j] = 2;
+      const auto& G = p->gt[p->grid_of[j]];
+      const auto& sgt = p->seg[j];
+      const double cost = sgt.S > 0 ? (double)(sgt.S + 1) * ((size_t)1 << sgt.logM) * sgt.logM : 2.0 * G.M * G.logM;
+      p->alpha_sg[d][j] = pairc && p->alpha_mode[d][j] != 0 && sg_alpha_faster(G.L, Lj, cost);
     }
+    p->alpha_default[d] = p->alpha_mode[d];
   }
+  // basis tables of the split products
+  std::vector<std::array<size_t, 5>> o_sg(p->gt.size());
+  for (size_t g = 0; g < p->gt.size(); ++g) {
+    auto& G = p->gt[g];
+    o_sg[g].fill(SIZE_MAX);
+    if (!pairc) continue;
+    const bool pow2 = 4 * G.L == G.M;
+    // (an MW analysis evaluates at the MW samples, whatever L)
+    G.sg_beta[0] = sg_beta_faster(G.L, pow2 && !p->mw);
+    G.sg_beta[1] = sg_beta_faster(G.L, pow2);
+    bool need[5] = {G.sg_beta[0], G.sg_beta[1], false, false, p->mw && sg_beta_faster(G.L, pow2)};
+    for (int j = 0; j <= p->nscale; ++j)
+      if (p->grid_of[j] == (int)g)
+        for (int d = 0; d < 2; ++d) need[2 + d] = need[2 + d] || p->alpha_sg[d][j];
+    for (int k = 0; k < 5; ++k)
+      if (need[k]) o_sg[g][k] = take(sg_table(k == 4 ? 0 : k, G.L).bytes);
+  }
+  // operand images of one product launch (shared by the five kinds), in the
+  // buffer of the synthesis partials: the contraction that writes those comes
+  // after every product launch of its call
+  size_t sgd_bytes = 0;
+  if (pairc) {
+    size_t most = 0;
+    for (int k = 0; k < 5; ++k) {
+      size_t n = 0;
+      for (int j = 0; j <= p->nscale; ++j) {
+        const auto& G = p->gt[p->grid_of[j]];
+        const bool used = k < 2 ? G.sg_beta[k] : (k < 4 ? p->alpha_sg[k - 2][j] != 0 : o_sg[p->grid_of[j]][4] != SIZE_MAX);
+        if (!used) continue;
+        const SgDims d = sg_dims(k == 4 ? 0 : k, G.L, p->Ycols[j], j == p->nscale ? 1 : N, G.nb);
+        n += (size_t)d.data_tiles * d.stages;
+      }
+      most = std::max(most, n);
+    }
+    sgd_bytes = most * kSgDataBytes;
+  }
+  const size_t o_P = take(std::max((size_t)p->nbr * L * p->Lp32 * sizeof(cx<T>), sgd_bytes));
   // tensor-core basis images of the direct alpha sums (FP32 plans)
   std::vector<size_t> o_ta(p->nscale + 1, SIZE_MAX), o_ts(p->nscale + 1, SIZE_MAX);
   if (sizeof(T) == sizeof(float)) {
@@ -1274,6 +1378,7 @@ void plan_build_typed(s2dw_plan_s* p, const double* kap_d, const double* phi_d, 
     G.Hs = b + go[g].H;
     G.pre_mw = b + go[g].pm;
     G.tw2 = b + go[g].tw2;
+    for (int k = 0; k < 5; ++k) G.sg[k] = o_sg[g][k] != SIZE_MAX ? b + o_sg[g][k] : nullptr;
   }
   for (int j = 0; j <= p->nscale; ++j) {
     auto& sgt = p->seg[j];
@@ -1282,6 +1387,7 @@ void plan_build_typed(s2dw_plan_s* p, const double* kap_d, const double* phi_d, 
     sgt.Ha = b + so[j].Ha;
     sgt.Hs = b + so[j].Hs;
   }
+  p->sg_data = sgd_bytes > 0 ? p->P : nullptr;
   p->tc_ana.assign(p->nscale + 1, nullptr);
   p->tc_syn.assign(p->nscale + 1, nullptr);
   for (int j = 0; j <= p->nscale; ++j) {
@@ -1325,6 +1431,7 @@ void plan_build_typed(s2dw_plan_s* p, const double* kap_d, const double* phi_d, 
       const size_t Lg = G.L, ng = 2 * Lg - 1;
       need = std::max(need, (size_t)G.M + ng + (2 * Lg - 1) + 2 * Lg + 2 * Lg + (2 * Lg - 1) + ng + (4 * Lg - 1) +
                                 4 * (size_t)G.M);
+      need = std::max(need, 8 * Lg);  // roots of the split products' basis
     }
     amalloc(&t64, need * sizeof(double2), st);
     amalloc(&qg, (size_t)2 * p->gt.back().L * sizeof(double), st);
@@ -1365,6 +1472,8 @@ void plan_build_typed(s2dw_plan_s* p, const double* kap_d, const double* phi_d, 
     put(G.pre_mw, tw64, ng);
     ck(launch_twiddles64(tw64, G.logM - 1, st));  // length 2Lg (half-length beta transforms)
     put(G.tw2, tw64, twiddle_entries(G.logM - 1));
+    for (int k = 0; k < 5; ++k)  // (roots in the same scratch)
+      if (G.sg[k]) ck(sg_build_table(k == 4 ? 0 : k, G.sg[k], tw64, q_g, Lg, p->mw && k == 0, st));
   }
   {
     size_t need = 0;
@@ -2018,6 +2127,9 @@ int s2dw_wait_timeouts(int* count) {
   e = pair_timeouts(&pc);
   if (e != cudaSuccess) return err_of(e);
   *count += pc;
+  e = split_gemm_timeouts(&pc);
+  if (e != cudaSuccess) return err_of(e);
+  *count += pc;
   return *count > 0 ? S2DW_ETIMEOUT : S2DW_OK;
 }
 
@@ -2037,10 +2149,10 @@ int s2dw_launch_counts(s2dw_plan_t p, int* analysis, int* synthesis) {
     return ls.items[k] > 0 ? 1 : 0;
   };
   const int fpack = (!p->fp64 && ls.njobs > 0 && ls.nbmax > 0) ? 1 : 0;  // f packing of the FP32 contraction
-  if (analysis) *analysis = fpack + contract + has(0) + has(1) + has(4) + has(6) + has(8) + has(13);
+  if (analysis) *analysis = fpack + contract + has(0) + has(1) + has(4) + has(6) + has(8) + has(13) + 2 * (has(16) + has(18));
   if (synthesis)
     *synthesis = contract + has(2) + has(3) + has(5) + has(7) + has(9) + has(10) + has(11) + has(12) + has(14) +
-                 has(15) + 1;
+                 has(15) + 2 * (has(17) + has(19) + has(20)) + 1;
   return S2DW_OK;
 }
 

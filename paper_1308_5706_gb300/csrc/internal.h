@@ -110,7 +110,12 @@ enum CztKind {
   CZT_BETA_RS = 12,          //   (single FFT, or chirp-z for non-power-of-two L)
   CZT_BETA_ANA_DCT = 13,     // beta sums as half-length transforms (L a power of two, L >= 16)
   CZT_BETA_SYN_DCT = 14,
-  CZT_BETA_RS_DCT = 15       //   (MW grid, synthesis: evaluation on the DH beta grid)
+  CZT_BETA_RS_DCT = 15,      //   (MW grid, synthesis: evaluation on the DH beta grid)
+  SG_KIND_BETA_ANA = 16,     // split matrix products on the tensor cores (FP32 plans)
+  SG_KIND_BETA_SYN = 17,
+  SG_KIND_ALPHA_ANA = 18,
+  SG_KIND_ALPHA_SYN = 19,
+  SG_KIND_BETA_RS = 20       //   (MW grid, synthesis: evaluation on the DH beta grid)
 };
 // Or-ed into an alpha chirp-z kind: the list may hold segments with an odd row
 // count N nb (MW grid), whose last row pair has one row.
@@ -157,6 +162,7 @@ struct CztSeg {
   const cx<T>* post;
   T scale;
   int P, nsegs;   // segmented chirp-z: samples per segment, segments
+  int tabP, tabK, tabD;  // split products: basis tiles and stages of the table, first data stage of the launch
   int nb;         // beta samples per gamma sample (rows of X, V and W per g): 2L, or L on the MW grid
 };
 
@@ -170,6 +176,39 @@ void launch_alpha_tc(bool syn, const CztSeg<float>* segs, int nseg, int total_it
 cudaError_t alpha_tc_prepare();
 cudaError_t alpha_tc_timeouts(int* count);  // reads and resets the device count
 cudaError_t alpha_tc_wait_probe(long long limit, cudaStream_t st);  // a wait that runs out
+
+// Beta and alpha sums as split FP16 matrix products on the tensor cores
+// (split_gemm.cu).  Modes 0 beta analysis, 1 beta synthesis, 2 alpha analysis, 3
+// alpha synthesis; basis tables per grid, laid out per stage of 32 terms.
+constexpr int kSgDataBytes = 4 * 16 * 512 + 512;  // one data stage of 128 rows: operand images, inverse row scales
+struct SgTable {
+  int sets, tiles, stages;
+  size_t bytes;
+};
+struct SgDims {
+  int data_tiles, basis_tiles, stages;
+};
+SgTable sg_table(int mode, int L);
+SgDims sg_dims(int mode, int L, int Lj, int N, int nb);
+float sg_out_scale(int mode, int L);
+int sg_period(int mode, int L, bool mw);  // double2 of scratch the build needs
+cudaError_t sg_build_table(int mode, void* out, double2* scratch, const double* qw, int L, bool mw, cudaStream_t st);
+void launch_split_gemm(int mode, const CztSeg<float>* segs, int nseg, int total, int stages, const CallPtrs& ptrs,
+                       cudaStream_t st);
+// Whether the products are the faster form.  beta: the chirp-z (other L than
+// powers of two) costs two FFTs of M >= 4L per column: 20.5 against 20 us at L =
+// 100, N = 3, 30 against 21 at L = 200; the half-length transforms of
+// power-of-two L one of 2L: 230 against 243 us at L = 1024, N = 5, 2807 against
+// 2144 at L = 2048, N = 8.
+inline bool sg_beta_faster(int L, bool pow2) { return pow2 ? L >= 2048 : L > 112; }
+// alpha, band L_j on a grid of band-limit L: a row costs L L_j terms here, a
+// chirp-z `fft_cost` = (FFTs) x (length) x log2(length) (two FFTs of M, or S + 1
+// of M' segmented).  Per row at L = 1024, N = 5: 16 ps per term against 0.1 ps
+// per unit of that cost; below L = 128 the two launches cost more than they save
+// (L = 64, N = 3 18 against 10.5 us, L = 128, N = 5 21 against 27).
+inline bool sg_alpha_faster(int L, int Lj, double fft_cost) { return L >= 128 && (double)L * Lj < 6.5 * fft_cost; }
+cudaError_t split_gemm_prepare();
+cudaError_t split_gemm_timeouts(int* count);  // reads and resets the device count
 
 // Per-job parameters of the batched final synthesis reduction.
 struct ReduceJobs {

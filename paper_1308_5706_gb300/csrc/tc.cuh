@@ -133,6 +133,19 @@ __device__ __forceinline__ void tmem_ld8(uint32_t ta, float (&v)[8]) {
   for (int j = 0; j < 8; ++j) v[j] = __uint_as_float(r[j]);
 }
 
+// one load of 16 columns
+__device__ __forceinline__ void tmem_ld16(uint32_t ta, float (&v)[16]) {
+  uint32_t r[16];
+  asm volatile(
+      "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%16];\n"
+      "tcgen05.wait::ld.sync.aligned;\n"
+      : S2DW_R8(0), S2DW_R8(8)
+      : "r"(ta)
+      : "memory");
+#pragma unroll
+  for (int j = 0; j < 16; ++j) v[j] = __uint_as_float(r[j]);
+}
+
 // one load of 32 columns
 __device__ __forceinline__ void tmem_ld32(uint32_t ta, float (&v)[32]) {
   uint32_t r[32];
