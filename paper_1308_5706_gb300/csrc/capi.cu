@@ -841,7 +841,10 @@ void build_segs(s2dw_plan_s* p, int job, int kind, std::vector<CztSeg<T>>& out, 
         s.items = alpha_tc_items(L, Nj * G.nb, syn);
         s.H = reinterpret_cast<const cx<T>*>(syn ? p->tc_syn[j] : p->tc_ana[j]);
       } else if (!syn) {
-        s.items = ((n + kAgCols - 1) / kAgCols) * ((Nj * G.nb + kAgChunk - 1) / kAgChunk);
+        const int tiles = (L + kAgCols - 1) / kAgCols, rows = Nj * G.nb;
+        s.P = 512;  // rows per CTA: fewer while a scale has less than a CTA per SM
+        while (s.P > kAgMinRows && tiles * ((rows + s.P - 1) / s.P) < 152) s.P /= 2;
+        s.items = tiles * ((rows + s.P - 1) / s.P);
       } else {
         s.items = (Nj * G.nb + direct_rows_syn(sizeof(T) == 8) - 1) / direct_rows_syn(sizeof(T) == 8);
       }

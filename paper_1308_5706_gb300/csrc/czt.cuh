@@ -1001,38 +1001,94 @@ __global__ void __launch_bounds__(256) k_beta_syn_dct(const CztSeg<T>* __restric
 // ---------------------------------------------------------------------------
 constexpr int kDirectMax = kDirectMaxLj;
 
+// 8 rows (As) at the 32 NI samples from a0 + 32 i0: nrow of them to Wb.
+template <typename T, int NI>
+__device__ __forceinline__ void alpha_ana_rows(const T* __restrict__ As, const T* __restrict__ Bs, int i0, int Lj, int L,
+                                               int a0, int nrow, T* __restrict__ Wb) {
+  const int lane = threadIdx.x & 31, n = 2 * L - 1;
+  T c[8][NI], s[8][NI];
+  const T* __restrict__ ap = As;
+  const T* __restrict__ bp = Bs + kAgCols + 4 * lane + i0;
+#pragma unroll
+  for (int r = 0; r < 8; ++r)
+#pragma unroll
+    for (int i = 0; i < NI; ++i) c[r][i] = ap[r], s[r][i] = T(0);
+  ap += kAgRows;
+#pragma unroll 1
+  for (int m = 1; m < Lj; ++m) {
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+      T av[8], bv[NI];
+#pragma unroll
+      for (int r = 0; r < 8; ++r) av[r] = ap[h * kAgRows + r];
+#pragma unroll
+      for (int i = 0; i < NI; ++i) bv[i] = bp[h * kAgCols + i];
+#pragma unroll
+      for (int r = 0; r < 8; ++r)
+#pragma unroll
+        for (int i = 0; i < NI; ++i) {
+          T& x = h ? s[r][i] : c[r][i];
+          x = fma(av[r], bv[i], x);
+        }
+    }
+    ap += 2 * kAgRows;
+    bp += 2 * kAgCols;
+  }
+#pragma unroll
+  for (int r = 0; r < 8; ++r) {
+    if (r >= nrow) break;
+    T* __restrict__ W = Wb + (size_t)r * n;
+#pragma unroll
+    for (int i = 0; i < NI; ++i) {
+      const int a = a0 + lane + 32 * (i0 + i);
+      if (a < L) W[a] = c[r][i] + s[r][i];
+      if (a > 0 && a < L) W[n - a] = c[r][i] - s[r][i];
+    }
+  }
+}
+
 // W[row][a] = X_0 + 2 sum_{m=1}^{Lj-1} Re(X_m e^{2 pi i m a / n})   (Eq. (30), Hermitian in m)
-// as a small matrix product W = A B over k < K = 2 Lj - 1 with
-//   A[row] = (X_0.x, X_1.x, X_1.y, X_2.x, ...),
-//   B[.][a] = (1, 2 cos(2 pi a/n), -2 sin(2 pi a/n), 2 cos(4 pi a/n), ...).
-// A CTA owns kAgCols consecutive samples a and kAgChunk rows: it builds its
-// B tile once in shared memory from the exact root table (index m a mod n
-// advanced by additions), then per pass of kAgRows rows stages A and
-// accumulates a register tile of 8 rows x 4 samples per thread, samples
-// lane + 32 i so that every store of a warp is one 128-byte line.  Layouts:
-// B[k][lane][i] (one 16-byte load per k), A[k][row].  FP64 plans only (FP32
-// plans run the tensor-core kernels of alpha_tc.cu).
+// folded over a <-> n - a: W_a = C + S, W_{n-a} = C - S with
+//   C = X_0 + sum_m (2 cos(2 pi m a/n)) Re X_m, S = sum_m (-2 sin(2 pi m a/n)) Im X_m,
+// two small matrix products over a < L, half the multiply-adds of one over all
+// n samples.  What bounds it: the FP64 pipes (two multiply-adds per cycle and
+// SM, a quarter of them in each quarter of the SM).  A CTA owns kAgCols
+// consecutive samples a and the segment's P rows: as many as leave a scale a
+// CTA per SM (512 rows per CTA left 20 CTAs at L = 100); it builds its B tile
+// once in shared memory from the exact root table (index m a mod n advanced by
+// additions), then per pass of kAgRows rows stages A.  A warp takes 8 rows x 32
+// NI samples, lane + 32 i so that every store of a warp is one 256-byte run;
+// with fewer than 64 rows the warps split the samples instead (all 8 busy: two
+// of 8 busy took twice as long).  Layouts: B[k][lane][i] (k = 2m - 1 cos, k = 2m
+// sin), A[k][row].  FP64 plans only (FP32 plans run the tensor-core kernels).
+// Measured (GB300, all scales of band <= 32, analysis / synthesis, us, one
+// unfolded product and a rotation recurrence -> now): L = 32, N = 3 392 / 20 ->
+// 30 / 14; L = 100, N = 3 809 / 69 -> 36 / 34; L = 512, N = 3 1132 / 1037 -> 353 / 403.
+// At least a CTA per SM against two (16-row CTAs rebuild more B): 353 against 371
+// at L = 512, N = 3, and 158 against 173 at L = 256, N = 5.
 template <typename T>
 __global__ void __launch_bounds__(256) k_alpha_ana_direct(const CztSeg<T>* __restrict__ segs, int nseg, CallPtrs ptrs) {
   static_assert(sizeof(T) == sizeof(double), "FP32 plans use the tensor-core kernels");
   extern __shared__ __align__(16) unsigned char smem_raw[];
   constexpr int KMAX = 2 * kDirectMaxLjAna - 1;
-  constexpr int AW = 1;                     // stored copies of each A value
   T* Bs = reinterpret_cast<T*>(smem_raw);  // [KMAX][32][4]
-  T* As = Bs + KMAX * kAgCols;              // [KMAX][kAgRows][AW]
+  T* As = Bs + KMAX * kAgCols;              // [KMAX][kAgRows]
   const CztSeg<T> sg = segs[czt_find_seg<T>(segs, nseg)];
   const int item = blockIdx.x - sg.start;
-  const int Lj = sg.Lj, L = sg.L, n = 2 * L - 1, K = 2 * Lj - 1;
-  const int ntile = (n + kAgCols - 1) / kAgCols;
+  const int Lj = sg.Lj, L = sg.L, n = 2 * L - 1;
+  const int ntile = (L + kAgCols - 1) / kAgCols;
   const int a0 = (item % ntile) * kAgCols;
-  const int nrows = sg.N * sg.nb, rbeg = (item / ntile) * kAgChunk, rend = min(nrows, rbeg + kAgChunk);
+  const int nrows = sg.N * sg.nb, rbeg = (item / ntile) * sg.P, rend = min(nrows, rbeg + sg.P);
   const int t = threadIdx.x, w = t >> 5, lane = t & 31;
   const cx<T>* __restrict__ root = sg.pre;  // e^{2 pi i u / n}, u < n
   T* __restrict__ Wb = reinterpret_cast<T*>(sg.is_phi ? ptrs.Wphi[sg.job] : ptrs.W[sg.job]) + sg.woff;
-  if (K <= 0) {  // empty scale: W = 0
+  if (Lj <= 0) {  // empty scale: W = 0
     for (int r = rbeg; r < rend; ++r)
-      for (int c = t; c < kAgCols; c += blockDim.x)
-        if (a0 + c < n) Wb[(size_t)r * n + a0 + c] = T(0);
+      for (int c = t; c < kAgCols; c += blockDim.x) {
+        const int a = a0 + c;
+        if (a < L) Wb[(size_t)r * n + a] = T(0);
+        if (a > 0 && a < L) Wb[(size_t)r * n + n - a] = T(0);
+      }
     return;
   }
   // B tile: thread t fills sample c = t % kAgCols for m = 1 + t / kAgCols, step 256 / kAgCols
@@ -1040,8 +1096,7 @@ __global__ void __launch_bounds__(256) k_alpha_ana_direct(const CztSeg<T>* __res
     constexpr int MS = 256 / kAgCols;
     const int c = t % kAgCols, a = a0 + c;
     const int pos = (c & 31) * 4 + (c >> 5);  // [lane][i] of sample c = lane + 32 i
-    const bool ok = a < n;
-    if (t < kAgCols) Bs[pos] = ok ? T(1) : T(0);
+    const bool ok = a < L;
     int m = 1 + t / kAgCols;
     int u = ok ? (int)(((long long)m * a) % n) : 0;
     const int du = ok ? (int)(((long long)MS * a) % n) : 0;
@@ -1061,96 +1116,71 @@ __global__ void __launch_bounds__(256) k_alpha_ana_direct(const CztSeg<T>* __res
     for (int i = t; i < kAgRows * Lj; i += blockDim.x) {
       const int m = i / kAgRows, r = i % kAgRows;  // consecutive threads: consecutive rows (no bank conflicts)
       const cx<T> x = r < nr ? sg.buf_in[(size_t)(r0 + r) * Lj + m] : mkc<T>(0, 0);
-      const int k1 = m == 0 ? 0 : 2 * m - 1;
-#pragma unroll
-      for (int d = 0; d < AW; ++d) As[(k1 * kAgRows + r) * AW + d] = x.x;
-      if (m > 0) {
-#pragma unroll
-        for (int d = 0; d < AW; ++d) As[((k1 + 1) * kAgRows + r) * AW + d] = x.y;
-      }
+      As[(m == 0 ? 0 : 2 * m - 1) * kAgRows + r] = x.x;
+      if (m > 0) As[(2 * m) * kAgRows + r] = x.y;
     }
     __syncthreads();
-    T out[8][4];
-    {
-#pragma unroll
-      for (int r = 0; r < 8; ++r)
-#pragma unroll
-        for (int i = 0; i < 4; ++i) out[r][i] = T(0);
-      const T* __restrict__ ap = As + 8 * w;
-      const T* __restrict__ bp = Bs + 4 * lane;
-#pragma unroll 2
-      for (int k = 0; k < K; ++k) {
-        T av[8], bv[4];
-#pragma unroll
-        for (int r = 0; r < 8; ++r) av[r] = ap[r];
-#pragma unroll
-        for (int i = 0; i < 4; ++i) bv[i] = bp[i];
-#pragma unroll
-        for (int r = 0; r < 8; ++r)
-#pragma unroll
-          for (int i = 0; i < 4; ++i) out[r][i] = fma(av[r], bv[i], out[r][i]);
-        ap += kAgRows;
-        bp += kAgCols;
-      }
-    }
-#pragma unroll
-    for (int r = 0; r < 8; ++r) {
-      const int row = 8 * w + r;
-      if (row < nr) {
-#pragma unroll
-        for (int i = 0; i < 4; ++i) {
-          const int a = a0 + lane + 32 * i;
-          if (a < n) Wb[(size_t)(r0 + row) * n + a] = out[r][i];
-        }
-      }
-    }
+    // warps: row groups of 8, and where a CTA has fewer than 64 rows column groups (every
+    // quarter of the SM has its own FP64 pipe)
+    const int nrg = min(kAgRows, sg.P) >> 3, rg = w % nrg;  // 2, 4 or 8 row groups
+    const int ni = nrg >> 1, i0 = (w / nrg) * ni;           // this warp's groups of 32 samples: [i0, i0 + ni)
+    if (8 * rg >= nr || a0 + 32 * i0 >= L) continue;  // (the whole warp; no barrier inside)
+    const int live = min(ni, (L - a0 - 32 * i0 + 31) / 32);      // groups of 32 samples in range
+    T* __restrict__ Wr = Wb + (size_t)(r0 + 8 * rg) * n;
+    const int nrow = min(8, nr - 8 * rg);
+    if (live == 4) alpha_ana_rows<T, 4>(As + 8 * rg, Bs, i0, Lj, L, a0, nrow, Wr);
+    else if (live == 3) alpha_ana_rows<T, 3>(As + 8 * rg, Bs, i0, Lj, L, a0, nrow, Wr);
+    else if (live == 2) alpha_ana_rows<T, 2>(As + 8 * rg, Bs, i0, Lj, L, a0, nrow, Wr);
+    else alpha_ana_rows<T, 1>(As + 8 * rg, Bs, i0, Lj, L, a0, nrow, Wr);
   }
 }
 
 // V[row][m] = (2 pi / n) sum_{a<n} W[row][a] e^{-2 pi i m a / n}, m < Lj   (Eq. (37))
-// A CTA takes R = 32 / sizeof(T) rows, staged in shared memory as one 32-byte
-// line per sample a (Ws[a][r]) so that a lane reads all R rows with two
-// 16-byte loads; loads are issued in unrolled batches (rows have odd length,
-// so neither 16-byte copies nor TMA tiles apply).  Warp w sums the a-range
-// chunk w; its lanes are (sub, m) with P = 32 / Lj lanes per m splitting the
-// chunk further.  Partials are reduced over sub by shuffles when Lj divides
-// 32, then over the chunks in shared memory.
+// folded like the analysis: with s, d = W_a +- W_{n-a} (a < L; W_0 alone),
+//   Re V = (2 pi/n) sum s cos, Im V = -(2 pi/n) sum d sin.
+// A CTA takes R = 4 rows, s and d staged in shared memory as one 64-byte line
+// per sample a; loads are issued in unrolled batches (rows have odd length, so
+// neither 16-byte copies nor TMA tiles apply).  The roots come from the table (a
+// rotation recurrence took a third of the FP64 operations).  Warp w sums the a-range chunk w;
+// its lanes are (sub, m) with P = 32 / Lj lanes per m splitting the chunk
+// further.  Partials are reduced over sub by shuffles when Lj divides 32, then
+// over the chunks in shared memory.
 // FP64 plans only (FP32 plans run the tensor-core kernels of alpha_tc.cu).
-template <typename T>
-__device__ __forceinline__ void syn_direct_line(const T* p, T (&x)[32 / sizeof(T)]) {
-  const double2 a = reinterpret_cast<const double2*>(p)[0], b = reinterpret_cast<const double2*>(p)[1];
-  x[0] = a.x; x[1] = a.y; x[2] = b.x; x[3] = b.y;
-}
-
 template <typename T>
 __global__ void __launch_bounds__(256) k_alpha_syn_direct(const CztSeg<T>* __restrict__ segs, int nseg, CallPtrs ptrs) {
   static_assert(sizeof(T) == sizeof(double), "FP32 plans use the tensor-core kernels");
   extern __shared__ __align__(16) unsigned char smem_raw[];
   constexpr int R = 32 / sizeof(T);
-  constexpr int U = 4;  // samples per thread per load batch (R * U loads in flight)
+  constexpr int U = 2;  // sample pairs per thread per load batch (2 R U loads in flight)
   const CztSeg<T> sg = segs[czt_find_seg<T>(segs, nseg)];
   const int item = blockIdx.x - sg.start;
   const int Lj = sg.Lj, L = sg.L, n = 2 * L - 1;
   const int nrows = sg.N * sg.nb, row0 = item * R, nr = min(R, nrows - row0);
-  T* Ws = reinterpret_cast<T*>(smem_raw);  // [n][R], later the partials
+  T* Ws = reinterpret_cast<T*>(smem_raw);  // [L][s: R, d: R], later the partials
   const T* __restrict__ Wb = reinterpret_cast<const T*>(sg.is_phi ? ptrs.Wphi[sg.job] : ptrs.W[sg.job]) + sg.woff +
                              (size_t)row0 * n;
   const int tid = threadIdx.x;
-  for (int a0 = 0; a0 < n; a0 += U * 256) {
-    T x[U][R];
+  for (int a0 = 0; a0 < L; a0 += U * 256) {
+    T x[U][R], y[U][R];
 #pragma unroll
     for (int u = 0; u < U; ++u) {
       const int a = a0 + u * 256 + tid;
 #pragma unroll
-      for (int r = 0; r < R; ++r) x[u][r] = (a < n && r < nr) ? __ldg(Wb + (size_t)r * n + a) : T(0);
+      for (int r = 0; r < R; ++r) {
+        const bool in = a < L && r < nr;
+        x[u][r] = in ? __ldg(Wb + (size_t)r * n + a) : T(0);
+        y[u][r] = (in && a > 0) ? __ldg(Wb + (size_t)r * n + n - a) : T(0);
+      }
     }
 #pragma unroll
     for (int u = 0; u < U; ++u) {
       const int a = a0 + u * 256 + tid;
-      if (a < n) {
-        double2* d = reinterpret_cast<double2*>(Ws + (size_t)a * R);
-        d[0] = make_double2(x[u][0], x[u][1]);
-        d[1] = make_double2(x[u][2], x[u][3]);
+      if (a < L) {
+        double2* d = reinterpret_cast<double2*>(Ws + (size_t)a * 2 * R);
+        d[0] = make_double2(x[u][0] + y[u][0], x[u][1] + y[u][1]);
+        d[1] = make_double2(x[u][2] + y[u][2], x[u][3] + y[u][3]);
+        d[2] = make_double2(x[u][0] - y[u][0], x[u][1] - y[u][1]);
+        d[3] = make_double2(x[u][2] - y[u][2], x[u][3] - y[u][3]);
       }
     }
   }
@@ -1163,21 +1193,21 @@ __global__ void __launch_bounds__(256) k_alpha_syn_direct(const CztSeg<T>* __res
 #pragma unroll
   for (int r = 0; r < R; ++r) acc[r] = mkc<T>(0, 0);
   if (active) {
-    const int c_lo = (int)(((long long)n * warp) / 8), c_hi = (int)(((long long)n * (warp + 1)) / 8);
+    const int c_lo = (int)(((long long)L * warp) / 8), c_hi = (int)(((long long)L * (warp + 1)) / 8);
     const int a_lo = c_lo + (int)(((long long)(c_hi - c_lo) * sub) / P);
     const int a_hi = c_lo + (int)(((long long)(c_hi - c_lo) * (sub + 1)) / P);
-    const cx<T> st = cconj<T>(ldk(root + m));
-    cx<T> w = mkc<T>(1, 0);
+    int u = (m * a_lo) % n;
+#pragma unroll 2
     for (int a = a_lo; a < a_hi; ++a) {
-      if (((a - a_lo) & 15) == 0) w = cconj<T>(ldk(root + (m * a) % n));
-      T x[R];
-      syn_direct_line<T>(Ws + (size_t)a * R, x);
-#pragma unroll
-      for (int r = 0; r < R; ++r) {
-        acc[r].x = fma(x[r], w.x, acc[r].x);
-        acc[r].y = fma(x[r], w.y, acc[r].y);
-      }
-      w = cmul<T>(w, st);
+      const cx<T> w = cconj<T>(ldk(root + u));
+      u += m;
+      if (u >= n) u -= n;
+      const double2* p = reinterpret_cast<const double2*>(Ws + (size_t)a * 2 * R);
+      const double2 s0 = p[0], s1 = p[1], d0 = p[2], d1 = p[3];
+      acc[0].x = fma(s0.x, w.x, acc[0].x), acc[1].x = fma(s0.y, w.x, acc[1].x);
+      acc[2].x = fma(s1.x, w.x, acc[2].x), acc[3].x = fma(s1.y, w.x, acc[3].x);
+      acc[0].y = fma(d0.x, w.y, acc[0].y), acc[1].y = fma(d0.y, w.y, acc[1].y);
+      acc[2].y = fma(d1.x, w.y, acc[2].y), acc[3].y = fma(d1.y, w.y, acc[3].y);
     }
   }
   // in-warp reduction over sub (lanes m, m + Lj, m + 2 Lj, ...) when Lj | 32
@@ -1213,8 +1243,7 @@ __global__ void __launch_bounds__(256) k_alpha_syn_direct(const CztSeg<T>* __res
 // rows, or the partials (at most 256 x R complex) if larger
 template <typename T>
 size_t alpha_syn_direct_smem(int L) {
-  const size_t n = 2 * (size_t)L - 1;
-  const size_t rows = n * 32, parts = (size_t)256 * (32 / sizeof(T)) * sizeof(cx<T>);
+  const size_t rows = (size_t)L * 64, parts = (size_t)256 * (32 / sizeof(T)) * sizeof(cx<T>);
   return rows > parts ? rows : parts;
 }
 

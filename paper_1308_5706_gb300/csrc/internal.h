@@ -126,8 +126,8 @@ template <typename T>
 constexpr size_t alpha_seg_smem() { return 2 * (size_t)(4096 + 4096 / 16) * 2 * sizeof(T); }
 constexpr int kDirectMaxLj = 32;     // synthesis: direct alpha sums for L_j <= 32
 constexpr int kDirectMaxLjAna = 32;  // analysis: direct (matrix-product) alpha sums for L_j <= 32
-// tile of the direct analysis kernel: samples per CTA, rows per pass, rows per CTA
-constexpr int kAgCols = 128, kAgRows = 64, kAgChunk = 512;
+// tile of the direct analysis kernel: samples per CTA, rows per pass, fewest rows per CTA
+constexpr int kAgCols = 128, kAgRows = 64, kAgMinRows = 16;
 template <typename T>  // B tile + A tile (FP32 stores each A value twice)
 constexpr size_t alpha_ana_direct_smem() {
   return (size_t)(2 * kDirectMaxLjAna - 1) * (kAgCols + kAgRows * (sizeof(T) == 4 ? 2 : 1)) * sizeof(T);
