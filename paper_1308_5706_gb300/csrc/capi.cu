@@ -113,11 +113,12 @@ void kernels_prepare(bool fp64, bool pair) {
   std::lock_guard<std::mutex> lk(g_prep_mu);
   if (!(done_czt[fp64 ? 1 : 0] & bit)) {
     ck(fp64 ? czt_prepare_f64(13) : czt_prepare_f32(13));
+    if (fp64) ck(contract_direct_prepare_f64());
     done_czt[fp64 ? 1 : 0] |= bit;
   }
   if (pair && !(done_pair & bit)) {
     ck(contract_tile_prepare());
-    ck(contract_direct_prepare());
+    ck(contract_direct_prepare_f32());
     ck(split_gemm_prepare());
     done_pair |= bit;
   }
@@ -158,6 +159,7 @@ struct DeltaTab {
   double* raw64 = nullptr;  // the allocations
   float* raw32 = nullptr;
   float* pair32 = nullptr;  // pair table of the FP32 contraction (built for the first FP32 plan)
+  double* pair64 = nullptr; // that of the direct FP64 contraction, l < min(Lmax, kContractDirectMaxL64)
 };
 std::mutex g_mu;
 std::vector<DeltaTab*> g_tabs;
@@ -229,7 +231,7 @@ void delta_pair_ensure(DeltaTab* t, cudaStream_t st) {
   if (t->pair32) return;
   float* pt = nullptr;
   amalloc(&pt, (size_t)pair_table_entries(t->Lmax) * sizeof(float), st);
-  cudaError_t e = launch_pair_table(pt, t->d64, t->Lmax, st);
+  cudaError_t e = launch_pair_table<float>(pt, t->d64, t->Lmax, st);
   if (e == cudaSuccess) e = cudaStreamSynchronize(st);
   if (e != cudaSuccess) {
     afree(pt, st);
@@ -237,6 +239,24 @@ void delta_pair_ensure(DeltaTab* t, cudaStream_t st) {
   }
   t->pair32 = pt;
   t->bytes += (size_t)pair_table_entries(t->Lmax) * sizeof(float);
+}
+
+// The FP64 pair table of the direct contraction (small band-limits only).
+int pair64_reach(const DeltaTab* t) { return std::min(t->Lmax, kContractDirectMaxL64); }
+void delta_pair64_ensure(DeltaTab* t, cudaStream_t st) {
+  std::lock_guard<std::mutex> lk(g_mu);
+  if (t->pair64) return;
+  double* pt = nullptr;
+  const size_t bytes = (size_t)pair_table_entries(pair64_reach(t)) * sizeof(double);
+  amalloc(&pt, bytes, st);
+  cudaError_t e = launch_pair_table<double>(pt, t->d64, pair64_reach(t), st);
+  if (e == cudaSuccess) e = cudaStreamSynchronize(st);
+  if (e != cudaSuccess) {
+    afree(pt, st);
+    throw CudaFail{e};
+  }
+  t->pair64 = pt;
+  t->bytes += bytes;
 }
 
 void delta_release(DeltaTab* t) {
@@ -247,6 +267,7 @@ void delta_release(DeltaTab* t) {
     afree(t->raw64, st);
     afree(t->raw32, st);
     afree(t->pair32, st);
+    afree(t->pair64, st);
     g_tabs.erase(std::remove(g_tabs.begin(), g_tabs.end(), t), g_tabs.end());
     delete t;
   }
@@ -378,7 +399,7 @@ struct s2dw_plan_s {
   // host copies of the static descriptors (device copies live in `own`)
   std::vector<unsigned char> desc_w_host, desc_phi_host;
   std::vector<TileTask> tiles_w_host, tiles_phi_host;  // FP64 plans
-  bool direct_w = false, direct_phi = false;  // FP32: the direct contraction (else the tile kernel)
+  bool direct_w = false, direct_phi = false;  // the direct contraction (else FP32: the tile kernel, FP64: k_contract)
   int pair_shape = kPairShapePair;  // FP32: CTA-shape value of s2dw_plan_choices
   Lists own;
   // stage timing (s2dw_profile): one set of events per call, up to kProfCalls
@@ -478,8 +499,9 @@ void fill_desc(s2dw_plan_s* p, ContractDesc<T>& dw, ContractDesc<T>& dp, const T
   std::memset(&dw, 0, sizeof(dw));
   std::memset(&dp, 0, sizeof(dp));
   dw.delta = delta;
-  dw.dpair = p->tab->pair32;
-  dw.RSp = reinterpret_cast<const float*>(p->RSp);
+  const T* pairs = sizeof(T) == 4 ? reinterpret_cast<const T*>(p->tab->pair32) : reinterpret_cast<const T*>(p->tab->pair64);
+  dw.dpair = pairs;
+  dw.RSp = reinterpret_cast<const T*>(p->RSp);
   dw.fP = reinterpret_cast<const cx<T>*>(p->fP);
   dw.Lr = p->Lr;
   dw.Lrf = p->Lrf;
@@ -532,8 +554,8 @@ void fill_desc(s2dw_plan_s* p, ContractDesc<T>& dw, ContractDesc<T>& dp, const T
   dw.nseg = ns;
   // scaling part: one N = 1 "scale" with kernel Phi on [0, lphi]
   dp.delta = delta;
-  dp.dpair = p->tab->pair32;
-  dp.RSp = reinterpret_cast<const float*>(p->RSphi_p);
+  dp.dpair = pairs;
+  dp.RSp = reinterpret_cast<const T*>(p->RSphi_p);
   dp.fP = reinterpret_cast<const cx<T>*>(p->fP);
   dp.Lr = p->Lrphi;
   dp.Lrf = p->Lrf;
@@ -580,7 +602,8 @@ CTask make_task(int prob, int p, int q, int half, int lstart, int lend, int j, i
 // scales 2i, 2i + 1 (one per slot) over the union of their l ranges, the
 // synthesis by l ranges on which each slot holds one scale (an l-segment
 // where a slot is empty joins its neighbour).
-void build_tile_tasks(const ContractDesc<float>& d, int prob, int Lband, int lend, int table_Lmax,
+template <typename T>
+void build_tile_tasks(const ContractDesc<T>& d, int prob, int Lband, int lend, int table_Lmax,
                       std::vector<CTask>& ana, std::vector<CTask>& syn) {
   if (Lband <= 0 || lend < 0) return;
   struct Range { int lo, hi, j, j2; };
@@ -633,7 +656,8 @@ void sort_tasks(std::vector<CTask>& v) {
 // its descriptor, band Lband, last l lend): every tile, for the analysis once
 // per scale over the scale's l (its [lo, hi] from the l-segments), for the
 // synthesis once per l-segment.
-void build_direct_tasks(const ContractDesc<float>& d, int prob, int Lband, int lend, int table_Lmax,
+template <typename T>
+void build_direct_tasks(const ContractDesc<T>& d, int prob, int Lband, int lend, int table_Lmax,
                         std::vector<CTask>& ana, std::vector<CTask>& syn) {
   if (Lband <= 0 || lend < 0) return;
   const int nb = (Lband + 31) / 32;
@@ -657,12 +681,16 @@ void build_direct_tasks(const ContractDesc<float>& d, int prob, int Lband, int l
 // Analysis: rt rows per thread, so 32 / (8 rt) CTAs of 8 warps per task (8 CTAs
 // of 4 warps at rt = 1): fewer rows per thread while the tasks alone would
 // leave SMs idle (a thread's R loads serve its rt rows).  Synthesis: pieces of
-// a multiple of 16 l, about four CTAs per SM over the launch.
-int direct_split(std::vector<CTask>& ana, std::vector<CTask>& syn, int sms) {
+// a multiple of 16 l, about four CTAs per SM over the launch.  FP64 (rt is not
+// used): pieces of a multiple of 4 l, two CTAs each; with N > 2 two CTAs per SM,
+// because each repeats the gamma step of its rows (four / one piece per SM, us:
+// L = 256, N = 1 125 / 152, N = 3 256 / 220, N = 8 682 / 427).
+int direct_split(std::vector<CTask>& ana, std::vector<CTask>& syn, int sms, bool fp64, int N) {
   const long long n = (long long)ana.size();
   long long total = 0;
   for (const CTask& t : syn) total += t.lend - t.lstart + 1;
-  const int ls = round_up((int)std::min<long long>(std::max<long long>((total + 4LL * sms - 1) / (4LL * sms), 1), 4096), 16);
+  const long long want = (fp64 && N > 2 ? 1LL : 4LL) * sms;
+  const int ls = round_up((int)std::min<long long>(std::max<long long>((total + want - 1) / want, 1), 4096), fp64 ? 4 : 16);
   std::vector<CTask> cut;
   for (const CTask& t : syn)
     for (int l = t.lstart; l <= t.lend; l += ls) {
@@ -886,7 +914,7 @@ Lists* build_lists(const std::vector<s2dw_plan_t>& plans) {
   std::vector<ContractDesc<T>> dw(nj), dp(nj);
   std::map<int, std::vector<Task>> tw_byN;
   std::vector<Task> tphi;
-  struct FpTasks {  // FP32 contraction: analysis and synthesis tasks
+  struct FpTasks {  // direct and tile contractions: analysis and synthesis tasks
     std::vector<CTask> task[2];
     int rt = 4;
     size_t off[2] = {0, 0};
@@ -901,12 +929,15 @@ Lists* build_lists(const std::vector<s2dw_plan_t>& plans) {
     s2dw_plan_s* p = plans[i];
     std::memcpy(&dw[i], p->desc_w_host.data(), sizeof(ContractDesc<T>));
     std::memcpy(&dp[i], p->desc_phi_host.data(), sizeof(ContractDesc<T>));
-    if constexpr (sizeof(T) == sizeof(float)) {
-      FpTasks& w = (p->direct_w ? dir_byN : tile_byN)[p->N];
-      (p->direct_w ? build_direct_tasks : build_tile_tasks)(dw[i], i, p->L0, p->lend_w, p->tab->Lmax, w.task[0], w.task[1]);
-      FpTasks& f = p->direct_phi ? dir_phi : tile_phi;
-      (p->direct_phi ? build_direct_tasks : build_tile_tasks)(dp[i], i, p->Lphi, p->lphi, p->tab->Lmax, f.task[0], f.task[1]);
-    }
+    const int reach = sizeof(T) == sizeof(float) ? p->tab->Lmax : pair64_reach(p->tab);
+    auto add = [&](FpTasks& w, const ContractDesc<T>& d, bool direct, int Lband, int lend) {
+      if (direct) build_direct_tasks<T>(d, i, Lband, lend, reach, w.task[0], w.task[1]);
+      else build_tile_tasks<T>(d, i, Lband, lend, reach, w.task[0], w.task[1]);
+    };
+    if (sizeof(T) == sizeof(float) || p->direct_w)
+      add((p->direct_w ? dir_byN : tile_byN)[p->N], dw[i], p->direct_w, p->L0, p->lend_w);
+    if (sizeof(T) == sizeof(float) || p->direct_phi)
+      add(p->direct_phi ? dir_phi : tile_phi, dp[i], p->direct_phi, p->Lphi, p->lphi);
     for (Task t : p->tiles_w_host) {  // (FP64 plans)
       t.prob = i;
       tw_byN[p->N].push_back(t);
@@ -954,9 +985,12 @@ Lists* build_lists(const std::vector<s2dw_plan_t>& plans) {
     if (cudaGetDevice(&dev) == cudaSuccess) cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
   }
   std::vector<FpTasks*> fp;
-  for (auto& kv : dir_byN) fp.push_back(&kv.second);
+  for (auto& kv : dir_byN) {
+    fp.push_back(&kv.second);
+    kv.second.rt = direct_split(kv.second.task[0], kv.second.task[1], sms, sizeof(T) == 8, kv.first);
+  }
   fp.push_back(&dir_phi);
-  for (FpTasks* b : fp) b->rt = direct_split(b->task[0], b->task[1], sms);
+  dir_phi.rt = direct_split(dir_phi.task[0], dir_phi.task[1], sms, sizeof(T) == 8, 1);
   const size_t ndir = fp.size();
   for (auto& kv : tile_byN) fp.push_back(&kv.second);
   fp.push_back(&tile_phi);
@@ -1060,22 +1094,23 @@ inline void mark_use(s2dw_plan_t p, cudaStream_t st) {
   if (!capturing(st)) cudaEventRecord(p->last_use, st);
 }
 
-// Direct FP32 contraction launches of one direction (the scaling parts ride
+// Direct contraction launches of one direction (the scaling parts ride
 // with the first group); the number of launches.
 int direct_groups(const Lists& ls) { return (int)ls.dir_w.size() + (ls.dir_w.empty() && ls.dir_phi.n[0] > 0 ? 1 : 0); }
-void run_direct(const Lists& ls, bool syn, const ContractDesc<float>* dw, const ContractDesc<float>* dp,
+template <typename T>
+void run_direct(const Lists& ls, bool syn, const ContractDesc<T>* dw, const ContractDesc<T>* dp,
                 const CallPtrs& ptrs, cudaStream_t st) {
   const int d = syn ? 1 : 0;
-  const DirTasks phi{dp, reinterpret_cast<const CTask*>(ls.dir_phi.task[d]), ls.dir_phi.n[d]};
-  DirTasks none = phi;
+  const DirTasks<T> phi{dp, reinterpret_cast<const CTask*>(ls.dir_phi.task[d]), ls.dir_phi.n[d]};
+  DirTasks<T> none = phi;
   none.n = 0;
   bool first = true;
   for (const auto& g : ls.dir_w) {
-    launch_contract_direct(g.N, syn, g.rt, DirTasks{dw, reinterpret_cast<const CTask*>(g.task[d]), g.n[d]},
+    launch_contract_direct<T>(g.N, syn, g.rt, DirTasks<T>{dw, reinterpret_cast<const CTask*>(g.task[d]), g.n[d]},
                            first ? phi : none, ptrs, st);
     first = false;
   }
-  if (first) launch_contract_direct(1, syn, ls.dir_phi.rt, DirTasks{dw, nullptr, 0}, phi, ptrs, st);
+  if (first) launch_contract_direct<T>(1, syn, ls.dir_phi.rt, DirTasks<T>{dw, nullptr, 0}, phi, ptrs, st);
 }
 
 // Analysis stages: [contraction + gamma | scaling contraction | beta | alpha chirp-z full-band | segmented
@@ -1103,7 +1138,9 @@ void run_analysis(const Lists& ls, const CallPtrs& ptrs, cudaStream_t st, cudaEv
   rec(ev, 0, st);
   if constexpr (sizeof(T) == sizeof(float)) {
     launch_fpack(dw, ls.njobs, ls.nbmax, ls.Lrmax, ptrs, st);
-    run_direct(ls, false, dw, dp, ptrs, st);
+  }
+  run_direct<T>(ls, false, dw, dp, ptrs, st);
+  if constexpr (sizeof(T) == sizeof(float)) {
     for (auto& g : ls.tile_w)
       launch_contract_tile(g.N, 2, false, dw, reinterpret_cast<const CTask*>(g.task[0]), g.n[0], st);
     rec(ev, 1, st);
@@ -1169,8 +1206,8 @@ void run_synthesis(const Lists& ls, const CallPtrs& ptrs, const ReduceJobs& rj, 
   launch_dct_parts<T>(ls, CZT_BETA_SYN_DCT, ptrs, st);
   launch_products<T>(ls, SG_KIND_BETA_SYN, ptrs, st);
   rec(ev, 4, st);
+  run_direct<T>(ls, true, dw, dp, ptrs, st);
   if constexpr (sizeof(T) == sizeof(float)) {
-    run_direct(ls, true, dw, dp, ptrs, st);
     for (auto& g : ls.tile_w)
       launch_contract_tile(g.N, 2, true, dw, reinterpret_cast<const CTask*>(g.task[1]), g.n[1], st);
     rec(ev, 5, st);
@@ -1234,18 +1271,18 @@ void plan_build_typed(s2dw_plan_s* p, const double* kap_d, const double* phi_d, 
     off = align256(off + bytes);
     return o;
   };
+  const bool dir64 = sizeof(T) == sizeof(double) && p->direct_w;
   const bool pairc = sizeof(T) == sizeof(float);  // FP32 contraction (pair table)
   const int NH = (N + 1) / 2;
   p->Lr = L + kPairPadL;  // read-ahead rows of the tile contraction
   p->Lrphi = p->Lphi + kPairPadL;
   p->Lrf = L + kPairPadL;
   const int nbw = (L + 31) / 32, nbp = (p->Lphi + 31) / 32;
-  const size_t o_RS = pairc ? take(0) : take((size_t)L * 2 * NH * p->Lp * sizeof(T));
-  const size_t o_RSphi = pairc ? take(0) : take((size_t)p->Lphi * p->Lphip * sizeof(T));
-  const size_t o_RSp = pairc ? take((size_t)nbw * p->Lr * 2 * NH * 32 * sizeof(float)) : take(0);
-  const size_t o_RSphi_p = pairc ? take((size_t)nbp * p->Lrphi * 32 * sizeof(float)) : take(0);
-  p->direct_w = pairc && p->L0 <= kContractDirectMaxL;
-  p->direct_phi = pairc && p->Lphi <= kContractDirectMaxL;
+  const bool pairt = pairc || dir64;  // R rows in the pair layout
+  const size_t o_RS = pairt ? take(0) : take((size_t)L * 2 * NH * p->Lp * sizeof(T));
+  const size_t o_RSphi = pairt ? take(0) : take((size_t)p->Lphi * p->Lphip * sizeof(T));
+  const size_t o_RSp = pairt ? take((size_t)nbw * p->Lr * 2 * NH * 32 * sizeof(T)) : take(0);
+  const size_t o_RSphi_p = pairt ? take((size_t)nbp * p->Lrphi * 32 * sizeof(T)) : take(0);
   const bool packf = pairc && !(p->direct_w && p->direct_phi);  // the direct contraction reads f itself
   const size_t o_fP = packf ? take((size_t)nbw * p->Lrf * 32 * sizeof(cx<T>)) : take(0);
   std::vector<size_t> o_Y(p->nscale + 1), o_X(p->nscale + 1);
@@ -1355,10 +1392,10 @@ void plan_build_typed(s2dw_plan_s* p, const double* kap_d, const double* phi_d, 
   p->ws_bytes = off;
   amalloc(&p->ws, off, st);
   char* b = reinterpret_cast<char*>(p->ws);
-  p->RS = pairc ? nullptr : b + o_RS;
-  p->RSphi = pairc ? nullptr : b + o_RSphi;
-  p->RSp = pairc ? b + o_RSp : nullptr;
-  p->RSphi_p = pairc ? b + o_RSphi_p : nullptr;
+  p->RS = pairt ? nullptr : b + o_RS;
+  p->RSphi = pairt ? nullptr : b + o_RSphi;
+  p->RSp = pairt ? b + o_RSp : nullptr;
+  p->RSphi_p = pairt ? b + o_RSphi_p : nullptr;
   p->fP = packf ? b + o_fP : nullptr;
   p->Y.resize(p->nscale + 1);
   p->X.resize(p->nscale + 1);
@@ -1415,11 +1452,10 @@ void plan_build_typed(s2dw_plan_s* p, const double* kap_d, const double* phi_d, 
   ck(cudaMemcpyAsync(slot_d, slot_w.data(), slot_w.size() * sizeof(int), cudaMemcpyHostToDevice, st));
   ck(cudaMemcpyAsync(slot_d + slot_w.size(), slot_p.data(), slot_p.size() * sizeof(int), cudaMemcpyHostToDevice,
                      st));
-  if (pairc) {
-    ck(launch_rtable_pair(reinterpret_cast<float*>(p->RSp), p->tab->d64, kap_d, sabs_d, slot_d, L, p->Lr, N, 2, L,
-                          st));
-    ck(launch_rtable_pair(reinterpret_cast<float*>(p->RSphi_p), p->tab->d64, phi_d, nullptr, slot_d + slot_w.size(),
-                          p->Lphi, p->Lrphi, 1, 1, L, st));
+  if (pairt) {
+    ck(launch_rtable_pair<T>(reinterpret_cast<T*>(p->RSp), p->tab->d64, kap_d, sabs_d, slot_d, L, p->Lr, N, 2, L, st));
+    ck(launch_rtable_pair<T>(reinterpret_cast<T*>(p->RSphi_p), p->tab->d64, phi_d, nullptr, slot_d + slot_w.size(),
+                             p->Lphi, p->Lrphi, 1, 1, L, st));
   } else {
     ck(launch_rtable<T>(reinterpret_cast<T*>(p->RS), p->tab->d64, kap_d, sabs_d, slot_d, L, p->Lp, N, 2, L, st));
     ck(launch_rtable<T>(reinterpret_cast<T*>(p->RSphi), p->tab->d64, phi_d, nullptr, slot_d + slot_w.size(),
@@ -1515,6 +1551,8 @@ void plan_build_typed(s2dw_plan_s* p, const double* kap_d, const double* phi_d, 
   if (pairc) {
     delta_pair_ensure(p->tab, st);
     kernels_prepare(false, true);
+  } else if (dir64) {
+    delta_pair64_ensure(p->tab, st);
   }
   ContractDesc<T> dw, dp;
   const T* delta = (sizeof(T) == sizeof(double)) ? reinterpret_cast<const T*>(p->tab->d64)
@@ -1535,7 +1573,7 @@ void plan_build_typed(s2dw_plan_s* p, const double* kap_d, const double* phi_d, 
       if (!pair_shapes_offered(N) || npairs < 3LL * sms) p->pair_shape = kPairShapeTile;
       else p->pair_shape = N >= 4 ? kPairShapePair : kPairShapeTile2;
     }
-  } else {
+  } else if (!dir64) {
     build_tiles(p->L0, p->lend_w, p->TMP, 0, p->tiles_w_host);
     build_tiles(p->Lphi, p->lphi, p->TMP, 0, p->tiles_phi_host);
     sort_tiles(p->tiles_w_host);
@@ -1638,8 +1676,16 @@ int plan_create(s2dw_plan_t* out, int L, int N, double lam, int J0, unsigned fla
     p->Lp32 = round_up(L, 32);
     p->Lphip = round_up(p->Lphi, 32);
     p->Lphip32 = round_up(p->Lphi, 32);
-    p->nbr = (p->L0 + p->TMP - 1) / p->TMP;
-    p->nbr_phi = (p->Lphi + p->TMP - 1) / p->TMP;
+    if (p->fp64) {
+      p->direct_w = p->direct_phi = L <= kContractDirectMaxL64;
+    } else {
+      p->direct_w = p->L0 <= kContractDirectMaxL;
+      p->direct_phi = p->Lphi <= kContractDirectMaxL;
+    }
+    // blocks of partials: TMP rows each; the direct contraction writes whole 32-row tiles
+    const int rows = p->direct_w ? 32 : p->TMP, rows_phi = p->direct_phi ? 32 : p->TMP;
+    p->nbr = (p->L0 + rows - 1) / rows * (rows / p->TMP);
+    p->nbr_phi = (p->Lphi + rows_phi - 1) / rows_phi * (rows_phi / p->TMP);
     // sampling grid of every scale (last: the scaling part): the full grid of
     // band-limit L, or with S2DW_MULTIRES the grid of the scale's own
     // band-limit (1 + the last l with a nonzero kernel)
@@ -1852,6 +1898,8 @@ int s2dw_sht_forward(s2dw_plan_t p, const void* fpix, void* flm, void* stream) {
   rj.dp[0] = c->own.desc_phi;
   rj.out[0] = flm;
   rj.L[0] = c->L;
+  rj.tmp[0] = c->TMP;
+  rj.halves[0] = c->fp64 && c->direct_w ? 1 : 0;
   rj.lend[0] = c->lend_w;
   rj.Lphi[0] = c->Lphi;
   rj.sht[0] = 1;
@@ -2011,6 +2059,8 @@ int s2dw_plan_tune(s2dw_plan_t p, int reps, int* choices, int* n) {
         rj.dp[0] = p->own.desc_phi;
         rj.out[0] = fr;
         rj.L[0] = p->L;
+        rj.tmp[0] = p->TMP;
+        rj.halves[0] = p->fp64 && p->direct_w ? 1 : 0;
         rj.lend[0] = p->lend_w;
         rj.Lphi[0] = p->Lphi;
         if (p->fp64) {
@@ -2197,6 +2247,8 @@ int s2dw_synthesis(s2dw_plan_t p, const void* W, const void* Wphi, void* flm, vo
   rj.dp[0] = p->own.desc_phi;
   rj.out[0] = flm;
   rj.L[0] = p->L;
+  rj.tmp[0] = p->TMP;
+  rj.halves[0] = p->fp64 && p->direct_w ? 1 : 0;
   rj.lend[0] = p->lend_w;
   rj.Lphi[0] = p->Lphi;
   cudaEvent_t* ev = nullptr;
@@ -2346,6 +2398,8 @@ int s2dw_synthesis_batch(const s2dw_plan_t* plans, const void* const* W, const v
     rj.dp[i] = reinterpret_cast<const char*>(ls->desc_phi) + i * dsz;
     rj.out[i] = flm[i];
     rj.L[i] = plans[i]->L;
+    rj.tmp[i] = plans[i]->TMP;
+    rj.halves[i] = plans[i]->fp64 && plans[i]->direct_w ? 1 : 0;
     rj.lend[i] = plans[i]->lend_w;
     rj.Lphi[i] = plans[i]->Lphi;
   }

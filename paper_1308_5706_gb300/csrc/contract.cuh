@@ -51,27 +51,32 @@ constexpr size_t kCtaSmemBudget = 112 * 1024;  // two CTAs per SM (228 KB, 1 KB 
 // four multiply-adds per pair and sample.  cg[k N + g]: the factors of n_k.
 // (Fused operations are explicit, so that every instantiation rounds alike: a
 // batched call equals the single one bit for bit.)
-template <int N>
-__device__ __forceinline__ void gamma_ana(const float2 (&b0)[(N + 1) / 2], const float2 (&b1)[(N + 1) / 2], bool plus,
-                                          const float2* cg, float2 (&y)[N]) {
+__device__ __forceinline__ float fma_rn(float a, float b, float c) { return __fmaf_rn(a, b, c); }
+__device__ __forceinline__ double fma_rn(double a, double b, double c) { return __fma_rn(a, b, c); }
+__device__ __forceinline__ float mul_rn(float a, float b) { return __fmul_rn(a, b); }
+__device__ __forceinline__ double mul_rn(double a, double b) { return __dmul_rn(a, b); }
+
+template <int N, typename T>
+__device__ __forceinline__ void gamma_ana(const cx<T> (&b0)[(N + 1) / 2], const cx<T> (&b1)[(N + 1) / 2], bool plus,
+                                          const cx<T>* cg, cx<T> (&y)[N]) {
   constexpr int NH = (N + 1) / 2, ZH = N & 1;
-  float2 P[NH], Q[NH];
+  cx<T> P[NH], Q[NH];
 #pragma unroll
   for (int q = ZH; q < NH; ++q) {
-    const float2 p = plus ? b0[q] : b1[q], r = plus ? b1[q] : b0[q];
-    P[q] = make_float2(2.f * p.x, 2.f * p.y);
-    Q[q] = make_float2(2.f * r.x, 2.f * r.y);
+    const cx<T> p = plus ? b0[q] : b1[q], r = plus ? b1[q] : b0[q];
+    P[q] = mkc<T>(T(2) * p.x, T(2) * p.y);
+    Q[q] = mkc<T>(T(2) * r.x, T(2) * r.y);
   }
 #pragma unroll
   for (int g = 0; g < N; ++g) {
-    float2 z = ZH ? make_float2(b0[0].x + b1[0].x, b0[0].y + b1[0].y) : make_float2(0.f, 0.f);
+    cx<T> z = ZH ? mkc<T>(b0[0].x + b1[0].x, b0[0].y + b1[0].y) : mkc<T>(0, 0);
 #pragma unroll
     for (int q = ZH; q < NH; ++q) {
-      const float2 c = cg[(N / 2 + q) * N + g];
-      z.x = __fmaf_rn(P[q].x, c.x, z.x);
-      z.x = __fmaf_rn(-Q[q].y, c.y, z.x);
-      z.y = __fmaf_rn(P[q].y, c.x, z.y);
-      z.y = __fmaf_rn(Q[q].x, c.y, z.y);
+      const cx<T> c = cg[(N / 2 + q) * N + g];
+      z.x = fma_rn(P[q].x, c.x, z.x);
+      z.x = fma_rn(-Q[q].y, c.y, z.x);
+      z.y = fma_rn(P[q].y, c.x, z.y);
+      z.y = fma_rn(Q[q].x, c.y, z.y);
     }
     y[g] = z;
   }
@@ -81,32 +86,26 @@ __device__ __forceinline__ void gamma_ana(const float2 (&b0)[(N + 1) / 2], const
 // the tile's sign applied): 2 Re(factor) v where plus (tau sgn = 1, with
 // l_start's parity or the other one for the other bank), else 2 i Im(factor) v;
 // n = 0: the factor itself.
-template <int N>
-__device__ __forceinline__ void gamma_syn_add(float2 (&h)[(N + 1) / 2], float2 v, bool plus, const float2* cg, int g) {
+template <int N, typename T>
+__device__ __forceinline__ void gamma_syn_add(cx<T> (&h)[(N + 1) / 2], cx<T> v, bool plus, const cx<T>* cg, int g) {
   constexpr int NH = (N + 1) / 2, ZH = N & 1;
   if (ZH) {
-    const float c = cg[(N / 2) * N + g].x;
-    h[0].x = __fmaf_rn(v.x, c, h[0].x);
-    h[0].y = __fmaf_rn(v.y, c, h[0].y);
+    const T c = cg[(N / 2) * N + g].x;
+    h[0].x = fma_rn(v.x, c, h[0].x);
+    h[0].y = fma_rn(v.y, c, h[0].y);
   }
-  const float2 u = plus ? make_float2(2.f * v.x, 2.f * v.y) : make_float2(-2.f * v.y, 2.f * v.x);
+  const cx<T> u = plus ? mkc<T>(T(2) * v.x, T(2) * v.y) : mkc<T>(T(-2) * v.y, T(2) * v.x);
 #pragma unroll
   for (int q = ZH; q < NH; ++q) {
-    const float2 f = cg[(N / 2 + q) * N + g];
-    const float c = plus ? f.x : f.y;
-    h[q].x = __fmaf_rn(u.x, c, h[q].x);
-    h[q].y = __fmaf_rn(u.y, c, h[q].y);
+    const cx<T> f = cg[(N / 2 + q) * N + g];
+    const T c = plus ? f.x : f.y;
+    h[q].x = fma_rn(u.x, c, h[q].x);
+    h[q].y = fma_rn(u.y, c, h[q].y);
   }
 }
 
 // E consecutive values from 16-byte aligned shared memory.
 template <typename T, int E> struct VecLdS;
-template <> struct VecLdS<float, 4> {
-  static __device__ __forceinline__ void ld(const float* p, float (&r)[4]) {
-    const float4 v = *reinterpret_cast<const float4*>(p);
-    r[0] = v.x; r[1] = v.y; r[2] = v.z; r[3] = v.w;
-  }
-};
 template <> struct VecLdS<double, 2> {
   static __device__ __forceinline__ void ld(const double* p, double (&r)[2]) {
     const double2 v = *reinterpret_cast<const double2*>(p);
@@ -115,36 +114,10 @@ template <> struct VecLdS<double, 2> {
 };
 
 // Accumulators of a thread: E elements x NSLOT slots x N orders, complex.
-// Generic form: cx<T> per entry.  float with E = 4: real and imaginary parts
-// of element pairs (0,1), (2,3) packed for f32x2 instructions.
-template <typename T, int E, int NSLOT, int N, bool PACK> struct Acc;
-template <typename T, int E, int NSLOT, int N> struct Acc<T, E, NSLOT, N, false> {
+template <typename T, int E, int NSLOT, int N> struct Acc {
   cx<T> v[E][NSLOT][N];
   __device__ __forceinline__ cx<T> get(int e, int s, int k) const { return v[e][s][k]; }
   __device__ __forceinline__ void set(int e, int s, int k, cx<T> x) { v[e][s][k] = x; }
-};
-template <int E, int NSLOT, int N> struct Acc<float, E, NSLOT, N, true> {
-  f2p x[E / 2][NSLOT][N], y[E / 2][NSLOT][N];
-  __device__ __forceinline__ cx<float> get(int e, int s, int k) const {
-    float a0, a1, b0, b1;
-    upk2(x[e >> 1][s][k], a0, a1);
-    upk2(y[e >> 1][s][k], b0, b1);
-    return (e & 1) ? mkc<float>(a1, b1) : mkc<float>(a0, b0);
-  }
-  __device__ __forceinline__ void set(int e, int s, int k, cx<float> v) {
-    float a0, a1, b0, b1;
-    upk2(x[e >> 1][s][k], a0, a1);
-    upk2(y[e >> 1][s][k], b0, b1);
-    if (e & 1) {
-      a1 = v.x;
-      b1 = v.y;
-    } else {
-      a0 = v.x;
-      b0 = v.y;
-    }
-    x[e >> 1][s][k] = pk2(a0, a1);
-    y[e >> 1][s][k] = pk2(b0, b1);
-  }
 };
 
 // Shared-memory geometry of one pipeline stage (element counts of T).
@@ -180,7 +153,7 @@ __host__ __device__ constexpr size_t contract_smem_bytes() {
 
 // Two CTAs per SM (128 registers) where the accumulators allow it (FP32, N <= 5).
 template <typename T, int N, int NSLOT, bool SYN, int E>
-__global__ void __launch_bounds__(256, (sizeof(T) == 4 && N <= 5 ? 2 : 1))
+__global__ void __launch_bounds__(256, 1)
 k_contract(const ContractDesc<T>* __restrict__ descs, const TileTask* __restrict__ tiles, CallPtrs ptrs) {
   using G = StageGeom<T, N, NSLOT, E>;
   constexpr int STAGES = contract_stages<T, N, NSLOT, SYN, E>();
@@ -302,8 +275,7 @@ k_contract(const ContractDesc<T>* __restrict__ descs, const TileTask* __restrict
 #pragma unroll
   for (int i = 0; i < STAGES - 2; ++i) issue();
 
-  constexpr bool PACK = std::is_same<T, float>::value && E == 4;
-  Acc<T, E, NSLOT, N, PACK> acc;
+  Acc<T, E, NSLOT, N> acc;
 #pragma unroll
   for (int e = 0; e < E; ++e)
 #pragma unroll
@@ -432,88 +404,47 @@ k_contract(const ContractDesc<T>* __restrict__ descs, const TileTask* __restrict
         for (int e = 0; e < E; ++e) dv[e] *= (e & 1) ? -sg0 : sg0;
       }
       const T* Rr = S + G::R_OFF + (mpb - mp0);
-      if constexpr (PACK) {
-        // float, E = 4: pairs (0,1) and (2,3) per f32x2 instruction
-        if (!SYN) {
-          const cx<T> fv = reinterpret_cast<const cx<T>*>(S + G::F_OFF)[c];
-          const f2p fx = pk2(fv.x, fv.x), fy = pk2(fv.y, fv.y);
-          const f2p d01 = pk2(dv[0], dv[1]), d23 = pk2(dv[2], dv[3]);
-          const f2p tx0 = mul2(d01, fx), tx1 = mul2(d23, fx), ty0 = mul2(d01, fy), ty1 = mul2(d23, fy);
+      if (!SYN) {
+        const cx<T> fv = reinterpret_cast<const cx<T>*>(S + G::F_OFF)[c];
+        cx<T> tt[E];
 #pragma unroll
-          for (int s = 0; s < NSLOT; ++s)
+        for (int e = 0; e < E; ++e) tt[e] = mkc<T>(dv[e] * fv.x, dv[e] * fv.y);
 #pragma unroll
-            for (int h = 0; h < NH; ++h) {
-              const int q = (ZH && h == 0) ? 2 * NP : BQ + h - ZH;
-              const ulonglong2 r = *reinterpret_cast<const ulonglong2*>(Rr + (s * NH + h) * TMP);
-              acc.x[0][s][q] = fma2(tx0, r.x, acc.x[0][s][q]);
-              acc.y[0][s][q] = fma2(ty0, r.x, acc.y[0][s][q]);
-              acc.x[1][s][q] = fma2(tx1, r.y, acc.x[1][s][q]);
-              acc.y[1][s][q] = fma2(ty1, r.y, acc.y[1][s][q]);
+        for (int s = 0; s < NSLOT; ++s)
+#pragma unroll
+          for (int h = 0; h < NH; ++h) {
+            const int q = (ZH && h == 0) ? 2 * NP : BQ + h - ZH;
+            T r[E];
+            VecLdS<T, E>::ld(Rr + (s * NH + h) * TMP, r);
+#pragma unroll
+            for (int e = 0; e < E; ++e) {
+              cx<T>& a = acc.v[e][s][q];
+              a.x = fma(tt[e].x, r[e], a.x);
+              a.y = fma(tt[e].y, r[e], a.y);
             }
-        } else {
-          f2p px0 = 0, py0 = 0, px1 = 0, py1 = 0;
-#pragma unroll
-          for (int s = 0; s < NSLOT; ++s)
-#pragma unroll
-            for (int h = 0; h < NH; ++h) {
-              const int q = (ZH && h == 0) ? 2 * NP : BQ + h - ZH;
-              const ulonglong2 r = *reinterpret_cast<const ulonglong2*>(Rr + (s * NH + h) * TMP);
-              px0 = fma2(acc.x[0][s][q], r.x, px0);
-              py0 = fma2(acc.y[0][s][q], r.x, py0);
-              px1 = fma2(acc.x[1][s][q], r.y, px1);
-              py1 = fma2(acc.y[1][s][q], r.y, py1);
-            }
-          const f2p d01 = pk2(dv[0], dv[1]), d23 = pk2(dv[2], dv[3]);
-          const f2p sx = fma2(d23, px1, mul2(d01, px0)), sy = fma2(d23, py1, mul2(d01, py0));
-          float a, b;
-          upk2(sx, a, b);
-          part.x = a + b;
-          upk2(sy, a, b);
-          part.y = a + b;
-        }
-      } else {
-        if (!SYN) {
-          const cx<T> fv = reinterpret_cast<const cx<T>*>(S + G::F_OFF)[c];
-          cx<T> tt[E];
-#pragma unroll
-          for (int e = 0; e < E; ++e) tt[e] = mkc<T>(dv[e] * fv.x, dv[e] * fv.y);
-#pragma unroll
-          for (int s = 0; s < NSLOT; ++s)
-#pragma unroll
-            for (int h = 0; h < NH; ++h) {
-              const int q = (ZH && h == 0) ? 2 * NP : BQ + h - ZH;
-              T r[E];
-              VecLdS<T, E>::ld(Rr + (s * NH + h) * TMP, r);
-#pragma unroll
-              for (int e = 0; e < E; ++e) {
-                cx<T>& a = acc.v[e][s][q];
-                a.x = fma(tt[e].x, r[e], a.x);
-                a.y = fma(tt[e].y, r[e], a.y);
-              }
-            }
-        } else {
-          cx<T> p[E];
-#pragma unroll
-          for (int e = 0; e < E; ++e) p[e] = mkc<T>(0, 0);
-#pragma unroll
-          for (int s = 0; s < NSLOT; ++s)
-#pragma unroll
-            for (int h = 0; h < NH; ++h) {
-              const int q = (ZH && h == 0) ? 2 * NP : BQ + h - ZH;
-              T r[E];
-              VecLdS<T, E>::ld(Rr + (s * NH + h) * TMP, r);
-#pragma unroll
-              for (int e = 0; e < E; ++e) {
-                const cx<T> a = acc.v[e][s][q];
-                p[e].x = fma(a.x, r[e], p[e].x);
-                p[e].y = fma(a.y, r[e], p[e].y);
-              }
-            }
-#pragma unroll
-          for (int e = 0; e < E; ++e) {
-            part.x = fma(dv[e], p[e].x, part.x);
-            part.y = fma(dv[e], p[e].y, part.y);
           }
+      } else {
+        cx<T> p[E];
+#pragma unroll
+        for (int e = 0; e < E; ++e) p[e] = mkc<T>(0, 0);
+#pragma unroll
+        for (int s = 0; s < NSLOT; ++s)
+#pragma unroll
+          for (int h = 0; h < NH; ++h) {
+            const int q = (ZH && h == 0) ? 2 * NP : BQ + h - ZH;
+            T r[E];
+            VecLdS<T, E>::ld(Rr + (s * NH + h) * TMP, r);
+#pragma unroll
+            for (int e = 0; e < E; ++e) {
+              const cx<T> a = acc.v[e][s][q];
+              p[e].x = fma(a.x, r[e], p[e].x);
+              p[e].y = fma(a.y, r[e], p[e].y);
+            }
+          }
+#pragma unroll
+        for (int e = 0; e < E; ++e) {
+          part.x = fma(dv[e], p[e].x, part.x);
+          part.y = fma(dv[e], p[e].y, part.y);
         }
       }
     }
@@ -551,22 +482,25 @@ k_contract(const ContractDesc<T>* __restrict__ descs, const TileTask* __restrict
 // f_lm = (2l+1)/(8 pi^2) * (sum of tile partials, fixed order), m >= 0, and
 // f_{l,-m} = (-1)^m conj(f_lm) (real signal).  blockIdx.z = job.
 template <typename T>
-__global__ void k_syn_reduce(ReduceJobs jobs, int tmp) {
+__global__ void k_syn_reduce(ReduceJobs jobs) {
   const int job = blockIdx.z;
   const int l = blockIdx.y;
   const int m = blockIdx.x * blockDim.x + threadIdx.x;
-  const int L = jobs.L[job];
+  const int L = jobs.L[job], tmp = jobs.tmp[job];
   if (l >= L || m > l) return;
   const ContractDesc<T>* dw = reinterpret_cast<const ContractDesc<T>*>(jobs.dw[job]);
   const ContractDesc<T>* dp = reinterpret_cast<const ContractDesc<T>*>(jobs.dp[job]);
+  // blocks of half a tile (direct FP64 contraction): tiles B, m' above m's block, fill the first half only
+  const bool halves = jobs.halves[job] != 0;
+  auto step = [&](int b) { return halves && !(b & 1) && (b >> 1) > (m >> 5) ? 2 : 1; };
   cx<T> sum = mkc<T>(0, 0);
   if (l <= jobs.lend[job]) {
     const int nb = min(l / tmp, dw->nbr - 1);
-    for (int b = 0; b <= nb; ++b) sum = cadd<T>(sum, dw->P[((size_t)b * dw->L + l) * dw->Lp32 + m]);
+    for (int b = 0; b <= nb; b += step(b)) sum = cadd<T>(sum, dw->P[((size_t)b * dw->L + l) * dw->Lp32 + m]);
   }
   if (l < jobs.Lphi[job]) {
     const int nb = min(l / tmp, dp->nbr - 1);
-    for (int b = 0; b <= nb; ++b) sum = cadd<T>(sum, dp->P[((size_t)b * dp->L + l) * dp->Lp32 + m]);
+    for (int b = 0; b <= nb; b += step(b)) sum = cadd<T>(sum, dp->P[((size_t)b * dp->L + l) * dp->Lp32 + m]);
   }
   // (2l+1)/(8 pi^2) of the synthesis (Eq. (32)); the forward SHT's plan has
   // Phi_l = sqrt((2l+1)/(4 pi)) and needs f_lm = Phi_l S where the partials

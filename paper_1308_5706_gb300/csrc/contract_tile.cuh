@@ -394,7 +394,7 @@ __device__ __forceinline__ void tile_ana_body(const TileCtx& x) {
           b1[q] = up ? make_float2(ax[EH + e][k].y, ay[EH + e][k].y) : make_float2(ax[EH + e][k].x, ay[EH + e][k].x);
         }
         // m and m' have the parities of u and r (CC/2 is even, mp0 and the column groups too)
-        gamma_ana<N>(b0, b1, ((r + l_start + N - 1) & 1) == 0, x.cg, y[r]);
+        gamma_ana<N, float>(b0, b1, ((r + l_start + N - 1) & 1) == 0, x.cg, y[r]);
         const float fs = (ISB && ((r + u) & 1)) ? -1.f : 1.f;
 #pragma unroll
         for (int g = 0; g < N; ++g) y[r][g] = cscale<float>(cmul_ipow<float>(y[r][g], (-m) & 3), fs);
@@ -486,7 +486,7 @@ __device__ __forceinline__ void tile_syn_body(const TileCtx& x) {
             // i^m: c0 is a multiple of C (m = c modulo 4 at C = 4, modulo 2 at C = 2)
             float2 u = cmul_ipow<float>(sb[(r0 + r) * PITCH + c0 + c], c & 3);
             if (C == 2 && (c0 & 2)) u = make_float2(-u.x, -u.y);
-            gamma_syn_add<N>(h[4 * c + r], cscale<float>(u, (ISB && ((r + c) & 1)) ? -1.f : 1.f), ub == ((r & 1) == 0), x.cg,
+            gamma_syn_add<N, float>(h[4 * c + r], cscale<float>(u, (ISB && ((r + c) & 1)) ? -1.f : 1.f), ub == ((r & 1) == 0), x.cg,
                              g);
           }
         }

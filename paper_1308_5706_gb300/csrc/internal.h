@@ -24,9 +24,9 @@ struct LSeg {
 template <typename T>
 struct ContractDesc {
   const T* delta;    // Delta table (padded eighth domain), working precision
-  // FP32 plans (contract_tile.cuh, contract_direct.cu):
-  const float* dpair;  // Delta pair table of the plan's shared table
-  const float* RSp;    // [nb][Lr][nslot][(N+1)/2][32]: R rows per 32-block of m', l outermost
+  // contract_direct.cuh and (FP32 plans) contract_tile.cuh:
+  const T* dpair;      // Delta pair table of the plan's shared table
+  const T* RSp;        // [nb][Lr][nslot][(N+1)/2][32]: R rows per 32-block of m', l outermost
   const cx<T>* fP;     // [nb][Lrf][re, im][32] (as floats): f_lm per 32-block of m (zero for m > l), packed per call
   int Lr, Lrf;         // l rows of RSp and fP (>= L + 7: a stage may read seven l past the last)
   const T* RS;       // [L][nslot][(N+1)/2][Lp]: Delta^l_{m',n_k} kappa^j(l) |s_{l,n_k}|, n_k >= 0
@@ -218,6 +218,8 @@ struct ReduceJobs {
   int L[MAXB];
   int lend[MAXB];
   int Lphi[MAXB];
+  int tmp[MAXB];  // rows m' per block of synthesis partials
+  int halves[MAXB];  // 1: blocks are halves of 32-row tiles (direct FP64 contraction)
   int sht[MAXB];  // 1: forward spherical harmonic transform (factor 1/(2 pi), see s2dw_sht_forward)
 };
 
@@ -233,17 +235,27 @@ void launch_contract_tile(int N, int nslot, bool syn, const ContractDesc<float>*
                           cudaStream_t st);
 void launch_fpack(const ContractDesc<float>* descs, int njobs, int nbmax, int Lrmax, const CallPtrs& ptrs,
                   cudaStream_t st);
-cudaError_t launch_pair_table(float* out, const double* d64, int Lmax, cudaStream_t st);
-cudaError_t launch_rtable_pair(float* RSp, const double* d64, const double* kap, const double* sabs,
+template <typename T>
+cudaError_t launch_pair_table(T* out, const double* d64, int Lmax, cudaStream_t st);
+template <typename T>
+cudaError_t launch_rtable_pair(T* RSp, const double* d64, const double* kap, const double* sabs,
                                const int* slotj, int L, int Lr, int N, int nslot, int kapL, cudaStream_t st);
-// FP32 contraction of small and middle band-limits (contract_direct.cu): one
-// launch over the tiles of the plans' wavelet scales (N orders) and of their
-// scaling parts.  rt: rows per thread of the analysis (1, 2 or 4).
+// Contraction of small and middle band-limits (contract_direct.cuh): one launch
+// over the tiles of the plans' wavelet scales (N orders) and of their scaling
+// parts.  rt: rows per thread of the analysis (1, 2 or 4).
+template <typename T>
 struct DirTasks {
-  const ContractDesc<float>* descs;
+  const ContractDesc<T>* descs;
   const CTask* tasks;
   int n;
 };
+template <typename T>
+void launch_contract_direct(int N, bool syn, int rt, const DirTasks<T>& w, const DirTasks<T>& p, const CallPtrs& ptrs,
+                            cudaStream_t st);
+extern template void launch_contract_direct<float>(int, bool, int, const DirTasks<float>&, const DirTasks<float>&,
+                                                   const CallPtrs&, cudaStream_t);
+extern template void launch_contract_direct<double>(int, bool, int, const DirTasks<double>&, const DirTasks<double>&,
+                                                    const CallPtrs&, cudaStream_t);
 // Band-limits up to this run it.  Contraction per call, GB300 (tile-pair ring
 // kernel with its scaling launch -> direct, analysis / synthesis, us): L = 32,
 // N = 3 34 / 38 -> 8 / 13; L = 128, N = 5 62 / 77 -> 15 / 17; L = 256, N = 5
@@ -252,9 +264,16 @@ struct DirTasks {
 // halves and the scales: L = 800, N = 3 246 / 268 against 250 / 205, L = 1024,
 // N = 5 406 / 400 against 648 / 705.
 constexpr int kContractDirectMaxL = 640;
-void launch_contract_direct(int N, bool syn, int rt, const DirTasks& w, const DirTasks& p, const CallPtrs& ptrs,
-                            cudaStream_t st);
-cudaError_t contract_direct_prepare();
+// FP64 (pair table of its own, 358 MB at 512): eighth-domain kernel with its
+// scaling launch -> direct, us: L = 32, N = 3 112 / 121 -> 13 / 25; L = 100, N = 3
+// 239 / 256 -> 37 / 45; L = 256, N = 1 280 / 351 -> 127 / 125, N = 3 500 / 545 ->
+// 195 / 220, N = 8 1212 / 1192 -> 299 / 427; L = 384, N = 5 1048 / 1108 -> 638 /
+// 725; L = 512, N = 3 1102 / 1195 -> 1044 / 1129, N = 8 2318 / 2257 -> 1831 /
+// 1989.  Above, the pair table would grow with L^3 for the
+// last few percent.
+constexpr int kContractDirectMaxL64 = 512;
+cudaError_t contract_direct_prepare_f32();
+cudaError_t contract_direct_prepare_f64();
 cudaError_t contract_tile_prepare();
 cudaError_t pair_timeouts(int* count);  // reads and resets the device count
 template <typename T>
@@ -263,8 +282,6 @@ void launch_czt(int kind, const CztSeg<T>* segs, int nseg, int total_items, int 
 template <typename T>
 void launch_syn_reduce(const ReduceJobs& jobs, int njobs, int Lmax, cudaStream_t st);
 
-template <> void launch_contract<float>(int, int, bool, const ContractDesc<float>*, const TileTask*, int,
-                                        const CallPtrs&, cudaStream_t);
 template <> void launch_contract<double>(int, int, bool, const ContractDesc<double>*, const TileTask*, int,
                                          const CallPtrs&, cudaStream_t);
 template <> void launch_czt<float>(int, const CztSeg<float>*, int, int, int, const CallPtrs&, cudaStream_t, int);

@@ -246,12 +246,12 @@ __global__ void k_rtable(T* RS, const double* d64, const double* kap, const doub
   RS[idx] = (T)v;
 }
 
-// Pair table (FP32) of the FP32 contraction from the FP64 table: block
+// Pair table of the direct and tile contractions from the FP64 table: block
 // (pair (p, q), l) is [r][c] = Delta^l_{32p+r, 32q+c}, zero where an index
 // exceeds l.  Grid (Lmax, number of pairs); CTAs with l < 32 q exit.  Each
-// thread writes 4 consecutive c (one 16-byte store).
-__global__ void __launch_bounds__(256) k_pair_table(float* __restrict__ out, const double* __restrict__ d64,
-                                                    int Lmax) {
+// thread writes 4 consecutive c.
+template <typename T>
+__global__ void __launch_bounds__(256) k_pair_table(T* __restrict__ out, const double* __restrict__ d64, int Lmax) {
   const int l = blockIdx.x;
   const int pi = blockIdx.y;
   int q = 0;
@@ -260,31 +260,40 @@ __global__ void __launch_bounds__(256) k_pair_table(float* __restrict__ out, con
   if (l < 32 * q) return;
   const int r = threadIdx.x >> 3, c0 = (threadIdx.x & 7) * 4;
   const int mp = 32 * p + r;
-  float v[4];
+  T v[4];
 #pragma unroll
   for (int i = 0; i < 4; ++i) {
     const int m = 32 * q + c0 + i;
-    v[i] = (mp <= l && m <= l) ? (float)delta_lookup(d64, l, mp, m) : 0.0f;
+    v[i] = (mp <= l && m <= l) ? (T)delta_lookup(d64, l, mp, m) : T(0);
   }
-  float* dst = out + pair_run_base(p, q, Lmax) + (long long)(l - 32 * q) * 1024 + r * 32 + c0;
-  *reinterpret_cast<float4*>(dst) = make_float4(v[0], v[1], v[2], v[3]);
+  T* dst = out + pair_run_base(p, q, Lmax) + (long long)(l - 32 * q) * 1024 + r * 32 + c0;
+  if constexpr (sizeof(T) == 4) {
+    *reinterpret_cast<float4*>(dst) = make_float4(v[0], v[1], v[2], v[3]);
+  } else {
+    reinterpret_cast<double2*>(dst)[0] = make_double2(v[0], v[1]);
+    reinterpret_cast<double2*>(dst)[1] = make_double2(v[2], v[3]);
+  }
 }
 
-cudaError_t launch_pair_table(float* out, const double* d64, int Lmax, cudaStream_t st) {
+template <typename T>
+cudaError_t launch_pair_table(T* out, const double* d64, int Lmax, cudaStream_t st) {
   const int B = Lmax / 32;
   if (B <= 0) return cudaSuccess;
   dim3 grid(Lmax, B * (B + 1) / 2);
-  k_pair_table<<<grid, 256, 0, st>>>(out, d64, Lmax);
+  k_pair_table<T><<<grid, 256, 0, st>>>(out, d64, Lmax);
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return e;
   // the read-ahead padding after the last run
-  return cudaMemsetAsync(out + pair_run_base(0, B, Lmax), 0, (size_t)kPairPadL * 1024 * sizeof(float), st);
+  return cudaMemsetAsync(out + pair_run_base(0, B, Lmax), 0, (size_t)kPairPadL * 1024 * sizeof(T), st);
 }
+template cudaError_t launch_pair_table<float>(float*, const double*, int, cudaStream_t);
+template cudaError_t launch_pair_table<double>(double*, const double*, int, cudaStream_t);
 
-// R rows in the layout of the FP32 contraction:
+// R rows in the layout of those contractions:
 // RSp[b][l][s][h][c] = R at (l, m' = 32 b + c, slot s, order n_k, k = N/2 + h),
 // as k_rtable (zero for l >= L, m' > l, inactive slots).
-__global__ void k_rtable_pair(float* RSp, const double* d64, const double* kap, const double* sabs, const int* slotj,
+template <typename T>
+__global__ void k_rtable_pair(T* RSp, const double* d64, const double* kap, const double* sabs, const int* slotj,
                               int L, int Lr, int N, int nslot, int kapL, int64_t total) {
   const int NH = (N + 1) / 2;
   const int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
@@ -306,17 +315,22 @@ __global__ void k_rtable_pair(float* RSp, const double* d64, const double* kap, 
       if (sa != 0.0 && kv != 0.0) v = delta_lookup(d64, l, mp, n) * kv * sa;
     }
   }
-  RSp[idx] = (float)v;
+  RSp[idx] = (T)v;
 }
 
-cudaError_t launch_rtable_pair(float* RSp, const double* d64, const double* kap, const double* sabs,
+template <typename T>
+cudaError_t launch_rtable_pair(T* RSp, const double* d64, const double* kap, const double* sabs,
                                const int* slotj, int L, int Lr, int N, int nslot, int kapL, cudaStream_t st) {
   const int nb = (L + 31) / 32;
   const int64_t total = (int64_t)nb * Lr * nslot * ((N + 1) / 2) * 32;
   if (total == 0) return cudaSuccess;
-  k_rtable_pair<<<(unsigned)((total + 255) / 256), 256, 0, st>>>(RSp, d64, kap, sabs, slotj, L, Lr, N, nslot, kapL, total);
+  k_rtable_pair<T><<<(unsigned)((total + 255) / 256), 256, 0, st>>>(RSp, d64, kap, sabs, slotj, L, Lr, N, nslot, kapL, total);
   return cudaGetLastError();
 }
+template cudaError_t launch_rtable_pair<float>(float*, const double*, const double*, const double*, const int*, int, int,
+                                               int, int, int, cudaStream_t);
+template cudaError_t launch_rtable_pair<double>(double*, const double*, const double*, const double*, const int*, int,
+                                                int, int, int, int, cudaStream_t);
 
 // Entry i of the twiddle table of length 2^logM: locate level d, then (k, j)
 // in it: e^{-2 pi i j k / S_d}.
