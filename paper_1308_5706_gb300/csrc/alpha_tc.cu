@@ -27,8 +27,16 @@ namespace {
 
 constexpr int kTcA = 128;       // analysis: samples a per tile (MMA M)
 constexpr int kTcRows = 128;    // analysis: rows per tile (MMA N)
-constexpr int kTcChunk = 1024;  // analysis: rows per CTA
-constexpr int kTcAnaThreads = 512;
+constexpr int kAnaProd = 8;     // analysis: producer warps
+constexpr int kAnaEpi = 8;      // analysis: epilogue warps
+// analysis: a CTA takes 2048 rows of a scale, halved down to one row tile while
+// the scale has fewer CTAs than this over the jobs of the launch (a launch
+// holds about five scales; a CTA starts with its 64 KB basis image).  1024 rows
+// always -> at least 40 / 64 / 160 CTAs, us: L = 128, N = 5 32 -> 11 / 11 / 11;
+// L = 361, N = 4 27 -> 15 / 15 / 19; L = 512, N = 3 34 -> 29 / 33 / 39; L = 1024,
+// N = 5 125 -> 123 / 123 / 126; L = 2048, N = 8 707 -> 678 / 677 / 663.
+constexpr int kTcAnaCtas = 40;
+constexpr int kTcAnaThreads = (kAnaProd + kAnaEpi) * 32;
 constexpr int kTcM = 128;       // synthesis: rows per CTA (MMA M)
 constexpr int kTcKc = 32;       // synthesis: samples per K chunk
 constexpr int kSynStages = 3;   // synthesis: shared-memory ring stages
@@ -52,18 +60,34 @@ constexpr size_t syn_tc_smem() {
   return (size_t)kSynStages * 2 * (tc::img_floats(kTcM, kTcKc) + tc::img_floats(64, kTcKc)) * sizeof(float);
 }
 
+// Analysis, warp-specialised (one CTA of 128 samples x up to 2048 rows per SM):
+//   warps 0-7   producers: rows of X (registers, two row tiles ahead) split
+//               into the row image of stage i % 2; arrive on full[stage];
+//               thread 0 then waits full[stage] and tempty[stage], issues the
+//               MMAs and commits to empty[stage] and tfull[stage] (a warp of its
+//               own would cap the registers at 96: spills)
+//   warps 8-15  epilogue: wait tfull[stage], read the sums (TMEM lanes =
+//               samples, half the rows per warp), arrive on tempty[stage] and
+//               store, every store one 128-byte run of a row of W
+// What bounds it: the stores of W.  With every warp staging, then storing (one
+// barrier per row tile) the store path idled while X was staged and the warps
+// queued for it afterwards; the roles keep both going.  Measured (scales of band
+// <= 32, with the rows per CTA of kTcAnaCtas, us, before -> now): L = 128, N = 5 31
+// -> 11, L = 361, N = 4 26 -> 15, L = 1024, N = 5 (503 MB of W) 144 -> 123, L = 2048,
+// N = 8 784 -> 678.
+// Every wait is bounded and a timeout in any role stops all of them.
 __global__ void __launch_bounds__(kTcAnaThreads, 1) k_alpha_ana_tc(const CztSeg<float>* __restrict__ segs,
                                                                    int nseg, CallPtrs ptrs) {
   extern __shared__ __align__(128) unsigned char smem_raw[];
-  __shared__ __align__(8) uint64_t mbar[2];
+  __shared__ __align__(8) uint64_t bar[8];  // full[2], empty[2], tfull[2], tempty[2]
   __shared__ uint32_t tbase;
-  __shared__ int fail;
+  __shared__ volatile int fail;
   const CztSeg<float> sg = segs[czt_find_seg<float>(segs, nseg)];
   const int item = blockIdx.x - sg.start;
-  const int Lj = sg.Lj, n = 2 * sg.L - 1, K = 2 * Lj, K8 = ana_k8(Lj);
+  const int Lj = sg.Lj, n = 2 * sg.L - 1, K8 = ana_k8(Lj);
   const int ntile = (n + kTcA - 1) / kTcA;
   const int ta = item % ntile, a0 = ta * kTcA;
-  const int nrows = sg.N * sg.nb, rbeg = (item / ntile) * kTcChunk, rend = min(nrows, rbeg + kTcChunk);
+  const int nrows = sg.N * sg.nb, rbeg = (item / ntile) * sg.P, rend = min(nrows, rbeg + sg.P);
   const int t = threadIdx.x, w = t >> 5, lane = t & 31;
   float* __restrict__ Wb = reinterpret_cast<float*>(sg.is_phi ? ptrs.Wphi[sg.job] : ptrs.W[sg.job]) + sg.woff;
   if (Lj <= 0) {  // empty scale: W = 0
@@ -76,148 +100,163 @@ __global__ void __launch_bounds__(kTcAnaThreads, 1) k_alpha_ana_tc(const CztSeg<
   float* Ahi = reinterpret_cast<float*>(smem_raw);
   float* Alo = Ahi + img;
   float* Bimg = Alo + img;  // [stage][hi, lo][img]
-  const uint32_t mb0 = tc::smem_u32(&mbar[0]), mb1 = tc::smem_u32(&mbar[1]);
+  auto full = [&](int b) { return tc::smem_u32(&bar[b]); };
+  auto empty = [&](int b) { return tc::smem_u32(&bar[2 + b]); };
+  auto tfull = [&](int b) { return tc::smem_u32(&bar[4 + b]); };
+  auto tempty = [&](int b) { return tc::smem_u32(&bar[6 + b]); };
   if (t == 0) {
-    tc::mbar_init(mb0, 1);
-    tc::mbar_init(mb1, 1);
+    for (int b = 0; b < 2; ++b) {
+      tc::mbar_init(full(b), kAnaProd * 32);
+      tc::mbar_init(empty(b), 1);
+      tc::mbar_init(tfull(b), 1);
+      tc::mbar_init(tempty(b), kAnaEpi);
+    }
     fail = 0;
   }
   // TMEM: the sums of stage s at column 128 s
   if (w == 0) tc::tmem_alloc(&tbase, 2 * kTcRows);
-  // basis image of this sample tile (built per plan, already split)
-  {
-    const float* src = reinterpret_cast<const float*>(sg.H) + (size_t)ta * 2 * img;
-    for (int i = 4 * t; i < 2 * img; i += 4 * kTcAnaThreads) cp16(Ahi + i, src + i);
-    asm volatile("cp.async.commit_group;" ::: "memory");
-  }
-  const int ntr = (rend - rbeg + kTcRows - 1) / kTcRows;  // row tiles of this CTA
-  // staging: thread t holds column k = t % KP of rows rl0 + q RS of a row
-  // tile (KP = K8 rounded up to a power of two, RS = 512 / KP >= 8 rows), so
-  // the image offset is linear in q and a warp reads consecutive k of a row
-  const int lk = K8 <= 8 ? 3 : (K8 <= 16 ? 4 : (K8 <= 32 ? 5 : 6));
-  const int k = t & ((1 << lk) - 1), rl0 = t >> lk, RS = kTcAnaThreads >> lk, NQ = kTcRows / RS;
-  const bool kin = k < K, kst = k < K8;
-  const int o0 = kst ? tc::img_off(rl0, k, K8) : 0, oq = (RS / 8) * (K8 / 4) * tc::kLboF;
-  const float* __restrict__ X = reinterpret_cast<const float*>(sg.buf_in);
-  const size_t rsk = (size_t)RS * K;  // elements between the rows q and q + 1 of a thread
-  auto load = [&](int i, float (&xr)[16]) {  // NQ <= 16
-    const int r = rbeg + i * kTcRows + rl0;
-    const float* src = X + (size_t)r * K + k;
-    const int qn = kin ? (rend - r + RS - 1) / RS : 0;  // rows r + q RS < rend exist
-#pragma unroll
-    for (int q = 0; q < 16; ++q) {
-      if (q < NQ) xr[q] = q < qn ? __ldg(src) : 0.f;
-      src += rsk;
-    }
-  };
-  auto store = [&](int stg, const float (&xr)[16]) {
-    float* hi = Bimg + (size_t)stg * 2 * img + o0;
-    float* lo = hi + img;
-    if (kst) {
-#pragma unroll
-      for (int q = 0; q < 16; ++q) {
-        if (q < NQ) {
-          float h, l;
-          tc::split_tf32(xr[q], h, l);
-          hi[q * oq] = h;
-          lo[q * oq] = l;
-        }
-      }
-    }
-  };
-  const uint32_t idesc = tc::idesc_tf32(kTcA, kTcRows);
-  const uint64_t kstep = (uint64_t)(tc::img_kstep_bytes(1) >> 4);  // start-address field per K-step
-  auto issue = [&](int stg, uint32_t tmem_d) {  // D = (A_hi B_lo + A_lo B_hi) + A_hi B_hi, cross terms first
-    const uint64_t aH = tc::smem_desc(tc::smem_u32(Ahi), K8), aL = tc::smem_desc(tc::smem_u32(Alo), K8);
-    const uint64_t bH = tc::smem_desc(tc::smem_u32(Bimg + (size_t)stg * 2 * img), K8);
-    const uint64_t bL = tc::smem_desc(tc::smem_u32(Bimg + (size_t)stg * 2 * img + img), K8);
-    for (int s = 0; s < K8 / 8; ++s) {
-      const uint64_t o = kstep * s;
-      tc::mma_tf32(tmem_d, aH + o, bL + o, idesc, s > 0);
-      tc::mma_tf32(tmem_d, aL + o, bH + o, idesc, 1);
-    }
-    for (int s = 0; s < K8 / 8; ++s) {
-      const uint64_t o = kstep * s;
-      tc::mma_tf32(tmem_d, aH + o, bH + o, idesc, 1);
-    }
-  };
-  // row tiles in registers one tile ahead of their store, two buffers used
-  // by name (the loop is unrolled by two), so no copy waits on loads in flight
-  float xa[16], xb[16];
-  load(0, xa);
-  if (ntr > 1) load(1, xb);
-  store(0, xa);
-  asm volatile("cp.async.wait_group 0;" ::: "memory");
-  tc::fence_async_smem();
   tc::fence_before();
   __syncthreads();
   tc::fence_after();
   const uint32_t tmem = tbase;
-  if (t == 0) {
-    issue(0, tmem);
-    tc::mma_commit(mb0);
-  }
-  int last = 0;  // last row tile whose MMAs were issued
-  // epilogue map: warp w holds samples a0 + 32 (w % 4) + lane and rows 32 (w / 4) .. + 31 of a tile
-  const int a = a0 + 32 * (w & 3) + lane, cg = 32 * (w >> 2);
-  // tile i: fill = the buffer of tile i (stored), reloaded with tile i + 2; use = tile i + 1
-  auto step = [&](int i, float (&use)[16], float (&fill)[16]) -> bool {
-    const int s = i & 1;
-    if (i + 2 < ntr) load(i + 2, fill);
-    if (i + 1 < ntr) store(s ^ 1, use);  // stage s ^ 1: tile i - 1 was waited for
-    // one thread waits for tile i's MMAs; the barrier below passes it on
-    if (t == 0 && !tc::mbar_wait(s ? mb1 : mb0, (i >> 1) & 1, tc::kWaitCycles)) fail = 1;
-    tc::fence_async_smem();
-    tc::fence_before();
-    __syncthreads();
-    tc::fence_after();
-    if (fail) return false;  // read after the barrier: the same decision in every thread
-    if (i + 1 < ntr) {
-      if (t == 0) {
-        issue(s ^ 1, tmem + (uint32_t)((s ^ 1) * kTcRows));
-        tc::mma_commit(s ^ 1 ? mb1 : mb0);
+  const int ntr = (rend - rbeg + kTcRows - 1) / kTcRows;  // row tiles of this CTA
+  if (w < kAnaProd) {
+    // basis image of this sample tile (built per plan, already split)
+    const float* src = reinterpret_cast<const float*>(sg.H) + (size_t)ta * 2 * img;
+    for (int i = 4 * t; i < 2 * img; i += 4 * kAnaProd * 32) cp16(Ahi + i, src + i);
+    asm volatile("cp.async.commit_group;" ::: "memory");
+    // thread t holds X_m, m = t % KP, of rows rl0 + q RS of a row tile (KP = K8 / 2
+    // rounded up to a power of two, RS = 256 / KP >= 8 rows), so the image
+    // offset is linear in q and a warp reads consecutive m of a row
+    const int lk = K8 <= 8 ? 2 : (K8 <= 16 ? 3 : (K8 <= 32 ? 4 : 5));
+    const int m = t & ((1 << lk) - 1), rl0 = t >> lk, RS = (kAnaProd * 32) >> lk, NQ = kTcRows / RS;
+    const bool kin = m < Lj, kst = 2 * m < K8;
+    const int o0 = kst ? tc::img_off(rl0, 2 * m, K8) : 0, oq = (RS / 8) * (K8 / 4) * tc::kLboF;
+    const float2* __restrict__ X = sg.buf_in;
+    const size_t rsk = (size_t)RS * Lj;  // values between the rows q and q + 1 of a thread
+    auto load = [&](int i, float2 (&xr)[16]) {  // NQ <= 16
+      const int r = rbeg + i * kTcRows + rl0;
+      const float2* p = X + (size_t)r * Lj + m;
+      const int qn = kin ? (rend - r + RS - 1) / RS : 0;  // rows r + q RS < rend exist
+#pragma unroll
+      for (int q = 0; q < 16; ++q) {
+        if (q < NQ) xr[q] = q < qn ? __ldg(p) : make_float2(0.f, 0.f);
+        p += rsk;
       }
-      last = i + 1;
-    }
-    const int r0 = rbeg + i * kTcRows + cg;
-    const uint32_t te = tmem + ((uint32_t)(32 * (w & 3)) << 16) + (uint32_t)(s * kTcRows + cg);
-    float* pw = Wb + (size_t)r0 * n + a;
-    {
-      float v[32];
-      tc::tmem_ld32(te, v);
-      // row j at pw + j n: the pointer advances by one row per store, and a
-      // full group of 32 rows (all but the last tile) needs no row test
-      const int jn = rend - r0;
-      if (a < n && jn > 0) {
-        float* q = pw;
-        if (jn >= 32) {
+    };
+    int last = -1;  // thread 0: last row tile whose MMAs were issued
+    auto issue = [&](int i) {
+      const int s = i & 1;
+      if (!tc::mbar_wait(full(s), (uint32_t)(i >> 1) & 1u, tc::kWaitCycles) ||
+          (i >= 2 && !tc::mbar_wait(tempty(s), (uint32_t)((i >> 1) - 1) & 1u, tc::kWaitCycles))) {
+        fail = 1;
+        return;
+      }
+      tc::fence_after();
+      // D = (A_hi B_lo + A_lo B_hi) + A_hi B_hi, cross terms first
+      const uint32_t idesc = tc::idesc_tf32(kTcA, kTcRows), d = tmem + (uint32_t)(s * kTcRows);
+      const uint64_t kstep = (uint64_t)(tc::img_kstep_bytes(1) >> 4);  // start-address field per K-step
+      const uint64_t aH = tc::smem_desc(tc::smem_u32(Ahi), K8), aL = tc::smem_desc(tc::smem_u32(Alo), K8);
+      const uint64_t bH = tc::smem_desc(tc::smem_u32(Bimg + (size_t)s * 2 * img), K8);
+      const uint64_t bL = tc::smem_desc(tc::smem_u32(Bimg + (size_t)s * 2 * img + img), K8);
+      for (int k = 0; k < K8 / 8; ++k) {
+        const uint64_t o = kstep * k;
+        tc::mma_tf32(d, aH + o, bL + o, idesc, k > 0);
+        tc::mma_tf32(d, aL + o, bH + o, idesc, 1);
+      }
+      for (int k = 0; k < K8 / 8; ++k) {
+        const uint64_t o = kstep * k;
+        tc::mma_tf32(d, aH + o, bH + o, idesc, 1);
+      }
+      tc::mma_commit(empty(s));
+      tc::mma_commit(tfull(s));
+      last = i;
+    };
+    auto step = [&](int i, float2 (&xr)[16]) -> bool {
+      const int s = i & 1;
+      if (fail) return false;
+      if (i >= 2 && !tc::mbar_wait(empty(s), (uint32_t)((i >> 1) - 1) & 1u, tc::kWaitCycles)) {
+        fail = 1;
+        return false;
+      }
+      float* hi = Bimg + (size_t)s * 2 * img + o0;
+      float* lo = hi + img;
+      if (kst) {
 #pragma unroll
-          for (int j = 0; j < 32; ++j) {
-            __stcs(q, v[j]);  // written once: streaming
-            q += n;
+        for (int q = 0; q < 16; ++q) {
+          if (q < NQ) {
+            float2 h, l;
+            tc::split_tf32(xr[q].x, h.x, l.x);
+            tc::split_tf32(xr[q].y, h.y, l.y);
+            *reinterpret_cast<float2*>(hi + q * oq) = h;
+            *reinterpret_cast<float2*>(lo + q * oq) = l;
           }
-        } else {
+        }
+      }
+      if (i + 2 < ntr) load(i + 2, xr);
+      if (i == 0) asm volatile("cp.async.wait_group 0;" ::: "memory");
+      tc::fence_async_smem();
+      tc::mbar_arrive(full(s));
+      if (t == 0) issue(i);
+      return true;
+    };
+    float2 xa[16], xb[16];
+    load(0, xa);
+    if (ntr > 1) load(1, xb);
+    for (int i = 0; i < ntr; i += 2) {
+      if (!step(i, xa)) break;
+      if (i + 1 < ntr && !step(i + 1, xb)) break;
+    }
+    asm volatile("cp.async.wait_group 0;" ::: "memory");
+    // after a timeout: a bounded wait for the MMAs in flight before TMEM is released
+    if (t == 0 && fail && last >= 0) tc::mbar_wait(tfull(last & 1), (uint32_t)(last >> 1) & 1u, tc::kWaitCycles);
+  } else {
+    // samples a0 + 32 (w % 4) + lane, rows 64 h .. 64 h + 63 of a tile
+    const int a = a0 + 32 * (w & 3) + lane, cg = 64 * ((w - kAnaProd) >> 2);
+    for (int i = 0; i < ntr; ++i) {
+      const int s = i & 1;
+      const bool got = !fail && tc::mbar_wait(tfull(s), (uint32_t)(i >> 1) & 1u, tc::kWaitCycles);
+      if (!__all_sync(0xffffffffu, got)) {  // warp-uniform: the TMEM loads below are warp-collective
+        fail = 1;
+        break;
+      }
+      tc::fence_after();
+      const uint32_t te = tmem + ((uint32_t)(32 * (w & 3)) << 16) + (uint32_t)(s * kTcRows + cg);
 #pragma unroll
-          for (int j = 0; j < 32; ++j) {
-            if (j < jn) __stcs(q, v[j]);
-            q += n;
+      for (int h = 0; h < 2; ++h) {
+        float v[32];
+        tc::tmem_ld32(te + 32 * h, v);
+        if (h == 1) {
+          tc::fence_before();
+          __syncwarp();
+          if (lane == 0) tc::mbar_arrive(tempty(s));
+        }
+        // row j at q + j n: the pointer advances by one row per store, and a
+        // full group of 32 rows (all but the last tile) needs no row test
+        const int r0 = rbeg + i * kTcRows + cg + 32 * h, jn = rend - r0;
+        if (a < n && jn > 0) {
+          float* q = Wb + (size_t)r0 * n + a;
+          if (jn >= 32) {
+#pragma unroll
+            for (int j = 0; j < 32; ++j) {
+              __stcs(q, v[j]);  // written once: streaming
+              q += n;
+            }
+          } else {
+#pragma unroll
+            for (int j = 0; j < 32; ++j) {
+              if (j < jn) __stcs(q, v[j]);
+              q += n;
+            }
           }
         }
       }
     }
-    tc::fence_before();
-    return true;
-  };
-  for (int i = 0; i < ntr; i += 2) {
-    if (!step(i, xb, xa)) break;
-    if (i + 1 < ntr && !step(i + 1, xa, xb)) break;
   }
-  if (fail && t == 0) {
-    atomicAdd(&g_tc_timeouts, 1);
-    // the MMAs in flight (the last commit covers all): a second bounded wait before freeing TMEM
-    tc::mbar_wait(last & 1 ? mb1 : mb0, (last >> 1) & 1, tc::kWaitCycles);
-  }
+  __syncwarp();
+  tc::fence_before();
   __syncthreads();
+  if (fail && t == 0) atomicAdd(&g_tc_timeouts, 1);
   if (w == 0) tc::tmem_free(tmem, 2 * kTcRows);
 }
 
@@ -534,10 +573,12 @@ cudaError_t alpha_tc_build_table(float* out, int L, int Lj, bool syn, cudaStream
   return cudaGetLastError();
 }
 
-int alpha_tc_items(int L, int rows, bool syn) {
+int alpha_tc_items(int L, int rows, int njobs, bool syn, int& P) {
+  P = kTcRows;
   if (syn) return (rows + kTcM - 1) / kTcM;
-  const int n = 2 * L - 1;
-  return ((n + kTcA - 1) / kTcA) * ((rows + kTcChunk - 1) / kTcChunk);
+  const int tiles = (2 * L - 1 + kTcA - 1) / kTcA;
+  for (P = 2048; P > kTcRows && (long long)njobs * tiles * ((rows + P - 1) / P) < kTcAnaCtas; P /= 2) {}
+  return tiles * ((rows + P - 1) / P);
 }
 
 void launch_alpha_tc(bool syn, const CztSeg<float>* segs, int nseg, int total_items, const CallPtrs& ptrs,

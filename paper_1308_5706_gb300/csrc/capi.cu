@@ -712,7 +712,7 @@ void sort_tiles(std::vector<TileTask>& t) {
 }
 
 template <typename T>
-void build_segs(s2dw_plan_s* p, int job, int kind, std::vector<CztSeg<T>>& out, int& start, int& stages) {
+void build_segs(s2dw_plan_s* p, int job, int njobs, int kind, std::vector<CztSeg<T>>& out, int& start, int& stages) {
   // kinds 4 / 5 collect the alpha segments of scales with Lj <= kDirectMaxLjAna
   // (analysis) or kDirectMaxLj (synthesis),
   // kinds 6 / 7 the beta segments of plans whose FFT length M is 4L
@@ -866,7 +866,7 @@ void build_segs(s2dw_plan_s* p, int job, int kind, std::vector<CztSeg<T>>& out, 
     if (direct) {
       const bool syn = base_kind == CZT_ALPHA_SYN;
       if (sizeof(T) == sizeof(float)) {  // tensor cores: the plan's basis image of this scale
-        s.items = alpha_tc_items(L, Nj * G.nb, syn);
+        s.items = alpha_tc_items(L, Nj * G.nb, njobs, syn, s.P);
         s.H = reinterpret_cast<const cx<T>*>(syn ? p->tc_syn[j] : p->tc_ana[j]);
       } else if (!syn) {
         const int tiles = (L + kAgCols - 1) / kAgCols, rows = Nj * G.nb;
@@ -946,7 +946,7 @@ Lists* build_lists(const std::vector<s2dw_plan_t>& plans) {
       t.prob = i;
       tphi.push_back(t);
     }
-    for (int k = 0; k < Lists::NK; ++k) build_segs<T>(p, i, k, segs[k], start[k], stages[k]);
+    for (int k = 0; k < Lists::NK; ++k) build_segs<T>(p, i, (int)plans.size(), k, segs[k], start[k], stages[k]);
     ls->maxlogM = std::max(ls->maxlogM, p->logM);
     ls->Lmax = std::max(ls->Lmax, p->L);
     if (p->fP) {  // packed f: plans that run the tile contraction

@@ -170,7 +170,7 @@ struct CztSeg {
 // alpha_tc.cu).  Basis tables: one per scale and direction, built per plan.
 size_t alpha_tc_table_floats(int L, int Lj, bool syn);
 cudaError_t alpha_tc_build_table(float* out, int L, int Lj, bool syn, cudaStream_t st);
-int alpha_tc_items(int L, int rows, bool syn);
+int alpha_tc_items(int L, int rows, int njobs, bool syn, int& P);  // CTAs; P: rows per CTA
 void launch_alpha_tc(bool syn, const CztSeg<float>* segs, int nseg, int total_items, const CallPtrs& ptrs,
                      cudaStream_t st);
 cudaError_t alpha_tc_prepare();
