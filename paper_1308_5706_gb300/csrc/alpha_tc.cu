@@ -78,6 +78,7 @@ constexpr size_t syn_tc_smem() {
 // Every wait is bounded and a timeout in any role stops all of them.
 __global__ void __launch_bounds__(kTcAnaThreads, 1) k_alpha_ana_tc(const CztSeg<float>* __restrict__ segs,
                                                                    int nseg, CallPtrs ptrs) {
+  begin_after();
   extern __shared__ __align__(128) unsigned char smem_raw[];
   __shared__ __align__(8) uint64_t bar[8];  // full[2], empty[2], tfull[2], tempty[2]
   __shared__ uint32_t tbase;
@@ -279,6 +280,7 @@ constexpr int kSynThreads = (kSynProd + kSynAcc + 1) * 32;  // + the MMA warp
 
 __global__ void __launch_bounds__(kSynThreads, 1) k_alpha_syn_tc(const CztSeg<float>* __restrict__ segs, int nseg,
                                                                  CallPtrs ptrs) {
+  begin_after();
   extern __shared__ __align__(128) unsigned char smem_raw[];
   __shared__ __align__(8) uint64_t bar[2 * kSynStages + 4];  // full[S], empty[S], tfull[2], tempty[2]
   __shared__ uint32_t tbase;
@@ -585,9 +587,9 @@ void launch_alpha_tc(bool syn, const CztSeg<float>* segs, int nseg, int total_it
                      cudaStream_t st) {
   if (total_items <= 0) return;
   if (syn)
-    k_alpha_syn_tc<<<total_items, kSynThreads, syn_tc_smem(), st>>>(segs, nseg, ptrs);
+    launch_after(k_alpha_syn_tc, total_items, kSynThreads, syn_tc_smem(), st, segs, nseg, ptrs);
   else
-    k_alpha_ana_tc<<<total_items, kTcAnaThreads, ana_tc_smem(), st>>>(segs, nseg, ptrs);
+    launch_after(k_alpha_ana_tc, total_items, kTcAnaThreads, ana_tc_smem(), st, segs, nseg, ptrs);
 }
 
 cudaError_t alpha_tc_prepare() {

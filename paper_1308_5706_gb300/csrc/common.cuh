@@ -109,6 +109,13 @@ template <int N>
 __device__ __forceinline__ void cp_async_wait() { asm volatile("cp.async.wait_group %0;\n" ::"n"(N) : "memory"); }
 
 
+// First statement of every kernel of a transform call.  The kernels are launched
+// with programmatic stream serialization (launch_after): the next one is set up
+// as the CTAs of this one exit, and starts its work here once the one before
+// has completed and its writes are visible.  Every kernel waits before it
+// reads or writes anything, so a completed kernel implies all earlier ones.
+__device__ __forceinline__ void begin_after() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+
 // Packed float pairs (two FP32 lanes per 64-bit register) for the sm_100+
 // f32x2 instructions: one instruction per two multiply-adds.
 typedef unsigned long long f2p;

@@ -155,6 +155,7 @@ __host__ __device__ constexpr size_t contract_smem_bytes() {
 template <typename T, int N, int NSLOT, bool SYN, int E>
 __global__ void __launch_bounds__(256, 1)
 k_contract(const ContractDesc<T>* __restrict__ descs, const TileTask* __restrict__ tiles, CallPtrs ptrs) {
+  begin_after();
   using G = StageGeom<T, N, NSLOT, E>;
   constexpr int STAGES = contract_stages<T, N, NSLOT, SYN, E>();
   // Order parity: R_{l m' -n} = (-1)^{l+m'} R_{l m' n}, so only n >= 0 is
@@ -483,6 +484,7 @@ k_contract(const ContractDesc<T>* __restrict__ descs, const TileTask* __restrict
 // f_{l,-m} = (-1)^m conj(f_lm) (real signal).  blockIdx.z = job.
 template <typename T>
 __global__ void k_syn_reduce(ReduceJobs jobs) {
+  begin_after();
   const int job = blockIdx.z;
   const int l = blockIdx.y;
   const int m = blockIdx.x * blockDim.x + threadIdx.x;
@@ -527,7 +529,7 @@ void launch_one(dim3 grid, const ContractDesc<T>* descs, const TileTask* tiles, 
     cudaFuncSetAttribute(k_contract<T, N, NSLOT, SYN, E>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (dev < 64) dev_done |= 1ull << dev;
   }
-  k_contract<T, N, NSLOT, SYN, E><<<grid, 256, smem, st>>>(descs, tiles, ptrs);
+  launch_after(k_contract<T, N, NSLOT, SYN, E>, grid, 256, smem, st, descs, tiles, ptrs);
 }
 
 template <typename T, int E>

@@ -207,6 +207,7 @@ template <typename T, int N, int RT, int NW>
 __global__ void __launch_bounds__(32 * NW)
 k_contract_dir_ana(const ContractDesc<T>* __restrict__ dw, const CTask* __restrict__ tw, int nw,
                    const ContractDesc<T>* __restrict__ dphi, const CTask* __restrict__ tp, CallPtrs ptrs) {
+  begin_after();
   constexpr int SUB = 32 / (RT * NW), RW = ((N + 1) / 2) * 32;
   __shared__ cx<T> cg[64];
   __shared__ __align__(16) T Rs[2 * kDirLC<T> * RW];
@@ -398,6 +399,7 @@ template <typename T, int N>
 __global__ void __launch_bounds__(256)
 k_contract_dir_syn(const ContractDesc<T>* __restrict__ dw, const CTask* __restrict__ tw, int nw,
                    const ContractDesc<T>* __restrict__ dphi, const CTask* __restrict__ tp) {
+  begin_after();
   extern __shared__ __align__(16) unsigned char dir_smem[];
   __shared__ cx<T> cg[64];
   cx<T>* red = reinterpret_cast<cx<T>*>(dir_smem);
@@ -419,11 +421,11 @@ void dir_launch(bool syn, int rt, const DirTasks<T>& w, const DirTasks<T>& p, co
   const int n = w.n + p.n;
   const ContractDesc<T>* dw = w.descs;
   const ContractDesc<T>* dp = p.descs;
-  if (syn) k_contract_dir_syn<T, N><<<kDirSynSub<T> * n, 256, dir_syn_smem<T, N>(), st>>>(dw, w.tasks, w.n, dp, p.tasks);
-  else if constexpr (sizeof(T) == 8) k_contract_dir_ana<T, N, 1, 4><<<8 * n, 128, 0, st>>>(dw, w.tasks, w.n, dp, p.tasks, ptrs);
-  else if (rt == 4) k_contract_dir_ana<T, N, 4, 8><<<n, 256, 0, st>>>(dw, w.tasks, w.n, dp, p.tasks, ptrs);
-  else if (rt == 2) k_contract_dir_ana<T, N, 2, 8><<<2 * n, 256, 0, st>>>(dw, w.tasks, w.n, dp, p.tasks, ptrs);
-  else k_contract_dir_ana<T, N, 1, 4><<<8 * n, 128, 0, st>>>(dw, w.tasks, w.n, dp, p.tasks, ptrs);
+  if (syn) launch_after(k_contract_dir_syn<T, N>, kDirSynSub<T> * n, 256, dir_syn_smem<T, N>(), st, dw, w.tasks, w.n, dp, p.tasks);
+  else if constexpr (sizeof(T) == 8) launch_after(k_contract_dir_ana<T, N, 1, 4>, 8 * n, 128, 0, st, dw, w.tasks, w.n, dp, p.tasks, ptrs);
+  else if (rt == 4) launch_after(k_contract_dir_ana<T, N, 4, 8>, n, 256, 0, st, dw, w.tasks, w.n, dp, p.tasks, ptrs);
+  else if (rt == 2) launch_after(k_contract_dir_ana<T, N, 2, 8>, 2 * n, 256, 0, st, dw, w.tasks, w.n, dp, p.tasks, ptrs);
+  else launch_after(k_contract_dir_ana<T, N, 1, 4>, 8 * n, 128, 0, st, dw, w.tasks, w.n, dp, p.tasks, ptrs);
 }
 
 template <typename T, int N>

@@ -7,7 +7,7 @@ template <>
 void launch_syn_reduce<float>(const ReduceJobs& jobs, int njobs, int Lmax, cudaStream_t st) {
   if (njobs <= 0) return;
   dim3 grid((Lmax + 127) / 128, Lmax, njobs), block(128);
-  k_syn_reduce<float><<<grid, block, 0, st>>>(jobs);
+  launch_after(k_syn_reduce<float>, grid, block, 0, st, jobs);
 }
 
 int contract_rows_per_thread(bool fp64) { return fp64 ? 2 : 4; }

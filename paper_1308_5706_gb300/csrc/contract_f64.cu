@@ -13,7 +13,7 @@ template <>
 void launch_syn_reduce<double>(const ReduceJobs& jobs, int njobs, int Lmax, cudaStream_t st) {
   if (njobs <= 0) return;
   dim3 grid((Lmax + 127) / 128, Lmax, njobs), block(128);
-  k_syn_reduce<double><<<grid, block, 0, st>>>(jobs);
+  launch_after(k_syn_reduce<double>, grid, block, 0, st, jobs);
 }
 
 }  // namespace s2dw

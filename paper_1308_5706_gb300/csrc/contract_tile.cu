@@ -7,6 +7,7 @@ namespace s2dw {
 // fP[b][l][re, im][c] = f_{l, 32 b + c} for 32 b + c <= l < L, else 0 (Lrf rows
 // per block).  Grid (ceil(Lrmax / 8), max blocks, jobs); 8 rows l per CTA.
 __global__ void __launch_bounds__(256) k_fpack(const ContractDesc<float>* __restrict__ descs, CallPtrs ptrs) {
+  begin_after();
   const int job = blockIdx.z, b = blockIdx.y;
   const ContractDesc<float>* D = descs + job;
   const int L = D->L, Lrf = D->Lrf;
@@ -25,7 +26,7 @@ void launch_fpack(const ContractDesc<float>* descs, int njobs, int nbmax, int Lr
                   cudaStream_t st) {
   if (njobs <= 0 || nbmax <= 0) return;
   dim3 grid((Lrmax + 7) / 8, nbmax, njobs);
-  k_fpack<<<grid, 256, 0, st>>>(descs, ptrs);
+  launch_after(k_fpack, grid, 256, 0, st, descs, ptrs);
 }
 
 bool tile_both_halves(int N) { return N <= 6; }
@@ -61,9 +62,9 @@ void launch_contract_tile(int N, int nslot, bool syn, const ContractDesc<float>*
   tile_pick(N, nslot, [&](auto n, auto s) {
     constexpr int NN = decltype(n)::value, NS = decltype(s)::value, H = NN <= 6 ? 2 : 1;
     if (syn)
-      k_contract_tile<NN, NS, true, H><<<ntasks, 256, TileGeom<NN, NS, true, H>::SMEM, st>>>(descs, tasks);
+      launch_after(k_contract_tile<NN, NS, true, H>, ntasks, 256, TileGeom<NN, NS, true, H>::SMEM, st, descs, tasks);
     else
-      k_contract_tile<NN, NS, false, H><<<ntasks, 256, TileGeom<NN, NS, false, H>::SMEM, st>>>(descs, tasks);
+      launch_after(k_contract_tile<NN, NS, false, H>, ntasks, 256, TileGeom<NN, NS, false, H>::SMEM, st, descs, tasks);
   });
 }
 

@@ -630,6 +630,7 @@ __device__ __forceinline__ void tile_syn_body(const TileCtx& x) {
 template <int N, int NSLOT, bool SYN, int HALVES>
 __global__ void __launch_bounds__(256, 1)
 k_contract_tile(const ContractDesc<float>* __restrict__ descs, const CTask* __restrict__ tasks) {
+  begin_after();
   using G = TileGeom<N, NSLOT, SYN, HALVES>;
   extern __shared__ __align__(128) unsigned char tile_smem[];
   __shared__ __align__(8) uint64_t full[G::STAGES], empty[G::STAGES];

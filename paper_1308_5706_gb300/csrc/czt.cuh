@@ -106,6 +106,7 @@ __device__ __forceinline__ void czt_beta_ana_body(const CztSeg<T>& sg, cx<T>* A)
 
 template <typename T>
 __global__ void __launch_bounds__(256, 2) k_czt_beta_ana(const CztSeg<T>* __restrict__ segs, int nseg) {
+  begin_after();
   extern __shared__ __align__(16) unsigned char smem_raw[];
   cx<T>* A = reinterpret_cast<cx<T>*>(smem_raw);
   const CztSeg<T> sg = segs[czt_find_seg<T>(segs, nseg)];
@@ -153,6 +154,7 @@ __device__ __forceinline__ void beta_mw_dft_body(const CztSeg<T>& sg, cx<T>* A) 
 
 template <typename T>
 __global__ void __launch_bounds__(256, 2) k_beta_mw_dft(const CztSeg<T>* __restrict__ segs, int nseg) {
+  begin_after();
   extern __shared__ __align__(16) unsigned char smem_raw[];
   cx<T>* A = reinterpret_cast<cx<T>*>(smem_raw);
   const CztSeg<T> sg = segs[czt_find_seg<T>(segs, nseg)];
@@ -186,6 +188,7 @@ __host__ __device__ constexpr size_t alpha_czt_smem(int maxlogM, bool staging) {
 template <typename T, bool ODD, int LOGM>
 __global__ void __launch_bounds__(256, sizeof(T) == 4 ? 3 : 2) k_czt_alpha_ana(const CztSeg<T>* __restrict__ segs, int nseg, int maxlogM,
                                                           CallPtrs ptrs, int ahead) {
+  begin_after();
   constexpr int NT = alpha_czt_nt(sizeof(T) == 8);
   extern __shared__ __align__(16) unsigned char smem_raw[];
   cx<T>* A = reinterpret_cast<cx<T>*>(smem_raw);
@@ -243,6 +246,7 @@ __global__ void __launch_bounds__(256, sizeof(T) == 4 ? 3 : 2) k_czt_alpha_ana(c
 template <typename T, int LOGM>
 __global__ void __launch_bounds__(256, sizeof(T) == 4 ? 3 : 2) k_czt_alpha_syn(const CztSeg<T>* __restrict__ segs, int nseg, int total,
                                                           int maxlogM, CallPtrs ptrs) {
+  begin_after();
   constexpr int NT = alpha_czt_nt(sizeof(T) == 8);
   extern __shared__ __align__(16) unsigned char smem_raw[];
   cx<T>* A = reinterpret_cast<cx<T>*>(smem_raw);
@@ -411,6 +415,7 @@ __device__ __forceinline__ void seg_prefetch_rows(const CztSeg<T>* __restrict__ 
 template <typename T, bool ODD>
 __global__ void __launch_bounds__(256) k_czt_alpha_ana_seg(const CztSeg<T>* __restrict__ segs, int nseg, CallPtrs ptrs,
                                                            int ahead) {
+  begin_after();
   extern __shared__ __align__(16) unsigned char smem_raw[];
   cx<T>* sm = reinterpret_cast<cx<T>*>(smem_raw);
   seg_prefetch_rows<T, T>(segs, nseg, ahead, nullptr, false, ptrs);
@@ -483,6 +488,7 @@ __device__ __forceinline__ void alpha_syn_seg_body(const CztSeg<T>& sg, const Ca
 template <typename T, bool ODD>
 __global__ void __launch_bounds__(256) k_czt_alpha_syn_seg(const CztSeg<T>* __restrict__ segs, int nseg, CallPtrs ptrs,
                                                            int ahead) {
+  begin_after();
   extern __shared__ __align__(16) unsigned char smem_raw[];
   cx<T>* sm = reinterpret_cast<cx<T>*>(smem_raw);
   seg_prefetch_rows<T, T>(segs, nseg, ahead, nullptr, true, ptrs);
@@ -532,6 +538,7 @@ __device__ __forceinline__ void czt_beta_syn_body(const CztSeg<T>& sg, cx<T>* A)
 
 template <typename T>
 __global__ void __launch_bounds__(256, 2) k_czt_beta_syn(const CztSeg<T>* __restrict__ segs, int nseg) {
+  begin_after();
   extern __shared__ __align__(16) unsigned char smem_raw[];
   cx<T>* A = reinterpret_cast<cx<T>*>(smem_raw);
   const CztSeg<T> sg = segs[czt_find_seg<T>(segs, nseg)];
@@ -562,6 +569,7 @@ __device__ __forceinline__ bool beta_ana_staged(int Lj) {
 template <typename T, int LOGM>
 __global__ void __launch_bounds__(256, 2) k_beta_ana_fft(const CztSeg<T>* __restrict__ segs, int nseg, int total,
                                                          int maxlogM) {
+  begin_after();
   constexpr int NT = beta_fft_nt(sizeof(T) == 8);
   constexpr int EPC = 16 / (int)sizeof(cx<T>);  // complex values per 16-byte copy
   extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -645,6 +653,7 @@ __device__ __forceinline__ bool beta_syn_staged(int Lj, int nt) {
 template <typename T, int LOGM>
 __global__ void __launch_bounds__(256, 2) k_beta_syn_fft(const CztSeg<T>* __restrict__ segs, int nseg, int total,
                                                          int maxlogM) {
+  begin_after();
   constexpr int NT = beta_fft_nt(sizeof(T) == 8);
   extern __shared__ __align__(16) unsigned char smem_raw[];
   cx<T>* A = reinterpret_cast<cx<T>*>(smem_raw);
@@ -792,6 +801,7 @@ __device__ __forceinline__ bool beta_dct_ana_staged(int Lj) {
 // compile-time length lets the stage loops and index maps fold); 0: any.
 template <typename T, int LOGN>
 __global__ void __launch_bounds__(256) k_beta_ana_dct(const CztSeg<T>* __restrict__ segs, int nseg, int total) {
+  begin_after();
   constexpr int EPC = 16 / (int)sizeof(cx<T>);
   extern __shared__ __align__(16) unsigned char smem_raw[];
   cx<T>* A = reinterpret_cast<cx<T>*>(smem_raw);
@@ -890,6 +900,7 @@ __global__ void __launch_bounds__(256) k_beta_ana_dct(const CztSeg<T>* __restric
 
 template <typename T, int LOGN>
 __global__ void __launch_bounds__(256) k_beta_syn_dct(const CztSeg<T>* __restrict__ segs, int nseg, int total) {
+  begin_after();
   extern __shared__ __align__(16) unsigned char smem_raw[];
   cx<T>* A = reinterpret_cast<cx<T>*>(smem_raw);
   cx<T>* stg = A + fft_smem_elems(kDctSpan);  // [gi][v]: column gi in FFT input order
@@ -1068,6 +1079,7 @@ __device__ __forceinline__ void alpha_ana_rows(const T* __restrict__ As, const T
 // at L = 512, N = 3, and 158 against 173 at L = 256, N = 5.
 template <typename T>
 __global__ void __launch_bounds__(256) k_alpha_ana_direct(const CztSeg<T>* __restrict__ segs, int nseg, CallPtrs ptrs) {
+  begin_after();
   static_assert(sizeof(T) == sizeof(double), "FP32 plans use the tensor-core kernels");
   extern __shared__ __align__(16) unsigned char smem_raw[];
   constexpr int KMAX = 2 * kDirectMaxLjAna - 1;
@@ -1148,6 +1160,7 @@ __global__ void __launch_bounds__(256) k_alpha_ana_direct(const CztSeg<T>* __res
 // FP64 plans only (FP32 plans run the tensor-core kernels of alpha_tc.cu).
 template <typename T>
 __global__ void __launch_bounds__(256) k_alpha_syn_direct(const CztSeg<T>* __restrict__ segs, int nseg, CallPtrs ptrs) {
+  begin_after();
   static_assert(sizeof(T) == sizeof(double), "FP32 plans use the tensor-core kernels");
   extern __shared__ __align__(16) unsigned char smem_raw[];
   constexpr int R = 32 / sizeof(T);
@@ -1294,17 +1307,17 @@ void launch_czt_impl(int kind, const CztSeg<T>* segs, int nseg, int total_items,
       if (!odd && ulog == 13) k = k_czt_alpha_ana<T, false, 13>;
     }
     const size_t sm = alpha_czt_smem<T>(maxlogM, false);
-    k<<<total_items, 256, sm, st>>>(segs, nseg, maxlogM, ptrs, alpha_czt_grid<T>(k, sm));
+    launch_after(k, total_items, 256, sm, st, segs, nseg, maxlogM, ptrs, alpha_czt_grid<T>(k, sm));
     return;
   }
   if (kind == CZT_ALPHA_ANA_SEG) {
     auto k = odd ? k_czt_alpha_ana_seg<T, true> : k_czt_alpha_ana_seg<T, false>;
-    k<<<total_items, 256, alpha_seg_smem<T>(), st>>>(segs, nseg, ptrs, alpha_czt_grid<T>(k, alpha_seg_smem<T>()));
+    launch_after(k, total_items, 256, alpha_seg_smem<T>(), st, segs, nseg, ptrs, alpha_czt_grid<T>(k, alpha_seg_smem<T>()));
     return;
   }
   if (kind == CZT_ALPHA_SYN_SEG) {
     auto k = odd ? k_czt_alpha_syn_seg<T, true> : k_czt_alpha_syn_seg<T, false>;
-    k<<<total_items, 256, alpha_seg_smem<T>(), st>>>(segs, nseg, ptrs, alpha_czt_grid<T>(k, alpha_seg_smem<T>()));
+    launch_after(k, total_items, 256, alpha_seg_smem<T>(), st, segs, nseg, ptrs, alpha_czt_grid<T>(k, alpha_seg_smem<T>()));
     return;
   }
   if (kind == CZT_ALPHA_SYN) {
@@ -1316,16 +1329,16 @@ void launch_czt_impl(int kind, const CztSeg<T>* segs, int nseg, int total_items,
       if (ulog == 13) k = k_czt_alpha_syn<T, 13>;
     }
     const int g = std::min(total_items, alpha_czt_grid<T>(k, sm));
-    k<<<g, 256, sm, st>>>(segs, nseg, total_items, maxlogM, ptrs);
+    launch_after(k, g, 256, sm, st, segs, nseg, total_items, maxlogM, ptrs);
     return;
   }
   const size_t smem = sizeof(cx<T>) * beta_czt_smem_elems(maxlogM, sizeof(T) == 8);
   dim3 grid(total_items), block(256);
   switch (kind) {
-    case CZT_BETA_ANA: k_czt_beta_ana<T><<<grid, block, smem, st>>>(segs, nseg); break;
-    case CZT_BETA_SYN: k_czt_beta_syn<T><<<grid, block, smem, st>>>(segs, nseg); break;
-    case CZT_BETA_MW_DFT: k_beta_mw_dft<T><<<grid, block, smem, st>>>(segs, nseg); break;
-    case CZT_BETA_RS: k_czt_beta_ana<T><<<grid, block, smem, st>>>(segs, nseg); break;
+    case CZT_BETA_ANA: launch_after(k_czt_beta_ana<T>, grid, block, smem, st, segs, nseg); break;
+    case CZT_BETA_SYN: launch_after(k_czt_beta_syn<T>, grid, block, smem, st, segs, nseg); break;
+    case CZT_BETA_MW_DFT: launch_after(k_beta_mw_dft<T>, grid, block, smem, st, segs, nseg); break;
+    case CZT_BETA_RS: launch_after(k_czt_beta_ana<T>, grid, block, smem, st, segs, nseg); break;
     case CZT_BETA_RS_FFT:
     case CZT_BETA_ANA_FFT: {  // persistent
       const size_t sm = beta_ana_fft_smem<T>(maxlogM);
@@ -1336,14 +1349,14 @@ void launch_czt_impl(int kind, const CztSeg<T>* segs, int nseg, int total_items,
         if (ulog == 13) k = k_beta_ana_fft<T, 13>;
       }
       const int g = std::min(total_items, alpha_czt_grid<T>(k, sm));
-      k<<<g, block, sm, st>>>(segs, nseg, total_items, maxlogM);
+      launch_after(k, g, block, sm, st, segs, nseg, total_items, maxlogM);
       break;
     }
     case CZT_ALPHA_ANA_DIRECT:
       if constexpr (sizeof(T) == sizeof(float))
         launch_alpha_tc(false, segs, nseg, total_items, ptrs, st);  // tensor cores
       else
-        k_alpha_ana_direct<T><<<grid, block, alpha_ana_direct_smem<T>(), st>>>(segs, nseg, ptrs);
+        launch_after(k_alpha_ana_direct<T>, grid, block, alpha_ana_direct_smem<T>(), st, segs, nseg, ptrs);
       break;
 
     case CZT_BETA_ANA_DCT:
@@ -1355,10 +1368,10 @@ void launch_czt_impl(int kind, const CztSeg<T>* segs, int nseg, int total_items,
       auto pick = [&](auto ana_k, auto syn_k) {
         if (syn) {
           const int g = std::min(total_items, alpha_czt_grid<T>(syn_k, sm));
-          syn_k<<<g, block, sm, st>>>(segs, nseg, total_items);
+          launch_after(syn_k, g, block, sm, st, segs, nseg, total_items);
         } else {
           const int g = std::min(total_items, alpha_czt_grid<T>(ana_k, sm));
-          ana_k<<<g, block, sm, st>>>(segs, nseg, total_items);
+          launch_after(ana_k, g, block, sm, st, segs, nseg, total_items);
         }
       };
       switch (logN) {
@@ -1379,14 +1392,14 @@ void launch_czt_impl(int kind, const CztSeg<T>* segs, int nseg, int total_items,
         if (ulog == 13) k = k_beta_syn_fft<T, 13>;
       }
       const int g = std::min(total_items, alpha_czt_grid<T>(k, sm));
-      k<<<g, block, sm, st>>>(segs, nseg, total_items, maxlogM);
+      launch_after(k, g, block, sm, st, segs, nseg, total_items, maxlogM);
       break;
     }
     case CZT_ALPHA_SYN_DIRECT:
       if constexpr (sizeof(T) == sizeof(float))
         launch_alpha_tc(true, segs, nseg, total_items, ptrs, st);  // tensor cores
       else
-        k_alpha_syn_direct<T><<<grid, block, alpha_syn_direct_smem<T>(1 << (maxlogM - 2)), st>>>(segs, nseg, ptrs);
+        launch_after(k_alpha_syn_direct<T>, grid, block, alpha_syn_direct_smem<T>(1 << (maxlogM - 2)), st, segs, nseg, ptrs);
       break;
     default: break;
   }

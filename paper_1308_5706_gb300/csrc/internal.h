@@ -19,6 +19,29 @@ struct LSeg {
   int j[2];
 };
 
+// Launch of a kernel that begins with begin_after(): its launch overlaps the end
+// of the kernel before it in the stream (under capture: a programmatic edge).
+// Measured, plain launches -> this, analysis / synthesis, us: L = 32, N = 3 21 / 32 ->
+// 14 / 24; L = 128, N = 5 50 / 60 -> 40 / 47; L = 361, N = 4 141 / 157 -> 128 / 140;
+// L = 1024, N = 5 1105 / 1338 -> 1083 / 1314.  No kernel asks for its successor
+// earlier (griddepcontrol.launch_dependents at its start): the waiting CTAs
+// then shared the SMs' resources and filled them unevenly, L = 128 46 / 50, L =
+// 1024 1169 / 1384.
+template <typename... P, typename... A>
+inline void launch_after(void (*k)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, A... args) {
+  cudaLaunchAttribute at;
+  at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at.val.programmaticStreamSerializationAllowed = 1;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = grid;
+  cfg.blockDim = block;
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = st;
+  cfg.attrs = &at;
+  cfg.numAttrs = 1;
+  cudaLaunchKernelEx(&cfg, k, static_cast<P>(args)...);
+}
+
 // Static, per-plan description of one contraction pass (wavelet scales with
 // N orders, or the scaling function with N = 1), device resident.
 template <typename T>

@@ -194,6 +194,7 @@ __device__ __forceinline__ void bulk_g2s(uint32_t dst, const void* src, int byte
 template <int MODE>
 __global__ void __launch_bounds__(32 * kCvWarps)
 k_sg_convert(const CztSeg<float>* __restrict__ segs, int nseg, CallPtrs ptrs) {
+  begin_after();
   extern __shared__ __align__(128) unsigned char sg_smem[];
   unsigned char* img = sg_smem;
   float* sinv = reinterpret_cast<float*>(sg_smem + kHalf);
@@ -362,6 +363,7 @@ k_sg_convert(const CztSeg<float>* __restrict__ segs, int nseg, CallPtrs ptrs) {
 template <int MODE>
 __global__ void __launch_bounds__(kSgThreads, 1)
 k_split_gemm(const CztSeg<float>* __restrict__ segs, int nseg, int total, CallPtrs ptrs) {
+  begin_after();
   extern __shared__ __align__(128) unsigned char sg_smem[];
   const float* scales = reinterpret_cast<const float*>(sg_smem + (size_t)kSgStages * 2 * kHalf);
   __shared__ __align__(8) uint64_t bar[2 * kSgStages + 4];  // full[S], empty[S], tfull[2], tempty[2]
@@ -695,8 +697,8 @@ cudaError_t sg_build_table(int mode, void* out, double2* scratch, const double* 
 namespace {
 template <int MODE>
 void sg_launch(const CztSeg<float>* segs, int nseg, int total, int stages, const CallPtrs& ptrs, cudaStream_t st) {
-  k_sg_convert<MODE><<<stages, 32 * kCvWarps, kData, st>>>(segs, nseg, ptrs);
-  k_split_gemm<MODE><<<std::min(total, sg_sms()), kSgThreads, kSgSmem, st>>>(segs, nseg, total, ptrs);
+  launch_after(k_sg_convert<MODE>, stages, 32 * kCvWarps, kData, st, segs, nseg, ptrs);
+  launch_after(k_split_gemm<MODE>, std::min(total, sg_sms()), kSgThreads, kSgSmem, st, segs, nseg, total, ptrs);
 }
 template <int MODE>
 cudaError_t sg_attr() {
