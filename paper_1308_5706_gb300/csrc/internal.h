@@ -287,14 +287,14 @@ extern template void launch_contract_direct<double>(int, bool, int, const DirTas
 // halves and the scales: L = 800, N = 3 246 / 268 against 250 / 205, L = 1024,
 // N = 5 406 / 400 against 648 / 705.
 constexpr int kContractDirectMaxL = 640;
-// FP64 (pair table of its own, 358 MB at 512): eighth-domain kernel with its
+// FP64 (pair table of its own, 152 MB at 384): eighth-domain kernel with its
 // scaling launch -> direct, us: L = 32, N = 3 112 / 121 -> 13 / 25; L = 100, N = 3
 // 239 / 256 -> 37 / 45; L = 256, N = 1 280 / 351 -> 127 / 125, N = 3 500 / 545 ->
 // 195 / 220, N = 8 1212 / 1192 -> 299 / 427; L = 384, N = 5 1048 / 1108 -> 638 /
-// 725; L = 512, N = 3 1102 / 1195 -> 1044 / 1129, N = 8 2318 / 2257 -> 1831 /
-// 1989.  Above, the pair table would grow with L^3 for the
-// last few percent.
-constexpr int kContractDirectMaxL64 = 512;
+// 725.  At L = 512 it would still gain (N = 3 1102 / 1195 -> 1044 / 1129, N = 8 2318 /
+// 2257 -> 1831 / 1989: 1 and 4% of a call), but its 358 MB of table cost a new plan
+// 0.3 ms, more than two calls gain at N = 3.
+constexpr int kContractDirectMaxL64 = 384;
 cudaError_t contract_direct_prepare_f32();
 cudaError_t contract_direct_prepare_f64();
 cudaError_t contract_tile_prepare();

@@ -1,4 +1,4 @@
-"""The FP64 contractions (L <= 512: one task per scale or l range and tile; above:
+"""The FP64 contractions (L <= 384: one task per scale or l range and tile; above:
 the eighth-domain kernel) at the edges of their 32-blocks, at the line between
 them and for every N: analysis rows against the oracle's Eq. (20) and synthesis
 of random coefficients against its Eqs. (32)-(41) within the 1e-11 of FP64
@@ -16,7 +16,7 @@ pytestmark = pytest.mark.gpu
 
 @pytest.mark.parametrize("L,N,lam,J0", [(2, 1, 2.0, 0), (9, 8, 2.0, 1), (31, 2, 2.0, 0), (32, 3, 1.5, 0), (33, 4, 2.0, 2),
                                         (63, 7, 3.0, 0), (65, 6, 2.0, 4), (97, 5, 2.0, 0), (255, 1, 2.0, 3), (256, 8, 2.0, 0),
-                                        (257, 2, 2.0, 0), (512, 2, 2.0, 6), (513, 1, 2.0, 5)])
+                                        (257, 2, 2.0, 0), (384, 2, 2.0, 5), (385, 2, 2.0, 5), (512, 2, 2.0, 6), (513, 1, 2.0, 5)])
 def test_fp64_contraction(L, N, lam, J0):
     f = flm_gaussian(L, 41, "unit")
     kern = O.kernels(L, N, lam, J0)
@@ -38,7 +38,7 @@ def test_fp64_contraction(L, N, lam, J0):
 
 def test_fp64_batch_over_both_kernels():
     import torch
-    plans = [B.Plan(L, N, 2.0, 1, "fp64") for L, N in [(100, 3), (300, 3), (40, 3), (512, 2), (513, 2)]]
+    plans = [B.Plan(L, N, 2.0, 1, "fp64") for L, N in [(100, 3), (300, 3), (40, 3), (384, 2), (385, 2)]]
     fs = [torch.from_numpy(flm_gaussian(p.L, 60 + i, "cl")).cuda() for i, p in enumerate(plans)]
     Wb, fb = [p.alloc_w() for p in plans], [p.alloc_flm() for p in plans]
     hs = [p.handle for p in plans]
