@@ -1679,8 +1679,8 @@ int plan_create(s2dw_plan_t* out, int L, int N, double lam, int J0, unsigned fla
     if (p->fp64) {
       p->direct_w = p->direct_phi = L <= kContractDirectMaxL64;
     } else {
-      p->direct_w = p->L0 <= kContractDirectMaxL;
-      p->direct_phi = p->Lphi <= kContractDirectMaxL;
+      p->direct_w = p->L0 <= contract_direct_max_l(N);
+      p->direct_phi = p->Lphi <= contract_direct_max_l(1);
     }
     // blocks of partials: TMP rows each; the direct contraction writes whole 32-row tiles
     const int rows = p->direct_w ? 32 : p->TMP, rows_phi = p->direct_phi ? 32 : p->TMP;

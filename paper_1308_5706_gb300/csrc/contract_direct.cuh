@@ -2,8 +2,8 @@
 // Sec. 3.3 Eqs. (34), (32)): the sums of contract_tile.cuh, organised for
 // latency instead of for one long stream per CTA.
 //
-// What bounds it.  At L <= kContractDirectMaxL a whole contraction is a few
-// microseconds of FP32 work; a ring kernel with one CTA per 32 x 32 tile (pair)
+// What bounds it.  At small L a whole contraction is a few microseconds of FP32
+// work; a ring kernel with one CTA per 32 x 32 tile (pair)
 // walks its l one stage after the other, at L = 128 on 16 of 152 SMs for 128
 // dependent steps.  Here
 //   analysis: a task is one scale of one tile over that scale's own l range, so

@@ -279,14 +279,18 @@ extern template void launch_contract_direct<float>(int, bool, int, const DirTask
                                                    const CallPtrs&, cudaStream_t);
 extern template void launch_contract_direct<double>(int, bool, int, const DirTasks<double>&, const DirTasks<double>&,
                                                     const CallPtrs&, cudaStream_t);
-// Band-limits up to this run it.  Contraction per call, GB300 (tile-pair ring
-// kernel with its scaling launch -> direct, analysis / synthesis, us): L = 32,
-// N = 3 34 / 38 -> 8 / 13; L = 128, N = 5 62 / 77 -> 15 / 17; L = 256, N = 5
-// 85 / 106 -> 28 / 40; L = 512, N = 5 144 / 170 -> 101 / 139; L = 640, N = 3
-// 149 / 161 -> 137 / 119.  Above, Delta no longer stays in L2 between the two
-// halves and the scales: L = 800, N = 3 246 / 268 against 250 / 205, L = 1024,
-// N = 5 406 / 400 against 648 / 705.
-constexpr int kContractDirectMaxL = 640;
+// FP32 band-limits up to this run it (both directions of a plan), above the tile
+// kernel (contract_tile.cuh), whose CTAs are fewer and longer but read Delta and
+// the R rows once for two scales.  Contraction per call, direct against tile,
+// analysis / synthesis, us:
+//   L      N = 1             N = 3             N = 5              N = 8
+//   320    27 / 20, 44 / 34  31 / 37, 55 / 45  36 / 60, 63 / 60   40 / 77, 51 / 48
+//   384    42 / 27, 53 / 41  57 / 48, 61 / 52  77 / 83, 73 / 69   67 / 106, 57 / 54
+//   448    56 / 39, 59 / 47  76 / 59, 69 / 58  104 / 111, 81 / 77 105 / 138, 63 / 75
+//   512    74 / 53, 64 / 55  91 / 75, 73 / 64  132 / 155, 90 / 84 138 / 190, 81 / 100
+// and at the small end direct against one CTA per tile pair: L = 32, N = 3 8 / 13,
+// 34 / 38; L = 128, N = 5 15 / 17, 62 / 77; L = 256, N = 5 28 / 40, 85 / 106.
+constexpr int contract_direct_max_l(int N) { return N <= 2 ? 448 : (N <= 4 ? 384 : (N <= 6 ? 320 : 288)); }
 // FP64 (pair table of its own, 152 MB at 384): eighth-domain kernel with its
 // scaling launch -> direct, us: L = 32, N = 3 112 / 121 -> 13 / 25; L = 100, N = 3
 // 239 / 256 -> 37 / 45; L = 256, N = 1 280 / 351 -> 127 / 125, N = 3 500 / 545 ->

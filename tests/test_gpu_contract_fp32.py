@@ -1,6 +1,6 @@
-"""The FP32 contractions (L <= 640 and above): Fourier cube, scaling
+"""The FP32 contractions (direct for small L, tile kernel above): Fourier cube, scaling
 part and synthesis against the FP64 plan at the edges of its 32-blocks, of its
-range (L = 640 | 641) and for every N, within the 1e-5 that the mixed path keeps
+ranges (L = 448 | 449 for N <= 2, 384 for N <= 4, 320, 288 for N > 6) and for every N, within the 1e-5 that the mixed path keeps
 (FP32 sums of at most L terms); and independence of how a launch cuts its tasks
 (rows per thread, l ranges): a job in a large batch equals the job alone."""
 import numpy as np
@@ -15,6 +15,8 @@ pytestmark = pytest.mark.gpu
 
 @pytest.mark.parametrize("L,N,lam,J0", [(2, 1, 2.0, 0), (9, 8, 2.0, 1), (31, 2, 2.0, 0), (32, 3, 1.5, 0), (33, 4, 2.0, 2),
                                         (63, 7, 3.0, 0), (65, 6, 2.0, 4), (97, 5, 2.0, 0), (193, 1, 2.0, 7),
+                                        (448, 2, 2.0, 0), (449, 2, 2.0, 0), (384, 4, 2.0, 0), (385, 4, 2.0, 1),
+                                        (320, 5, 2.0, 0), (321, 6, 2.0, 0), (288, 7, 2.0, 1), (289, 8, 2.0, 0),
                                         (640, 3, 2.0, 1), (641, 2, 2.0, 1), (655, 7, 2.0, 0), (672, 8, 3.0, 0),
                                         (705, 6, 1.7, 2), (800, 5, 2.0, 0), (673, 1, 2.0, 0)])
 def test_direct_contraction_vs_fp64(L, N, lam, J0):
