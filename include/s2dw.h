@@ -229,9 +229,9 @@ const char* s2dw_strerror(int status);
 /*
  * s2dw_wait_timeouts: number of bounded waits in the library's kernels that
  * gave up since the last call (0 in normal operation).  The tensor-core
- * kernels of the small-band alpha sums (FP32 plans) wait on an mbarrier for
- * their matrix products, and the FP32 contraction for the bulk copies of its
- * operands, about one second at most; one that gives up skips the rest of
+ * kernels of the alpha and beta sums (FP32 plans) wait on mbarriers for their
+ * matrix products and copies, and the FP32 contraction for the bulk copies of
+ * its operands, about one second at most; one that gives up skips the rest of
  * its work (and releases its tensor memory, or waits for its copies in
  * flight), so the output of that call is invalid.  Synchronous (waits for the device); reads and resets the
  * count.  Returns S2DW_ETIMEOUT when the count is nonzero (the count is
@@ -292,18 +292,20 @@ int s2dw_profile_read(s2dw_plan_t plan, double* ms, int* ncalls);
  *   [0] beta sums of the analysis, [1] beta sums of the synthesis:
  *       0 = one FFT of length 4L per column, 1 = one complex DCT/DST of length
  *       2L per column on the grids where it measured faster (L >= 128 in the
- *       analysis, 128 <= L <= 1024 in the synthesis), the FFT on the others
- *       (both where L is a power of two; a grid with other L keeps its
- *       chirp-z; the DCT/DST is launched once per transform length);
- *       default 1;
+ *       analysis, 128 <= L <= 1024 in the synthesis) and matrix products on the
+ *       tensor cores for L >= 2048 (FP32 plans), the FFT on the others (both
+ *       where L is a power of two; a grid with other L runs the products for L >
+ *       112 in FP32 plans, else its chirp-z; the DCT/DST is launched once per
+ *       transform length); default 1;
  *   [2 + 2j] alpha sums of the analysis of scale j (j = J+1: scaling part),
  *   [3 + 2j] of the synthesis: 0 = direct sums (L_j <= 32), 1 = chirp-z of
  *       the grid's length, 2 = segmented chirp-z (where the plan built its
- *       tables, s2dw_alpha_method);
- *   [last] the contraction's CTA shape (FP32 plans): 0 = both tiles of a
- *       pair of 32-wide blocks per CTA (N <= 5), 1 = one tile per CTA (the
- *       only shape for N > 5), 2 = one tile per CTA at two CTAs per SM
- *       (N <= 5); FP64 plans: 0.
+ *       tables, s2dw_alpha_method).  The default of an FP32 plan's scale above
+ *       32 runs matrix products on the tensor cores instead where those are
+ *       faster (mid bands, L >= 128); any other value runs as named;
+ *   [last] the contraction's CTA shape (FP32 plans): 0, 1, 2 for N <= 5, 1 for N >
+ *       5; FP64 plans: 0.  Kept for saved choices: the contraction now follows
+ *       from L and N and every value runs the same kernels;
  *   s2dw_plan_choices(plan, choices, n): *n in = capacity, out = entries;
  *     choices == NULL only queries *n; S2DW_EINVAL if the capacity is short.
  *   s2dw_plan_set_choices(plan, choices, n): n must be the plan's count and
@@ -314,8 +316,7 @@ int s2dw_profile_read(s2dw_plan_t plan, double* ms, int* ncalls);
  *     plan's private stream with scratch buffers it allocates and frees (a
  *     pseudo-random f_lm and the W its analysis writes; coordinate descent:
  *     each direction's beta method, then each scale's alpha method, largest
- *     band first, then the contraction's CTA shape (both directions' times),
- *     the minimum of `reps` round trips per trial, a candidate
+ *     band first, the minimum of `reps` round trips per trial, a candidate
  *     kept when it is 3% faster in two measurements with the incumbent
  *     re-timed between them), applies the best and writes it to choices (may
  *     be NULL).  Synchronous; 1 <= reps <= 64.

@@ -400,7 +400,7 @@ struct s2dw_plan_s {
   std::vector<unsigned char> desc_w_host, desc_phi_host;
   std::vector<TileTask> tiles_w_host, tiles_phi_host;  // FP64 plans
   bool direct_w = false, direct_phi = false;  // the direct contraction (else FP32: the tile kernel, FP64: k_contract)
-  int pair_shape = kPairShapePair;  // FP32: CTA-shape value of s2dw_plan_choices
+  int pair_shape = kPairShapePair;  // FP32: last value of s2dw_plan_choices (selects nothing)
   Lists own;
   // stage timing (s2dw_profile): one set of events per call, up to kProfCalls
   static constexpr int kProfCalls = 256;
@@ -1561,10 +1561,7 @@ void plan_build_typed(s2dw_plan_s* p, const double* kap_d, const double* phi_d, 
   p->desc_w_host.assign(reinterpret_cast<unsigned char*>(&dw), reinterpret_cast<unsigned char*>(&dw) + sizeof(dw));
   p->desc_phi_host.assign(reinterpret_cast<unsigned char*>(&dp), reinterpret_cast<unsigned char*>(&dp) + sizeof(dp));
   if (pairc) {
-    // default CTA shape (measured on GB300): below about 3 pairs per SM one
-    // tile per CTA with every value in registers; above it both tiles of a
-    // pair (each Delta block read once) for N >= 4, one tile at two CTAs per
-    // SM for N <= 3
+    // the reported value of the last choice; it no longer selects a kernel
     {
       int dev = 0, sms = 0;
       ck(cudaGetDevice(&dev));
@@ -1948,7 +1945,7 @@ static int choices_count(s2dw_plan_t p) { return 3 + 2 * (p->nscale + 1); }
 // Whether method v is available for choice idx of the plan (layout of s2dw_plan_choices).
 static bool choice_valid(s2dw_plan_t p, int idx, int v) {
   if (idx < 2) return v == 0 || v == 1;  // grids without half-length transforms keep the FFT
-  if (idx == choices_count(p) - 1) {  // contraction CTA shape (FP32 plans with N <= 5 have three)
+  if (idx == choices_count(p) - 1) {  // accepted for saved choices (FP32 plans with N <= 5 have three values)
     if (p->fp64) return v == 0;
     return pair_shapes_offered(p->N) ? (v >= kPairShapePair && v <= kPairShapeTile2) : v == kPairShapeTile;
   }
