@@ -309,7 +309,11 @@ def recorded_traffic(stage: str):
         return None, None
     if not rec:
         return None, None
-    if source_fingerprint(rec["files"]) != rec["fingerprint"]:
+    try:
+        same = source_fingerprint(rec["files"]) == rec["fingerprint"]
+    except OSError:  # a source file is gone
+        same = False
+    if not same:
         return None, "sources changed since the capture of " + rec["date"]
     return rec["bytes_per_launch"], f"ncu capture of {rec['date']} ({rec['kernel']})"
 
