@@ -1338,7 +1338,7 @@ void plan_build_typed(s2dw_plan_s* p, const double* kap_d, const double* phi_d, 
       const auto& G = p->gt[p->grid_of[j]];
       const auto& sgt = p->seg[j];
       const double cost = sgt.S > 0 ? (double)(sgt.S + 1) * ((size_t)1 << sgt.logM) * sgt.logM : 2.0 * G.M * G.logM;
-      p->alpha_sg[d][j] = pairc && p->alpha_mode[d][j] != 0 && sg_alpha_faster(G.L, Lj, cost);
+      p->alpha_sg[d][j] = pairc && p->alpha_mode[d][j] != 0 && sg_alpha_faster(G.L, Lj, cost, sgt.S > 0);
     }
     p->alpha_default[d] = p->alpha_mode[d];
   }

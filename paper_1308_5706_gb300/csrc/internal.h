@@ -228,8 +228,14 @@ inline bool sg_beta_faster(int L, bool pow2) { return pow2 ? L >= 2048 : L > 112
 // chirp-z `fft_cost` = (FFTs) x (length) x log2(length) (two FFTs of M, or S + 1
 // of M' segmented).  Per row at L = 1024, N = 5: 16 ps per term against 0.1 ps
 // per unit of that cost; below L = 128 the two launches cost more than they save
-// (L = 64, N = 3 18 against 10.5 us, L = 128, N = 5 21 against 27).
-inline bool sg_alpha_faster(int L, int Lj, double fft_cost) { return L >= 128 && (double)L * Lj < 6.5 * fft_cost; }
+// (L = 64, N = 3 18 against 10.5 us, L = 128, N = 5 21 against 27).  Lines at 4 / 6.5 /
+// 9 / 13 times the cost, analysis and synthesis of the whole call, us: where 9
+// moves segmented scales, L = 1024, N = 5 2452 / 2400 / 2364 / 2526, L = 1500, N = 3
+// 4741 / 4705 / 4652 / 4655; where it moves a full chirp-z, L = 900, N = 3 1383 /
+// 1357 / 1415 / 1414.
+inline bool sg_alpha_faster(int L, int Lj, double fft_cost, bool segmented) {
+  return L >= 128 && (double)L * Lj < (segmented ? 9.0 : 6.5) * fft_cost;
+}
 cudaError_t split_gemm_prepare();
 cudaError_t split_gemm_timeouts(int* count);  // reads and resets the device count
 
