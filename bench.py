@@ -887,7 +887,7 @@ def main():
                    "parallelism": f"replicas x{world}",
                    "launch_methods": {"choices": pm.tuned[0], "source": pm.tuned[1],
                                       "layout": "beta ana, beta syn, alpha ana / syn per scale, then the contraction CTA shape (s2dw.h)"},
-                   "l2": "inputs larger than L2 (W 0.92 GB, Delta table 0.72 GB per step)"},
+                   "l2": "inputs larger than L2 (W 0.92 GB, Delta pair table 0.78 GB per direction)"},
         "latency_ms": {"p50": per_sorted[len(per) // 2],
                        "p99": per_sorted[min(len(per) - 1, int(round(0.99 * (len(per) - 1))))]},
         "fp64": ({"value": args.fp64_steps / (total64 / 1e3), "ms_per_step": total64 / args.fp64_steps,

@@ -153,11 +153,9 @@ struct DeltaTab {
   int Lmax;
   int device;
   double* d64;  // entry 0 of the table (kDeltaFront zero entries precede it)
-  float* d32;
   int refs;
   size_t bytes;
   double* raw64 = nullptr;  // the allocations
-  float* raw32 = nullptr;
   float* pair32 = nullptr;  // pair table of the FP32 contraction (built for the first FP32 plan)
   double* pair64 = nullptr; // that of the direct FP64 contraction, l < min(Lmax, kContractDirectMaxL64)
 };
@@ -185,30 +183,23 @@ DeltaTab* delta_acquire(int L, cudaStream_t st) {
     if (u->device == dev && u->Lmax < Lmax && (!donor || u->Lmax > donor->Lmax)) donor = u;
   const int l_first = donor ? donor->Lmax : 0;
   const int64_t entries = delta_table_entries(Lmax) + 64;  // + read-ahead pad
-  DeltaTab* t = new DeltaTab{Lmax, dev, nullptr, nullptr, 1, 0};
+  DeltaTab* t = new DeltaTab{Lmax, dev, nullptr, 1, 0};
   double* em = nullptr;
   int* ee = nullptr;
   try {
     // kDeltaPad spare entries: the contraction copies 16-byte chunks of row
     // segments that may run past the last row of the last slab
     amalloc(&t->raw64, (kDeltaFront + entries + kDeltaPad) * sizeof(double), st);
-    amalloc(&t->raw32, (kDeltaFront + entries + kDeltaPad) * sizeof(float), st);
     ck(cudaMemsetAsync(t->raw64, 0, kDeltaFront * sizeof(double), st));
-    ck(cudaMemsetAsync(t->raw32, 0, kDeltaFront * sizeof(float), st));
     t->d64 = t->raw64 + kDeltaFront;
-    t->d32 = t->raw32 + kDeltaFront;
-    t->bytes = entries * (sizeof(double) + sizeof(float));
+    t->bytes = entries * sizeof(double);
     const int64_t kept = delta_slab_offset(l_first);
-    if (donor) {
-      ck(cudaMemcpyAsync(t->d64, donor->d64, kept * sizeof(double), cudaMemcpyDeviceToDevice, st));
-      ck(cudaMemcpyAsync(t->d32, donor->d32, kept * sizeof(float), cudaMemcpyDeviceToDevice, st));
-    }
+    if (donor) ck(cudaMemcpyAsync(t->d64, donor->d64, kept * sizeof(double), cudaMemcpyDeviceToDevice, st));
     ck(cudaMemsetAsync(t->d64 + kept, 0, (entries + kDeltaPad - kept) * sizeof(double), st));
-    ck(cudaMemsetAsync(t->d32 + kept, 0, (entries + kDeltaPad - kept) * sizeof(float), st));
     const size_t ne = (size_t)Lmax * (Lmax + 1) / 2;
     amalloc(&em, ne * sizeof(double), st);
     amalloc(&ee, ne * sizeof(int), st);
-    ck(launch_delta_build(t->d64, t->d32, em, ee, Lmax, l_first, st));
+    ck(launch_delta_build(t->d64, nullptr, em, ee, Lmax, l_first, st));
     afree(em, st);
     afree(ee, st);
     ck(cudaStreamSynchronize(st));
@@ -217,7 +208,6 @@ DeltaTab* delta_acquire(int L, cudaStream_t st) {
     afree(em, st);
     afree(ee, st);
     afree(t->raw64, st);
-    afree(t->raw32, st);
     delete t;
     throw;
   }
@@ -265,7 +255,6 @@ void delta_release(DeltaTab* t) {
   if (--t->refs == 0) {
     cudaStream_t st = setup_stream();
     afree(t->raw64, st);
-    afree(t->raw32, st);
     afree(t->pair32, st);
     afree(t->pair64, st);
     g_tabs.erase(std::remove(g_tabs.begin(), g_tabs.end(), t), g_tabs.end());
@@ -1555,8 +1544,8 @@ void plan_build_typed(s2dw_plan_s* p, const double* kap_d, const double* phi_d, 
     delta_pair64_ensure(p->tab, st);
   }
   ContractDesc<T> dw, dp;
-  const T* delta = (sizeof(T) == sizeof(double)) ? reinterpret_cast<const T*>(p->tab->d64)
-                                                 : reinterpret_cast<const T*>(p->tab->d32);
+  // (FP32 plans read the pair table only)
+  const T* delta = sizeof(T) == sizeof(double) ? reinterpret_cast<const T*>(p->tab->d64) : nullptr;
   fill_desc<T>(p, dw, dp, delta);
   p->desc_w_host.assign(reinterpret_cast<unsigned char*>(&dw), reinterpret_cast<unsigned char*>(&dw) + sizeof(dw));
   p->desc_phi_host.assign(reinterpret_cast<unsigned char*>(&dp), reinterpret_cast<unsigned char*>(&dp) + sizeof(dp));

@@ -46,7 +46,7 @@ inline void launch_after(void (*k)(P...), dim3 grid, dim3 block, size_t smem, cu
 // N orders, or the scaling function with N = 1), device resident.
 template <typename T>
 struct ContractDesc {
-  const T* delta;    // Delta table (padded eighth domain), working precision
+  const T* delta;    // Delta table (padded eighth domain; FP64 plans)
   // contract_direct.cuh and (FP32 plans) contract_tile.cuh:
   const T* dpair;      // Delta pair table of the plan's shared table
   const T* RSp;        // [nb][Lr][nslot][(N+1)/2][32]: R rows per 32-block of m', l outermost
