@@ -17,13 +17,19 @@
 // run on pipes 50 times as fast.
 //
 // FP32 accuracy from FP16 products: x = hi + lo with hi = x rounded to FP16 (11
-// bits) and lo = x - hi rounded to FP16, so that x is held to 2^-24 like an FP32
-// value, and x y = hi hi + hi lo + lo hi + O(2^-24).  Range: the basis is scaled
-// by a power of two per table; the data rows by a power of two per row and
-// stage (32 values of each of the two products), chosen from their maximum, so
-// any finite FP32 input works.  The tensor cores' FP32 accumulation truncates,
-// so a stage's sums (cross products first) leave TMEM after its 32 terms and
-// are added, scaled back, in FP32 registers with rounding to nearest.
+// bits) and lo = x - hi rounded to FP16, so that x is held to 2^-23 (an FP32
+// value to 2^-24), and x y = hi hi + hi lo + lo hi up to 2^-21, 2^-23.7 in the
+// mean square: single terms are worse than FP32 products, sums of whole calls
+// are closer to 64 bits than the transforms' were (3.3e-7 -> 2.4e-7 at L = 723,
+// 2.6e-7 -> 2.0e-7 at L = 361), as few roundings follow one another.  Range: the
+// basis is scaled by a power of two per table; the data by a power of two per row
+// and stage (32 values of each of the two products), chosen from their maximum;
+// in the beta synthesis per tile and stage, whose 64 columns m come out of one
+// alpha sum per row b with errors relative to its largest (a column 2^-16 below
+// its neighbours still keeps 24 bits).  The tensor cores' FP32 accumulation
+// truncates, so a stage's sums (cross products first) leave TMEM after its 32
+// terms and are added, with both scales taken back, in FP32 registers with
+// rounding to nearest: any input whose partial sums are finite works.
 //
 // Two kernels.  k_sg_convert folds, scales and splits the data once, a CTA per
 // tile of 128 rows and stage, into the operand images the products read (in
@@ -76,6 +82,8 @@ constexpr int kSgScales = 6;                  // stages of row scales kept: thre
 constexpr size_t kSgSmem = (size_t)kSgStages * 2 * kHalf + (size_t)kSgScales * kScaleB;
 static_assert(kSgDataBytes == kData, "bytes of a data stage");
 constexpr int kCvWarps = 8;                   // warps of the conversion kernel
+constexpr float kSgAnaScale = 8192.f;         // scale of the analysis bases (values up to 2), a power of two
+constexpr float kSgAlphaSynScale = 16384.f;   // of the alpha synthesis basis (values up to 1)
 
 enum SgMode { SG_BETA_ANA = 0, SG_BETA_SYN = 1, SG_ALPHA_ANA = 2, SG_ALPHA_SYN = 3 };
 
@@ -118,7 +126,8 @@ __device__ __forceinline__ bool sg_wait(uint32_t mbar, uint32_t parity, volatile
 }
 
 // 2^(14 - e) for a row maximum in [2^e, 2^(e+1)), as a float (1 for 0, Inf and
-// NaN), and its inverse; clamped so that both stay normal
+// NaN), and its inverse; clamped so that both stay normal (the inverse times the
+// basis scale, 2^-23 at least, is then 2^-136 at least: exact)
 __device__ __forceinline__ float sg_scale(uint32_t maxbits, float& inv) {
   const int e = (int)(maxbits >> 23);  // biased exponent; the sign bit is clear
   if (maxbits == 0u || e == 255) {
@@ -210,6 +219,9 @@ k_sg_convert(const CztSeg<float>* __restrict__ segs, int nseg, CallPtrs ptrs) {
   const int i0 = blockIdx.x - sg.tabD, c = i0 % sg.nsegs, rt = i0 / sg.nsegs;
   const SgTile T = sg_data_tile<MODE>(sg, rt);
   const int Lj = sg.Lj, L = sg.L, n = 2 * L - 1;
+  // 1 / (scale of the basis): the sums are scaled back by it stage by stage, with
+  // the row's own scale (kept to the end it brought sums above 2^104 to Inf)
+  const float unbasis = MODE == SG_ALPHA_SYN ? 1.f / kSgAlphaSynScale : sg.scale;
   const int hl = lane >> 4, tl = lane & 15;  // half-warp, position in it
   if constexpr (MODE == SG_BETA_SYN) {
     // lanes: 32 of the tile's 64 columns; a task is one half of the columns and
@@ -241,7 +253,7 @@ k_sg_convert(const CztSeg<float>* __restrict__ segs, int nseg, CallPtrs ptrs) {
     __syncthreads();
     float inv;
     const float s = sg_scale(smax, inv);
-    if (t < 128) sinv[t] = inv;
+    if (t < 128) sinv[t] = inv * unbasis;
 #pragma unroll
     for (int i = 0; i < 2; ++i) {
       const int task = w + kCvWarps * i;
@@ -339,12 +351,12 @@ k_sg_convert(const CztSeg<float>* __restrict__ segs, int nseg, CallPtrs ptrs) {
           put2(img + 2 * p * kImg, o, T.minus ? -a1 : a0, T.minus ? -b1 : b0, s);
           put2(img + 2 * p * kImg, o + 16, T.minus ? a0 : a1, T.minus ? b0 : b1, s);
         }
-        if (tl < 2) sinv[2 * r + tl] = inv;
+        if (tl < 2) sinv[2 * r + tl] = inv * unbasis;
       } else {
         const int o = sg_off(r, 2 * tl);
         put2(img, o, x[0], x[2], s);
         put2(img + 2 * kImg, o, x[1], x[3], s);
-        if (tl == 0) sinv[r] = inv;
+        if (tl == 0) sinv[r] = inv * unbasis;
       }
     }
   }
@@ -509,13 +521,12 @@ k_split_gemm(const CztSeg<float>* __restrict__ segs, int nseg, int total, CallPt
       if (!ok) break;
       const CztSeg<float>& sg = *T.sg;
       const int Lj = sg.Lj, L = sg.L, n = 2 * L - 1;
-      const float os = sg.scale;
       if constexpr (MODE == SG_BETA_ANA) {
         const int m = 2 * (64 * T.mt + (ml >> 1)) + T.par, b0 = 128 * T.nt + 64 * h, jn = min(64, L - b0);
         const bool reflect = sg.nb == 2 * L;
         if (m < Lj) {
           float* X = reinterpret_cast<float*>(sg.buf_out + (size_t)T.g * sg.nb * Lj + m) + (ml & 1);
-          const float so = T.minus ? -os : os;
+          const float so = T.minus ? -1.f : 1.f;
           const size_t rl = 2 * (size_t)Lj;
           float* up = X + (size_t)b0 * rl;
           float* dn = X + (size_t)(2 * L - 1 - b0) * rl;
@@ -525,7 +536,7 @@ k_split_gemm(const CztSeg<float>* __restrict__ segs, int nseg, int total, CallPt
 #pragma unroll
           for (int j = 0; j < 64; ++j) {
             if (j < jn) {
-              *up = (acc[0][j] + acc[1][j]) * os;
+              *up = acc[0][j] + acc[1][j];
               if (reflect) *dn = (acc[0][j] - acc[1][j]) * so;
             }
             up += rl;
@@ -540,8 +551,8 @@ k_split_gemm(const CztSeg<float>* __restrict__ segs, int nseg, int total, CallPt
           for (int j = 0; j < 64; ++j) {
             // product 0 (sums): even m' with cos, odd with sin; product 1 the others
             const int m0 = 2 * (i0 + j) + (T.minus ? 1 : 0), m1 = 2 * (i0 + j) + (T.minus ? 0 : 1);
-            if (m0 < Lj) V[(size_t)m0 * 2 * Lj] = acc[0][j] * os;
-            if (m1 < Lj) V[(size_t)m1 * 2 * Lj] = acc[1][j] * os;
+            if (m0 < Lj) V[(size_t)m0 * 2 * Lj] = acc[0][j];
+            if (m1 < Lj) V[(size_t)m1 * 2 * Lj] = acc[1][j];
           }
         }
       } else if constexpr (MODE == SG_ALPHA_ANA) {
@@ -552,7 +563,7 @@ k_split_gemm(const CztSeg<float>* __restrict__ segs, int nseg, int total, CallPt
 #pragma unroll
           for (int j = 0; j < 64; ++j) {
             if (j < jn) {
-              const float c = acc[0][j] * os, s = acc[1][j] * os;
+              const float c = acc[0][j], s = acc[1][j];
               if (a > 0) __stcs(dn, c - s);
               __stcs(up, c + s);
             }
@@ -564,6 +575,7 @@ k_split_gemm(const CztSeg<float>* __restrict__ segs, int nseg, int total, CallPt
         const int m = 128 * T.nt + ml, r = T.r0 + 64 * h, jn = min(64, T.rows - r);
         if (m < Lj && jn > 0) {
           float2* V = sg.buf_out + (size_t)r * Lj + m;
+          const float os = sg.scale;  // 2 pi / n
 #pragma unroll
           for (int j = 0; j < 64; ++j) {
             if (j < jn) *V = make_float2(acc[0][j] * os, acc[1][j] * os);
@@ -654,11 +666,12 @@ SgTable sg_table(int mode, int L) {
   t.bytes = (size_t)t.sets * t.tiles * t.stages * kHalf;
   return t;
 }
-// output scale of a segment (Eq. (37)'s 2 pi / n included)
+// scale of a segment: the inverse of the basis scale (a power of two); alpha
+// synthesis: Eq. (37)'s 2 pi / n
 float sg_out_scale(int mode, int L) {
   if (mode == SG_BETA_SYN) return (float)(1.0 / beta_syn_scale(L));
-  if (mode == SG_ALPHA_SYN) return (float)(2.0 * 3.14159265358979323846 / (2 * L - 1) / 16384.0);
-  return (float)(1.0 / 8192.0);
+  if (mode == SG_ALPHA_SYN) return (float)(2.0 * 3.14159265358979323846 / (2 * L - 1));
+  return 1.f / kSgAnaScale;
 }
 // tiles of one segment: prod of data tiles and basis tiles (P), stages
 SgDims sg_dims(int mode, int L, int Lj, int N, int nb) {
@@ -686,10 +699,10 @@ cudaError_t sg_build_table(int mode, void* out, double2* scratch, const double* 
   const unsigned grid = (unsigned)((total + 255) / 256);
   unsigned char* o = reinterpret_cast<unsigned char*>(out);
   switch (mode) {
-    case SG_BETA_ANA: k_sg_basis<SG_BETA_ANA><<<grid, 256, 0, st>>>(o, scratch, qw, L, period, t.tiles, t.stages, t.sets, 8192.0, mw); break;
+    case SG_BETA_ANA: k_sg_basis<SG_BETA_ANA><<<grid, 256, 0, st>>>(o, scratch, qw, L, period, t.tiles, t.stages, t.sets, kSgAnaScale, mw); break;
     case SG_BETA_SYN: k_sg_basis<SG_BETA_SYN><<<grid, 256, 0, st>>>(o, scratch, qw, L, period, t.tiles, t.stages, t.sets, beta_syn_scale(L), mw); break;
-    case SG_ALPHA_ANA: k_sg_basis<SG_ALPHA_ANA><<<grid, 256, 0, st>>>(o, scratch, qw, L, period, t.tiles, t.stages, t.sets, 8192.0, mw); break;
-    default: k_sg_basis<SG_ALPHA_SYN><<<grid, 256, 0, st>>>(o, scratch, qw, L, period, t.tiles, t.stages, t.sets, 16384.0, mw); break;
+    case SG_ALPHA_ANA: k_sg_basis<SG_ALPHA_ANA><<<grid, 256, 0, st>>>(o, scratch, qw, L, period, t.tiles, t.stages, t.sets, kSgAnaScale, mw); break;
+    default: k_sg_basis<SG_ALPHA_SYN><<<grid, 256, 0, st>>>(o, scratch, qw, L, period, t.tiles, t.stages, t.sets, kSgAlphaSynScale, mw); break;
   }
   return cudaGetLastError();
 }
