@@ -249,6 +249,17 @@ int s2dw_wait_timeouts(int* count);
 int s2dw_wait_probe(long long limit_cycles, void* stream);
 
 /*
+ * s2dw_plan_wait_probe: the same in the kernels themselves.  Launches on `stream`
+ * the plan's kernels with bounded waits that touch nothing but its workspace
+ * (matrix products of the beta sums), with waits that
+ * give up after limit_cycles SM cycles (clamped to [0, 2e9]; 0: at the first
+ * look).  What gave up is counted for s2dw_wait_timeouts; the intermediates of the plan's
+ * last call are lost (s2dw_stage), later calls are not affected.  FP32 plans
+ * (S2DW_ENOTSUP for FP64 ones, which have no such waits); S2DW_EINVAL for NULL.
+ */
+int s2dw_plan_wait_probe(s2dw_plan_t plan, long long limit_cycles, void* stream);
+
+/*
  * Introspection used by the tests (synchronous, host outputs).
  *   s2dw_scale_support: l-range [lo, hi] on which kappa^j(l) > 0 (j = J+1
  *     gives Phi's range, lo = 0).

@@ -55,6 +55,7 @@ _SIGNATURES = {
     "s2dw_plan_set_choices": (_c_i, [_c_p, _c_ip, _c_i]),
     "s2dw_plan_tune": (_c_i, [_c_p, _c_i, _c_ip, _c_ip]),
     "s2dw_wait_probe": (_c_i, [ctypes.c_longlong, _c_p]),
+    "s2dw_plan_wait_probe": (_c_i, [_c_p, ctypes.c_longlong, _c_p]),
 }
 
 STAGES = ["ana_contract", "ana_contract_phi", "ana_beta", "ana_alpha_czt", "ana_alpha_seg", "ana_alpha_direct",
@@ -188,6 +189,12 @@ def s2dw_wait_probe(limit_cycles: int, stream=None) -> None:
     """One warp waits, at most limit_cycles SM cycles, on an mbarrier nothing
     arrives on and counts the give-up (the failure path of the bounded waits)."""
     _check(lib().s2dw_wait_probe(int(limit_cycles), _stream(stream)), "s2dw_wait_probe")
+
+
+def s2dw_plan_wait_probe(plan: int, limit_cycles: int, stream=None) -> None:
+    """The plan's own kernels with bounded waits, over its workspace, with waits
+    that give up after limit_cycles SM cycles (mixed plans)."""
+    _check(lib().s2dw_plan_wait_probe(plan, int(limit_cycles), _stream(stream)), "s2dw_plan_wait_probe")
 
 
 def s2dw_kernels(plan: int, J: int, L: int, N: int):

@@ -1114,10 +1114,10 @@ void launch_dct_parts(const Lists& ls, int kind, const CallPtrs& ptrs, cudaStrea
 
 // split matrix products of a kind (FP32 plans)
 template <typename T>
-void launch_products(const Lists& ls, int kind, const CallPtrs& ptrs, cudaStream_t st) {
+void launch_products(const Lists& ls, int kind, const CallPtrs& ptrs, cudaStream_t st, long long limit = kWaitLimit) {
   if constexpr (sizeof(T) == sizeof(float))
     launch_split_gemm(kind == SG_KIND_BETA_RS ? 0 : kind - SG_KIND_BETA_ANA, reinterpret_cast<const CztSeg<T>*>(ls.segs[kind]),
-                      ls.nseg[kind], ls.items[kind], ls.stages[kind], ptrs, st);
+                      ls.nseg[kind], ls.items[kind], ls.stages[kind], ptrs, st, limit);
 }
 
 template <typename T>
@@ -2175,6 +2175,18 @@ int s2dw_wait_timeouts(int* count) {
 int s2dw_wait_probe(long long limit_cycles, void* stream) {
   const long long lim = std::min(std::max(limit_cycles, 1000LL), 2000000000LL);
   return err_of(alpha_tc_wait_probe(lim, reinterpret_cast<cudaStream_t>(stream)));
+}
+
+int s2dw_plan_wait_probe(s2dw_plan_t p, long long limit_cycles, void* stream) {
+  if (!p) return S2DW_EINVAL;
+  if (p->fp64) return S2DW_ENOTSUP;
+  const long long lim = std::min(std::max(limit_cycles, 0LL), kWaitLimit);
+  cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
+  CallPtrs ptrs;  // (these launches read and write the workspace only)
+  std::memset(&ptrs, 0, sizeof(ptrs));
+  for (int kind : {SG_KIND_BETA_ANA, SG_KIND_BETA_RS, SG_KIND_BETA_SYN}) launch_products<float>(p->own, kind, ptrs, st, lim);
+  mark_use(p, st);
+  return err_of(cudaGetLastError());
 }
 
 int s2dw_launch_counts(s2dw_plan_t p, int* analysis, int* synthesis) {

@@ -11,6 +11,7 @@ constexpr int MAXS = 66;   // wavelet scales (<= 64) plus headroom
 constexpr int MAXB = 64;   // transforms per batched launch
 constexpr int TILE = 32;   // contraction tile edge (m' and m)
 constexpr int LCH = 8;     // l-chunk of the synthesis in-tile reduction
+constexpr long long kWaitLimit = 2000000000LL;  // cycles of a bounded wait: about one second at the maximum SM clock
 
 // One l-segment on which the scale held by each of the two accumulator
 // slots is constant (slot s holds the scale j with j % 2 == s, or -1).
@@ -217,7 +218,7 @@ float sg_out_scale(int mode, int L);
 int sg_period(int mode, int L, bool mw);  // double2 of scratch the build needs
 cudaError_t sg_build_table(int mode, void* out, double2* scratch, const double* qw, int L, bool mw, cudaStream_t st);
 void launch_split_gemm(int mode, const CztSeg<float>* segs, int nseg, int total, int stages, const CallPtrs& ptrs,
-                       cudaStream_t st);
+                       cudaStream_t st, long long limit = kWaitLimit);
 // Whether the products are the faster form.  beta: the chirp-z (other L than
 // powers of two) costs two FFTs of M >= 4L per column: 20.5 against 20 us at L =
 // 100, N = 3, 30 against 21 at L = 200; the half-length transforms of

@@ -56,8 +56,9 @@
 // L = 511, N = 3 91 / 280 -> 39 / 189; alpha of all scales above 32: L = 256, N =
 // 5 57 / 55 -> 33 / 29, L = 512, N = 3 102 / 98 -> 70 / 65, L = 723, N = 6 361 /
 // 411 -> 304 / 309, L = 1024, N = 5 512 / 540 -> 447 / 521.
-// Every wait is bounded; a CTA that gives up stops all roles, waits for its MMAs
-// and copies in flight (bounded), frees its TMEM and counts the event.
+// Every wait is bounded; a CTA that gives up stops all roles, and once they have
+// met waits for its MMAs and copies in flight (bounded), counts the event and
+// frees its TMEM.
 #include <cuda_fp16.h>
 
 #include "czt.cuh"
@@ -112,12 +113,12 @@ __device__ __forceinline__ bool sg_poll(uint32_t mbar, uint32_t parity) {
       : "memory");
   return ok != 0;
 }
-__device__ __forceinline__ bool sg_wait(uint32_t mbar, uint32_t parity, volatile int* fail) {
+__device__ __forceinline__ bool sg_wait(uint32_t mbar, uint32_t parity, volatile int* fail, long long limit) {
   if (sg_poll(mbar, parity)) return true;
   const long long t0 = clock64();
   while (!sg_poll(mbar, parity)) {
     if (*fail) return false;
-    if (clock64() - t0 > tc::kWaitCycles) {
+    if (clock64() - t0 > limit) {
       *fail = 1;
       return false;
     }
@@ -374,13 +375,16 @@ k_sg_convert(const CztSeg<float>* __restrict__ segs, int nseg, CallPtrs ptrs) {
 
 template <int MODE>
 __global__ void __launch_bounds__(kSgThreads, 1)
-k_split_gemm(const CztSeg<float>* __restrict__ segs, int nseg, int total, CallPtrs ptrs) {
+k_split_gemm(const CztSeg<float>* __restrict__ segs, int nseg, int total, CallPtrs ptrs, long long wait_limit) {
   begin_after();
+  // (as a constant here, or the register allocation costs the kernel 2%: L = 723, N = 6 309 against 316 us;
+  // that of the alpha analysis has room for it and spills less, 305 -> 283)
+  const long long limit = MODE == SG_ALPHA_SYN ? kWaitLimit : wait_limit;
   extern __shared__ __align__(128) unsigned char sg_smem[];
   const float* scales = reinterpret_cast<const float*>(sg_smem + (size_t)kSgStages * 2 * kHalf);
   __shared__ __align__(8) uint64_t bar[2 * kSgStages + 4];  // full[S], empty[S], tfull[2], tempty[2]
   __shared__ uint32_t tbase;
-  __shared__ int s_fail;
+  __shared__ int s_fail, s_loaded, s_issued;  // a role gave up; stages whose copies, whose products were issued
   volatile int* fail = &s_fail;
   constexpr bool DATA_A = MODE == SG_BETA_ANA || MODE == SG_BETA_SYN;
   const int t = threadIdx.x, w = t >> 5, lane = t & 31;
@@ -417,7 +421,7 @@ k_split_gemm(const CztSeg<float>* __restrict__ segs, int nseg, int total, CallPt
         const unsigned char* dat = reinterpret_cast<const unsigned char*>(T.sg->pre) + (size_t)T.rt * T.nk * kData;
         for (int c = 0; c < T.nk; ++c, ++gc) {
           const int s = gc % kSgStages;
-          if (gc >= kSgStages && !sg_wait(bempty(s), (uint32_t)(gc / kSgStages - 1) & 1u, fail)) {
+          if (gc >= kSgStages && !sg_wait(bempty(s), (uint32_t)(gc / kSgStages - 1) & 1u, fail, limit)) {
             ok = false;
             break;
           }
@@ -431,9 +435,7 @@ k_split_gemm(const CztSeg<float>* __restrict__ segs, int nseg, int total, CallPt
           bulk_g2s(dsc, dat + (size_t)c * kData + kHalf, kScaleB, mb);
         }
       }
-      if (*fail)  // copies in flight (bounded waits)
-        for (int g = max(0, gc - kSgStages); g < gc; ++g)
-          tc::mbar_wait(bfull(g % kSgStages), (uint32_t)(g / kSgStages) & 1u, tc::kWaitCycles);
+      s_loaded = gc;
     }
     __syncwarp();
   } else if (w == 1) {
@@ -445,8 +447,8 @@ k_split_gemm(const CztSeg<float>* __restrict__ segs, int nseg, int total, CallPt
         const int nk = sg_tile<MODE>(segs, nseg, tile).nk;
         for (int c = 0; c < nk; ++c, ++gc) {
           const int s = gc % kSgStages, b = gc & 1;
-          if (!sg_wait(bfull(s), (uint32_t)(gc / kSgStages) & 1u, fail) ||
-              (gc >= 2 && !sg_wait(btempty(b), (uint32_t)(gc / 2 - 1) & 1u, fail))) {
+          if (!sg_wait(bfull(s), (uint32_t)(gc / kSgStages) & 1u, fail, limit) ||
+              (gc >= 2 && !sg_wait(btempty(b), (uint32_t)(gc / 2 - 1) & 1u, fail, limit))) {
             ok = false;
             break;
           }
@@ -469,10 +471,7 @@ k_split_gemm(const CztSeg<float>* __restrict__ segs, int nseg, int total, CallPt
           tc::mma_commit(btfull(b));
         }
       }
-      if (*fail) {  // MMAs in flight (a bounded wait)
-        if (gc > 0) tc::mbar_wait(btfull((gc - 1) & 1), (uint32_t)((gc - 1) / 2) & 1u, tc::kWaitCycles);
-        atomicAdd(&g_sg_timeouts, 1);
-      }
+      s_issued = gc;
     }
     __syncwarp();
   } else {
@@ -491,7 +490,9 @@ k_split_gemm(const CztSeg<float>* __restrict__ segs, int nseg, int total, CallPt
       for (int c = 0; c < T.nk; ++c) {
         const int b = gc & 1;
         const float* sc = scales + (gc % kSgScales) * (kScaleB / 4);
-        if (!sg_wait(btfull(b), (uint32_t)(gc / 2) & 1u, fail)) {
+        // one decision per warp: the TMEM loads and the barrier below are warp-collective
+        if (!__all_sync(0xffffffffu, sg_wait(btfull(b), (uint32_t)(gc / 2) & 1u, fail, limit))) {
+          *fail = 1;
           ok = false;
           break;
         }
@@ -588,7 +589,18 @@ k_split_gemm(const CztSeg<float>* __restrict__ segs, int nseg, int total, CallPt
   tc::fence_before();
   __syncthreads();
   tc::fence_after();
-  if (w == 1) tc::tmem_free(tmem, 512);
+  if (w == 1) {
+    // After a give-up, whichever role's it was (every role has left its loop): the
+    // copies and products in flight, in bounded waits, before TMEM goes
+    if (lane == 0 && s_fail) {
+      for (int g = max(0, s_loaded - kSgStages); g < s_loaded; ++g)
+        tc::mbar_wait(bfull(g % kSgStages), (uint32_t)(g / kSgStages) & 1u, tc::kWaitCycles);
+      if (s_issued > 0) tc::mbar_wait(btfull((s_issued - 1) & 1), (uint32_t)((s_issued - 1) / 2) & 1u, tc::kWaitCycles);
+      atomicAdd(&g_sg_timeouts, 1);
+    }
+    __syncwarp();
+    tc::tmem_free(tmem, 512);
+  }
 }
 
 // Basis images.  root: e^{2 pi i u / period}, u < period (FP64).  One thread per
@@ -709,9 +721,10 @@ cudaError_t sg_build_table(int mode, void* out, double2* scratch, const double* 
 
 namespace {
 template <int MODE>
-void sg_launch(const CztSeg<float>* segs, int nseg, int total, int stages, const CallPtrs& ptrs, cudaStream_t st) {
+void sg_launch(const CztSeg<float>* segs, int nseg, int total, int stages, const CallPtrs& ptrs, cudaStream_t st,
+               long long limit) {
   launch_after(k_sg_convert<MODE>, stages, 32 * kCvWarps, kData, st, segs, nseg, ptrs);
-  launch_after(k_split_gemm<MODE>, std::min(total, sg_sms()), kSgThreads, kSgSmem, st, segs, nseg, total, ptrs);
+  launch_after(k_split_gemm<MODE>, std::min(total, sg_sms()), kSgThreads, kSgSmem, st, segs, nseg, total, ptrs, limit);
 }
 template <int MODE>
 cudaError_t sg_attr() {
@@ -719,15 +732,16 @@ cudaError_t sg_attr() {
 }
 }  // namespace
 
-// total: output tiles, stages: data stages of the launch (two launches)
+// total: output tiles, stages: data stages of the launch (two launches); limit:
+// cycles of the products' bounded waits
 void launch_split_gemm(int mode, const CztSeg<float>* segs, int nseg, int total, int stages, const CallPtrs& ptrs,
-                       cudaStream_t st) {
+                       cudaStream_t st, long long limit) {
   if (total <= 0) return;
   switch (mode) {
-    case SG_BETA_ANA: sg_launch<SG_BETA_ANA>(segs, nseg, total, stages, ptrs, st); break;
-    case SG_BETA_SYN: sg_launch<SG_BETA_SYN>(segs, nseg, total, stages, ptrs, st); break;
-    case SG_ALPHA_ANA: sg_launch<SG_ALPHA_ANA>(segs, nseg, total, stages, ptrs, st); break;
-    default: sg_launch<SG_ALPHA_SYN>(segs, nseg, total, stages, ptrs, st); break;
+    case SG_BETA_ANA: sg_launch<SG_BETA_ANA>(segs, nseg, total, stages, ptrs, st, limit); break;
+    case SG_BETA_SYN: sg_launch<SG_BETA_SYN>(segs, nseg, total, stages, ptrs, st, limit); break;
+    case SG_ALPHA_ANA: sg_launch<SG_ALPHA_ANA>(segs, nseg, total, stages, ptrs, st, limit); break;
+    default: sg_launch<SG_ALPHA_SYN>(segs, nseg, total, stages, ptrs, st, limit); break;
   }
 }
 

@@ -18,6 +18,8 @@
 
 #include <cstdint>
 
+#include "internal.h"
+
 namespace s2dw {
 namespace tc {
 
@@ -96,8 +98,7 @@ __device__ __forceinline__ bool mbar_wait(uint32_t mbar, uint32_t parity, long l
   return true;
 }
 
-// about one second at the maximum SM clock
-constexpr long long kWaitCycles = 2000000000LL;
+constexpr long long kWaitCycles = kWaitLimit;
 
 // TMEM columns (power of two >= 32), allocated by one whole warp; the base
 // address is written to *dst (shared memory).
