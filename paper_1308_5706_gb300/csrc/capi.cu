@@ -2184,7 +2184,17 @@ int s2dw_plan_wait_probe(s2dw_plan_t p, long long limit_cycles, void* stream) {
   cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
   CallPtrs ptrs;  // (these launches read and write the workspace only)
   std::memset(&ptrs, 0, sizeof(ptrs));
-  for (int kind : {SG_KIND_BETA_ANA, SG_KIND_BETA_RS, SG_KIND_BETA_SYN}) launch_products<float>(p->own, kind, ptrs, st, lim);
+  const Lists& ls = p->own;
+  const ContractDesc<float>* dw = reinterpret_cast<const ContractDesc<float>*>(ls.desc_w);
+  const ContractDesc<float>* dp = reinterpret_cast<const ContractDesc<float>*>(ls.desc_phi);
+  auto contract = [&](bool syn) {
+    for (auto& g : ls.tile_w)
+      launch_contract_tile(g.N, 2, syn, dw, reinterpret_cast<const CTask*>(g.task[syn]), g.n[syn], st, lim);
+    launch_contract_tile(1, 1, syn, dp, reinterpret_cast<const CTask*>(ls.tile_phi.task[syn]), ls.tile_phi.n[syn], st, lim);
+  };
+  contract(false);
+  for (int kind : {SG_KIND_BETA_ANA, SG_KIND_BETA_RS, SG_KIND_BETA_SYN}) launch_products<float>(ls, kind, ptrs, st, lim);
+  contract(true);
   mark_use(p, st);
   return err_of(cudaGetLastError());
 }

@@ -57,14 +57,14 @@ void tile_pick(int N, int nslot, F&& f) {
 }  // namespace
 
 void launch_contract_tile(int N, int nslot, bool syn, const ContractDesc<float>* descs, const CTask* tasks, int ntasks,
-                          cudaStream_t st) {
+                          cudaStream_t st, long long limit) {
   if (ntasks <= 0) return;
   tile_pick(N, nslot, [&](auto n, auto s) {
     constexpr int NN = decltype(n)::value, NS = decltype(s)::value, H = NN <= 6 ? 2 : 1;
     if (syn)
-      launch_after(k_contract_tile<NN, NS, true, H>, ntasks, 256, TileGeom<NN, NS, true, H>::SMEM, st, descs, tasks);
+      launch_after(k_contract_tile<NN, NS, true, H>, ntasks, 256, TileGeom<NN, NS, true, H>::SMEM, st, descs, tasks, limit);
     else
-      launch_after(k_contract_tile<NN, NS, false, H>, ntasks, 256, TileGeom<NN, NS, false, H>::SMEM, st, descs, tasks);
+      launch_after(k_contract_tile<NN, NS, false, H>, ntasks, 256, TileGeom<NN, NS, false, H>::SMEM, st, descs, tasks, limit);
   });
 }
 

@@ -50,8 +50,9 @@
 // the sums without copies 0.27 ms: two warps per scheduler leave fixed
 // latencies exposed, more do not fit beside the accumulators.
 //
-// Every wait is bounded (about a second): a CTA that gives up stops computing,
-// waits for its own copies and counts the event for s2dw_wait_timeouts.
+// Every wait is bounded (about a second): a CTA that gives up issues no more
+// copies, runs through what is left, waits for its own copies and counts the event
+// for s2dw_wait_timeouts.
 #pragma once
 
 #include <type_traits>
@@ -98,10 +99,15 @@ __device__ __forceinline__ bool mbar_ready(uint32_t mbar, uint32_t par) {
 }
 // Blocking wait (try_wait, system-dependent suspension) for the phase of
 // parity `par`; false once *abort is set (by this or another thread) or after
-// tc::kWaitCycles, which sets it.
-__device__ __noinline__ bool pair_wait_slow(uint32_t mbar, uint32_t par, volatile int* abort) {
+// `limit` cycles, which sets it.
+__device__ __noinline__ bool pair_wait_slow(uint32_t mbar, uint32_t par, volatile int* abort, long long limit) {
   const long long t0 = clock64();
   for (;;) {
+    if (*abort) return false;
+    if (clock64() - t0 >= limit) {
+      *abort = 1;
+      return false;
+    }
     uint32_t ok;
     asm volatile(
         "{\n.reg .pred p;\nmbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\nselp.u32 %0, 1, 0, p;\n}\n"
@@ -109,15 +115,10 @@ __device__ __noinline__ bool pair_wait_slow(uint32_t mbar, uint32_t par, volatil
         : "r"(mbar), "r"(par)
         : "memory");
     if (ok) return true;
-    if (*abort) return false;
-    if (clock64() - t0 > tc::kWaitCycles) {
-      *abort = 1;
-      return false;
-    }
   }
 }
-__device__ __forceinline__ bool pair_wait(uint32_t mbar, uint32_t par, volatile int* abort) {
-  return mbar_ready(mbar, par) || pair_wait_slow(mbar, par, abort);
+__device__ __forceinline__ bool pair_wait(uint32_t mbar, uint32_t par, volatile int* abort, long long limit) {
+  return mbar_ready(mbar, par) || pair_wait_slow(mbar, par, abort, limit);
 }
 __device__ __forceinline__ void mbar_expect(uint32_t mbar, uint32_t bytes) {
   asm volatile("{\n.reg .b64 st;\nmbarrier.arrive.expect_tx.shared::cta.b64 st, [%0], %1;\n}\n" ::"r"(mbar), "r"(bytes)
@@ -152,6 +153,7 @@ struct TileCtx {
   TileSrc* src;
   uint32_t ring_s, full_s, empty_s;
   volatile int* abort;
+  long long limit;       // cycles of a bounded wait
   int lo[2], hi[2];      // l range of each slot's scale (empty: hi < lo)
 };
 
@@ -160,6 +162,7 @@ template <typename G, bool SYN, int HALVES>
 struct TileRing {
   const TileCtx& x;
   int issued = 0;
+  bool live = true;  // none of this thread's waits for a stage has given up
   __device__ __forceinline__ explicit TileRing(const TileCtx& c) : x(c) {}
   __device__ __forceinline__ void issue() {
     const uint32_t slot = (uint32_t)issued % G::STAGES, mb = x.full_s + 8u * slot;
@@ -196,28 +199,34 @@ struct TileRing {
     }
     for (int i = 0; i < min(nst, G::STAGES); ++i) issue();
   }
-  // data of stage i, or nullptr after a wait that gave up
-  __device__ __forceinline__ const float* wait(int i) const {
+  // Data of stage i.  A wait that gave up changes nothing in the control flow (the
+  // sums that follow shuffle over the whole warp, and stay in bounds whatever the
+  // ring holds); the CTA's results are lost and counted.
+  __device__ __forceinline__ const float* wait(int i) {
     const uint32_t slot = (uint32_t)i % G::STAGES;
-    return pair_wait(x.full_s + 8u * slot, ((uint32_t)i / G::STAGES) & 1u, x.abort) ? x.ring + slot * G::SIZE : nullptr;
+    if (!pair_wait(x.full_s + 8u * slot, ((uint32_t)i / G::STAGES) & 1u, x.abort, x.limit)) live = false;
+    return x.ring + slot * G::SIZE;
   }
-  // this warp has read stage i; thread 0 refills the slot read LAG stages ago
+  // This warp has read stage i; thread 0 refills the slot read LAG stages ago.  Not
+  // after a give-up: the slot's last copy may be in flight, and its barrier takes
+  // one arrival per phase.
   __device__ __forceinline__ void release(int i, int nst) {
     __syncwarp();
     if ((threadIdx.x & 31) == 0) tc::mbar_arrive(x.empty_s + 8u * ((uint32_t)i % G::STAGES));
     const int r = i - G::LAG;
-    if (threadIdx.x == 0 && r >= 0 && r + G::STAGES < nst &&
-        pair_wait(x.empty_s + 8u * ((uint32_t)r % G::STAGES), ((uint32_t)r / G::STAGES) & 1u, x.abort))
+    if (threadIdx.x == 0 && live && r >= 0 && r + G::STAGES < nst &&
+        pair_wait(x.empty_s + 8u * ((uint32_t)r % G::STAGES), ((uint32_t)r / G::STAGES) & 1u, x.abort, x.limit))
       issue();
   }
-  // a CTA that gave up waits for its own copies before it may leave
+  // once every warp has left its loop: a CTA that gave up, whichever warp's wait it
+  // was, waits for its own copies before it may leave, and is counted
   __device__ __forceinline__ void finish() {
-    if (*x.abort && threadIdx.x == 0) {
+    __syncthreads();
+    if (threadIdx.x == 0 && *x.abort) {
       for (int i = max(0, issued - G::STAGES); i < issued; ++i)
         tc::mbar_wait(x.full_s + 8u * ((uint32_t)i % G::STAGES), ((uint32_t)i / G::STAGES) & 1u, tc::kWaitCycles);
       atomicAdd(&g_pair_timeouts, 1);
     }
-    __syncthreads();
   }
 };
 
@@ -329,7 +338,7 @@ __device__ __forceinline__ void tile_ana_body(const TileCtx& x) {
   for (int i = 0; i < nst; ++i) {
     const int l0 = l_start + KL * i;
     const float* S = ring.wait(i);
-    if (S && !idle) {
+    if (!idle) {
       if (l0 >= fa && l0 + KL - 1 <= fb) {
 #pragma unroll 1
         for (int ii = 0; ii < KL / 2; ++ii) one(S, 2 * ii + par, std::integral_constant<int, FULL>());
@@ -590,7 +599,7 @@ __device__ __forceinline__ void tile_syn_body(const TileCtx& x) {
     const int l0 = l_start + KL * i;
     float2* redb = x.red + (size_t)(((i & 1) * 2 + par) * (KL / 2)) * G::NWA * 32;
     const float* S = ring.wait(i);
-    if (S && !idle) {
+    if (!idle) {
       if (l0 >= fa && l0 + KL - 1 <= fb) {
 #pragma unroll 1
         for (int ii = 0; ii < KL / 2; ++ii)
@@ -629,7 +638,7 @@ __device__ __forceinline__ void tile_syn_body(const TileCtx& x) {
 
 template <int N, int NSLOT, bool SYN, int HALVES>
 __global__ void __launch_bounds__(256, 1)
-k_contract_tile(const ContractDesc<float>* __restrict__ descs, const CTask* __restrict__ tasks) {
+k_contract_tile(const ContractDesc<float>* __restrict__ descs, const CTask* __restrict__ tasks, long long limit) {
   begin_after();
   using G = TileGeom<N, NSLOT, SYN, HALVES>;
   extern __shared__ __align__(128) unsigned char tile_smem[];
@@ -650,6 +659,7 @@ k_contract_tile(const ContractDesc<float>* __restrict__ descs, const CTask* __re
   x.full_s = tc::smem_u32(&full[0]);
   x.empty_s = tc::smem_u32(&empty[0]);
   x.abort = &s_abort;
+  x.limit = limit;
 #pragma unroll
   for (int s = 0; s < 2; ++s) {
     const int j = s == 0 ? x.tk.j : x.tk.j2;

@@ -262,7 +262,7 @@ bool tile_both_halves(int N);  // a CTA computes both tiles of a block pair
 constexpr int kPairShapePair = 0, kPairShapeTile = 1, kPairShapeTile2 = 2;
 inline bool pair_shapes_offered(int N) { return N <= 5; }
 void launch_contract_tile(int N, int nslot, bool syn, const ContractDesc<float>* descs, const CTask* tasks, int ntasks,
-                          cudaStream_t st);
+                          cudaStream_t st, long long limit = kWaitLimit);
 void launch_fpack(const ContractDesc<float>* descs, int njobs, int nbmax, int Lrmax, const CallPtrs& ptrs,
                   cudaStream_t st);
 template <typename T>

@@ -20,7 +20,8 @@ def _roundtrip(p, f):
     return W, Wp, g
 
 
-@pytest.mark.parametrize("L,N,kw", [(200, 2, {}), (361, 5, {}), (300, 3, {"mw": True})])
+@pytest.mark.parametrize("L,N,kw", [(200, 2, {}), (361, 5, {}), (300, 3, {"mw": True}),
+                                    (512, 1, {}), (512, 5, {}), (512, 8, {})])
 def test_kernels_give_up_in_every_role(L, N, kw):
     import torch
     f = torch.from_numpy(flm_gaussian(L, 3, "cl")).to(torch.complex64).cuda()
