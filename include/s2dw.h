@@ -250,12 +250,14 @@ int s2dw_wait_probe(long long limit_cycles, void* stream);
 
 /*
  * s2dw_plan_wait_probe: the same in the kernels themselves.  Launches on `stream`
- * the plan's kernels with bounded waits that touch nothing but its workspace
- * (contraction of large band-limits, matrix products of the beta sums), with
- * waits that give up after limit_cycles SM cycles (clamped to [0, 2e9]; 0: at the first
- * look).  What gave up is counted for s2dw_wait_timeouts; the intermediates of the plan's
- * last call are lost (s2dw_stage), later calls are not affected.  FP32 plans
- * (S2DW_ENOTSUP for FP64 ones, which have no such waits); S2DW_EINVAL for NULL.
+ * the plan's kernels with bounded waits (contraction of large band-limits, matrix
+ * products, direct alpha sums) over its workspace and a scratch W, allocated and
+ * freed in stream order, with waits that give up after limit_cycles SM cycles
+ * (clamped to [0, 2e9]; 0: at once; the products of the alpha synthesis keep
+ * their own limit).  What gave up is counted for s2dw_wait_timeouts; the
+ * intermediates of the plan's last call are lost (s2dw_stage), later calls are
+ * not affected.  FP32 plans (S2DW_ENOTSUP for FP64 ones, which have no such
+ * waits); S2DW_EINVAL for NULL.
  */
 int s2dw_plan_wait_probe(s2dw_plan_t plan, long long limit_cycles, void* stream);
 

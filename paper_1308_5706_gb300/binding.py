@@ -192,7 +192,7 @@ def s2dw_wait_probe(limit_cycles: int, stream=None) -> None:
 
 
 def s2dw_plan_wait_probe(plan: int, limit_cycles: int, stream=None) -> None:
-    """The plan's own kernels with bounded waits, over its workspace, with waits
+    """The plan's own kernels with bounded waits, over scratch data, with waits
     that give up after limit_cycles SM cycles (mixed plans)."""
     _check(lib().s2dw_plan_wait_probe(plan, int(limit_cycles), _stream(stream)), "s2dw_plan_wait_probe")
 

@@ -76,13 +76,18 @@ constexpr size_t syn_tc_smem() {
 // -> 11, L = 361, N = 4 26 -> 15, L = 1024, N = 5 (503 MB of W) 144 -> 123, L = 2048,
 // N = 8 784 -> 678.
 // Every wait is bounded and a timeout in any role stops all of them.
+// PROBE: waits of wait_limit cycles (s2dw_plan_wait_probe); a run-time limit in the
+// kernels themselves costs them 1%.
+template <bool PROBE>
 __global__ void __launch_bounds__(kTcAnaThreads, 1) k_alpha_ana_tc(const CztSeg<float>* __restrict__ segs,
-                                                                   int nseg, CallPtrs ptrs) {
+                                                                   int nseg, CallPtrs ptrs, long long wait_limit) {
   begin_after();
+  const long long limit = PROBE ? wait_limit : tc::kWaitCycles;
   extern __shared__ __align__(128) unsigned char smem_raw[];
   __shared__ __align__(8) uint64_t bar[8];  // full[2], empty[2], tfull[2], tempty[2]
   __shared__ uint32_t tbase;
   __shared__ volatile int fail;
+  __shared__ int issued;  // last row tile whose MMAs were issued, -1: none
   const CztSeg<float> sg = segs[czt_find_seg<float>(segs, nseg)];
   const int item = blockIdx.x - sg.start;
   const int Lj = sg.Lj, n = 2 * sg.L - 1, K8 = ana_k8(Lj);
@@ -148,8 +153,8 @@ __global__ void __launch_bounds__(kTcAnaThreads, 1) k_alpha_ana_tc(const CztSeg<
     int last = -1;  // thread 0: last row tile whose MMAs were issued
     auto issue = [&](int i) {
       const int s = i & 1;
-      if (!tc::mbar_wait(full(s), (uint32_t)(i >> 1) & 1u, tc::kWaitCycles) ||
-          (i >= 2 && !tc::mbar_wait(tempty(s), (uint32_t)((i >> 1) - 1) & 1u, tc::kWaitCycles))) {
+      if (!tc::mbar_wait(full(s), (uint32_t)(i >> 1) & 1u, limit) ||
+          (i >= 2 && !tc::mbar_wait(tempty(s), (uint32_t)((i >> 1) - 1) & 1u, limit))) {
         fail = 1;
         return;
       }
@@ -176,7 +181,7 @@ __global__ void __launch_bounds__(kTcAnaThreads, 1) k_alpha_ana_tc(const CztSeg<
     auto step = [&](int i, float2 (&xr)[16]) -> bool {
       const int s = i & 1;
       if (fail) return false;
-      if (i >= 2 && !tc::mbar_wait(empty(s), (uint32_t)((i >> 1) - 1) & 1u, tc::kWaitCycles)) {
+      if (i >= 2 && !tc::mbar_wait(empty(s), (uint32_t)((i >> 1) - 1) & 1u, limit)) {
         fail = 1;
         return false;
       }
@@ -209,14 +214,13 @@ __global__ void __launch_bounds__(kTcAnaThreads, 1) k_alpha_ana_tc(const CztSeg<
       if (i + 1 < ntr && !step(i + 1, xb)) break;
     }
     asm volatile("cp.async.wait_group 0;" ::: "memory");
-    // after a timeout: a bounded wait for the MMAs in flight before TMEM is released
-    if (t == 0 && fail && last >= 0) tc::mbar_wait(tfull(last & 1), (uint32_t)(last >> 1) & 1u, tc::kWaitCycles);
+    if (t == 0) issued = last;
   } else {
     // samples a0 + 32 (w % 4) + lane, rows 64 h .. 64 h + 63 of a tile
     const int a = a0 + 32 * (w & 3) + lane, cg = 64 * ((w - kAnaProd) >> 2);
     for (int i = 0; i < ntr; ++i) {
       const int s = i & 1;
-      const bool got = !fail && tc::mbar_wait(tfull(s), (uint32_t)(i >> 1) & 1u, tc::kWaitCycles);
+      const bool got = !fail && tc::mbar_wait(tfull(s), (uint32_t)(i >> 1) & 1u, limit);
       if (!__all_sync(0xffffffffu, got)) {  // warp-uniform: the TMEM loads below are warp-collective
         fail = 1;
         break;
@@ -257,8 +261,15 @@ __global__ void __launch_bounds__(kTcAnaThreads, 1) k_alpha_ana_tc(const CztSeg<
   __syncwarp();
   tc::fence_before();
   __syncthreads();
-  if (fail && t == 0) atomicAdd(&g_tc_timeouts, 1);
-  if (w == 0) tc::tmem_free(tmem, 2 * kTcRows);
+  if (w == 0) {
+    // after a give-up, whichever role's it was: a bounded wait for the MMAs in flight before TMEM is released
+    if (t == 0 && fail) {
+      if (issued >= 0) tc::mbar_wait(tfull(issued & 1), (uint32_t)(issued >> 1) & 1u, tc::kWaitCycles);
+      atomicAdd(&g_tc_timeouts, 1);
+    }
+    __syncwarp();
+    tc::tmem_free(tmem, 2 * kTcRows);
+  }
 }
 
 // Synthesis, warp-specialised (one CTA of 128 rows per SM):
@@ -278,13 +289,16 @@ constexpr int kSynProd = 8;                          // producer warps
 constexpr int kSynAcc = 8;                            // accumulator warps
 constexpr int kSynThreads = (kSynProd + kSynAcc + 1) * 32;  // + the MMA warp
 
+template <bool PROBE>
 __global__ void __launch_bounds__(kSynThreads, 1) k_alpha_syn_tc(const CztSeg<float>* __restrict__ segs, int nseg,
-                                                                 CallPtrs ptrs) {
+                                                                 CallPtrs ptrs, long long wait_limit) {
   begin_after();
+  const long long limit = PROBE ? wait_limit : tc::kWaitCycles;
   extern __shared__ __align__(128) unsigned char smem_raw[];
   __shared__ __align__(8) uint64_t bar[2 * kSynStages + 4];  // full[S], empty[S], tfull[2], tempty[2]
   __shared__ uint32_t tbase;
   __shared__ volatile int fail;
+  __shared__ int issued;  // last chunk whose MMAs were issued, -1: none
   const CztSeg<float> sg = segs[czt_find_seg<float>(segs, nseg)];
   const int item = blockIdx.x - sg.start;
   const int Lj = sg.Lj, n = 2 * sg.L - 1, NP = syn_npad(Lj);
@@ -352,7 +366,7 @@ __global__ void __launch_bounds__(kSynThreads, 1) k_alpha_syn_tc(const CztSeg<fl
       if (c + 1 < nchunk) {
         const int c1 = c + 1;
         if (c1 >= kSynStages &&
-            !tc::mbar_wait(empty(c1 % kSynStages), (c1 / kSynStages - 1) & 1, tc::kWaitCycles)) {
+            !tc::mbar_wait(empty(c1 % kSynStages), (c1 / kSynStages - 1) & 1, limit)) {
           fail = 1;
           return false;
         }
@@ -395,12 +409,8 @@ __global__ void __launch_bounds__(kSynThreads, 1) k_alpha_syn_tc(const CztSeg<fl
     for (int j = 0; j < 32; ++j) acc[j] = 0.f;
     bool ok = true;
     for (int c = 0; c < nchunk; ++c) {
-      if (fail) {
-        ok = false;
-        break;
-      }
       const int b = c & 1;
-      const bool got = tc::mbar_wait(tfull(b), (c >> 1) & 1, tc::kWaitCycles);
+      const bool got = !fail && tc::mbar_wait(tfull(b), (c >> 1) & 1, limit);
       if (!__all_sync(0xffffffffu, got)) {  // warp-uniform: the TMEM loads below are warp-collective
         fail = 1;
         ok = false;
@@ -450,8 +460,8 @@ __global__ void __launch_bounds__(kSynThreads, 1) k_alpha_syn_tc(const CztSeg<fl
     for (int c = 0; c < nchunk; ++c) {
       if (fail) break;
       const int st = c % kSynStages, b = c & 1;
-      if (!tc::mbar_wait(full(st), (c / kSynStages) & 1, tc::kWaitCycles) ||
-          (c >= 2 && !tc::mbar_wait(tempty(b), ((c >> 1) - 1) & 1, tc::kWaitCycles))) {
+      if (!tc::mbar_wait(full(st), (c / kSynStages) & 1, limit) ||
+          (c >= 2 && !tc::mbar_wait(tempty(b), ((c >> 1) - 1) & 1, limit))) {
         fail = 1;
         break;
       }
@@ -476,14 +486,20 @@ __global__ void __launch_bounds__(kSynThreads, 1) k_alpha_syn_tc(const CztSeg<fl
       tc::mma_commit(tfull(b));
       last = c;
     }
-    // after a timeout: a bounded wait for the MMAs in flight before TMEM is released
-    if (fail && last >= 0) tc::mbar_wait(tfull(last & 1), (last >> 1) & 1, tc::kWaitCycles);
+    issued = last;
   }
   __syncwarp();
   tc::fence_before();
   __syncthreads();
-  if (fail && t == 0) atomicAdd(&g_tc_timeouts, 1);
-  if (w == kSynProd) tc::tmem_free(tmem, ncols);
+  if (w == kSynProd) {
+    // after a give-up, whichever role's it was: a bounded wait for the MMAs in flight before TMEM is released
+    if (lane == 0 && fail) {
+      if (issued >= 0) tc::mbar_wait(tfull(issued & 1), (issued >> 1) & 1, tc::kWaitCycles);
+      atomicAdd(&g_tc_timeouts, 1);
+    }
+    __syncwarp();
+    tc::tmem_free(tmem, ncols);
+  }
 }
 
 // Basis images.  Analysis: [tile][hi, lo][img_floats(128, K8)], sample a =
@@ -584,18 +600,23 @@ int alpha_tc_items(int L, int rows, int njobs, bool syn, int& P) {
 }
 
 void launch_alpha_tc(bool syn, const CztSeg<float>* segs, int nseg, int total_items, const CallPtrs& ptrs,
-                     cudaStream_t st) {
+                     cudaStream_t st, long long limit) {
   if (total_items <= 0) return;
+  const bool probe = limit != kWaitLimit;
   if (syn)
-    launch_after(k_alpha_syn_tc, total_items, kSynThreads, syn_tc_smem(), st, segs, nseg, ptrs);
+    launch_after(probe ? k_alpha_syn_tc<true> : k_alpha_syn_tc<false>, total_items, kSynThreads, syn_tc_smem(), st, segs, nseg, ptrs, limit);
   else
-    launch_after(k_alpha_ana_tc, total_items, kTcAnaThreads, ana_tc_smem(), st, segs, nseg, ptrs);
+    launch_after(probe ? k_alpha_ana_tc<true> : k_alpha_ana_tc<false>, total_items, kTcAnaThreads, ana_tc_smem(), st, segs, nseg, ptrs, limit);
 }
 
 cudaError_t alpha_tc_prepare() {
-  cudaError_t e = cudaFuncSetAttribute(k_alpha_ana_tc, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)ana_tc_smem());
-  if (e != cudaSuccess) return e;
-  return cudaFuncSetAttribute(k_alpha_syn_tc, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)syn_tc_smem());
+  for (auto k : {k_alpha_ana_tc<false>, k_alpha_ana_tc<true>})
+    if (cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)ana_tc_smem()); e != cudaSuccess)
+      return e;
+  for (auto k : {k_alpha_syn_tc<false>, k_alpha_syn_tc<true>})
+    if (cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)syn_tc_smem()); e != cudaSuccess)
+      return e;
+  return cudaSuccess;
 }
 
 cudaError_t alpha_tc_timeouts(int* count) {

@@ -2182,8 +2182,16 @@ int s2dw_plan_wait_probe(s2dw_plan_t p, long long limit_cycles, void* stream) {
   if (p->fp64) return S2DW_ENOTSUP;
   const long long lim = std::min(std::max(limit_cycles, 0LL), kWaitLimit);
   cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
-  CallPtrs ptrs;  // (these launches read and write the workspace only)
+  int64_t wphi = 0;
+  s2dw_query(p, nullptr, nullptr, &wphi, nullptr, nullptr);
+  const size_t wbytes = ((size_t)p->woff[p->nscale] + (size_t)wphi) * sizeof(float);
+  void* W = nullptr;  // scratch: the alpha sums' W and W^Phi
+  if (cudaError_t e = cudaMallocAsync(&W, wbytes, st); e != cudaSuccess) return err_of(e);
+  cudaMemsetAsync(W, 0, wbytes, st);
+  CallPtrs ptrs;
   std::memset(&ptrs, 0, sizeof(ptrs));
+  ptrs.W[0] = W;
+  ptrs.Wphi[0] = reinterpret_cast<float*>(W) + p->woff[p->nscale];
   const Lists& ls = p->own;
   const ContractDesc<float>* dw = reinterpret_cast<const ContractDesc<float>*>(ls.desc_w);
   const ContractDesc<float>* dp = reinterpret_cast<const ContractDesc<float>*>(ls.desc_phi);
@@ -2192,9 +2200,20 @@ int s2dw_plan_wait_probe(s2dw_plan_t p, long long limit_cycles, void* stream) {
       launch_contract_tile(g.N, 2, syn, dw, reinterpret_cast<const CTask*>(g.task[syn]), g.n[syn], st, lim);
     launch_contract_tile(1, 1, syn, dp, reinterpret_cast<const CTask*>(ls.tile_phi.task[syn]), ls.tile_phi.n[syn], st, lim);
   };
+  auto direct = [&](bool syn) {
+    const int k = syn ? CZT_ALPHA_SYN_DIRECT : CZT_ALPHA_ANA_DIRECT;
+    launch_alpha_tc(syn, reinterpret_cast<const CztSeg<float>*>(ls.segs[k]), ls.nseg[k], ls.items[k], ptrs, st, lim);
+  };
   contract(false);
-  for (int kind : {SG_KIND_BETA_ANA, SG_KIND_BETA_RS, SG_KIND_BETA_SYN}) launch_products<float>(ls, kind, ptrs, st, lim);
+  launch_products<float>(ls, SG_KIND_BETA_ANA, ptrs, st, lim);
+  launch_products<float>(ls, SG_KIND_ALPHA_ANA, ptrs, st, lim);
+  direct(false);
+  direct(true);
+  launch_products<float>(ls, SG_KIND_ALPHA_SYN, ptrs, st, lim);
+  launch_products<float>(ls, SG_KIND_BETA_RS, ptrs, st, lim);
+  launch_products<float>(ls, SG_KIND_BETA_SYN, ptrs, st, lim);
   contract(true);
+  cudaFreeAsync(W, st);
   mark_use(p, st);
   return err_of(cudaGetLastError());
 }

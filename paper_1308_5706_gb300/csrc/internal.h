@@ -196,7 +196,7 @@ size_t alpha_tc_table_floats(int L, int Lj, bool syn);
 cudaError_t alpha_tc_build_table(float* out, int L, int Lj, bool syn, cudaStream_t st);
 int alpha_tc_items(int L, int rows, int njobs, bool syn, int& P);  // CTAs; P: rows per CTA
 void launch_alpha_tc(bool syn, const CztSeg<float>* segs, int nseg, int total_items, const CallPtrs& ptrs,
-                     cudaStream_t st);
+                     cudaStream_t st, long long limit = kWaitLimit);
 cudaError_t alpha_tc_prepare();
 cudaError_t alpha_tc_timeouts(int* count);  // reads and resets the device count
 cudaError_t alpha_tc_wait_probe(long long limit, cudaStream_t st);  // a wait that runs out

@@ -90,8 +90,10 @@ __device__ __forceinline__ void mbar_arrive(uint32_t mbar) {
   asm volatile("{\n.reg .b64 st;\nmbarrier.arrive.shared::cta.b64 st, [%0];\n}\n" ::"r"(mbar) : "memory");
 }
 
-// Wait for the phase of the given parity to complete; false after `limit` SM cycles.
+// Wait for the phase of the given parity to complete; false after `limit` SM
+// cycles (0: at once, without a look).
 __device__ __forceinline__ bool mbar_wait(uint32_t mbar, uint32_t parity, long long limit) {
+  if (limit == 0) return false;
   const long long t0 = clock64();
   while (!mbar_test(mbar, parity))
     if (clock64() - t0 > limit) return false;

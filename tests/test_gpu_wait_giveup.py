@@ -1,5 +1,5 @@
 """Give-up path of the bounded waits inside the kernels: with waits that end at
-the first look the products and contractions of a plan stop in every role, are
+once the products, direct sums and contractions of a plan stop in every role, are
 counted, and leave tensor memory, barriers and context in order: the same plan
 then transforms as before, and waits of ordinary length count nothing."""
 import pytest
@@ -20,7 +20,7 @@ def _roundtrip(p, f):
     return W, Wp, g
 
 
-@pytest.mark.parametrize("L,N,kw", [(200, 2, {}), (361, 5, {}), (300, 3, {"mw": True}),
+@pytest.mark.parametrize("L,N,kw", [(32, 2, {}), (200, 2, {}), (361, 5, {}), (300, 3, {"mw": True}),
                                     (512, 1, {}), (512, 5, {}), (512, 8, {})])
 def test_kernels_give_up_in_every_role(L, N, kw):
     import torch
@@ -32,7 +32,8 @@ def test_kernels_give_up_in_every_role(L, N, kw):
         for limit in (0, 50, 1500):  # cycles: less than a bulk copy takes, up to about as long
             B.s2dw_plan_wait_probe(p.handle, limit)
             n = B.s2dw_wait_timeouts()  # synchronises: the launches have ended
-            assert n > 0 or limit > 50
+            # (at L = 32 only the direct alpha sums have such waits; they look once, suspended, before a limit ends them)
+            assert n > 0 or limit > (0 if L == 32 else 50)
         B.s2dw_plan_wait_probe(p.handle, 2_000_000_000)
         assert B.s2dw_wait_timeouts() == 0
         for a, b in zip(before, _roundtrip(p, f)):
