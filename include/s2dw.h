@@ -139,6 +139,9 @@ int s2dw_scale_grid(s2dw_plan_t plan, int j, int* Lgrid, int64_t* offset, int64_
  *             2: segmented chirp-z: *segments convolutions of length
  *                *fft_len, each covering *seg_len samples, sharing one
  *                forward FFT (analysis) or one inverse FFT (synthesis).
+ * Where the scale's choice is 3 (s2dw_plan_choices: matrix products) the call
+ * describes the transform that would run in their place, choice 2 if the plan has
+ * it, else 1.
  * Host only; any output may be NULL.  S2DW_EINVAL for a bad j or dir.
  */
 int s2dw_alpha_method(s2dw_plan_t plan, int j, int dir, int* method, int* fft_len, int* segments, int* seg_len);
@@ -287,10 +290,10 @@ int s2dw_stage(s2dw_plan_t plan, int stage, int j, void* host_out, int64_t* nbyt
  *   s2dw_profile_read(plan, ms, ncalls) waits for the recorded calls and
  *   fills ms[13] with per-launch durations (ms) summed over them:
  *   [0] analysis contraction + gamma step, [1] scaling contraction,
- *   [2] beta step, [3] alpha step, chirp-z of the full-band scales,
+ *   [2] beta step, [3] alpha step, matrix products and chirp-z of the full-band scales,
  *   [4] alpha step, segmented chirp-z of the mid-band scales, [5] alpha
  *   step, direct sums of the small-band scales; [6] synthesis alpha step
- *   (direct sums), [7] alpha step (full-band chirp-z), [8] alpha step
+ *   (direct sums), [7] alpha step (products, full-band chirp-z), [8] alpha step
  *   (segmented chirp-z), [9] beta step, [10] contraction, [11] scaling
  *   contraction, [12] final reduction (an empty launch reads 0);
  *   ncalls[2] (may be NULL) gets the numbers of analysis and synthesis calls.
@@ -313,9 +316,9 @@ int s2dw_profile_read(s2dw_plan_t plan, double* ms, int* ncalls);
  *   [2 + 2j] alpha sums of the analysis of scale j (j = J+1: scaling part),
  *   [3 + 2j] of the synthesis: 0 = direct sums (L_j <= 32), 1 = chirp-z of
  *       the grid's length, 2 = segmented chirp-z (where the plan built its
- *       tables, s2dw_alpha_method).  The default of an FP32 plan's scale above
- *       32 runs matrix products on the tensor cores instead where those are
- *       faster (mid bands, L >= 128); any other value runs as named;
+ *       tables, s2dw_alpha_method), 3 = matrix products on the tensor cores (the
+ *       default of an FP32 plan's scales above 32 where they are faster: L >= 128,
+ *       mid bands and, at smaller L, full ones; not available elsewhere);
  *   [last] the contraction's CTA shape (FP32 plans): 0, 1, 2 for N <= 5, 1 for N >
  *       5; FP64 plans: 0.  Kept for saved choices: the contraction now follows
  *       from L and N and every value runs the same kernels;

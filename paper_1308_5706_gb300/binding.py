@@ -160,7 +160,8 @@ def s2dw_scale_grid(plan: int, j: int):
 def s2dw_alpha_method(plan: int, j: int, direction: int):
     """(method, fft_len, segments, seg_len) of the alpha sums of scale j;
     direction 0 analysis, 1 synthesis; method 0 direct, 1 chirp-z,
-    2 segmented chirp-z."""
+    2 segmented chirp-z (for a scale that runs matrix products, choice 3 of
+    ``s2dw_plan_choices``, the transform in their place)."""
     vals = [ctypes.c_int() for _ in range(4)]
     _check(lib().s2dw_alpha_method(plan, j, direction, *[ctypes.byref(v) for v in vals]), "s2dw_alpha_method")
     return tuple(v.value for v in vals)

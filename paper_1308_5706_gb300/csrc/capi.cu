@@ -372,10 +372,11 @@ struct s2dw_plan_s {
   // FFT of length 4L, 1 = half-length transforms on the grids where they are
   // faster (power-of-two L >= 128; synthesis up to 1024);
   // alpha_mode[dir][j] 0 = direct sums (L_j <= 32), 1 = chirp-z of the grid's
-  // length, 2 = segmented chirp-z (where its tables exist); dir 0 = analysis
+  // length, 2 = segmented chirp-z (where its tables exist), 3 = split products
+  // (where alpha_sg: FP32 plans, the scales on which they are faster; their
+  // default); dir 0 = analysis
   int beta_mode[2] = {1, 1};
-  std::vector<int> alpha_mode[2], alpha_default[2];
-  // FP32: the alpha sums of scale j run as split products (while its method is the default one)
+  std::vector<int> alpha_mode[2];
   std::vector<char> alpha_sg[2];
   void* sg_data = nullptr;  // operand images of the product launch under way
   // [nscale + 1]: tensor-core basis images of the direct alpha sums (FP32 plans)
@@ -775,12 +776,7 @@ void build_segs(s2dw_plan_s* p, int job, int njobs, int kind, std::vector<CztSeg
     const int amode = is_alpha ? p->alpha_mode[base_kind == CZT_ALPHA_SYN ? 1 : 0][j] : -1;
     const bool direct = is_alpha && amode == 0;
     if (direct != direct_list) continue;
-    if (is_alpha && !direct) {
-      const int d = base_kind == CZT_ALPHA_SYN ? 1 : 0;
-      const bool sg = p->alpha_sg[d][j] && amode == p->alpha_default[d][j];
-      if (sg != sg_list) continue;
-      if (!sg && (amode == 2) != seg_list) continue;
-    }
+    if (is_alpha && !direct && ((amode == 3) != sg_list || (amode == 2) != seg_list)) continue;
     switch (base_kind) {
       case CZT_BETA_ANA:
         s.P = beta_czt_cols(G.logM, sizeof(T) == 8);  // columns per CTA of the chirp-z beta kernels
@@ -1315,8 +1311,8 @@ void plan_build_typed(s2dw_plan_s* p, const double* kap_d, const double* phi_d, 
     so[j].Ha = take((size_t)sgt.S * Ms * sizeof(cx<T>));
     so[j].Hs = take((size_t)sgt.S * Ms * sizeof(cx<T>));
   }
-  // default launch methods: direct sums for L_j <= 32, segmented chirp-z where it
-  // was chosen above, else the grid's chirp-z
+  // default launch methods: direct sums for L_j <= 32, split products where they are
+  // faster, segmented chirp-z where it was chosen above, else the grid's chirp-z
   for (int d = 0; d < 2; ++d) {
     p->alpha_mode[d].assign(p->nscale + 1, 1);
     p->alpha_sg[d].assign(p->nscale + 1, 0);
@@ -1328,8 +1324,8 @@ void plan_build_typed(s2dw_plan_s* p, const double* kap_d, const double* phi_d, 
       const auto& sgt = p->seg[j];
       const double cost = sgt.S > 0 ? (double)(sgt.S + 1) * ((size_t)1 << sgt.logM) * sgt.logM : 2.0 * G.M * G.logM;
       p->alpha_sg[d][j] = pairc && p->alpha_mode[d][j] != 0 && sg_alpha_faster(G.L, Lj, cost, sgt.S > 0);
+      if (p->alpha_sg[d][j]) p->alpha_mode[d][j] = 3;
     }
-    p->alpha_default[d] = p->alpha_mode[d];
   }
   // basis tables of the split products
   std::vector<std::array<size_t, 5>> o_sg(p->gt.size());
@@ -1907,16 +1903,13 @@ int s2dw_scale_grid(s2dw_plan_t p, int j, int* Lgrid, int64_t* offset, int64_t* 
 
 int s2dw_alpha_method(s2dw_plan_t p, int j, int dir, int* method, int* fft_len, int* segments, int* seg_len) {
   if (!p || j < 0 || j > p->nscale || dir < 0 || dir > 1) return S2DW_EINVAL;
-  const int Lj = p->Ycols[j];
   const auto& G = p->gt[p->grid_of[j]];
   const auto& sgt = p->seg[j];
-  int m = 1, len = G.M, ns = 1, sl = 2 * G.L - 1;
-  (void)Lj;
-  if (p->alpha_mode[dir][j] == 0) {
-    m = 0;
+  int m = p->alpha_mode[dir][j], len = G.M, ns = 1, sl = 2 * G.L - 1;
+  if (m == 3) m = sgt.S > 0 ? 2 : 1;  // products: the transform in their place
+  if (m == 0) {
     len = ns = sl = 0;
-  } else if (p->alpha_mode[dir][j] == 2) {
-    m = 2;
+  } else if (m == 2) {
     len = 1 << sgt.logM;
     ns = sgt.S;
     sl = sgt.P;
@@ -1943,6 +1936,7 @@ static bool choice_valid(s2dw_plan_t p, int idx, int v) {
   if (v == 0) return Lj <= (d == 0 ? kDirectMaxLjAna : kDirectMaxLj);  // direct kernels sized for L_j <= 32
   if (v == 1) return true;
   if (v == 2) return p->seg[j].S > 0;  // segment tables built at plan creation
+  if (v == 3) return p->alpha_sg[d][j] != 0;  // basis tables built at plan creation
   return false;
 }
 
@@ -2115,7 +2109,7 @@ int s2dw_plan_tune(s2dw_plan_t p, int reps, int* choices, int* n) {
     for (int d = 0; d < 2; ++d)
       for (int j : order) {
         const int idx = 2 + 2 * j + d;
-        for (int v = 0; v < 3; ++v) {
+        for (int v = 0; v < 4; ++v) {
           if (v == cur[idx] || !choice_valid(p, idx, v) || p->Ycols[j] <= 0) continue;
           std::vector<int> trial(cur);
           trial[idx] = v;
