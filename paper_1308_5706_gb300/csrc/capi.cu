@@ -1455,7 +1455,7 @@ void plan_build_typed(s2dw_plan_s* p, const double* kap_d, const double* phi_d, 
       const size_t Lg = G.L, ng = 2 * Lg - 1;
       need = std::max(need, (size_t)G.M + ng + (2 * Lg - 1) + 2 * Lg + 2 * Lg + (2 * Lg - 1) + ng + (4 * Lg - 1) +
                                 4 * (size_t)G.M);
-      need = std::max(need, 8 * Lg);  // roots of the split products' basis
+      need = std::max(need, sg_build_scratch(G.L));  // roots of the split products' basis
     }
     amalloc(&t64, need * sizeof(double2), st);
     amalloc(&qg, (size_t)2 * p->gt.back().L * sizeof(double), st);
@@ -1496,8 +1496,7 @@ void plan_build_typed(s2dw_plan_s* p, const double* kap_d, const double* phi_d, 
     put(G.pre_mw, tw64, ng);
     ck(launch_twiddles64(tw64, G.logM - 1, st));  // length 2Lg (half-length beta transforms)
     put(G.tw2, tw64, twiddle_entries(G.logM - 1));
-    for (int k = 0; k < 5; ++k)  // (roots in the same scratch)
-      if (G.sg[k]) ck(sg_build_table(k == 4 ? 0 : k, G.sg[k], tw64, q_g, Lg, p->mw && k == 0, st));
+    ck(sg_build_tables(G.sg, tw64, q_g, Lg, p->mw, st));  // (its roots in the same scratch)
   }
   {
     size_t need = 0;

@@ -215,8 +215,8 @@ struct SgDims {
 SgTable sg_table(int mode, int L);
 SgDims sg_dims(int mode, int L, int Lj, int N, int nb);
 float sg_out_scale(int mode, int L);
-int sg_period(int mode, int L, bool mw);  // double2 of scratch the build needs
-cudaError_t sg_build_table(int mode, void* out, double2* scratch, const double* qw, int L, bool mw, cudaStream_t st);
+size_t sg_build_scratch(int L);  // double2
+cudaError_t sg_build_tables(void* const* out, double2* scratch, const double* qw, int L, bool mw, cudaStream_t st);
 void launch_split_gemm(int mode, const CztSeg<float>* segs, int nseg, int total, int stages, const CallPtrs& ptrs,
                        cudaStream_t st, long long limit = kWaitLimit);
 // Whether the products are the faster form.  beta: the chirp-z (other L than

@@ -603,50 +603,89 @@ k_split_gemm(const CztSeg<float>* __restrict__ segs, int nseg, int total, CallPt
   }
 }
 
-// Basis images.  root: e^{2 pi i u / period}, u < period (FP64).  One thread per
-// (set, tile, stage, product, row r, position k); term of position k: 2 t + u
-// holds term t + 16 u of the stage.  The synthesis of beta keeps its terms in
-// order (four b per store).
-template <int MODE>
-__global__ void k_sg_basis(unsigned char* out, const double2* __restrict__ root, const double* __restrict__ qw, int L,
-                           int period, int tiles, int nk, int sets, double bscale, int mw) {
-  const long long idx = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-  const int k = (int)(idx & 31), r = (int)((idx >> 5) & 127), p = (int)((idx >> 12) & 1);
-  const long long st = idx >> 13;  // (set * tiles + tile) * nk + stage
-  if (st >= (long long)sets * tiles * nk) return;
-  const int c = (int)(st % nk), tile = (int)((st / nk) % tiles), set = (int)(st / ((long long)nk * tiles));
-  const int term = kSgK * c + (MODE == SG_BETA_SYN ? k : (k >> 1) + 16 * (k & 1)), row = 128 * tile + r;
-  double v = 0.0;
-  auto trig = [&](long long u, bool sine) {
-    const double2 e = root[(int)(u % period)];
-    return sine ? e.y : e.x;
-  };
-  if (MODE == SG_BETA_ANA) {  // row: b, term: i of m' = 2 i + p; set 1: sin
-    const long long mp = 2 * term + p;
-    if (row < L && mp < L) v = (mp == 0 ? 1.0 : 2.0) * trig(mp * (2 * row + 1), set == 1);
-  } else if (MODE == SG_BETA_SYN) {  // row: i of m', term: b; product 0: even m' (cos) or odd (sin)
-    const long long mp = 2 * row + (p ^ set);
-    if (term < L && mp < L) v = (mp == 0 ? 1.0 : 2.0) * qw[term] * trig(mp * (2 * term + 1), set == 1);
-  } else if (MODE == SG_ALPHA_ANA) {  // row: a, term: m
-    if (row < L && term < L) v = (term == 0 ? 1.0 : 2.0) * (p == 0 ? 1.0 : -1.0) * trig((long long)term * row, p == 1);
-  } else {  // row: m, term: a
-    if (row < L && term < L) v = (p == 0 ? 1.0 : -1.0) * trig((long long)term * row, p == 1);
-  }
-  (void)mw;
-  v *= bscale;
+// Basis images of a grid, all its tables in one launch (a launch per table, with
+// FP64 arithmetic and 2-byte stores per element, took 63 us of a new plan at L =
+// 723 and 425 at L = 2048; now with the roots 25 and 152).
+// Roots: trig values of the three periods, split once per root instead of once
+// per element: {cos hi, cos lo, sin hi, sin lo} of 2^14 e^{2 pi i u / period}, the
+// scaled coefficient 2 of the analyses (1 only where the angle is 0) and 1 of the
+// alpha synthesis; FP64 values for the beta synthesis, whose terms carry q_b.
+struct SgRoots {
+  double2* beta64;                 // 8 L
+  uint2 *beta, *beta_mw, *alpha;   // 8 L, 2 (2L - 1), 2L - 1
+  int n[3];
+};
+__device__ __forceinline__ uint32_t sg_split(double v) {  // hi | lo << 16
   const __half hi = __double2half(v);
   const __half lo = __double2half(v - (double)__half2float(hi));
-  unsigned char* q = out + (size_t)st * kHalf + (size_t)(2 * p) * kImg + sg_off(r, k);
-  *reinterpret_cast<__half*>(q) = hi;
-  *reinterpret_cast<__half*>(q + kImg) = lo;
+  return (uint32_t)__half_as_ushort(hi) | ((uint32_t)__half_as_ushort(lo) << 16);
+}
+__global__ void __launch_bounds__(256) k_sg_roots(SgRoots t) {
+  int u = blockIdx.x * 256 + threadIdx.x, k = 0;
+  while (k < 3 && u >= t.n[k]) u -= t.n[k++];
+  if (k == 3) return;
+  double s, c;
+  sincospi(2.0 * u / t.n[k], &s, &c);
+  (k == 0 ? t.beta : (k == 1 ? t.beta_mw : t.alpha))[u] =
+      make_uint2(sg_split(c * kSgAlphaSynScale), sg_split(s * kSgAlphaSynScale));
+  if (k == 0) t.beta64[u] = make_double2(c, s);
 }
 
-__global__ void k_sg_roots(double2* out, int period) {
-  const int u = blockIdx.x * blockDim.x + threadIdx.x;
-  if (u >= period) return;
-  double s, c;
-  sincospi(2.0 * u / period, &s, &c);
-  out[u] = make_double2(c, s);
+struct SgBuild {  // one table of the launch
+  unsigned char* out;
+  int mode, mw, tiles, stages, first;  // first block
+};
+struct SgBuilds {
+  SgBuild t[5];
+  int n;
+};
+// A thread writes 16 bytes of both images: eight positions k of one row r of (set,
+// tile, stage, product).  Term of position k: 2 t + u holds term t + 16 u of the
+// stage; the synthesis of beta keeps its terms in order (four b per store).
+__global__ void __launch_bounds__(256) k_sg_basis(SgBuilds b, SgRoots roots, const double* __restrict__ qw, int L, double syn_scale) {
+  int job = 0;
+  while (job + 1 < b.n && (int)blockIdx.x >= b.t[job + 1].first) ++job;
+  const SgBuild& t = b.t[job];
+  const int idx = (blockIdx.x - t.first) * 256 + threadIdx.x;
+  const int r = idx & 127, kc = (idx >> 7) & 3, p = (idx >> 9) & 1, st = idx >> 10;  // st: (set * tiles + tile) * stages + stage
+  const int c = st % t.stages, tile = (st / t.stages) % t.tiles, set = st / (t.stages * t.tiles);
+  const int row = 128 * tile + r, mode = t.mode, period = roots.n[t.mw ? 1 : (mode >= SG_ALPHA_ANA ? 2 : 0)];
+  const uint2* __restrict__ tab = t.mw ? roots.beta_mw : (mode >= SG_ALPHA_ANA ? roots.alpha : roots.beta);
+  uint32_t w[8];
+#pragma unroll
+  for (int i = 0; i < 8; ++i) {
+    const int k = 8 * kc + i, term = kSgK * c + (mode == SG_BETA_SYN ? k : (k >> 1) + 16 * (k & 1));
+    w[i] = 0;
+    if (mode == SG_BETA_ANA) {  // row: b, term: i of m' = 2 i + p; set 1: sin
+      const int mp = 2 * term + p;
+      if (row < L && mp < L) {
+        const uint2 e = tab[mp * (2 * row + 1) % period];
+        w[i] = mp == 0 ? (set ? 0u : sg_split(kSgAnaScale)) : (set ? e.y : e.x);
+      }
+    } else if (mode == SG_BETA_SYN) {  // row: i of m', term: b; product 0: even m' (cos) or odd (sin)
+      const int mp = 2 * row + (p ^ set);
+      if (term < L && mp < L) {
+        const double2 e = roots.beta64[mp * (2 * term + 1) % period];
+        w[i] = sg_split((mp == 0 ? 1.0 : 2.0) * qw[term] * (set ? e.y : e.x) * syn_scale);
+      }
+    } else {  // alpha, analysis: row a, term m; synthesis: row m, term a; product 1: -sin
+      if (row < L && term < L) {
+        const uint2 e = tab[term * row % period];
+        w[i] = p ? e.y ^ 0x80008000u : (mode == SG_ALPHA_ANA && term == 0 ? sg_split(kSgAnaScale) : e.x);
+      }
+    }
+  }
+  unsigned char* q = t.out + (size_t)st * kHalf + (size_t)(2 * p) * kImg + sg_off(r, 8 * kc);
+  uint4 hi, lo;
+  uint32_t* h = &hi.x;
+  uint32_t* l = &lo.x;
+#pragma unroll
+  for (int i = 0; i < 4; ++i) {
+    h[i] = __byte_perm(w[2 * i], w[2 * i + 1], 0x5410);
+    l[i] = __byte_perm(w[2 * i], w[2 * i + 1], 0x7632);
+  }
+  *reinterpret_cast<uint4*>(q) = hi;
+  *reinterpret_cast<uint4*>(q + kImg) = lo;
 }
 
 // power of two that brings the synthesis beta basis, |2 q_b| < 4 / L, up to 2^14
@@ -699,23 +738,31 @@ SgDims sg_dims(int mode, int L, int Lj, int N, int nb) {
   return d;
 }
 
-// scratch: `period` double2 (beta: 8 L, or 2 (2L-1) on the MW grid; alpha: 2L-1)
-int sg_period(int mode, int L, bool mw) {
-  return (mode == SG_BETA_ANA || mode == SG_BETA_SYN) ? (mw ? 2 * (2 * L - 1) : 8 * L) : 2 * L - 1;
-}
-cudaError_t sg_build_table(int mode, void* out, double2* scratch, const double* qw, int L, bool mw, cudaStream_t st) {
-  const SgTable t = sg_table(mode, L);
-  const int period = sg_period(mode, L, mw);
-  k_sg_roots<<<(period + 255) / 256, 256, 0, st>>>(scratch, period);
-  const long long total = (long long)t.sets * t.tiles * t.stages * 8192;
-  const unsigned grid = (unsigned)((total + 255) / 256);
-  unsigned char* o = reinterpret_cast<unsigned char*>(out);
-  switch (mode) {
-    case SG_BETA_ANA: k_sg_basis<SG_BETA_ANA><<<grid, 256, 0, st>>>(o, scratch, qw, L, period, t.tiles, t.stages, t.sets, kSgAnaScale, mw); break;
-    case SG_BETA_SYN: k_sg_basis<SG_BETA_SYN><<<grid, 256, 0, st>>>(o, scratch, qw, L, period, t.tiles, t.stages, t.sets, beta_syn_scale(L), mw); break;
-    case SG_ALPHA_ANA: k_sg_basis<SG_ALPHA_ANA><<<grid, 256, 0, st>>>(o, scratch, qw, L, period, t.tiles, t.stages, t.sets, kSgAnaScale, mw); break;
-    default: k_sg_basis<SG_ALPHA_SYN><<<grid, 256, 0, st>>>(o, scratch, qw, L, period, t.tiles, t.stages, t.sets, kSgAlphaSynScale, mw); break;
+// scratch of the build, double2
+size_t sg_build_scratch(int L) { return 16 * (size_t)L; }
+// Tables out[k] (null: not wanted) of a grid of band-limit L, k the modes and 4: mode 0
+// on the DH samples of an MW grid, whose own mode 0 evaluates at the MW samples.
+// qw: quadrature weights q_b.
+cudaError_t sg_build_tables(void* const* out, double2* scratch, const double* qw, int L, bool mw, cudaStream_t st) {
+  SgRoots r;
+  r.n[0] = 8 * L, r.n[1] = 2 * (2 * L - 1), r.n[2] = 2 * L - 1;
+  r.beta64 = scratch;
+  r.beta = reinterpret_cast<uint2*>(scratch + r.n[0]);
+  r.beta_mw = r.beta + r.n[0];
+  r.alpha = r.beta_mw + r.n[1];
+  SgBuilds b;
+  b.n = 0;
+  int blocks = 0;
+  for (int k = 0; k < 5; ++k) {
+    if (!out[k]) continue;
+    const int mode = k == 4 ? 0 : k;
+    const SgTable t = sg_table(mode, L);
+    b.t[b.n++] = SgBuild{reinterpret_cast<unsigned char*>(out[k]), mode, mw && k == 0, t.tiles, t.stages, blocks};
+    blocks += t.sets * t.tiles * t.stages * 4;
   }
+  if (blocks == 0) return cudaSuccess;
+  k_sg_roots<<<(r.n[0] + r.n[1] + r.n[2] + 255) / 256, 256, 0, st>>>(r);
+  k_sg_basis<<<blocks, 256, 0, st>>>(b, r, qw, L, beta_syn_scale(L));
   return cudaGetLastError();
 }
 
