@@ -98,6 +98,23 @@ void gauss_legendre(int Q, std::vector<double>& x, std::vector<double>& w) {
 // of a serving process).
 std::mutex g_setup_mu;
 cudaStream_t g_setup_stream[64] = {};
+// Freed blocks that the pool keeps: up to 16 GiB beside what is in use.  The pool's
+// threshold counts what is in use as well, so it moves with the live tables and
+// workspaces: at a fixed 16 GiB the Delta tables of L = 2048 alone (17.4 GB) were above
+// it, and every plan mapped and unmapped its workspace (1 ms per GB each; create
+// + destroy, L = 723, N = 6 2.46 -> 1.14 ms, L = 2048, N = 8 12.7 -> 2.75).
+constexpr uint64_t kPoolCache = 16ull << 30;
+uint64_t g_pool_live[64] = {};  // bytes of live tables and workspaces
+void pool_live(int dev, int64_t delta) {
+  if (dev < 0 || dev >= 64) return;
+  std::lock_guard<std::mutex> lk(g_setup_mu);
+  g_pool_live[dev] += (uint64_t)delta;
+  cudaMemPool_t pool;
+  if (cudaDeviceGetDefaultMemPool(&pool, dev) == cudaSuccess) {
+    uint64_t thr = kPoolCache + g_pool_live[dev];
+    cudaMemPoolSetAttribute(pool, cudaMemPoolAttrReleaseThreshold, &thr);
+  }
+}
 
 // Kernel attributes (shared-memory limits sized for every plan, L <= 2048)
 // are set once per device and precision under a lock, so that creating a plan
@@ -132,7 +149,7 @@ cudaStream_t setup_stream() {
     ck(cudaStreamCreateWithFlags(&g_setup_stream[dev], cudaStreamNonBlocking));
     cudaMemPool_t pool;
     if (cudaDeviceGetDefaultMemPool(&pool, dev) == cudaSuccess) {
-      uint64_t thr = 16ull << 30;  // keep up to 16 GiB of freed blocks cached
+      uint64_t thr = kPoolCache + g_pool_live[dev];
       cudaMemPoolSetAttribute(pool, cudaMemPoolAttrReleaseThreshold, &thr);
     }
   }
@@ -140,7 +157,15 @@ cudaStream_t setup_stream() {
 }
 template <typename P>
 void amalloc(P** p, size_t bytes, cudaStream_t st) {
-  ck(cudaMallocAsync(reinterpret_cast<void**>(p), bytes, st));
+  cudaError_t e = cudaMallocAsync(reinterpret_cast<void**>(p), bytes, st);
+  if (e == cudaErrorMemoryAllocation) {  // once more without the cached blocks
+    cudaGetLastError();
+    int dev = 0;
+    cudaMemPool_t pool;
+    if (cudaGetDevice(&dev) == cudaSuccess && cudaDeviceGetDefaultMemPool(&pool, dev) == cudaSuccess) cudaMemPoolTrimTo(pool, 0);
+    e = cudaMallocAsync(reinterpret_cast<void**>(p), bytes, st);
+  }
+  ck(e);
 }
 inline void afree(void* p, cudaStream_t st) {
   if (p) cudaFreeAsync(p, st);
@@ -212,6 +237,7 @@ DeltaTab* delta_acquire(int L, cudaStream_t st) {
     throw;
   }
   g_tabs.push_back(t);
+  pool_live(dev, (int64_t)t->bytes);
   return t;
 }
 
@@ -228,7 +254,9 @@ void delta_pair_ensure(DeltaTab* t, cudaStream_t st) {
     throw CudaFail{e};
   }
   t->pair32 = pt;
-  t->bytes += (size_t)pair_table_entries(t->Lmax) * sizeof(float);
+  const size_t bytes = (size_t)pair_table_entries(t->Lmax) * sizeof(float);
+  t->bytes += bytes;
+  pool_live(t->device, (int64_t)bytes);
 }
 
 // The FP64 pair table of the direct contraction (small band-limits only).
@@ -247,6 +275,7 @@ void delta_pair64_ensure(DeltaTab* t, cudaStream_t st) {
   }
   t->pair64 = pt;
   t->bytes += bytes;
+  pool_live(t->device, (int64_t)bytes);
 }
 
 void delta_release(DeltaTab* t) {
@@ -257,6 +286,7 @@ void delta_release(DeltaTab* t) {
     afree(t->raw64, st);
     afree(t->pair32, st);
     afree(t->pair64, st);
+    pool_live(t->device, -(int64_t)t->bytes);
     g_tabs.erase(std::remove(g_tabs.begin(), g_tabs.end(), t), g_tabs.end());
     delete t;
   }
@@ -408,7 +438,10 @@ struct s2dw_plan_s {
       cudaEventSynchronize(last_use);  // only this plan's work, not the device
       cudaEventDestroy(last_use);
     }
-    if (ws) cudaFreeAsync(ws, pst);
+    if (ws) {
+      cudaFreeAsync(ws, pst);
+      pool_live(device, -(int64_t)ws_bytes);
+    }
     own.mem = nullptr;
     if (own_mem) cudaFreeAsync(own_mem, pst);
     if (pst) cudaStreamDestroy(pst);  // releases after the queued frees
@@ -1376,6 +1409,7 @@ void plan_build_typed(s2dw_plan_s* p, const double* kap_d, const double* phi_d, 
   }
   p->ws_bytes = off;
   amalloc(&p->ws, off, st);
+  pool_live(p->device, (int64_t)off);
   char* b = reinterpret_cast<char*>(p->ws);
   p->RS = pairt ? nullptr : b + o_RS;
   p->RSphi = pairt ? nullptr : b + o_RSphi;
