@@ -512,44 +512,28 @@ __device__ __forceinline__ void put_split(float* hi, float* lo, int o, double v)
   lo[o] = tc::to_tf32((float)(v - (double)h));
 }
 
-__global__ void k_tc_basis_ana(float* out, int n, int Lj) {
-  const int K8 = ana_k8(Lj), img = tc::img_floats(kTcA, K8);
-  const int ntile = (n + kTcA - 1) / kTcA;
-  const long long total = (long long)ntile * kTcA * K8;
-  for (long long idx = blockIdx.x * (long long)blockDim.x + threadIdx.x; idx < total;
-       idx += (long long)gridDim.x * blockDim.x) {
-    const int tile = (int)(idx / (kTcA * K8)), r = (int)(idx / K8 % kTcA), k = (int)(idx % K8);
-    const int a = tile * kTcA + r, m = k >> 1;
+struct TcBasisJobs {
+  TcBasis t[2 * MAXS];
+};
+// blockIdx.y: table
+__global__ void __launch_bounds__(256) k_tc_basis(TcBasisJobs jobs) {
+  const TcBasis& b = jobs.t[blockIdx.y];
+  const int n = 2 * b.L - 1, Lj = b.Lj, RC = b.syn ? syn_npad(Lj) : kTcA, KC = b.syn ? kTcKc : ana_k8(Lj);
+  const int img = tc::img_floats(RC, KC), ntile = (n + (b.syn ? kTcKc : kTcA) - 1) / (b.syn ? kTcKc : kTcA);
+  const long long total = (long long)ntile * RC * KC;
+  for (long long idx = blockIdx.x * 256ll + threadIdx.x; idx < total; idx += gridDim.x * 256ll) {
+    const int tile = (int)(idx / (RC * KC)), r = (int)(idx / KC % RC), k = (int)(idx % KC);
+    const int a = b.syn ? tile * kTcKc + k : tile * kTcA + r, q = b.syn ? r : k, m = q >> 1;
     double v = 0.0;
-    if (a < n && k < 2 * Lj) {
+    if (a < n && q < 2 * Lj) {
       const long long u = ((long long)m * a) % n;
       double sn, cs;
       sincospi(2.0 * (double)u / (double)n, &sn, &cs);
-      const double cm = m == 0 ? 1.0 : 2.0;
-      v = (k & 1) ? -cm * sn : cm * cs;
+      const double c = b.syn ? 2.0 * 3.14159265358979323846 / n : (m == 0 ? 1.0 : 2.0);
+      v = (q & 1) ? -c * sn : c * cs;
     }
-    float* hi = out + (size_t)tile * 2 * img;
-    put_split(hi, hi + img, tc::img_off(r, k, K8), v);
-  }
-}
-
-__global__ void k_tc_basis_syn(float* out, int n, int Lj, double scale) {
-  const int NP = syn_npad(Lj), img = tc::img_floats(NP, kTcKc);
-  const int nchunk = (n + kTcKc - 1) / kTcKc;
-  const long long total = (long long)nchunk * NP * kTcKc;
-  for (long long idx = blockIdx.x * (long long)blockDim.x + threadIdx.x; idx < total;
-       idx += (long long)gridDim.x * blockDim.x) {
-    const int c = (int)(idx / (NP * kTcKc)), j = (int)(idx / kTcKc % NP), k = (int)(idx % kTcKc);
-    const int a = c * kTcKc + k, m = j >> 1;
-    double v = 0.0;
-    if (a < n && j < 2 * Lj) {
-      const long long u = ((long long)m * a) % n;
-      double sn, cs;
-      sincospi(2.0 * (double)u / (double)n, &sn, &cs);
-      v = (j & 1) ? -scale * sn : scale * cs;
-    }
-    float* hi = out + (size_t)c * 2 * img;
-    put_split(hi, hi + img, tc::img_off(j, k, kTcKc), v);
+    float* hi = b.out + (size_t)tile * 2 * img;
+    put_split(hi, hi + img, tc::img_off(r, k, KC), v);
   }
 }
 
@@ -578,16 +562,13 @@ size_t alpha_tc_table_floats(int L, int Lj, bool syn) {
   return (size_t)((n + kTcKc - 1) / kTcKc) * 2 * tc::img_floats(syn_npad(Lj), kTcKc);
 }
 
-cudaError_t alpha_tc_build_table(float* out, int L, int Lj, bool syn, cudaStream_t st) {
-  const size_t nf = alpha_tc_table_floats(L, Lj, syn);
-  if (nf == 0) return cudaSuccess;
-  cudaError_t e = cudaMemsetAsync(out, 0, nf * sizeof(float), st);  // image pads
-  if (e != cudaSuccess) return e;
-  const int n = 2 * L - 1;
-  if (syn)
-    k_tc_basis_syn<<<256, 256, 0, st>>>(out, n, Lj, 2.0 * 3.14159265358979323846 / n);
-  else
-    k_tc_basis_ana<<<256, 256, 0, st>>>(out, n, Lj);
+// All basis tables of a plan in one launch (a memset and a launch each: 28 in a
+// plan of L = 32; their pads are zeroed by the caller).
+cudaError_t alpha_tc_build_tables(const TcBasis* tables, int n, cudaStream_t st) {
+  if (n <= 0) return cudaSuccess;
+  TcBasisJobs jobs;
+  for (int i = 0; i < n; ++i) jobs.t[i] = tables[i];
+  k_tc_basis<<<dim3(128, n), 256, 0, st>>>(jobs);
   return cudaGetLastError();
 }
 

@@ -1449,16 +1449,20 @@ void plan_build_typed(s2dw_plan_s* p, const double* kap_d, const double* phi_d, 
   p->sg_data = sgd_bytes > 0 ? p->P : nullptr;
   p->tc_ana.assign(p->nscale + 1, nullptr);
   p->tc_syn.assign(p->nscale + 1, nullptr);
+  std::vector<TcBasis> tcb;
   for (int j = 0; j <= p->nscale; ++j) {
     const int Lj = p->Ycols[j], Lg = p->gt[p->grid_of[j]].L;
-    if (o_ta[j] != SIZE_MAX) {
-      p->tc_ana[j] = b + o_ta[j];
-      ck(alpha_tc_build_table(reinterpret_cast<float*>(p->tc_ana[j]), Lg, Lj, false, st));
+    for (int d = 0; d < 2; ++d) {
+      const size_t o = d ? o_ts[j] : o_ta[j];
+      if (o == SIZE_MAX) continue;
+      (d ? p->tc_syn : p->tc_ana)[j] = b + o;
+      tcb.push_back(TcBasis{reinterpret_cast<float*>(b + o), Lg, (short)Lj, (short)d});
     }
-    if (o_ts[j] != SIZE_MAX) {
-      p->tc_syn[j] = b + o_ts[j];
-      ck(alpha_tc_build_table(reinterpret_cast<float*>(p->tc_syn[j]), Lg, Lj, true, st));
-    }
+  }
+  if (!tcb.empty()) {  // (the last part of the workspace)
+    char* first = reinterpret_cast<char*>(tcb[0].out);
+    ck(cudaMemsetAsync(first, 0, b + off - first, st));  // image pads
+    ck(alpha_tc_build_tables(tcb.data(), (int)tcb.size(), st));
   }
 
   // ---- R tables ----

@@ -193,7 +193,12 @@ struct CztSeg {
 // Direct alpha sums on the tensor cores (FP32 plans, scales with L_j <= 32;
 // alpha_tc.cu).  Basis tables: one per scale and direction, built per plan.
 size_t alpha_tc_table_floats(int L, int Lj, bool syn);
-cudaError_t alpha_tc_build_table(float* out, int L, int Lj, bool syn, cudaStream_t st);
+struct TcBasis {
+  float* out;
+  int L;
+  short Lj, syn;
+};
+cudaError_t alpha_tc_build_tables(const TcBasis* tables, int n, cudaStream_t st);  // n <= 2 MAXS
 int alpha_tc_items(int L, int rows, int njobs, bool syn, int& P);  // CTAs; P: rows per CTA
 void launch_alpha_tc(bool syn, const CztSeg<float>* segs, int nseg, int total_items, const CallPtrs& ptrs,
                      cudaStream_t st, long long limit = kWaitLimit);

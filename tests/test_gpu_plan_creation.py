@@ -1,5 +1,6 @@
 """What creating a plan costs on the device: the basis tables of the matrix
-products of a grid are built in two launches, whatever number of tables, and a
+products of a grid are built in two launches, those of the direct alpha sums in
+one, whatever number of tables, and a
 closed plan's workspace stays with the library for the next one (mapping it anew
 costs 1 ms per GB) also beside the largest shared tables."""
 import pytest
@@ -18,6 +19,7 @@ def test_basis_tables_take_two_launches(L, N, kw):
     if not names:
         pytest.skip("profiler recorded no CUDA kernels")
     assert len([n for n in names if "k_sg_" in n]) == 2, names
+    assert len([n for n in names if "k_tc_basis" in n]) == 1, names
 
 
 def test_workspace_stays_mapped_beside_the_largest_tables():
