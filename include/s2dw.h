@@ -100,6 +100,14 @@ typedef struct s2dw_plan_s* s2dw_plan_t;
  */
 int s2dw_plan(s2dw_plan_t* out, int L, int N, double lambda, int J0, unsigned flags);
 
+/*
+ * s2dw_plan_bytes: an upper bound of the workspace_bytes (s2dw_query) of a plan with
+ * these arguments, without creating it (admission of requests by footprint): the
+ * workspace layout for the kernels' analytic supports.  Host only, no CUDA call;
+ * status as s2dw_plan, S2DW_EINVAL for bytes == NULL.
+ */
+int s2dw_plan_bytes(int L, int N, double lambda, int J0, unsigned flags, int64_t* bytes);
+
 /* Release a plan (NULL is accepted).  Waits only for this plan's last
  * recorded call (not the whole device), then frees its workspace.  Calls
  * captured into a CUDA graph are not tracked: destroy a plan only once no

@@ -28,6 +28,7 @@ _c_dp = ctypes.POINTER(ctypes.c_double)
 
 _SIGNATURES = {
     "s2dw_plan": (_c_i, [ctypes.POINTER(_c_p), _c_i, _c_i, ctypes.c_double, _c_i, ctypes.c_uint]),
+    "s2dw_plan_bytes": (_c_i, [_c_i, _c_i, ctypes.c_double, _c_i, ctypes.c_uint, _c_i64p]),
     "s2dw_plan_destroy": (_c_i, [_c_p]),
     "s2dw_query": (_c_i, [_c_p, _c_ip, _c_i64p, _c_i64p, _c_i64p, _c_i64p]),
     "s2dw_launch_counts": (_c_i, [_c_p, _c_ip, _c_ip]),
@@ -118,6 +119,13 @@ def s2dw_plan(L: int, N: int, lam: float, J0: int, flags: int) -> int:
     h = _c_p()
     _check(lib().s2dw_plan(ctypes.byref(h), L, N, float(lam), J0, flags), "s2dw_plan")
     return h.value
+
+
+def s2dw_plan_bytes(L: int, N: int, lam: float, J0: int, flags: int) -> int:
+    """Upper bound of the workspace bytes of a plan, without creating it (host only)."""
+    b = ctypes.c_int64()
+    _check(lib().s2dw_plan_bytes(L, N, float(lam), J0, flags, ctypes.byref(b)), "s2dw_plan_bytes")
+    return b.value
 
 
 def s2dw_plan_destroy(plan: int) -> None:

@@ -1278,16 +1278,31 @@ void own_lists_build(s2dw_plan_s* p) {
   delete ls;
 }
 
+// Byte offsets of a plan's workspace.
+struct PlanLayout {
+  size_t RS, RSphi, RSp, RSphi_p, fP, P, Pphi, images = 0, bytes = 0;  // images: operand images, in P
+  std::vector<size_t> Y, X, ta, ts;
+  struct GridOff { size_t tw, ca, pb, qb, pS, qS, root, bf, H, pm, tw2; };
+  std::vector<GridOff> grid;
+  struct SegOff { size_t tw, Ha, Hs; };
+  std::vector<SegOff> seg;
+  std::vector<std::array<size_t, 5>> sg;
+};
+
+// Workspace layout and launch methods of a plan whose bands and grids are set.
+// bound: bands are upper bounds (s2dw_plan_bytes), so every table and buffer that
+// bands up to kBandSlack below them could need (kappa underflows within 4e-4 of
+// its support's end).
+constexpr int kBandSlack = 5;
 template <typename T>
-void plan_build_typed(s2dw_plan_s* p, const double* kap_d, const double* phi_d, const double* sabs_d,
-                      const double* q_d, cudaStream_t st) {
+PlanLayout plan_layout(s2dw_plan_s* p, bool bound) {
   const int L = p->L, N = p->N;
-  // ---- workspace layout ----
+  PlanLayout o;
   size_t off = 0;
   auto take = [&](size_t bytes) {
-    const size_t o = off;
+    const size_t at = off;
     off = align256(off + bytes);
-    return o;
+    return at;
   };
   const bool dir64 = sizeof(T) == sizeof(double) && p->direct_w;
   const bool pairc = sizeof(T) == sizeof(float);  // FP32 contraction (pair table)
@@ -1297,46 +1312,56 @@ void plan_build_typed(s2dw_plan_s* p, const double* kap_d, const double* phi_d, 
   p->Lrf = L + kPairPadL;
   const int nbw = (L + 31) / 32, nbp = (p->Lphi + 31) / 32;
   const bool pairt = pairc || dir64;  // R rows in the pair layout
-  const size_t o_RS = pairt ? take(0) : take((size_t)L * 2 * NH * p->Lp * sizeof(T));
-  const size_t o_RSphi = pairt ? take(0) : take((size_t)p->Lphi * p->Lphip * sizeof(T));
-  const size_t o_RSp = pairt ? take((size_t)nbw * p->Lr * 2 * NH * 32 * sizeof(T)) : take(0);
-  const size_t o_RSphi_p = pairt ? take((size_t)nbp * p->Lrphi * 32 * sizeof(T)) : take(0);
+  o.RS = pairt ? take(0) : take((size_t)L * 2 * NH * p->Lp * sizeof(T));
+  o.RSphi = pairt ? take(0) : take((size_t)p->Lphi * p->Lphip * sizeof(T));
+  o.RSp = pairt ? take((size_t)nbw * p->Lr * 2 * NH * 32 * sizeof(T)) : take(0);
+  o.RSphi_p = pairt ? take((size_t)nbp * p->Lrphi * 32 * sizeof(T)) : take(0);
   const bool packf = pairc && !(p->direct_w && p->direct_phi);  // the direct contraction reads f itself
-  const size_t o_fP = packf ? take((size_t)nbw * p->Lrf * 32 * sizeof(cx<T>)) : take(0);
-  std::vector<size_t> o_Y(p->nscale + 1), o_X(p->nscale + 1);
+  o.fP = packf ? take((size_t)nbw * p->Lrf * 32 * sizeof(cx<T>)) : take(0);
+  o.Y.resize(p->nscale + 1);
+  o.X.resize(p->nscale + 1);
   for (int j = 0; j <= p->nscale; ++j) {
     const int Nj = (j == p->nscale) ? 1 : N;
     const int Lj = p->Ycols[j];
-    o_Y[j] = take((size_t)Nj * Lj * Lj * sizeof(cx<T>));
-    o_X[j] = take((size_t)Nj * 2 * p->gt[p->grid_of[j]].L * Lj * sizeof(cx<T>));
+    o.Y[j] = take((size_t)Nj * Lj * Lj * sizeof(cx<T>));
+    o.X[j] = take((size_t)Nj * 2 * p->gt[p->grid_of[j]].L * Lj * sizeof(cx<T>));
   }
-  const size_t o_Pphi = take((size_t)p->nbr_phi * p->Lphi * p->Lphip32 * sizeof(cx<T>));
+  o.Pphi = take((size_t)p->nbr_phi * p->Lphi * p->Lphip32 * sizeof(cx<T>));
   // per grid: twiddles, chirps, roots, beta phases and weights, spectra
-  struct GridOff { size_t tw, ca, pb, qb, pS, qS, root, bf, H, pm, tw2; };
-  std::vector<GridOff> go(p->gt.size());
-  for (size_t g = 0; g < p->gt.size(); ++g) {
-    const int Lg = p->gt[g].L, ng = 2 * Lg - 1, Mg = p->gt[g].M;
-    go[g].tw = take((size_t)Mg * sizeof(cx<T>));
-    go[g].ca = take((size_t)ng * sizeof(cx<T>));
-    go[g].pb = take((size_t)(2 * Lg - 1) * sizeof(cx<T>));
-    go[g].qb = take((size_t)2 * Lg * sizeof(cx<T>));
-    go[g].pS = take((size_t)2 * Lg * sizeof(cx<T>));
-    go[g].qS = take((size_t)(2 * Lg - 1) * sizeof(cx<T>));
-    go[g].root = take((size_t)ng * sizeof(cx<T>));
-    go[g].bf = take((size_t)(4 * Lg - 1) * sizeof(cx<T>));
-    go[g].H = take((size_t)4 * Mg * sizeof(cx<T>));
-    go[g].pm = take((size_t)ng * sizeof(cx<T>));
-    go[g].tw2 = take((size_t)twiddle_entries(p->gt[g].logM - 1) * sizeof(cx<T>));
-  }
+  auto& go = o.grid;
+  go.resize(p->gt.size());
+  // sets of tables of a grid (bound: scales whose bounds share a grid may have their own)
+  auto sets = [&](size_t g) {
+    return bound && p->multires ? (int)std::count(p->grid_of.begin(), p->grid_of.end(), (int)g) : 1;
+  };
+  for (size_t g = 0; g < p->gt.size(); ++g)
+    for (int k = 0; k < sets(g); ++k) {
+      const int Lg = p->gt[g].L, ng = 2 * Lg - 1, Mg = p->gt[g].M;
+      go[g].tw = take((size_t)Mg * sizeof(cx<T>));
+      go[g].ca = take((size_t)ng * sizeof(cx<T>));
+      go[g].pb = take((size_t)(2 * Lg - 1) * sizeof(cx<T>));
+      go[g].qb = take((size_t)2 * Lg * sizeof(cx<T>));
+      go[g].pS = take((size_t)2 * Lg * sizeof(cx<T>));
+      go[g].qS = take((size_t)(2 * Lg - 1) * sizeof(cx<T>));
+      go[g].root = take((size_t)ng * sizeof(cx<T>));
+      go[g].bf = take((size_t)(4 * Lg - 1) * sizeof(cx<T>));
+      go[g].H = take((size_t)4 * Mg * sizeof(cx<T>));
+      go[g].pm = take((size_t)ng * sizeof(cx<T>));
+      go[g].tw2 = take((size_t)twiddle_entries(p->gt[g].logM - 1) * sizeof(cx<T>));
+    }
   // segmented chirp-z tables of the scales that use it (chirp-z bands only)
   p->seg.assign(p->nscale + 1, s2dw_plan_s::SegTables());
-  struct SegOff { size_t tw, Ha, Hs; };
-  std::vector<SegOff> so(p->nscale + 1);
+  auto& so = o.seg;
+  so.resize(p->nscale + 1);
   for (int j = 0; j <= p->nscale; ++j) {
     const auto& G = p->gt[p->grid_of[j]];
     const int Lj = p->Ycols[j];
     if (Lj <= kDirectMaxLj) continue;  // direct sums
     auto& sgt = p->seg[j];
+    if (bound) {  // any choice: twiddles and two times S M' <= 1.7 M log2 M / 9 entries
+      take((size_t)8 * G.M * sizeof(cx<T>));
+      continue;
+    }
     seg_choice(G.L, Lj, G.logM, sgt.logM, sgt.P, sgt.S);
     if (sgt.S == 0) continue;
     const size_t Ms = (size_t)1 << sgt.logM;
@@ -1354,19 +1379,25 @@ void plan_build_typed(s2dw_plan_s* p, const double* kap_d, const double* phi_d, 
       if (Lj <= (d == 0 ? kDirectMaxLjAna : kDirectMaxLj)) p->alpha_mode[d][j] = 0;
       else if (p->seg[j].S > 0) p->alpha_mode[d][j] = 2;
       const auto& G = p->gt[p->grid_of[j]];
-      const auto& sgt = p->seg[j];
-      const double cost = sgt.S > 0 ? (double)(sgt.S + 1) * ((size_t)1 << sgt.logM) * sgt.logM : 2.0 * G.M * G.logM;
-      p->alpha_sg[d][j] = pairc && p->alpha_mode[d][j] != 0 && sg_alpha_faster(G.L, Lj, cost, sgt.S > 0);
+      // (bound: for any band up to kBandSlack below)
+      for (int b = Lj; pairc && p->alpha_mode[d][j] != 0 && b >= Lj - (bound ? kBandSlack : 0); --b) {
+        int lm, P, S;
+        seg_choice(G.L, b, G.logM, lm, P, S);
+        const double cost = S > 0 ? (double)(S + 1) * ((size_t)1 << lm) * lm : 2.0 * G.M * G.logM;
+        if (sg_alpha_faster(G.L, b, cost, S > 0)) p->alpha_sg[d][j] = 1;
+      }
       if (p->alpha_sg[d][j]) p->alpha_mode[d][j] = 3;
     }
   }
   // basis tables of the split products
-  std::vector<std::array<size_t, 5>> o_sg(p->gt.size());
+  auto& o_sg = o.sg;
+  o_sg.resize(p->gt.size());
   for (size_t g = 0; g < p->gt.size(); ++g) {
     auto& G = p->gt[g];
     o_sg[g].fill(SIZE_MAX);
     if (!pairc) continue;
-    const bool pow2 = 4 * G.L == G.M;
+    // (the bound of a scale's own grid may be a power of two where the grid is none)
+    const bool pow2 = !(bound && p->multires) && 4 * G.L == G.M;
     // (an MW analysis evaluates at the MW samples, whatever L)
     G.sg_beta[0] = sg_beta_faster(G.L, pow2 && !p->mw);
     G.sg_beta[1] = sg_beta_faster(G.L, pow2);
@@ -1375,12 +1406,12 @@ void plan_build_typed(s2dw_plan_s* p, const double* kap_d, const double* phi_d, 
       if (p->grid_of[j] == (int)g)
         for (int d = 0; d < 2; ++d) need[2 + d] = need[2 + d] || p->alpha_sg[d][j];
     for (int k = 0; k < 5; ++k)
-      if (need[k]) o_sg[g][k] = take(sg_table(k == 4 ? 0 : k, G.L).bytes);
+      if (need[k]) o_sg[g][k] = take(sets(g) * sg_table(k == 4 ? 0 : k, G.L).bytes);
   }
   // operand images of one product launch (shared by the five kinds), in the
   // buffer of the synthesis partials: the contraction that writes those comes
   // after every product launch of its call
-  size_t sgd_bytes = 0;
+  size_t& sgd_bytes = o.images;
   if (pairc) {
     size_t most = 0;
     for (int k = 0; k < 5; ++k) {
@@ -1396,67 +1427,85 @@ void plan_build_typed(s2dw_plan_s* p, const double* kap_d, const double* phi_d, 
     }
     sgd_bytes = most * kSgDataBytes;
   }
-  const size_t o_P = take(std::max((size_t)p->nbr * L * p->Lp32 * sizeof(cx<T>), sgd_bytes));
+  o.P = take(std::max((size_t)p->nbr * L * p->Lp32 * sizeof(cx<T>), sgd_bytes));
   // tensor-core basis images of the direct alpha sums (FP32 plans)
-  std::vector<size_t> o_ta(p->nscale + 1, SIZE_MAX), o_ts(p->nscale + 1, SIZE_MAX);
+  auto &o_ta = o.ta, &o_ts = o.ts;
+  o_ta.assign(p->nscale + 1, SIZE_MAX);
+  o_ts.assign(p->nscale + 1, SIZE_MAX);
   if (sizeof(T) == sizeof(float)) {
     for (int j = 0; j <= p->nscale; ++j) {
-      const int Lj = p->Ycols[j], Lg = p->gt[p->grid_of[j]].L;
+      int Lj = p->Ycols[j];
+      const int Lg = p->gt[p->grid_of[j]].L;
       if (Lj <= 0) continue;
+      if (bound && Lj <= kDirectMaxLj + kBandSlack) Lj = std::min(Lj, kDirectMaxLj);
       if (Lj <= kDirectMaxLjAna) o_ta[j] = take(alpha_tc_table_floats(Lg, Lj, false) * sizeof(float));
       if (Lj <= kDirectMaxLj) o_ts[j] = take(alpha_tc_table_floats(Lg, Lj, true) * sizeof(float));
     }
   }
+  o.bytes = off;
+  return o;
+}
+
+template <typename T>
+void plan_build_typed(s2dw_plan_s* p, const double* kap_d, const double* phi_d, const double* sabs_d,
+                      const double* q_d, cudaStream_t st) {
+  const int L = p->L, N = p->N;
+  const bool dir64 = sizeof(T) == sizeof(double) && p->direct_w;
+  const bool pairc = sizeof(T) == sizeof(float);  // FP32 contraction (pair table)
+  const bool pairt = pairc || dir64;              // R rows in the pair layout
+  const bool packf = pairc && !(p->direct_w && p->direct_phi);
+  const PlanLayout o = plan_layout<T>(p, false);
+  const size_t off = o.bytes;
   p->ws_bytes = off;
   amalloc(&p->ws, off, st);
   pool_live(p->device, (int64_t)off);
   char* b = reinterpret_cast<char*>(p->ws);
-  p->RS = pairt ? nullptr : b + o_RS;
-  p->RSphi = pairt ? nullptr : b + o_RSphi;
-  p->RSp = pairt ? b + o_RSp : nullptr;
-  p->RSphi_p = pairt ? b + o_RSphi_p : nullptr;
-  p->fP = packf ? b + o_fP : nullptr;
+  p->RS = pairt ? nullptr : b + o.RS;
+  p->RSphi = pairt ? nullptr : b + o.RSphi;
+  p->RSp = pairt ? b + o.RSp : nullptr;
+  p->RSphi_p = pairt ? b + o.RSphi_p : nullptr;
+  p->fP = packf ? b + o.fP : nullptr;
   p->Y.resize(p->nscale + 1);
   p->X.resize(p->nscale + 1);
   for (int j = 0; j <= p->nscale; ++j) {
-    p->Y[j] = b + o_Y[j];
-    p->X[j] = b + o_X[j];
+    p->Y[j] = b + o.Y[j];
+    p->X[j] = b + o.X[j];
   }
-  p->P = b + o_P;
-  p->Pphi = b + o_Pphi;
+  p->P = b + o.P;
+  p->Pphi = b + o.Pphi;
   for (size_t g = 0; g < p->gt.size(); ++g) {
     auto& G = p->gt[g];
-    G.tw = b + go[g].tw;
-    G.chirp_a = b + go[g].ca;
-    G.pre_b = b + go[g].pb;
-    G.post_b = b + go[g].qb;
-    G.preS_b = b + go[g].pS;
-    G.postS_b = b + go[g].qS;
-    G.root_a = b + go[g].root;
-    G.bfft = b + go[g].bf;
-    G.Hs = b + go[g].H;
-    G.pre_mw = b + go[g].pm;
-    G.tw2 = b + go[g].tw2;
-    for (int k = 0; k < 5; ++k) G.sg[k] = o_sg[g][k] != SIZE_MAX ? b + o_sg[g][k] : nullptr;
+    G.tw = b + o.grid[g].tw;
+    G.chirp_a = b + o.grid[g].ca;
+    G.pre_b = b + o.grid[g].pb;
+    G.post_b = b + o.grid[g].qb;
+    G.preS_b = b + o.grid[g].pS;
+    G.postS_b = b + o.grid[g].qS;
+    G.root_a = b + o.grid[g].root;
+    G.bfft = b + o.grid[g].bf;
+    G.Hs = b + o.grid[g].H;
+    G.pre_mw = b + o.grid[g].pm;
+    G.tw2 = b + o.grid[g].tw2;
+    for (int k = 0; k < 5; ++k) G.sg[k] = o.sg[g][k] != SIZE_MAX ? b + o.sg[g][k] : nullptr;
   }
   for (int j = 0; j <= p->nscale; ++j) {
     auto& sgt = p->seg[j];
     if (sgt.S == 0) continue;
-    sgt.tw = b + so[j].tw;
-    sgt.Ha = b + so[j].Ha;
-    sgt.Hs = b + so[j].Hs;
+    sgt.tw = b + o.seg[j].tw;
+    sgt.Ha = b + o.seg[j].Ha;
+    sgt.Hs = b + o.seg[j].Hs;
   }
-  p->sg_data = sgd_bytes > 0 ? p->P : nullptr;
+  p->sg_data = o.images > 0 ? p->P : nullptr;
   p->tc_ana.assign(p->nscale + 1, nullptr);
   p->tc_syn.assign(p->nscale + 1, nullptr);
   std::vector<TcBasis> tcb;
   for (int j = 0; j <= p->nscale; ++j) {
     const int Lj = p->Ycols[j], Lg = p->gt[p->grid_of[j]].L;
     for (int d = 0; d < 2; ++d) {
-      const size_t o = d ? o_ts[j] : o_ta[j];
-      if (o == SIZE_MAX) continue;
-      (d ? p->tc_syn : p->tc_ana)[j] = b + o;
-      tcb.push_back(TcBasis{reinterpret_cast<float*>(b + o), Lg, (short)Lj, (short)d});
+      const size_t at = d ? o.ts[j] : o.ta[j];
+      if (at == SIZE_MAX) continue;
+      (d ? p->tc_syn : p->tc_ana)[j] = b + at;
+      tcb.push_back(TcBasis{reinterpret_cast<float*>(b + at), Lg, (short)Lj, (short)d});
     }
   }
   if (!tcb.empty()) {  // (the last part of the workspace)
@@ -1604,6 +1653,63 @@ void plan_build_typed(s2dw_plan_s* p, const double* kap_d, const double* phi_d, 
   kernels_prepare(sizeof(T) == sizeof(double), false);
 }
 
+// Sizes, kernels and grids that follow from the bands (p->Lj, L0, lphi).
+void plan_shape(s2dw_plan_s* p) {
+  const int L = p->L, N = p->N;
+  const unsigned flags = p->flags;
+  p->Lphi = p->lphi + 1;
+  p->Ycols = p->Lj;
+  p->Ycols.push_back(p->Lphi);
+  p->Lp = round_up(L, 32);  // R-table row pitch: whole 32-row tiles are staged
+  p->Lp32 = round_up(L, 32);
+  p->Lphip = round_up(p->Lphi, 32);
+  p->Lphip32 = round_up(p->Lphi, 32);
+  if (p->fp64) {
+    p->direct_w = p->direct_phi = L <= kContractDirectMaxL64;
+  } else {
+    p->direct_w = p->L0 <= contract_direct_max_l(N);
+    p->direct_phi = p->Lphi <= contract_direct_max_l(1);
+  }
+  // blocks of partials: TMP rows each; the direct contraction writes whole 32-row tiles
+  const int rows = p->direct_w ? 32 : p->TMP, rows_phi = p->direct_phi ? 32 : p->TMP;
+  p->nbr = (p->L0 + rows - 1) / rows * (rows / p->TMP);
+  p->nbr_phi = (p->Lphi + rows_phi - 1) / rows_phi * (rows_phi / p->TMP);
+  // sampling grid of every scale (last: the scaling part): the full grid of
+  // band-limit L, or with S2DW_MULTIRES the grid of the scale's own
+  // band-limit (1 + the last l with a nonzero kernel)
+  p->multires = (flags & S2DW_MULTIRES) != 0;
+  p->mw = (flags & S2DW_MW) != 0;
+  if (p->mw && p->multires) throw CudaFail{cudaErrorInvalidValue};
+  std::vector<int> Lg(p->nscale + 1);
+  for (int j = 0; j < p->nscale; ++j) Lg[j] = p->multires ? std::max(1, p->Lj[j]) : L;
+  Lg[p->nscale] = p->multires ? p->Lphi : L;
+  std::vector<int> uniq(Lg);
+  std::sort(uniq.begin(), uniq.end());
+  uniq.erase(std::unique(uniq.begin(), uniq.end()), uniq.end());
+  p->gt.resize(uniq.size());
+  p->logM = 0;
+  for (size_t g = 0; g < uniq.size(); ++g) {
+    auto& G = p->gt[g];
+    G.L = uniq[g];
+    G.logM = 5;  // the radix-16 convolution engine needs M >= 32
+    while ((1 << G.logM) < 4 * G.L - 2) ++G.logM;
+    G.M = 1 << G.logM;
+    G.nb = p->mw ? G.L : 2 * G.L;
+    p->logM = std::max(p->logM, G.logM);
+  }
+  p->M = 1 << p->logM;
+  p->grid_of.resize(p->nscale + 1);
+  for (int j = 0; j <= p->nscale; ++j)
+    p->grid_of[j] = (int)(std::lower_bound(uniq.begin(), uniq.end(), Lg[j]) - uniq.begin());
+  p->woff.resize(p->nscale + 1);
+  int64_t wacc = 0;
+  for (int j = 0; j < p->nscale; ++j) {
+    p->woff[j] = wacc;
+    wacc += (int64_t)N * p->gt[p->grid_of[j]].nb * (2 * Lg[j] - 1);
+  }
+  p->woff[p->nscale] = wacc;
+}
+
 // sht_mode: the companion plan of s2dw_sht_*: no wavelet scales, N = 1 and
 // Phi_l = sqrt((2l+1)/(4 pi)) for every l < L, so that its scaling part is
 // the spherical harmonic transform pair on the DH sphere grid.
@@ -1688,57 +1794,7 @@ int plan_create(s2dw_plan_t* out, int L, int N, double lam, int J0, unsigned fla
     p->lphi = 0;
     for (int l = 0; l < L; ++l)
       if (p->phi_host[l] > 0.0) p->lphi = l;
-    p->Lphi = p->lphi + 1;
-    p->Ycols = p->Lj;
-    p->Ycols.push_back(p->Lphi);
-    p->Lp = round_up(L, 32);  // R-table row pitch: whole 32-row tiles are staged
-    p->Lp32 = round_up(L, 32);
-    p->Lphip = round_up(p->Lphi, 32);
-    p->Lphip32 = round_up(p->Lphi, 32);
-    if (p->fp64) {
-      p->direct_w = p->direct_phi = L <= kContractDirectMaxL64;
-    } else {
-      p->direct_w = p->L0 <= contract_direct_max_l(N);
-      p->direct_phi = p->Lphi <= contract_direct_max_l(1);
-    }
-    // blocks of partials: TMP rows each; the direct contraction writes whole 32-row tiles
-    const int rows = p->direct_w ? 32 : p->TMP, rows_phi = p->direct_phi ? 32 : p->TMP;
-    p->nbr = (p->L0 + rows - 1) / rows * (rows / p->TMP);
-    p->nbr_phi = (p->Lphi + rows_phi - 1) / rows_phi * (rows_phi / p->TMP);
-    // sampling grid of every scale (last: the scaling part): the full grid of
-    // band-limit L, or with S2DW_MULTIRES the grid of the scale's own
-    // band-limit (1 + the last l with a nonzero kernel)
-    p->multires = (flags & S2DW_MULTIRES) != 0;
-    p->mw = (flags & S2DW_MW) != 0;
-    if (p->mw && p->multires) throw CudaFail{cudaErrorInvalidValue};
-    std::vector<int> Lg(p->nscale + 1);
-    for (int j = 0; j < p->nscale; ++j) Lg[j] = p->multires ? std::max(1, p->Lj[j]) : L;
-    Lg[p->nscale] = p->multires ? p->Lphi : L;
-    std::vector<int> uniq(Lg);
-    std::sort(uniq.begin(), uniq.end());
-    uniq.erase(std::unique(uniq.begin(), uniq.end()), uniq.end());
-    p->gt.resize(uniq.size());
-    p->logM = 0;
-    for (size_t g = 0; g < uniq.size(); ++g) {
-      auto& G = p->gt[g];
-      G.L = uniq[g];
-      G.logM = 5;  // the radix-16 convolution engine needs M >= 32
-      while ((1 << G.logM) < 4 * G.L - 2) ++G.logM;
-      G.M = 1 << G.logM;
-      G.nb = p->mw ? G.L : 2 * G.L;
-      p->logM = std::max(p->logM, G.logM);
-    }
-    p->M = 1 << p->logM;
-    p->grid_of.resize(p->nscale + 1);
-    for (int j = 0; j <= p->nscale; ++j)
-      p->grid_of[j] = (int)(std::lower_bound(uniq.begin(), uniq.end(), Lg[j]) - uniq.begin());
-    p->woff.resize(p->nscale + 1);
-    int64_t wacc = 0;
-    for (int j = 0; j < p->nscale; ++j) {
-      p->woff[j] = wacc;
-      wacc += (int64_t)N * p->gt[p->grid_of[j]].nb * (2 * Lg[j] - 1);
-    }
-    p->woff[p->nscale] = wacc;
+    plan_shape(p);
     p->tab = delta_acquire(L, st);
     if (p->fp64) plan_build_typed<double>(p, kap, phi, sabs, q, st);
     else plan_build_typed<float>(p, kap, phi, sabs, q, st);
@@ -1766,6 +1822,21 @@ int plan_create(s2dw_plan_t* out, int L, int N, double lam, int J0, unsigned fla
     return rc;
   }
   *out = p;
+  return S2DW_OK;
+}
+
+int plan_args(int L, int N, double lambda, int J0, unsigned flags) {
+  const unsigned prec = flags & (S2DW_FP64 | S2DW_MIXED);
+  if (prec != S2DW_FP64 && prec != S2DW_MIXED) return S2DW_EINVAL;
+  if (flags & ~(unsigned)(S2DW_FP64 | S2DW_MIXED | S2DW_REAL_SIGNAL | S2DW_MULTIRES | S2DW_MW)) return S2DW_EINVAL;
+  if ((flags & S2DW_MW) && (flags & S2DW_MULTIRES)) return S2DW_EINVAL;
+  // invalid requests (no transform exists) before limits of this build
+  if (L < 2 || N < 1 || N > L) return S2DW_EINVAL;
+  if (!(lambda > 1.0) || !std::isfinite(lambda)) return S2DW_EINVAL;
+  const int jm = jmax_of(L, lambda);
+  if (jm < 0) return S2DW_ENOTSUP;  // over a million scales
+  if (J0 < 0 || J0 > jm) return S2DW_EINVAL;
+  if (L > 2048 || N > 8) return S2DW_ENOTSUP;
   return S2DW_OK;
 }
 
@@ -1798,22 +1869,43 @@ const char* s2dw_strerror(int status) {
 int s2dw_plan(s2dw_plan_t* out, int L, int N, double lambda, int J0, unsigned flags) {
   if (!out) return S2DW_EINVAL;
   *out = nullptr;
-  const unsigned prec = flags & (S2DW_FP64 | S2DW_MIXED);
-  if (prec != S2DW_FP64 && prec != S2DW_MIXED) return S2DW_EINVAL;
-  if (flags & ~(unsigned)(S2DW_FP64 | S2DW_MIXED | S2DW_REAL_SIGNAL | S2DW_MULTIRES | S2DW_MW)) return S2DW_EINVAL;
-  if ((flags & S2DW_MW) && (flags & S2DW_MULTIRES)) return S2DW_EINVAL;
-  // invalid requests (no transform exists) before limits of this build
-  if (L < 2 || N < 1 || N > L) return S2DW_EINVAL;
-  if (!(lambda > 1.0) || !std::isfinite(lambda)) return S2DW_EINVAL;
-  const int jm = jmax_of(L, lambda);
-  if (jm < 0) return S2DW_ENOTSUP;  // over a million scales
-  if (J0 < 0 || J0 > jm) return S2DW_EINVAL;
-  if (L > 2048 || N > 8) return S2DW_ENOTSUP;
+  if (int rc = plan_args(L, N, lambda, J0, flags); rc != S2DW_OK) return rc;
   try {
     return plan_create(out, L, N, lambda, J0, flags);
   } catch (...) {
     return S2DW_ECUDA;
   }
+}
+
+int s2dw_plan_bytes(int L, int N, double lambda, int J0, unsigned flags, int64_t* bytes) {
+  if (!bytes) return S2DW_EINVAL;
+  if (int rc = plan_args(L, N, lambda, J0, flags); rc != S2DW_OK) return rc;
+  try {
+    s2dw_plan_s p;
+    p.L = L, p.N = N, p.J0 = J0, p.lam = lambda, p.flags = flags | S2DW_REAL_SIGNAL;
+    p.J = jmax_of(L, lambda) - J0;
+    p.nscale = p.J + 1;
+    if (p.nscale > 64) return S2DW_ENOTSUP;
+    p.fp64 = (flags & S2DW_FP64) != 0;
+    p.E = contract_rows_per_thread(p.fp64);
+    p.TMP = 8 * p.E;
+    // kappa^j is supported in L lambda^-(j+1) < l < L lambda^(1-j), Phi in l < L lambda^-J
+    // (one more where the power is rounded)
+    auto band = [&](int e) { return (int)std::min<double>(L, std::floor(L * std::pow(lambda, e)) + 2); };
+    p.lo.assign(p.nscale, -1);
+    p.hi.assign(p.nscale, -1);
+    p.Lj.assign(p.nscale, 0);
+    for (int j = 0; j < p.nscale; ++j) {
+      p.Lj[j] = band(1 - j);
+      p.L0 = std::max(p.L0, p.Lj[j]);
+    }
+    p.lphi = band(-p.J) - 1;
+    plan_shape(&p);
+    *bytes = (int64_t)(p.fp64 ? plan_layout<double>(&p, true).bytes : plan_layout<float>(&p, true).bytes);
+  } catch (...) {
+    return S2DW_ENOMEM;
+  }
+  return S2DW_OK;
 }
 
 int s2dw_plan_destroy(s2dw_plan_t plan) {

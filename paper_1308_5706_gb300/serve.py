@@ -30,6 +30,7 @@ from __future__ import annotations
 import collections
 import concurrent.futures
 import dataclasses
+import functools
 import math
 import time
 from typing import Dict, List, Optional
@@ -330,7 +331,11 @@ def B_jmax(L: int, lam: float) -> int:
     return J
 
 
+@functools.lru_cache(maxsize=65536)
+def _plan_bytes(L: int, N: int, lam: float, J0: int, flags: int) -> int:
+    return B.s2dw_plan_bytes(L, N, lam, J0, flags)
+
+
 def _workspace_estimate(r: Request, el: int) -> int:
-    # conservative: Fourier cubes, beta outputs and synthesis partials of a plan
-    L, N = r.L, r.N
-    return int(2 * (3 * N * L * L + 2 * N * 2 * L * L) * el + (L // 32 + 1) * L * L * 2 * el + 2 * L * N * L * el)
+    """Upper bound of the workspace of a plan for r (el: bytes per real number)."""
+    return _plan_bytes(r.L, r.N, r.lam, r.J0, B.S2DW_MIXED if el == 4 else B.S2DW_FP64)
