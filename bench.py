@@ -319,8 +319,9 @@ def recorded_traffic(stage: str):
 
 
 def roofline(pm, mean_stage, ms_per_step):
-    """Roofline of every timed launch and of the dominant one (largest mean
-    duration), from the live CUDA-event durations; and the round trip against
+    """Roofline of every timed stage and of the dominant one (largest mean
+    duration), from the live CUDA-event durations (a stage is one launch or a few:
+    f packing and contraction, conversion and products, products and chirp-z); and the round trip against
     the sum of the stage roofs: per direction the
     contraction at max(Delta bytes / HBM, 2+4N flops per triple / FP32 peak)
     and the FFT passes at (W + f bytes) / HBM."""
@@ -352,10 +353,10 @@ def roofline(pm, mean_stage, ms_per_step):
             a = w / (ms * 1e-3) / 1e9
             per[k] = {"bound": "hbm", "ms": round(ms, 4), "achieved": a, "peak": hbm, "unit": "GB/s",
                       "frac": a / hbm}
-    # the longest single launch: the contraction (the czt+seg group is two to four launches)
-    dom = max((k for k in per if not k.endswith("czt+seg")), key=lambda k: per[k]["ms"], default=max(per))
+    dom = max(per, key=lambda k: per[k]["ms"])
     r = dict(per[dom])
     r["kernel"] = dom
+    r["timed"] = "stage"
     r["traffic"], r["traffic_source"] = recorded_traffic(dom)
     r["peak_source"] = alu_src if r["bound"] == "alu" else f"hbm_gbs of {peak_src} peaks"
     r["work_per_launch"] = work[dom][1]
@@ -886,7 +887,7 @@ def main():
                    "grid": "full-resolution DH SO(3) grid per scale: 5 x 2048 x 2047",
                    "parallelism": f"replicas x{world}",
                    "launch_methods": {"choices": pm.tuned[0], "source": pm.tuned[1],
-                                      "layout": "beta ana, beta syn, alpha ana / syn per scale, then the contraction CTA shape (s2dw.h)"},
+                                      "layout": "beta ana, beta syn, alpha ana / syn per scale, then a value kept for saved choices (s2dw.h)"},
                    "l2": "inputs larger than L2 (W 0.92 GB, Delta pair table 0.78 GB per direction)"},
         "latency_ms": {"p50": per_sorted[len(per) // 2],
                        "p99": per_sorted[min(len(per) - 1, int(round(0.99 * (len(per) - 1))))]},
