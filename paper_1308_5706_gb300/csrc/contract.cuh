@@ -151,7 +151,7 @@ __host__ __device__ constexpr size_t contract_smem_bytes() {
   return contract_stages<T, N, NSLOT, SYN, E>() * StageGeom<T, N, NSLOT, E>::BYTES + contract_red_bytes<T, SYN>();
 }
 
-// Two CTAs per SM (128 registers) where the accumulators allow it (FP32, N <= 5).
+// (256, 1): the FP64 accumulators need more than the 128 registers of two CTAs per SM.
 template <typename T, int N, int NSLOT, bool SYN, int E>
 __global__ void __launch_bounds__(256, 1)
 k_contract(const ContractDesc<T>* __restrict__ descs, const TileTask* __restrict__ tiles, CallPtrs ptrs) {

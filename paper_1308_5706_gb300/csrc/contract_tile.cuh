@@ -19,7 +19,7 @@
 // thread that owns 4 rows x 1 column reads 30 words per l for 14 packed FMA
 // pairs of work; one that owns 2 rows x 8 columns reads 44 for 56.  Sixteen
 // elements fit in 255 registers only because a warp handles the l of one
-// parity: the sums over even and odd l of an order pair +-n are separate banks
+// parity (N = 5 and 6 spill 12 to 24 bytes): the sums over even and odd l of an order pair +-n are separate banks
 // (R_{l m' -n} = (-1)^{l+m'} R_{l m' n}), and here the two banks live in
 // different warps, which exchange halves through shared memory at the end
 // (analysis) or fold H for their parity at the start (synthesis).

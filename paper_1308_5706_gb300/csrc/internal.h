@@ -152,9 +152,9 @@ constexpr int kDirectMaxLj = 32;     // synthesis: direct alpha sums for L_j <= 
 constexpr int kDirectMaxLjAna = 32;  // analysis: direct (matrix-product) alpha sums for L_j <= 32
 // tile of the direct analysis kernel: samples per CTA, rows per pass, fewest rows per CTA
 constexpr int kAgCols = 128, kAgRows = 64, kAgMinRows = 16;
-template <typename T>  // B tile + A tile (FP32 stores each A value twice)
+template <typename T>  // B tile + A tile
 constexpr size_t alpha_ana_direct_smem() {
-  return (size_t)(2 * kDirectMaxLjAna - 1) * (kAgCols + kAgRows * (sizeof(T) == 4 ? 2 : 1)) * sizeof(T);
+  return (size_t)(2 * kDirectMaxLjAna - 1) * (kAgCols + kAgRows) * sizeof(T);
 }
 // row pairs (complex transforms) per CTA of the alpha chirp-z kernels: one
 // (FP32 measured 9% faster at three CTAs per SM than two transforms per CTA
