@@ -19,10 +19,11 @@
 // thread that owns 4 rows x 1 column reads 30 words per l for 14 packed FMA
 // pairs of work; one that owns 2 rows x 8 columns reads 44 for 56.  Sixteen
 // elements fit in 255 registers only because a warp handles the l of one
-// parity (N = 5 and 6 spill 12 to 24 bytes): the sums over even and odd l of an order pair +-n are separate banks
-// (R_{l m' -n} = (-1)^{l+m'} R_{l m' n}), and here the two banks live in
-// different warps, which exchange halves through shared memory at the end
-// (analysis) or fold H for their parity at the start (synthesis).
+// parity (N = 5 and 6 spill 12 to 24 bytes per thread all the same): the sums
+// over even and odd l of an order pair +-n are separate banks (R_{l m' -n} =
+// (-1)^{l+m'} R_{l m' n}), and here the two banks live in different warps, which
+// exchange halves through shared memory at the end (analysis) or fold H for
+// their parity at the start (synthesis).
 // Task: in the analysis two adjacent scales (one per slot) over the union of
 // their l ranges, so that no accumulator changes scale on the way; in the
 // synthesis an l range on which each slot holds one scale.  Where only one of
@@ -43,10 +44,10 @@
 //
 // Measured (GB300, ms per call, analysis / synthesis; before: one tile pair per
 // 512-thread CTA, 4 x 1 elements per thread, cp.async ring): L = 1024, N = 5
-// 0.401 / 0.394 -> 0.314 / 0.395, N = 3 0.341 / 0.353 -> 0.246 / 0.283, N = 1
-// 0.245 / 0.283 -> 0.210 / 0.226; L = 723, N = 6 0.229 / 0.240 -> 0.152 / 0.176;
-// L = 2048, N = 8 4.26 / 4.89 -> 2.95 / 3.46.  At N = 5 the FP32 pipe is 48%
-// (38%) busy, DRAM at 3.4 (2.7) TB/s; the copies alone take 0.19 (0.15) ms and
+// 0.401 / 0.394 -> 0.307 / 0.380, N = 3 0.341 / 0.353 -> 0.239 / 0.279, N = 1
+// 0.245 / 0.283 -> 0.205 / 0.221; L = 723, N = 6 0.229 / 0.240 -> 0.148 / 0.165;
+// L = 2048, N = 8 4.26 / 4.89 -> 2.92 / 3.49.  At N = 5 the FP32 pipe is 48%
+// (41%) busy, DRAM at 3.3 (2.7) TB/s; the copies alone take 0.19 (0.15) ms and
 // the sums without copies 0.27 ms: two warps per scheduler leave fixed
 // latencies exposed, more do not fit beside the accumulators.
 //

@@ -45,17 +45,18 @@
 // Images: no-swizzle K-major core matrices of 8 rows x 16 bytes (padding them
 // apart for conflict-free stores in the conversion made the products no faster
 // and the traffic larger).
-// What bounds it (L = 1000, N = 5, analysis beta, 249 us where the chirp-z took
+// What bounds it (L = 1000, N = 5, analysis beta, 248 us where the chirp-z took
 // 417): conversion 35 us; the products 133 us, 0.85 us per stage, near what
 // shared memory allows (it feeds each MMA 128 bytes per cycle and takes the
 // images at the same time: 164 KB per stage, 1280 cycles); the stores of X 80
-// us, half-filled sectors as a tile holds the columns of one parity.
+// us, half-filled sectors as a tile holds the columns of one parity.  The alpha
+// analysis spills 8 bytes per thread, the alpha synthesis 4.
 // Measured (GB300, us, analysis / synthesis, before -> now).  beta: L = 361, N =
-// 4 72 / 64 -> 31 / 33, L = 723, N = 6 337 / 320 -> 149 / 183, L = 1900, N = 4
-// 1834 / 1756 -> 912 / 1023, L = 2048, N = 8 2807 / 2991 -> 2144 / 2308, MW grid
-// L = 511, N = 3 91 / 280 -> 39 / 189; alpha of all scales above 32: L = 256, N =
-// 5 57 / 55 -> 33 / 29, L = 512, N = 3 102 / 98 -> 70 / 65, L = 723, N = 6 361 /
-// 411 -> 304 / 309, L = 1024, N = 5 512 / 540 -> 447 / 521.
+// 4, lambda = 3 72 / 64 -> 31 / 33, L = 723, N = 6 337 / 320 -> 152 / 184, L = 1900,
+// N = 4 1834 / 1756 -> 948 / 1050, L = 2048, N = 8 2807 / 2991 -> 2188 / 2330, MW
+// grid L = 511, N = 3 91 / 280 -> 39 / 179; alpha of all scales above 32: L = 256,
+// N = 5 57 / 55 -> 29 / 27, L = 512, N = 3 102 / 98 -> 66 / 64, L = 723, N = 6 361 /
+// 411 -> 283 / 309, L = 1024, N = 5 512 / 540 -> 401 / 495.
 // Every wait is bounded; a CTA that gives up stops all roles, and once they have
 // met waits for its MMAs and copies in flight (bounded), counts the event and
 // frees its TMEM.
